@@ -103,7 +103,17 @@ enum {
      *     256-column layers of a 2.4 M-node, 126 M-entry graph, bits and beta only: 4.9 / 5.2 ms for 3,
      *     5.7-5.9 / 5.9-6.1 ms for 1, 8.0 / 8.3 ms for 2.  All paths meet the same tolerance; their fp32 sums differ
      *     in rounding, so a re-binarized bit at the threshold may differ between them. */
-    BIGCN_OPT_BYTE_AGGREGATION = 4
+    BIGCN_OPT_BYTE_AGGREGATION = 4,
+    /* Order of a layer's two products, H' = A_tilde (diag(beta) F B diag(alpha)).
+     * 1 = the contraction F B first, then the aggregation of its rows (the kernels the options above choose among);
+     * 2 = the aggregation of the packed bits first, P = (A_tilde diag(beta)) F, then P B, both as exact integer products of
+     *     fixed-point weights; for d_out <= 256 and weights that fit shared memory (d_in <= 1280, or 640 above 128
+     *     columns), graphs of fewer than about 2^31 entries and rows, and a workspace of bigcn_workspace_bytes();
+     *     otherwise 1.  Edge values of either sign;
+     * 0 = default: whichever is expected to be the faster, by the sizes of the layer and the graph.
+     * A layer keeps to 1 when one of the options above is set or a debug tap is asked for.  Both orders meet the same
+     * tolerance; their fp32 sums differ in rounding. */
+    BIGCN_OPT_ORDER = 5
 };
 
 /* Context: binds a device and a stream.  `cuda_stream` is a cudaStream_t (0 = default stream). */

@@ -1,4 +1,5 @@
 // C ABI of libbigcn: contexts, argument validation, workspace carving and the launch sequences.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -21,6 +22,7 @@ struct bigcn_ctx {
     int zeta_format;             // 0 = auto
     int64_t long_row;            // 0 = default
     int contraction;             // 0 = auto, 1 = bit-count pipe, 2 = tensor cores wherever covered
+    int order;                   // 0 = the faster one, 1 = contraction first, 2 = aggregation first wherever covered
     int byte_path;               // aggregation of 129..256 byte columns: 0 / 1 = fp32 FMA stream, 2 = integer tensor-core products
     cudaEvent_t ev[2 * BIGCN_MAX_LAYERS + 2];
     bool ev_ready;
@@ -131,17 +133,60 @@ bigcn_status check_layer(bigcn_ctx* ctx, const bigcn_layer* l, const char* name)
     return BIGCN_OK;
 }
 
-// One layer on already validated arguments.  `zeta` is scratch for n * zeta_ld(d_out) elements.
+// Whether a layer aggregates the packed bits before the contraction (spmm_bits.cu), in `room` bytes of scratch.  Options that
+// name a storage format or a kernel of the other order, and the debug taps on the contraction, keep to that order.
+bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer, size_t room, bool bits_only, bool taps)
+{
+    return ctx->order != 1 && ctx->zeta_format == 0 && ctx->contraction == 0 && ctx->byte_path == 0 && ctx->long_row == 0 && !taps &&
+           spmm_bits_covers(g->n, g->nnz, layer->d_in, layer->d_out) &&
+           (ctx->order == 2 || spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out, bits_only)) &&
+           spmm_bits_scratch_bytes(g->n, g->nnz, layer->d_in) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
+}
+// The plan of the graph sits at the end of the scratch.
+void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
+{
+    return static_cast<char*>(scratch) + (room - spmm_bits_plan_bytes(g->n, g->nnz)) / kAlign * kAlign;
+}
+
+// One layer on already validated arguments.  `zeta` is `room` bytes of scratch: the contraction's rows in its first zbytes and
+// the aggregation's counter behind them, or (bits first) what spmm_bits_scratch_bytes() counts and the graph's plan, made here
+// unless `planned`.
 bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer,
-                       const uint32_t* in_bits, const float* in_beta, void* zeta, void* scratch,
+                       const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool planned,
                        float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,
                        float* next_beta, int32_t* dbg_dot, float* dbg_zeta,
                        cudaEvent_t ev_mid /*nullable*/)
 {
+    const int64_t stride_in = bigcn_packed_stride_words(layer->d_in);
+    if (bits_first(ctx, g, layer, room, h_out == nullptr, dbg_dot || dbg_zeta) && (!next || aligned(next_bits, 16))) {
+        if (ev_mid) BIGCN_CUDA(ctx, cudaEventRecord(ev_mid, ctx->stream));
+        SpmmArgs a = {};
+        a.n = g->n;
+        a.nnz = g->nnz;
+        a.rowptr = g->rowptr;
+        a.colidx = g->colidx;
+        a.val = g->val;
+        a.d_out = layer->d_out;
+        a.node_w = in_beta;
+        a.col_w = layer->alpha;
+        a.h_out = h_out;
+        a.ldh = ldh;
+        a.next_bits = next ? next_bits : nullptr;
+        a.next_stride = next ? bigcn_packed_stride_words(layer->d_out) : 0;
+        a.next_beta = next ? next_beta : nullptr;
+        a.next_shift = next ? next->in_shift : nullptr;
+        a.next_scale = next ? next->in_scale : nullptr;
+        a.scratch = zeta;
+        void* plan = plan_at(g, zeta, room);
+        cudaError_t e = planned ? cudaSuccess : launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
+        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, &ctx->launches_i);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
+        return BIGCN_OK;
+    }
+    void* const scratch = static_cast<char*>(zeta) + zbytes;
     const bool lane_stream = (next == nullptr && h_out != nullptr) || (next != nullptr && g->nnz >= 8 * g->n);
     const int fmt = pick_format(ctx, layer->d_in, layer->d_out, g->n, /*allow_half=*/true, /*narrow_bytes=*/lane_stream);
     const bool half = fmt == kZetaI8H;
-    const int64_t stride_in = bigcn_packed_stride_words(layer->d_in);
     // 33..60 byte columns for the lane-per-entry stream, on the tensor-core contraction: 64-byte rows that carry the node
     // factor in their last four bytes, so that the aggregation needs two lookups per entry, not four or five
     const bool row_tail = (fmt == kZetaI8 || half) && lane_stream && layer->d_out > 32 && layer->d_out <= 60 &&
@@ -202,6 +247,15 @@ size_t zeta_bytes_max(int64_t n, const int32_t* dims, int n_layers)
     return m;
 }
 
+// Scratch between the kernels of a layer, the larger of the two orders over all layers.
+size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers)
+{
+    size_t m = up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
+    for (int l = 0; l < n_layers; ++l)
+        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1])) m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]) + spmm_bits_plan_bytes(n, nnz) + kAlign);
+    return m;
+}
+
 // Bytes of a slot's input staging buffer: the fp32 features, or -- whichever is larger -- the packed input
 // (bits, then beta behind them at the next 256-byte boundary).
 size_t staging_in_bytes(int64_t n, int32_t d0)
@@ -228,15 +282,19 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     for (int l = 0; l < n_layers; ++l) dims[l + 1] = layers[l].d_out;
     int64_t stride_max = 0;
     for (int l = 0; l < n_layers; ++l) stride_max = stride_max > bigcn_packed_stride_words(dims[l]) ? stride_max : bigcn_packed_stride_words(dims[l]);
-    void* zeta = ws.take(zeta_bytes_max(n, dims, n_layers));
-    void* scratch = ws.take(spmm_scratch_bytes(n, graph->nnz, 0));
+    const size_t zbytes = up(zeta_bytes_max(n, dims, n_layers));
+    size_t others = 0;                                       // what else the step keeps
+    for (int i = 0; i < 2; ++i) others += up((size_t)n * stride_max * 4) + up((size_t)n * 4);
+    size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers);
+    if (up(ws.off) + room + others > ws.size) room = zbytes + up(spmm_scratch_bytes(n, graph->nnz, 0));   // a workspace without room for P
+    void* zeta = ws.take(room);
     uint32_t* bits[2];
     float* beta[2];
     for (int i = 0; i < 2; ++i) {
         bits[i] = static_cast<uint32_t*>(ws.take((size_t)n * stride_max * 4));
         beta[i] = static_cast<float*>(ws.take((size_t)n * 4));
     }
-    if (!zeta || !scratch || !bits[0] || !beta[0] || !bits[1] || !beta[1])
+    if (!zeta || !bits[0] || !beta[0] || !bits[1] || !beta[1])
         return fail(ctx, BIGCN_ERR_WORKSPACE, "workspace of %zu bytes is too small (see bigcn_workspace_bytes)", ws.size);
 
     cudaEvent_t* ev = ctx->ev;
@@ -250,11 +308,17 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
         cur_bits = bits[0];
         cur_beta = beta[0];
     }
+    bool planned = false;                                    // the layers share the graph's plan
+    for (int l = 0; l < n_layers && !planned; ++l) planned = bits_first(ctx, graph, &layers[l], room, l < n_layers - 1, false);
+    if (planned) {
+        cudaError_t e = launch_spmm_bits_plan(ctx->stream, n, graph->nnz, graph->rowptr, plan_at(graph, zeta, room), &ctx->launches_i);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");
+    }
     if (stats) BIGCN_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
     for (int l = 0; l < n_layers; ++l) {
         const bool last = (l == n_layers - 1);
         const int o = (l + 1) & 1;
-        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, scratch,
+        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, zbytes, room, planned,
                                     last ? logits_out : nullptr, ldo, last ? nullptr : &layers[l + 1],
                                     bits[o], beta[o], nullptr, nullptr, stats ? ev[2 + 2 * l] : nullptr);
         if (st != BIGCN_OK) return st;
@@ -374,6 +438,10 @@ bigcn_status bigcn_set_option(bigcn_ctx* ctx, int32_t option, int64_t value)
             if (value < 0 || value > 2) return fail(ctx, BIGCN_ERR_SHAPE, "contraction path %lld not in 0..2", (long long)value);
             ctx->contraction = (int)value;
             return BIGCN_OK;
+        case BIGCN_OPT_ORDER:
+            if (value < 0 || value > 2) return fail(ctx, BIGCN_ERR_SHAPE, "order %lld not in 0..2", (long long)value);
+            ctx->order = (int)value;
+            return BIGCN_OK;
         case BIGCN_OPT_BYTE_AGGREGATION:
             if (value < 0 || value > 3) return fail(ctx, BIGCN_ERR_SHAPE, "byte aggregation path %lld not in 0..3", (long long)value);
             ctx->byte_path = (int)value;
@@ -393,6 +461,7 @@ bigcn_status bigcn_sync_check(bigcn_ctx* ctx)
     if (bitgemm_tc_timeouts() != 0) return fail(ctx, BIGCN_ERR_INTERNAL, "a bounded wait on the tensor cores ran out (contraction kernel)");
     if (backward_tc_timeouts() != 0) return fail(ctx, BIGCN_ERR_INTERNAL, "a bounded wait on the tensor cores ran out (backward kernel)");
     if (spmm_tc_timeouts() != 0) return fail(ctx, BIGCN_ERR_INTERNAL, "a bounded wait ran out (tensor-core aggregation kernel)");
+    if (spmm_bits_timeouts() != 0) return fail(ctx, BIGCN_ERR_INTERNAL, "a bounded wait ran out (layer kernel on packed bits)");
     return BIGCN_OK;
 }
 
@@ -412,7 +481,7 @@ size_t bigcn_workspace_bytes(int64_t n, int64_t nnz, const int32_t* dims, int32_
         if (l < n_layers && bigcn_packed_stride_words(dims[l]) > stride_max) stride_max = bigcn_packed_stride_words(dims[l]);
         if (dims[l] > d_max) d_max = dims[l];
     }
-    size_t total = up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
+    size_t total = layer_scratch_bytes(n, nnz, dims, n_layers);
     total += 2 * (up((size_t)n * stride_max * 4) + up((size_t)n * 4));
     size_t aux = up(normalize_scratch_bytes(n));
     if (up(col_stats_scratch_bytes(d_max)) > aux) aux = up(col_stats_scratch_bytes(d_max));
@@ -557,7 +626,7 @@ bigcn_status bigcn_layer_forward(bigcn_ctx* ctx, const bigcn_graph* graph, const
     const size_t zbytes = up(zeta_bytes_max(graph->n, dims, 1));
     const size_t need = zbytes + up(spmm_scratch_bytes(graph->n, graph->nnz, layer->d_out));
     if (!ctx->ws || ctx->ws_bytes < need) return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace, has %zu", need, ctx->ws_bytes);
-    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, static_cast<char*>(ctx->ws) + zbytes, h_out, ldh, next, next_bits, next_beta,
+    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, zbytes, ctx->ws_bytes, false, h_out, ldh, next, next_bits, next_beta,
                    dbg_dot, dbg_zeta, nullptr);
     finish_call(ctx);
     return st;
@@ -951,25 +1020,16 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     cudaError_t e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out,
                                    in_beta, self_layer->alpha, kZetaF32, zeta_self, ld_self, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
     if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
-    const int fmt = pick_format(ctx, d_in, d_out, n);
-    const int64_t ldz = zeta_ld(d_out, fmt);
-    e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out,
-                       in_beta, nbr_layer->alpha, fmt, zeta_nbr, ldz, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
-    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (neighbour term) launch"); }
-    SpmmArgs a;
+    SpmmArgs a = {};
     a.n = n;
     a.nnz = mean_graph->nnz;
     a.rowptr = mean_graph->rowptr;
     a.colidx = mean_graph->colidx;
     a.val = mean_graph->val;
-    a.fmt = fmt;
-    a.zeta = zeta_nbr;
-    a.ldz = ldz;
     a.d_out = d_out;
     a.node_w = in_beta;
     a.col_w = nbr_layer->alpha;
     a.add = zeta_self;
-    a.byte_path = ctx->byte_path;
     a.ld_add = ld_self;
     a.h_out = h_out;
     a.ldh = ldh;
@@ -978,6 +1038,24 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.next_beta = next ? next_beta : nullptr;
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
+    if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, h_out == nullptr, false) && (!next || aligned(next_bits, 16))) {
+        a.scratch = zeta_nbr;
+        void* plan = plan_at(mean_graph, zeta_nbr, ctx->ws_bytes - zbytes);
+        e = launch_spmm_bits_plan(ctx->stream, n, mean_graph->nnz, mean_graph->rowptr, plan, &ctx->launches_i);
+        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, d_in, nbr_layer->w_bitsT, &ctx->launches_i);
+        finish_call(ctx);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
+        return BIGCN_OK;
+    }
+    const int fmt = pick_format(ctx, d_in, d_out, n);
+    const int64_t ldz = zeta_ld(d_out, fmt);
+    e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out,
+                       in_beta, nbr_layer->alpha, fmt, zeta_nbr, ldz, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
+    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (neighbour term) launch"); }
+    a.fmt = fmt;
+    a.zeta = zeta_nbr;
+    a.ldz = ldz;
+    a.byte_path = ctx->byte_path;
     a.long_row = ctx->long_row > 0 ? ctx->long_row : kDefaultLongRow;
     a.scratch = counter;
     a.scratch_bytes = spmm_scratch_bytes(n, mean_graph->nnz, d_out);

@@ -79,6 +79,19 @@ struct SpmmArgs {
 cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches);
 size_t spmm_scratch_bytes(int64_t n, int64_t nnz, int d_out);
 
+// A layer with the aggregation before the contraction, on the packed bits (spmm_bits.cu).  `plan` (spmm_bits_plan_bytes(), made by
+// launch_spmm_bits_plan() from the graph alone) serves any number of layers.  `a` as for launch_spmm(), its zeta fields
+// unused and a.scratch of spmm_bits_scratch_bytes(); stride: words per row of `bits` and of `w_bits`.
+bool spmm_bits_covers(int64_t n, int64_t nnz, int d_in, int d_out);
+// Whether this order of a layer is expected to be the faster one.
+bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out, bool bits_only);
+size_t spmm_bits_plan_bytes(int64_t n, int64_t nnz);
+cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rowptr, void* plan, int* launches);
+size_t spmm_bits_scratch_bytes(int64_t n, int64_t nnz, int d_in);
+cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan, const uint32_t* bits, int64_t stride, int d_in,
+                             const uint32_t* w_bits, int* launches);
+int spmm_bits_timeouts();
+
 cudaError_t launch_normalize_adjacency(cudaStream_t s, int64_t n, int64_t nnz_in,
                                        const int64_t* rowptr_A, const int32_t* colidx_A,
                                        int64_t* rowptr, int32_t* colidx, float* val, float* dinv,
