@@ -110,7 +110,8 @@ enum {
      *     fixed-point weights; for d_out <= 256 and weights that fit shared memory (d_in <= 1280, or 640 above 128
      *     columns), graphs of fewer than about 2^31 entries and rows, and a workspace of bigcn_workspace_bytes();
      *     otherwise 1.  Edge values of either sign;
-     * 0 = default: whichever is expected to be the faster, by the sizes of the layer and the graph.
+     * 0 = default: 2 for a launch that wants only the next layer's sign bits and beta, where the sizes of the layer and the
+     *     graph let it expect to be the faster; 1 otherwise.
      * A layer keeps to 1 when one of the options above is set or a debug tap is asked for.  Both orders meet the same
      * tolerance; their fp32 sums differ in rounding. */
     BIGCN_OPT_ORDER = 5

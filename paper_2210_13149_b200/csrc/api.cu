@@ -134,12 +134,13 @@ bigcn_status check_layer(bigcn_ctx* ctx, const bigcn_layer* l, const char* name)
 }
 
 // Whether a layer aggregates the packed bits before the contraction (spmm_bits.cu), in `room` bytes of scratch.  Options that
-// name a storage format or a kernel of the other order, and the debug taps on the contraction, keep to that order.
-bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer, size_t room, bool bits_only, bool taps)
+// name a storage format or a kernel of the other order, and the debug taps on the contraction, keep to that order; so does
+// by default a launch that writes H' in fp32 (not bits_only), whose values then round as they always did.
+bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer, size_t room, bool bits_only, bool taps, bool own = false)
 {
     return ctx->order != 1 && ctx->zeta_format == 0 && ctx->contraction == 0 && ctx->byte_path == 0 && ctx->long_row == 0 && !taps &&
-           spmm_bits_covers(g->n, g->nnz, layer->d_in, layer->d_out) &&
-           (ctx->order == 2 || spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out, bits_only)) &&
+           spmm_bits_covers(g->n, g->nnz, layer->d_in, layer->d_out, own) &&
+           (ctx->order == 2 || (bits_only && spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out))) &&
            spmm_bits_scratch_bytes(g->n, g->nnz, layer->d_in) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
 }
 // The plan of the graph sits at the end of the scratch.
@@ -179,7 +180,7 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
         a.scratch = zeta;
         void* plan = plan_at(g, zeta, room);
         cudaError_t e = planned ? cudaSuccess : launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
-        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, &ctx->launches_i);
+        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, nullptr, &ctx->launches_i);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
@@ -252,7 +253,7 @@ size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_la
 {
     size_t m = up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
     for (int l = 0; l < n_layers; ++l)
-        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1])) m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]) + spmm_bits_plan_bytes(n, nnz) + kAlign);
+        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]) + spmm_bits_plan_bytes(n, nnz) + kAlign);
     return m;
 }
 
@@ -1016,10 +1017,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     void* zeta_nbr = base + zbytes;
     void* counter = base + 2 * zbytes;
     const int64_t stride_in = bigcn_packed_stride_words(d_in);
-    const int64_t ld_self = zeta_ld(d_out, kZetaF32);
-    cudaError_t e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out,
-                                   in_beta, self_layer->alpha, kZetaF32, zeta_self, ld_self, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
-    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
+    cudaError_t e;
     SpmmArgs a = {};
     a.n = n;
     a.nnz = mean_graph->nnz;
@@ -1029,8 +1027,6 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.d_out = d_out;
     a.node_w = in_beta;
     a.col_w = nbr_layer->alpha;
-    a.add = zeta_self;
-    a.ld_add = ld_self;
     a.h_out = h_out;
     a.ldh = ldh;
     a.next_bits = next ? next_bits : nullptr;
@@ -1038,15 +1034,24 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.next_beta = next ? next_beta : nullptr;
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
-    if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, h_out == nullptr, false) && (!next || aligned(next_bits, 16))) {
+    if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, h_out == nullptr, false, /*own=*/true) && (!next || aligned(next_bits, 16))) {
+        const OwnTerm own = {reinterpret_cast<const int16_t*>(base), zeta_ld(d_out, kZetaI16), self_layer->alpha};
         a.scratch = zeta_nbr;
         void* plan = plan_at(mean_graph, zeta_nbr, ctx->ws_bytes - zbytes);
-        e = launch_spmm_bits_plan(ctx->stream, n, mean_graph->nnz, mean_graph->rowptr, plan, &ctx->launches_i);
-        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, d_in, nbr_layer->w_bitsT, &ctx->launches_i);
+        e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, self_layer->alpha,
+                           kZetaI16, base, own.ld, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
+        if (e == cudaSuccess) e = launch_spmm_bits_plan(ctx->stream, n, mean_graph->nnz, mean_graph->rowptr, plan, &ctx->launches_i);
+        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, d_in, nbr_layer->w_bitsT, &own, &ctx->launches_i);
         finish_call(ctx);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
+    const int64_t ld_self = zeta_ld(d_out, kZetaF32);
+    e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out,
+                                   in_beta, self_layer->alpha, kZetaF32, zeta_self, ld_self, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
+    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
+    a.add = zeta_self;
+    a.ld_add = ld_self;
     const int fmt = pick_format(ctx, d_in, d_out, n);
     const int64_t ldz = zeta_ld(d_out, fmt);
     e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out,

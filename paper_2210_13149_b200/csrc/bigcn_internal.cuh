@@ -82,14 +82,21 @@ size_t spmm_scratch_bytes(int64_t n, int64_t nnz, int d_out);
 // A layer with the aggregation before the contraction, on the packed bits (spmm_bits.cu).  `plan` (spmm_bits_plan_bytes(), made by
 // launch_spmm_bits_plan() from the graph alone) serves any number of layers.  `a` as for launch_spmm(), its zeta fields
 // unused and a.scratch of spmm_bits_scratch_bytes(); stride: words per row of `bits` and of `w_bits`.
-bool spmm_bits_covers(int64_t n, int64_t nnz, int d_in, int d_out);
+// `own`: a term of the node itself (Bi-GraphSAGE) is added: beta_i alpha_j dot_ij, its dots as rows of ld (a multiple of 8)
+// 16-bit integers.
+struct OwnTerm {
+    const int16_t* dots;
+    int64_t ld;
+    const float* alpha;
+};
+bool spmm_bits_covers(int64_t n, int64_t nnz, int d_in, int d_out, bool own);
 // Whether this order of a layer is expected to be the faster one.
-bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out, bool bits_only);
+bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out);
 size_t spmm_bits_plan_bytes(int64_t n, int64_t nnz);
 cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rowptr, void* plan, int* launches);
 size_t spmm_bits_scratch_bytes(int64_t n, int64_t nnz, int d_in);
 cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan, const uint32_t* bits, int64_t stride, int d_in,
-                             const uint32_t* w_bits, int* launches);
+                             const uint32_t* w_bits, const OwnTerm* own, int* launches);
 int spmm_bits_timeouts();
 
 cudaError_t launch_normalize_adjacency(cudaStream_t s, int64_t n, int64_t nnz_in,

@@ -537,13 +537,15 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
 // ---- P B diag(alpha) -----------------------------------------------------------------------------------------------
 
 constexpr int kGemmStages = 3;
+constexpr int kOwnElts = 2 * kTileRows * 256;       // two tiles of up to 256 columns or four of up to 128
 constexpr int kEpiGroups = 4;                       // warpgroups that read accumulators back
 constexpr int kGemmThreads = 128 * kEpiGroups + 64; // + a copying and an issuing warp
 constexpr int kTries = 1 << 20;                     // bound of every wait: tries of up to 1 us
 
 struct GemmMisc {
     uint64_t full[kGemmStages], empty[kGemmStages];
-    uint64_t acc_full[4], acc_empty[4];
+    uint64_t acc_full[4], acc_empty[4], own_full[4];
+    alignas(16) float rows[16][2][kTileRows];       // per epilogue warp: row scales of the tile, and the nodes' own factors
     uint32_t tmem;
     int abort;
     alignas(16) uint32_t words[2][4][kTileRows][4]; // by turn, warpgroup: packed words of 32 rows, one per warp
@@ -573,6 +575,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
+// Waits for a copy of this thread's own before the block ends (bounded; at once unless the block gave up).
+__device__ __forceinline__ void wait_landed(uint64_t* bar, uint32_t parity)
+{
+    uint32_t done = 0;
+    for (int it = 0; it < kTries && !done; ++it)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, 1000;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+}
+__device__ __forceinline__ void copy_bulk(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
 struct GemmDev {
     const uint8_t* p;
     int n_kc, d_in;
@@ -580,10 +597,17 @@ struct GemmDev {
     const uint32_t* w_bits;
     int w_stride;
     int tiles;
+    const int16_t* own;                             // kOwn: the nodes' own dots, rows of own_ld
+    int own_ld;
+    const float* own_alpha;
+    const float* own_beta;
 };
 
 // NM: blocks of 128 output columns.  Accumulators: 4 / NM tiles in tensor memory, each with a warpgroup per block of columns.
-template <int NM, bool kBitsOnly>
+// kOwn (Bi-GraphSAGE): the node's own term, beta_i alpha_j dot_ij, is added to the row.  Its dots come as 16-bit integers by bulk
+// copies, a tile ahead of their use; read from fp32 rows by the epilogue itself, the latency of each read bounded the
+// kernel (2.4 M rows of 256 columns: 4.9 ms against 0.9 ms without the term).
+template <int NM, bool kBitsOnly, bool kOwn>
 __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDev p, const GemmDev d)
 {
     constexpr int kAcc = 4 / NM;
@@ -591,7 +615,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
     unsigned char* sm = gemm_raw + ((1024u - (smem_u32(gemm_raw) & 1023u)) & 1023u);
     unsigned char* stages = sm;                                       // kGemmStages x kTileChunk
     unsigned char* a_op = stages + kGemmStages * kTileChunk;          // NM x [128 x 128 n_kc]
-    GemmMisc* m = reinterpret_cast<GemmMisc*>(a_op + NM * 128 * 128 * d.n_kc);
+    int16_t* own_s = reinterpret_cast<int16_t*>(a_op + NM * 128 * 128 * d.n_kc);      // kAcc x [32 x own_ld]
+    GemmMisc* m = reinterpret_cast<GemmMisc*>(own_s + (kOwn ? kOwnElts : 0));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort = &m->abort;
     if (warp == 0) tc::tmem_alloc(&m->tmem, 512);
@@ -603,6 +628,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
         for (int i = 0; i < 4; ++i) {
             mbar_init(&m->acc_full[i], 1);
             mbar_init(&m->acc_empty[i], 4 * NM);
+            mbar_init(&m->own_full[i], 1);
         }
         m->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -643,22 +669,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                     const int st = s % kGemmStages;
                     if (s >= kGemmStages) ok = mbar_wait(&m->empty[st], (uint32_t)(s / kGemmStages + 1) & 1u, abort);
                     if (!ok) break;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(&m->full[st])), "r"(kTileChunk) : "memory");
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                                 ::"r"(smem_u32(stages + st * kTileChunk)), "l"(src + (int64_t)kc * kTileChunk), "r"(kTileChunk), "r"(smem_u32(&m->full[st])) : "memory");
+                    copy_bulk(smem_u32(stages + st * kTileChunk), src + (int64_t)kc * kTileChunk, kTileChunk, &m->full[st]);
                 }
                 if (!ok) break;
             }
+            for (int q = max(0, s - kGemmStages); q < s; ++q) wait_landed(&m->full[q % kGemmStages], (uint32_t)(q / kGemmStages) & 1u);
         }
     } else if (warp == 4 * kEpiGroups + 1) {                          // products
         if (lane == 0) {
             // D = s32, A = B = s8, both K-major, N = 128, M = 128
             const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
             const uint32_t a_base = smem_u32(a_op), s_base = smem_u32(stages);
-            int s = 0;
-            for (int i = 0; i < my_tiles; ++i) {
+            int s = 0, i = 0;
+            for (; i < my_tiles; ++i) {
                 const int acc = i % kAcc;
                 if (i >= kAcc && !mbar_wait(&m->acc_empty[acc], (uint32_t)(i / kAcc + 1) & 1u, abort)) break;
+                if constexpr (kOwn) {
+                    const int64_t r0 = (int64_t)(blockIdx.x + i * gridDim.x) * kTileRows;
+                    const uint32_t bytes = (uint32_t)min((int64_t)kTileRows, p.n - r0) * (uint32_t)(2 * d.own_ld);
+                    copy_bulk(smem_u32(own_s + acc * kTileRows * d.own_ld), d.own + r0 * d.own_ld, bytes, &m->own_full[acc]);
+                }
                 bool ok = true;
                 for (int kc = 0; kc < d.n_kc; ++kc, ++s) {
                     const int st = s % kGemmStages;
@@ -677,18 +707,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                 if (!ok) break;
                 tc::commit_to(&m->acc_full[acc]);
             }
+            if constexpr (kOwn)
+                for (int q = max(0, i + 1 - kAcc); q < min(i + 1, my_tiles); ++q) wait_landed(&m->own_full[q % kAcc], (uint32_t)(q / kAcc) & 1u);
         }
     } else {                                                          // epilogue
         const int wg = warp >> 2, wq = warp & 3, h = wg % NM, acc = wg / NM;
         const int ch = 128 * h + 32 * wq + lane;
         const bool in = ch < p.d_out;
         const float alpha = in ? __ldg(p.col_w + ch) : 0.f;
+        const float own_alpha = kOwn && in ? __ldg(d.own_alpha + ch) : 0.f;
         const float shift = (in && p.next_shift) ? __ldg(p.next_shift + ch) : 0.f;
         const float scale = in ? (p.next_shift ? __ldg(p.next_scale + ch) : 1.f) : 0.f;   // 0: columns that do not exist add nothing to beta
         const uint32_t t_addr = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)((acc * NM + h) * 128);
         for (int i = acc; i < my_tiles; i += kAcc) {
             const int row0 = (int)(blockIdx.x + i * gridDim.x) * kTileRows, turn = (i / kAcc) & 1;
+            const int my_row = (int)min((int64_t)row0 + lane, p.n - 1);
+            m->rows[warp][0][lane] = __ldg(d.row_scale + my_row);
+            if constexpr (kOwn) m->rows[warp][1][lane] = __ldg(d.own_beta + my_row);
+            __syncwarp();
             if (!mbar_wait(&m->acc_full[acc], (uint32_t)(i / kAcc) & 1u, abort)) break;
+            if constexpr (kOwn) {
+                if (!mbar_wait(&m->own_full[acc], (uint32_t)(i / kAcc) & 1u, abort)) break;
+            }
+            const int16_t* own = own_s + acc * kTileRows * d.own_ld + ch;
             tc::fence_after_sync();
             uint32_t word = 0u;
             float l1_row = 0.f;                                       // lane r: the warp's sum of |x| over row r
@@ -697,18 +738,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                 uint32_t v[16];
                 tc::tmem_ld16(t_addr + (uint32_t)(rb * 16), v);
                 float l1[4];
-                const float4 rs4 = __ldg(reinterpret_cast<const float4*>(d.row_scale + row0 + 4 * rb));
+                const float4 rs4 = *reinterpret_cast<const float4*>(&m->rows[warp][0][4 * rb]);
                 const float rs[4] = {rs4.x, rs4.y, rs4.z, rs4.w};
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const int lo = (int)v[4 * r] + ((int)v[4 * r + 1] << 8), hi = (int)v[4 * r + 2] + ((int)v[4 * r + 3] << 8);
                     float x = fmaf((float)hi, 65536.f, (float)lo) * (rs[r] * alpha);
+                    if constexpr (kOwn) {
+                        if (in) x += __fmul_rn(__fmul_rn(m->rows[warp][1][4 * rb + r], own_alpha), (float)own[(4 * rb + r) * d.own_ld]);
+                    }
                     if constexpr (!kBitsOnly) {
                         const int row = row0 + 4 * rb + r;
-                        if (row < p.n && in) {
-                            if (p.add) x += __ldg(p.add + (int64_t)row * p.ld_add + ch);
-                            if (p.h_out) p.h_out[(int64_t)row * p.ldh + ch] = x;
-                        }
+                        if (row < p.n && in && p.h_out) p.h_out[(int64_t)row * p.ldh + ch] = x;
                     }
                     const float xh = __fmul_rn(__fsub_rn(x, shift), scale);
                     const uint32_t b = __ballot_sync(0xffffffffu, in && xh >= 0.f);
@@ -726,7 +767,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                 }
             }
             tc::fence_before_sync();
-            __syncwarp();
+            __syncwarp();                                             // (also: rows[] is written again for the next tile)
             if (lane == 0) mbar_arrive(&m->acc_empty[acc]);
             if (kBitsOnly || p.next_bits) {
                 m->words[turn][wg][lane][wq] = word;
@@ -748,7 +789,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
     if (warp == 0) tc::tmem_free(m->tmem, 512);
 }
 
-int gemm_smem(int nm, int n_kc) { return kGemmStages * kTileChunk + nm * 128 * 128 * n_kc + (int)sizeof(GemmMisc) + 1024; }
+int gemm_smem(int nm, int n_kc, bool own) { return kGemmStages * kTileChunk + nm * 128 * 128 * n_kc + (own ? kOwnElts * 2 : 0) + (int)sizeof(GemmMisc) + 1024; }
 
 // How the work of agg_bits_kernel is split, and the scratch of a layer.
 constexpr int kUnitsWanted = 4 * 16 * 148;           // four units for every warp that a B200 holds
@@ -789,35 +830,39 @@ Plan make_plan(int64_t n, int64_t nnz, int d_in)
 
 }  // namespace
 
-bool spmm_bits_covers(int64_t n, int64_t nnz, int d_in, int d_out)
+bool spmm_bits_covers(int64_t n, int64_t nnz, int d_in, int d_out, bool own)
 {
     const int64_t row_bytes = round_up(ceil_div(d_in, 32), 4) * 4;
     return d_out <= 256 && n * row_bytes < (int64_t(1) << 32) && nnz + kRowCost * (n + 2) < (int64_t(1) << 31) - 4096 &&
-           gemm_smem(d_out > 128 ? 2 : 1, (int)ceil_div(d_in, 128)) <= 227 * 1024;
+           gemm_smem(d_out > 128 ? 2 : 1, (int)ceil_div(d_in, 128), own) <= 227 * 1024;
 }
 
-// Predicted picoseconds on one B200, fitted to both orders' layers of d_in 64..602, d_out 16..256 on graphs of 3,000 to
-// 1,000,000 nodes with 4 to 500 entries a row (spread of the measurements about the model: 20 %).  This order pays per
-// stored entry and input column and, above all, per row (the read-back of P and the second kernel); the other per stored
-// entry and output column: this one is the better for long rows and wide outputs (256 -> 256 on 28 M entries in rows of
-// 490: 0.51 against 1.13 ms), the other for short rows and narrow outputs (256 -> 47 in rows of 5: 0.97 against 0.48 ms).
-bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out, bool bits_only)
+// Predicted picoseconds on one B200, fitted to hidden layers (bits and beta wanted) of d_in 64..602, d_out 16..256 on graphs of
+// 20,000 to 2,400,000 nodes with 4 to 490 entries a row; the model is within 15 % of nearly all of them.  This order pays
+// per stored entry and input column and, above all, per row (the read-back of P and the second kernel); the other per
+// stored entry and output column.  So this one is the better for long rows and wide outputs (256 -> 256, 28 M entries in
+// rows of 490: 0.56 against 1.12 ms), the other for short rows (256 -> 256, 2.6 M entries in rows of 15: 0.30 against 0.21 ms).
+bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out)
 {
+    if (d_out <= 32) return false;                   // level at best
     const int full = d_in / 256 + (d_in % 256 > 128 ? 1 : 0), rest = d_in % 256 > 128 ? 0 : d_in % 256;
-    const double here_entry = 17.5 * full + (rest == 0 ? 0.0 : (rest > 64 ? 12.5 : 11.3));
-    const double here_row = 850.0 * full + (rest == 0 ? 0.0 : 550.0) + (d_out > 128 ? 120.0 : 0.0) + (bits_only ? 0.0 : 0.6 * d_out);
+    const double here_entry = 15.0 * full + (rest == 0 ? 0.0 : (rest > 64 ? 10.0 : 8.0));
+    const double here_row = 800.0 * full + (rest == 0 ? 0.0 : 520.0) + (d_out > 128 ? 230.0 : 0.0);
     double there_entry, there_row;
-    if (d_out > 128) {
-        there_entry = d_in > 256 ? 56.0 : (bits_only ? 38.0 : 48.0);
-        there_row = d_in > 256 ? 1200.0 : 700.0;
+    if (d_out > 128 && d_in > 256) {                 // fp16 rows, in the L2 or not
+        there_entry = (double)n * d_out * 2 <= 125e6 ? 48.0 : 63.0;
+        there_row = 1100.0;
+    } else if (d_out > 128) {
+        there_entry = 32.0;
+        there_row = nnz >= 8 * n ? 550.0 : 800.0;
     } else if (d_out > 64) {
-        there_entry = 45.0;
-        there_row = d_in > 256 ? 700.0 : 300.0;
+        there_entry = 36.0;
+        there_row = d_in > 256 ? 720.0 : 290.0;
     } else {
-        there_entry = d_out > 32 ? (d_in > 256 ? 27.0 : 20.0) : 12.5;
-        there_row = d_in > 256 ? 500.0 : 360.0;
+        there_entry = d_in > 256 ? 24.0 : 15.0;
+        there_row = d_in > 256 ? 500.0 : 680.0;
     }
-    return 25e6 + here_entry * nnz + here_row * n < there_entry * nnz + there_row * n;
+    return 65e6 + here_entry * nnz + here_row * n < 0.95 * (10e6 + there_entry * nnz + there_row * n);
 }
 
 size_t spmm_bits_plan_bytes(int64_t n, int64_t nnz) { return make_plan(n, nnz, 1).graph_bytes(); }
@@ -838,7 +883,7 @@ cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const 
 }
 
 cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan, const uint32_t* bits, int64_t stride, int d_in,
-                             const uint32_t* w_bits, int* launches)
+                             const uint32_t* w_bits, const OwnTerm* own, int* launches)
 {
     if (a.n == 0) return cudaSuccess;
     const Plan pl = make_plan(a.n, a.nnz, d_in);
@@ -890,8 +935,6 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
     p.n = a.n;
     p.d_out = a.d_out;
     p.col_w = a.col_w;
-    p.add = a.add;
-    p.ld_add = a.ld_add;
     p.h_out = a.h_out;
     p.ldh = a.ldh;
     p.next_bits = a.next_bits;
@@ -908,9 +951,13 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
     d.w_bits = w_bits;
     d.w_stride = (int)stride;
     d.tiles = (int)ceil_div(a.n, kTileRows);
+    d.own = own ? own->dots : nullptr;
+    d.own_ld = own ? (int)own->ld : 0;
+    d.own_alpha = own ? own->alpha : nullptr;
+    d.own_beta = a.node_w;
     const int nm = a.d_out > 128 ? 2 : 1;
-    const int smem = gemm_smem(nm, pl.n_kc);
-    const bool bits_only = p.next_bits && !p.h_out && !p.add;
+    const int smem = gemm_smem(nm, pl.n_kc, own != nullptr);
+    const bool bits_only = p.next_bits && !p.h_out;
     auto gemm = [&](auto kernel) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (err != cudaSuccess) return err;
@@ -918,8 +965,12 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
         if (launches) ++*launches;
         return cudaGetLastError();
     };
-    if (nm == 2) return bits_only ? gemm(bits_gemm_kernel<2, true>) : gemm(bits_gemm_kernel<2, false>);
-    return bits_only ? gemm(bits_gemm_kernel<1, true>) : gemm(bits_gemm_kernel<1, false>);
+    if (own) {
+        if (nm == 2) return bits_only ? gemm(bits_gemm_kernel<2, true, true>) : gemm(bits_gemm_kernel<2, false, true>);
+        return bits_only ? gemm(bits_gemm_kernel<1, true, true>) : gemm(bits_gemm_kernel<1, false, true>);
+    }
+    if (nm == 2) return bits_only ? gemm(bits_gemm_kernel<2, true, false>) : gemm(bits_gemm_kernel<2, false, false>);
+    return bits_only ? gemm(bits_gemm_kernel<1, true, false>) : gemm(bits_gemm_kernel<1, false, false>);
 }
 
 int spmm_bits_timeouts()

@@ -75,3 +75,20 @@ def test_bits_first_signed_edge_values_of_wide_range(ctx, n, e, span):
     wmax = np.maximum.reduceat(w, g.rowptr[:-1].astype(np.int64))
     unit = np.where(deg <= 128, 2.0 ** -22 * wmax, 2.0 ** -26 * wmax) * deg + 2.0 ** -21 * wsum
     assert np.all(np.abs(out["h"].cpu().numpy() - t.H_out) <= unit[:, None] * d_in * np.abs(t.alpha)[None, :] + 1e-30)
+
+
+# the node's own term: one and several tiles, mostly empty rows, one and two blocks of 128 output columns, more tiles than
+# a block's buffers hold
+@pytest.mark.parametrize("n,e,d_in,d_out", [(1, 0, 5, 1), (33, 60, 64, 7), (300, 200, 64, 200), (500, 6000, 300, 129),
+                                             (4200, 50000, 127, 256), (30000, 60000, 40, 128)])
+def test_bits_first_sage_layer(ctx, n, e, d_in, d_out):
+    from paper_2210_13149_b200 import binding as B
+    from test_gpu_sage import check_sage_layer
+    check_sage_layer(ctx, 0, n, e, d_in, d_out)
+    rng = np.random.default_rng(n)
+    G = ctx.mean_adjacency(*(t.cuda() for t in synth.power_law_graph(n, e, 3)))
+    own, nbr = ctx.prepare_layers([dev((rng.standard_normal((d_in, d_out)) * d_in ** -0.5).astype(np.float32)) for _ in range(2)])
+    nxt = B.make_layer(d_out, 1, torch.zeros((1, 16), dtype=torch.int32, device="cuda"), dev(np.ones(1, np.float32)))
+    bits, beta = ctx.pack_features(dev(rng.standard_normal((n, d_in)).astype(np.float32)))
+    both, only = (ctx.sage_layer_forward(G, own, nbr, bits, beta, want_h=h, next_layer=nxt) for h in (True, False))
+    assert torch.equal(both["next_bits"], only["next_bits"]) and torch.equal(both["next_beta"], only["next_beta"])
