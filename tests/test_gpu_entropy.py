@@ -50,6 +50,12 @@ def test_entropy_bins_matches_oracle(ctx, n, d, M):
     check(ctx, activations(n, d, n * 31 + d), M)
 
 
+@pytest.mark.parametrize("M", [1750, 1751, 3500, 3501, 7000, 7001])
+@pytest.mark.parametrize("n,d", [(1023, 33), (9001, 31)])
+def test_entropy_bins_at_the_ends_of_every_strip_width(ctx, n, d, M):
+    check(ctx, activations(n, d, n + M), M)
+
+
 def test_entropy_bins_strided_rows_and_repeat(ctx):
     rng = np.random.default_rng(3)
     buf = rng.standard_normal((5000, 40)).astype(np.float32)
