@@ -13,15 +13,15 @@ namespace {
 
 constexpr int kGemmThreads = 256;
 constexpr int kGemmWarps = kGemmThreads / kWarp;
-constexpr int kRowsPerWarp = 8;
-constexpr int kTileRows = kGemmWarps * kRowsPerWarp;   // 64 rows of A per tile
-constexpr int kTM = 4;                                  // rows held in registers at a time
 
 // Shared memory: the packed weight panel of this channel block (row pitch ldb words, odd, so that
 // the 32 lanes of a warp - 32 consecutive channels - hit 32 different banks) and one tile of packed
 // feature rows (read as warp-wide broadcasts).  Each lane owns channels lane, lane+32, ... (TN of
-// them) and kTM rows at a time: kTM x TN integer accumulators of popc(a XOR b).
-template <int TN, int FMT, bool DBG>
+// them) and kTM rows at a time: kTM x TN integer accumulators of popc(a XOR b).  The panel is read 16 bytes at a time: word
+// by word, its 116 words x 64 rows took longer than the products of a small graph.
+// RW: rows a warp takes of a tile: 8, or 2 on graphs so small that tiles of 64 rows would leave multiprocessors without work
+// (3,327 rows, 3,703 -> 64: 32 us on 52 blocks).
+template <int TN, int FMT, bool DBG, int RW>
 __global__ void __launch_bounds__(kGemmThreads)
 bitgemm_kernel(const uint32_t* __restrict__ A, int64_t stride_a,
                const uint32_t* __restrict__ BT, int64_t stride_b,
@@ -30,6 +30,7 @@ bitgemm_kernel(const uint32_t* __restrict__ A, int64_t stride_a,
                void* __restrict__ zeta, int64_t ldz,
                int32_t* __restrict__ dbg_dot, float* __restrict__ dbg_zeta)
 {
+    constexpr int kTM = RW < 4 ? RW : 4, kRowsPerWarp = RW, kTileRows = RW * kGemmWarps;
     extern __shared__ __align__(16) uint32_t smem[];
     uint32_t* Bs = smem;                                   // [TN*32][ldb]
     uint32_t* As = smem + (size_t)TN * 32 * ldb;           // [kTileRows][stride_a]  (16-byte aligned: see launcher)
@@ -37,10 +38,16 @@ bitgemm_kernel(const uint32_t* __restrict__ A, int64_t stride_a,
     const int warp = threadIdx.x >> 5;
     const int jblock = blockIdx.y * (TN * 32);
 
-    for (int idx = threadIdx.x; idx < TN * 32 * kw; idx += kGemmThreads) {
-        const int c = idx / kw, k = idx - c * kw;
+    const int kq = (int)(stride_b >> 2);                   // 16-byte pieces per packed row (words past kw are not stored)
+    for (int idx = threadIdx.x; idx < TN * 32 * kq; idx += kGemmThreads) {
+        const int c = idx / kq, k = 4 * (idx - c * kq);
         const int j = jblock + c;
-        Bs[c * ldb + k] = (j < d_out) ? __ldg(BT + (int64_t)j * stride_b + k) : 0u;
+        const uint4 v = (j < d_out) ? __ldg(reinterpret_cast<const uint4*>(BT + (int64_t)j * stride_b + k)) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t* dst = Bs + c * ldb + k;
+        dst[0] = v.x;
+        if (k + 1 < ldb) dst[1] = v.y;
+        if (k + 2 < ldb) dst[2] = v.z;
+        if (k + 3 < ldb) dst[3] = v.w;
     }
     float al[TN];
 #pragma unroll
@@ -126,22 +133,23 @@ bitgemm_kernel(const uint32_t* __restrict__ A, int64_t stride_a,
     }
 }
 
-template <int TN, int FMT, bool DBG>
+template <int TN, int FMT, bool DBG, int RW>
 cudaError_t launch_inst(cudaStream_t s, const uint32_t* A, int64_t stride_a, const uint32_t* BT,
                         int64_t stride_b, int64_t n, int d_in, int d_out, const float* beta,
                         const float* alpha, void* zeta, int64_t ldz, int32_t* dbg_dot,
                         float* dbg_zeta, size_t smem_bytes, int ldb)
 {
     const int kw = (d_in + 31) / 32;
+    smem_bytes -= (size_t)(8 - RW) * kGemmWarps * stride_a * 4;
     if (smem_bytes > 48 * 1024) {                          // opt in to large dynamic shared memory
-        cudaError_t e = cudaFuncSetAttribute(bitgemm_kernel<TN, FMT, DBG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(bitgemm_kernel<TN, FMT, DBG, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem_bytes);
         if (e != cudaSuccess) return e;
     }
-    const int64_t n_tiles = ceil_div(n, kTileRows);
+    const int64_t n_tiles = ceil_div(n, RW * kGemmWarps);
     const unsigned gy = (unsigned)ceil_div(d_out, TN * 32);
     const unsigned gx = (unsigned)std::min<int64_t>(n_tiles, sm_count() * 8);
-    bitgemm_kernel<TN, FMT, DBG><<<dim3(gx, gy), kGemmThreads, smem_bytes, s>>>(
+    bitgemm_kernel<TN, FMT, DBG, RW><<<dim3(gx, gy), kGemmThreads, smem_bytes, s>>>(
         A, stride_a, BT, stride_b, n, d_in, d_out, kw, ldb, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta);
     return cudaGetLastError();
 }
@@ -152,8 +160,10 @@ cudaError_t launch_tn(cudaStream_t s, const uint32_t* A, int64_t stride_a, const
                       const float* alpha, int fmt, void* zeta, int64_t ldz, int32_t* dbg_dot,
                       float* dbg_zeta, size_t smem_bytes, int ldb)
 {
+    const bool small = ceil_div(n, 8 * kGemmWarps) * ceil_div(d_out, TN * 32) < 2 * sm_count();
 #define BIGCN_GEMM_CALL(FMT, DBG) \
-    launch_inst<TN, FMT, DBG>(s, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, smem_bytes, ldb)
+    (small ? launch_inst<TN, FMT, DBG, 2>(s, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, smem_bytes, ldb) \
+           : launch_inst<TN, FMT, DBG, 8>(s, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, smem_bytes, ldb))
     const bool dbg = dbg_dot || dbg_zeta;
     switch (fmt) {
         case kZetaF32: return dbg ? BIGCN_GEMM_CALL(kZetaF32, true) : BIGCN_GEMM_CALL(kZetaF32, false);
@@ -198,7 +208,7 @@ cudaError_t launch_bitgemm(cudaStream_t s, const uint32_t* A, int64_t stride_a,
     while (tn > 1 && tn * 16 >= d_out) tn >>= 1;           // smallest power of two with tn*32 >= d_out (max 8)
     auto bytes = [&](int t) {
         // the A tile starts at a 16-byte boundary: the panel size is rounded up to 4 words
-        return (size_t)(round_up((int64_t)t * 32 * ldb, 4) + (int64_t)kTileRows * stride_a) * 4;
+        return (size_t)(round_up((int64_t)t * 32 * ldb, 4) + (int64_t)(8 * kGemmWarps) * stride_a) * 4;
     };
     while (tn > 1 && bytes(tn) > 200 * 1024) tn >>= 1;
     if (bytes(tn) > 200 * 1024) return cudaErrorInvalidConfiguration;

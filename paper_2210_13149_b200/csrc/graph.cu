@@ -184,6 +184,7 @@ col_partial_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, in
     double s = 0.0, q = 0.0;
     if (j < d) {
         const double pivot = (double)__ldg(H + j);
+#pragma unroll 8
         for (int64_t r = r0 + ty; r < r1; r += 8) {
             const double x = (double)__ldg(H + r * ld + j) - pivot;
             s += x;
@@ -201,15 +202,32 @@ col_partial_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, in
     }
 }
 
-__global__ void col_final_kernel(const float* __restrict__ H, const double* __restrict__ partial, int chunks, int d, int64_t n, double eps,
-                                 float* __restrict__ shift, float* __restrict__ scale)
+// A block per 32 columns; thread (tx, ty) adds chunks ty, ty + 32, ... of column tx, the 32 sums are added in order.  (A
+// thread per column walked through all chunks alone: 18 us for 78 chunks.)
+__global__ void __launch_bounds__(1024)
+col_final_kernel(const float* __restrict__ H, const double* __restrict__ partial, int chunks, int d, int64_t n, double eps,
+                 float* __restrict__ shift, float* __restrict__ scale)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
+    __shared__ double s_sum[32][33], s_sq[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int j = blockIdx.x * 32 + tx;
     double s = 0.0, q = 0.0;
-    for (int c = 0; c < chunks; ++c) {
-        s += partial[((int64_t)c * d + j) * 2];
-        q += partial[((int64_t)c * d + j) * 2 + 1];
+    if (j < d) {
+#pragma unroll 4
+        for (int c = ty; c < chunks; c += 32) {
+            const double2 v = __ldg(reinterpret_cast<const double2*>(partial) + (int64_t)c * d + j);
+            s += v.x;
+            q += v.y;
+        }
+    }
+    s_sum[ty][tx] = s;
+    s_sq[ty][tx] = q;
+    __syncthreads();
+    if (ty != 0 || j >= d) return;
+    s = q = 0.0;
+    for (int r = 0; r < 32; ++r) {
+        s += s_sum[r][tx];
+        q += s_sq[r][tx];
     }
     const double off = n > 0 ? s / (double)n : 0.0;                       // mean of x - pivot
     const double mean = n > 0 ? (double)__ldg(H + j) + off : 0.0;
@@ -253,14 +271,14 @@ size_t col_stats_scratch_bytes(int d) { return (size_t)kStatChunksMax * (size_t)
 cudaError_t launch_col_stats(cudaStream_t s, const float* H, int64_t n, int d, int64_t ld, float eps,
                              float* shift, float* scale, void* scratch, int* launches)
 {
-    const int64_t rows_per_chunk = std::max<int64_t>(256, ceil_div(n, kStatChunksMax));
+    const int64_t rows_per_chunk = std::max<int64_t>(64, ceil_div(n, kStatChunksMax));
     const int chunks = (int)std::max<int64_t>(1, ceil_div(n, rows_per_chunk));
     double* partial = reinterpret_cast<double*>(scratch);
     col_partial_kernel<<<dim3((unsigned)ceil_div(d, 32), (unsigned)chunks), 256, 0, s>>>(H, n, d, ld, rows_per_chunk, partial);
     ++*launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    col_final_kernel<<<(unsigned)ceil_div(d, 128), 128, 0, s>>>(H, partial, chunks, d, n, (double)eps, shift, scale);
+    col_final_kernel<<<(unsigned)ceil_div(d, 32), 1024, 0, s>>>(H, partial, chunks, d, n, (double)eps, shift, scale);
     ++*launches;
     return cudaGetLastError();
 }

@@ -37,8 +37,8 @@ pack_rows_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld,
 #pragma unroll
             for (int r = 0; r < R; ++r) mine[r] = 0u;
             const int wlast = min(w0 + 32, kw);
-            for (int c0 = w0; c0 < wlast; c0 += WC) {
-                float x[R][WC];
+            float x[R][WC], nsh[kNorm ? WC : 1], nsc[kNorm ? WC : 1];
+            auto load = [&](int c0) {
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
@@ -46,15 +46,37 @@ pack_rows_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld,
                         const int j = ((c0 + q) << 5) + lane;
                         x[r][q] = (row0 + r < n && j < d) ? __ldg(H + (row0 + r) * ld + j) : 0.f;
                     }
+                if constexpr (kNorm) {
+#pragma unroll
+                    for (int q = 0; q < WC; ++q) {
+                        const int j = ((c0 + q) << 5) + lane;
+                        nsh[q] = j < d ? __ldg(shift + j) : 0.f;
+                        nsc[q] = j < d ? __ldg(scale + j) : 1.f;
+                    }
+                }
+            };
+            // rows of many words: the next chunk is asked for before this one is packed
+            constexpr bool kAhead = R <= 2;
+            if (kAhead) load(w0);
+            for (int c0 = w0; c0 < wlast; c0 += WC) {
+                if (!kAhead) load(c0);
+                float y[R][WC], ysh[kNorm ? WC : 1], ysc[kNorm ? WC : 1];
+#pragma unroll
+                for (int q = 0; q < WC; ++q) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) y[r][q] = x[r][q];
+                    if constexpr (kNorm) { ysh[q] = nsh[q]; ysc[q] = nsc[q]; }
+                }
+                if (kAhead && c0 + WC < wlast) load(c0 + WC);
 #pragma unroll
                 for (int q = 0; q < WC; ++q) {
                     const int j = ((c0 + q) << 5) + lane;
                     const bool in = j < d;
                     float sh = 0.f, sc = 1.f;
-                    if (kNorm && in) { sh = __ldg(shift + j); sc = __ldg(scale + j); }
+                    if constexpr (kNorm) { sh = ysh[q]; sc = ysc[q]; }
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        float v = x[r][q];
+                        float v = y[r][q];
                         if (kNorm) v = __fmul_rn(__fsub_rn(v, sh), sc);
                         const bool pos = in && (v >= 0.f);
                         if (in) l1[r] += fabsf(v);
@@ -237,6 +259,7 @@ weight_scale_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ld
     const int j = blockIdx.x * 32 + tx;
     double s = 0.0;
     if (j < d_out)
+#pragma unroll 8
         for (int k = ty; k < d_in; k += 32) s += (double)fabsf(__ldg(W + (int64_t)k * ldw + j));
     part[ty][tx] = s;
     __syncthreads();
