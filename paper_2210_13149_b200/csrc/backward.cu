@@ -789,6 +789,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     sa.long_row = long_row;
     sa.scratch = counter;
     sa.scratch_bytes = spmm_scratch_bytes(n, 0, 0);
+    sa.any_order = true;
     cudaError_t e = launch_spmm(s, sa, launches);
     if (e != cudaSuccess) return e;
 

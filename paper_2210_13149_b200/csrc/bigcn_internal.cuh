@@ -65,6 +65,7 @@ struct SpmmArgs {
     bool row_tail = false;           // byte rows of 64 bytes whose last four bytes hold the source's node factor (see bitgemm_tc.cu)
     const float* add = nullptr;   // optional fp32 [n x ld_add] added to every aggregated row (Bi-GraphSAGE self term)
     int64_t ld_add = 0;
+    bool any_order = false;          // h_out: the order of summation is free (see spmm.cu)
     float* h_out;            // nullable
     int64_t ldh;
     uint32_t* next_bits;     // nullable: fused re-binarization of the output

@@ -149,18 +149,19 @@ __device__ __forceinline__ void fill_col_table(const SpmmDev& p, float* ctab)
 }
 
 // Writes one finished row: optional fp32 store, optional sign/scale packing for the next layer.
-// Called by a full warp; every lane holds the totals of vector(s) c*32 + (lane % LPR).
+// Called by a full warp; every lane holds the totals of vector(s) c*32 + (lane % LPR).  S < 32: 32 / S rows at once, one per
+// S lanes; `on` says whether this lane's row exists.
 // kHalf (half-dot bytes): the accumulators hold sum_k w_k s_kj with s = (dot' - 1) / 2; the row's sum of the
 // edge weights `wsum` and their sum signed by the sources' first feature sign `wsgn` give back
 // sum_k w_k dot_kj = 2 acc_j + wsum + b0_j wsgn before the column factor is applied.
-template <typename T, int NCH, int LPR, bool kHalf = false>
+template <typename T, int NCH, int LPR, bool kHalf = false, int S = 32>
 __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, int64_t row, int lane,
-                                           float (&acc)[NCH][Elt<T>::kPerVec], float wsum = 0.f, float wsgn = 0.f)
+                                           float (&acc)[NCH][Elt<T>::kPerVec], float wsum = 0.f, float wsgn = 0.f, bool on = true)
 {
     constexpr int EPV = Elt<T>::kPerVec;
     constexpr int LW = 32 / EPV;                  // lanes that share one packed word
     constexpr int kCols = NCH * (LPR < 32 ? LPR : 32) * EPV;
-    const int g = lane / LPR, l = lane % LPR;
+    const int g = (lane % S) / LPR, l = lane % LPR;
     float l1 = 0.f;
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
@@ -186,9 +187,9 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
         if (p.add) {
 #pragma unroll
             for (int i = 0; i < EPV; ++i)
-                if (col0 + i < p.d_out) x[i] += __ldg(p.add + row * p.ld_add + col0 + i);
+                if ((S == 32 || on) && col0 + i < p.d_out) x[i] += __ldg(p.add + row * p.ld_add + col0 + i);
         }
-        if (p.h_out && g == 0 && vec < p.nv_fin) {
+        if (p.h_out && g == 0 && vec < p.nv_fin && (S == 32 || on)) {
             float* dst = p.h_out + row * p.ldh + col0;
             if (EPV == 4 && p.h_vec && col0 + 3 < p.d_out) {
                 *reinterpret_cast<float4*>(dst) = make_float4(x[0], x[1], x[2], x[3]);
@@ -221,16 +222,17 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
 #pragma unroll
             for (int o = 1; o < LW; o <<= 1) word |= __shfl_xor_sync(0xffffffffu, word, o);
             const int widx = col0 >> 5;
-            if (g == 0 && (l % LW) == 0 && vec < p.nv_fin && widx < p.next_stride)
+            if (g == 0 && (l % LW) == 0 && vec < p.nv_fin && widx < p.next_stride && (S == 32 || on))
                 p.next_bits[row * p.next_stride + widx] = word;
         }
     }
     if (p.next_bits) {
-        for (int w = p.covered_words + lane; w < p.next_stride; w += 32) p.next_bits[row * p.next_stride + w] = 0u;
+        if (S == 32 || on)
+            for (int w = p.covered_words + lane % S; w < p.next_stride; w += S) p.next_bits[row * p.next_stride + w] = 0u;
         if (g != 0) l1 = 0.f;                     // the other lane groups hold copies of the same totals
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-        if (lane == 0) p.next_beta[row] = l1 * p.inv_d_out;
+        for (int o = S / 2; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+        if (lane % S == 0 && (S == 32 || on)) p.next_beta[row] = l1 * p.inv_d_out;
     }
 }
 
@@ -1537,6 +1539,211 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
     return cudaGetLastError();
 }
 
+// ---- short rows ----------------------------------------------------------------------------------------------------
+// The aggregation of rows of up to 32 vectors with everything in registers: S lanes take a row (8, or the LPR lanes that
+// hold its vectors where those are more), so a warp takes 32 / S rows at once, and their bookkeeping, gathers and epilogues
+// share instructions.  A chunk is S stored entries of each of the rows: lane i of the S loads entry i's column, value and
+// factor -- column and value one chunk ahead, across rows -- and then every entry's row is fetched by the LPR lanes of one
+// of the S / LPR lane groups, up to eight fetches in flight.  Rows of more than 8 S entries are taken by the whole warp,
+// those above long_row by the block.  The order of summation differs from stream_entries()'s: for launches that write no H'
+// and for gradients (any_order).
+//
+// Against stream_entries(), which its ring in shared memory and the bookkeeping around it bound at 21 instructions per
+// entry and 110 per row: see rows_pays().
+template <typename T, int LPR, int S>
+struct RowSet {                                               // the rows that a warp's 32 / S lane groups have open
+    static constexpr int EPV = Elt<T>::kPerVec, PG = S / LPR;
+    // chunks taken together: enough of them for four fetches per lane where the whole warp takes a row
+    static constexpr int U = S == 32 && LPR < 4 ? 4 / LPR : 1;
+    static constexpr int H = U * LPR < 4 ? U * LPR : 4;       // fetches issued together
+
+    // acc += the next `left` entries of the lane's row, at most U S; col, val: of entry u S + lane % S
+    template <typename Next>
+    static __device__ __forceinline__ void chunk(const SpmmDev& p, int lane, int left, const int (&col)[U], const float (&val)[U], float (&acc)[EPV], Next next)
+    {
+        const int l = lane % LPR, pg = (lane % S) / LPR;
+        const bool vec_in = l < p.nv;
+        const uint4* zeta_l = p.zeta + (vec_in ? l : 0);
+        float w_[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) w_[u] = p.node_w ? __ldg(p.node_w + col[u]) : 1.f;
+#pragma unroll
+        for (int j0 = 0; j0 < U * LPR; j0 += H) {
+            if (j0 > 0 && !__any_sync(0xffffffffu, left > j0 * PG)) break;
+            uint4 v[H];
+#pragma unroll
+            for (int b = 0; b < H; ++b) {
+                const int k = __shfl_sync(0xffffffffu, col[(j0 + b) / LPR], (j0 + b) % LPR * PG + pg, S);
+                v[b] = __ldg(zeta_l + (int64_t)k * p.nv);
+            }
+            if (j0 == 0) {
+                next();                                       // the next chunk's columns and values, behind these fetches
+#pragma unroll
+                for (int u = 0; u < U; ++u) w_[u] *= val[u];
+            }
+#pragma unroll
+            for (int b = 0; b < H; ++b) {
+                const float w = __shfl_sync(0xffffffffu, w_[(j0 + b) / LPR], (j0 + b) % LPR * PG + pg, S);
+                if ((j0 + b) * PG + pg < left && vec_in) fma_any<T>(w, v[b], acc);
+            }
+        }
+    }
+    static __device__ __forceinline__ void reduce(float (&acc)[EPV])
+    {
+#pragma unroll
+        for (int o = LPR; o < S; o <<= 1)
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+    }
+};
+
+__host__ __device__ constexpr int row_lanes(int lpr) { return lpr <= 8 ? 8 : lpr; }
+__host__ __device__ constexpr int row_blocks(int elt_bytes) { return elt_bytes == 1 ? 3 : 4; }
+
+template <typename T, int LPR>
+__global__ void __launch_bounds__(kSpmmThreads, row_blocks(sizeof(T)))
+spmm_rows_kernel(const SpmmDev p, int rows_per_take, int dynamic)
+{
+    constexpr int EPV = Elt<T>::kPerVec, kCols = LPR * EPV, S = row_lanes(LPR), R = 32 / S;
+    using Set = RowSet<T, LPR, S>;
+    using Wide = RowSet<T, LPR, 32>;
+    __shared__ __align__(16) float ctab[4 * kCols];
+    __shared__ float part[kSpmmWarps][kCols];
+    __shared__ int64_t long_rows[kLongQueue];
+    __shared__ int n_long;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    fill_col_table<kCols, EPV>(p, ctab);
+    if (threadIdx.x == 0) n_long = 0;
+    __syncthreads();
+
+    const int n_takes = (int)ceil_div(p.n, rows_per_take);
+    float acc[1][EPV];
+    // [e, e + n_ent) by the whole warp, into acc (totals in every lane)
+    auto whole = [&](int64_t e, int64_t n_ent) {
+        zero_acc<1, EPV>(acc);
+        constexpr int U = Wide::U;
+        int col[U] = {};
+        float val[U] = {};
+        auto load = [&](int64_t at) {                         // (lanes past the row's end repeat its last entry)
+            if (at < n_ent) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t x = e + min(at + 32 * u + lane, n_ent - 1);
+                    col[u] = __ldg(p.colidx + x);
+                    val[u] = __ldg(p.val + x);
+                }
+            }
+        };
+        load(0);
+        for (int64_t at = 0; at < n_ent; at += 32 * U) {
+            int c[U];
+            float v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) c[u] = col[u], v[u] = val[u];
+            Wide::chunk(p, lane, (int)min(n_ent - at, (int64_t)(32 * U)), c, v, acc[0], [&]() { load(at + 32 * U); });
+        }
+        Wide::reduce(acc[0]);
+    };
+    for (int take = (int)blockIdx.x * kSpmmWarps + warp;;) {
+        if (dynamic) {
+            if (lane == 0) take = atomicAdd(p.run_counter, 1);
+            take = __shfl_sync(0xffffffffu, take, 0);
+        }
+        if (take >= n_takes) break;
+        const int64_t row0 = (int64_t)take * rows_per_take;
+        const int n_rows = (int)min((int64_t)rows_per_take, p.n - row0);
+        const int64_t rp = __ldg(p.rowptr + row0 + min(lane, n_rows));
+        const int64_t rp_next = __shfl_down_sync(0xffffffffu, rp, 1);
+        bool is_long = lane < n_rows && p.long_row > 0 && (rp_next - rp) > p.long_row;
+        if (is_long) {                                        // queue it for the block; if the queue is full, the warp takes it
+            const int slot = atomicAdd(&n_long, 1);
+            if (slot < kLongQueue) long_rows[slot] = row0 + lane;
+            else is_long = false;
+        }
+        const bool wide = lane < n_rows && !is_long && (S == 32 || rp_next - rp > 8 * S);
+        unsigned wide_mask = __ballot_sync(0xffffffffu, wide);
+        if constexpr (S < 32) {
+            // lane i: row i's entries, or -1 where the rows below do not take it
+            const int len = lane < n_rows && !is_long && !wide ? (int)(rp_next - rp) : -1;
+            int64_t e = 0;
+            int n_ent = -1, col = 0;
+            float val = 0.f;
+            auto open = [&](int r0) {                         // the row of this lane's group: its first chunk
+                const int r = min(r0 + lane / S, 31);
+                e = __shfl_sync(0xffffffffu, rp, r);
+                n_ent = r0 < n_rows ? __shfl_sync(0xffffffffu, len, r) : -1;
+            };
+            auto load = [&](int at) {
+                if (n_ent > at) {
+                    const int64_t x = e + min(at + lane % S, n_ent - 1);
+                    col = __ldg(p.colidx + x);
+                    val = __ldg(p.val + x);
+                }
+            };
+            open(0);
+            load(0);
+            for (int r0 = 0; r0 < n_rows; r0 += R) {
+                const int n_cur = n_ent;
+                const int most = __reduce_max_sync(0xffffffffu, n_cur);
+                if (most <= 0) {                              // nothing to add: rows without entries, or taken elsewhere
+                    zero_acc<1, EPV>(acc);
+                    open(r0 + R);
+                    load(0);
+                } else {
+                    zero_acc<1, EPV>(acc);
+                    for (int at = 0; at < most; at += S) {
+                        const int c[1] = {col};
+                        const float v[1] = {val};
+                        Set::chunk(p, lane, n_cur - at, c, v, acc[0], [&]() {
+                            if (at + S < most) {
+                                load(at + S);
+                            } else {
+                                open(r0 + R);
+                                load(0);
+                            }
+                        });
+                    }
+                    Set::reduce(acc[0]);
+                }
+                if (__any_sync(0xffffffffu, n_cur >= 0))
+                    finish_row<T, 1, LPR, false, S>(p, ctab, row0 + r0 + lane / S, lane, acc, 0.f, 0.f, n_cur >= 0);
+            }
+        }
+        for (; wide_mask; wide_mask &= wide_mask - 1) {
+            const int r = __ffs(wide_mask) - 1;
+            const int64_t s = __shfl_sync(0xffffffffu, rp, r);
+            whole(s, __shfl_sync(0xffffffffu, rp_next, r) - s);
+            finish_row<T, 1, LPR>(p, ctab, row0 + r, lane, acc);
+        }
+        if (!dynamic) take += (int)gridDim.x * kSpmmWarps;
+    }
+    __syncthreads();
+    // Long rows of this block, one after the other, each by all warps together.
+    const int nl = min(n_long, kLongQueue);
+    for (int q = 0; q < nl; ++q) {
+        const int64_t lrow = long_rows[q];
+        const int64_t ls = __ldg(p.rowptr + lrow), le = __ldg(p.rowptr + lrow + 1);
+        const int64_t slice = round_up(ceil_div(le - ls, kSpmmWarps), 32);
+        const int64_t s0 = min(le, ls + warp * slice), s1 = min(le, s0 + slice);
+        whole(s0, s1 - s0);
+        if (lane < LPR) {
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) part[warp][lane * EPV + i] = acc[0][i];
+        }
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int i = 0; i < EPV; ++i) {
+                float s = 0.f;
+                for (int w = 0; w < kSpmmWarps; ++w) s += part[w][(lane % LPR) * EPV + i];
+                acc[0][i] = s;
+            }
+            finish_row<T, 1, LPR>(p, ctab, lrow, lane, acc);
+        }
+        __syncthreads();
+    }
+}
+
 // Thread blocks per SM the kernel is compiled for (register budget) and launched with (grid size).
 template <int NCH, int LPR, bool kAligned, int kEltBytes>
 constexpr int spmm_blocks_per_sm()
@@ -1667,6 +1874,39 @@ cudaError_t launch_one(cudaStream_t s, const SpmmDev& p)
     return cudaGetLastError();
 }
 
+// Where spmm_rows_kernel takes the place of the general stream.  Measured, a layer with its contraction, before -> now
+// (fp16 rows, bits only): 2.4 M rows of 13 entries, 16 / 32 / 64 / 128 columns 1,283 / 1,562 / 1,974 / 2,873 -> 907 / 1,022 /
+// 1,636 / 2,774 us; 600 K rows of 51, 32 columns 807 -> 523 us; 20 K rows of 6, 3 columns 30 -> 20 us; gradients, 1.4 M rows of
+// 21, 32 columns 1,556 -> 1,153 us.  Not for rows of 32 vectors (2.4 M rows of 13, 256 columns 4.6 -> 5.1 ms), nor for 8 and
+// more on graphs that leave most warps without a row, where the ring keeps more fetches of a longer row in flight (2,500
+// rows of 31, 64 columns: 24 -> 30 us); nor, beyond one vector, where H' is written (the order of summation differs).
+bool rows_pays(const SpmmDev& p, int elt_bytes, double mean_row)
+{
+    if (p.half_dots || p.nv > 16) return false;
+    if (p.h_out && !p.any_order && p.nv > 1) return false;
+    if (elt_bytes == 1 && p.nv > 8 && !(mean_row > 0.0 && mean_row < 8.0)) return false;   // the row-aligned byte stream
+    return !(p.nv > 4 && p.n < 12000 && mean_row > 12.0);
+}
+
+template <typename T, int LPR>
+cudaError_t launch_rows(cudaStream_t s, const SpmmDev& p, double mean_row)
+{
+    constexpr int R = 32 / row_lanes(LPR);
+    const int64_t warps = (int64_t)sm_count() * row_blocks(sizeof(T)) * kSpmmWarps;
+    // rows that a warp takes at a time: four sets (four rows where most of them take a whole warp), fewer where that would
+    // leave warps without rows
+    const int unit = mean_row > 32.0 ? 1 : R;
+    const int rows_per_take = (int)std::min<int64_t>(4, std::max<int64_t>(1, p.n / (2 * warps * unit))) * unit;
+    const int64_t takes = ceil_div(p.n, rows_per_take);
+    const int dynamic = takes > 2 * warps ? 1 : 0;            // (on small graphs the counter's latency is not worth it)
+    if (dynamic) {
+        cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
+    spmm_rows_kernel<T, LPR><<<(unsigned)ceil_div(std::min(takes, warps), kSpmmWarps), kSpmmThreads, 0, s>>>(p, rows_per_take, dynamic);
+    return cudaGetLastError();
+}
+
 // mean_row: stored entries per row (0 = unknown).  256-byte rows of signed bytes take the row-aligned
 // multi-entry stream (the general stream has no fast unpack for bytes) unless the rows are known to be
 // much shorter than its groups of 8 entries.  For 2- and 4-byte elements in rows of 8 or 16 vectors the
@@ -1710,6 +1950,13 @@ cudaError_t dispatch(cudaStream_t s, const SpmmDev& p, double mean_row)
             if (short_rows) return launch_one<T, 1, 8, false, false, true>(s, p);
             return nv == 8 ? launch_one<T, 1, 8, true, true, true>(s, p) : launch_one<T, 1, 8, false, true, true>(s, p);
         }
+    }
+    if (rows_pays(p, (int)sizeof(T), mean_row)) {
+        if (nv <= 1) return launch_rows<T, 1>(s, p, mean_row);
+        if (nv <= 2) return launch_rows<T, 2>(s, p, mean_row);
+        if (nv <= 4) return launch_rows<T, 4>(s, p, mean_row);
+        if (nv <= 8) return launch_rows<T, 8>(s, p, mean_row);
+        return launch_rows<T, 16>(s, p, mean_row);
     }
     if (nv <= 1) return launch_one<T, 1, 1>(s, p);
     if (nv <= 2) return launch_one<T, 1, 2>(s, p);
@@ -1774,6 +2021,7 @@ cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches)
     p.next_beta = a.next_beta;
     p.next_shift = a.next_shift;
     p.next_scale = a.next_scale;
+    p.any_order = a.any_order;
     p.long_row = a.long_row;
     p.covered_words = (int)ceil_div(a.ldz, 32);
     p.inv_d_out = 1.f / (float)a.d_out;

@@ -31,6 +31,7 @@ struct SpmmDev {
     float* next_beta;
     const float* next_shift;
     const float* next_scale;
+    bool any_order;          // fp32 output whose order of summation is free
     int64_t long_row;
     int covered_words;       // packed words of the next layer that the zeta columns cover
     float inv_d_out;
