@@ -32,14 +32,43 @@ __global__ void pad_rows_kernel(const float* __restrict__ src, int64_t n, int d,
     }
 }
 
-// G_W~ = sum of the slabs, in slab order (double accumulation: the slabs can differ by orders of magnitude).
-__global__ void grad_wt_reduce_kernel(const float* __restrict__ part, int n_splits, int64_t elems, float* __restrict__ g_wt)
+// G_W~ = sum of the slabs (double accumulation: the slabs can differ by orders of magnitude), and for Eq. bp-W the sums
+// sum_k G_W~_kj sign(W_kj) over four inputs k.  A block takes 32 channels x 4 inputs; of its 1,024 threads eight share
+// an element and take every eighth slab each, eight loads in flight; their sums are added in order.  (One thread per element
+// walked through all slabs alone: 15 to 28 us whatever the sizes.)
+constexpr int kRedRows = 4, kRedGroups = 8;
+__global__ void __launch_bounds__(32 * kRedRows * kRedGroups)
+grad_wt_reduce_kernel(const float* __restrict__ part, int n_splits, int d_in, int d_out, const float* __restrict__ W, int64_t ldw,
+                      float* __restrict__ g_wt, double* __restrict__ col_part /* [ceil(d_in / 4)][d_out] */)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= elems) return;
+    __shared__ double s_sum[kRedGroups][kRedRows][33];
+    const int tx = threadIdx.x & 31, r = (threadIdx.x >> 5) % kRedRows, zg = threadIdx.x / (32 * kRedRows);
+    const int j = blockIdx.x * 32 + tx, k = blockIdx.y * kRedRows + r;
+    const int64_t elems = (int64_t)d_in * d_out;
     double s = 0.0;
-    for (int z = 0; z < n_splits; ++z) s += (double)part[(int64_t)z * elems + t];
-    g_wt[t] = (float)s;
+    if (j < d_out && k < d_in) {
+        const float* src = part + (int64_t)k * d_out + j;
+#pragma unroll 8
+        for (int z = zg; z < n_splits; z += kRedGroups) s += (double)__ldg(src + z * elems);
+    }
+    s_sum[zg][r][tx] = s;
+    __syncthreads();
+    if (zg == 0) {
+        for (int q = 1; q < kRedGroups; ++q) s += s_sum[q][r][tx];
+        const float g = (float)s;
+        double sg = 0.0;
+        if (j < d_out && k < d_in) {
+            g_wt[(int64_t)k * d_out + j] = g;
+            sg = __ldg(W + (int64_t)k * ldw + j) >= 0.f ? (double)g : -(double)g;
+        }
+        s_sum[0][r][tx] = sg;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 && j < d_out) {
+        double c = 0.0;
+        for (int q = 0; q < kRedRows; ++q) c += s_sum[0][q][tx];
+        col_part[(int64_t)blockIdx.y * d_out + j] = c;
+    }
 }
 
 // ---- the two dense products, on the tensor cores ------------------------------------------------------
@@ -180,109 +209,6 @@ grad_h_mma_kernel(const float* __restrict__ gz, int64_t ldz, const float* __rest
                     const int k = k0 + wc * 64 + nb * 8 + 2 * t + q;
                     const float v = acc[mb][nb][2 * half + q];
                     if (k < d_in) g_h[row * ldh + k] = fabsf(v) < 1.f ? v : 0.f;            // Eq. bp-H
-                }
-        }
-}
-
-// G_W~ partial sums on the tensor cores.  The product is taken transposed, C^T[j][k] = sum over nodes
-// of (beta_i G_zeta[i][j]) * F[i][k], so that the fp32 operand is again the row operand: A[j][node]
-// (split in three), B[node][k] = +-1 from the packed bits.  Both operands are stored node-major in
-// global memory and the reduction runs over the nodes, so the staging transposes them: a thread takes
-// two consecutive nodes and writes them as one 32-bit pair.  Block (x, y, z): channels j in
-// [128 x, +128), inputs k in [128 y, +128), nodes [z * rows_per_split, +rows_per_split); slab z of
-// `part` receives the tile as [k][j].
-__global__ void __launch_bounds__(kBwThreads)
-grad_wt_mma_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float* __restrict__ beta,
-                   const float* __restrict__ gz, int64_t ldz, int64_t n, int d_in, int d_out,
-                   int64_t rows_per_split, float* __restrict__ part)
-{
-    __shared__ __align__(16) unsigned short As[3 * kMmaTile * kMmaPitch];   // [term][j][node]
-    __shared__ __align__(16) unsigned short Bs[kMmaTile * kMmaPitch];       // [k][node]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wr = warp >> 1, wc = warp & 1;
-    const int j0 = blockIdx.x * kMmaTile, k0 = blockIdx.y * kMmaTile;
-    const int64_t r_begin = (int64_t)blockIdx.z * rows_per_split;
-    const int64_t r_end = min(n, r_begin + rows_per_split);
-    const bool vec_ok = (ldz % 4 == 0) && (reinterpret_cast<uintptr_t>(gz) % 16 == 0);
-    float acc[2][8][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-    for (int64_t r0 = r_begin; r0 < r_end; r0 += kMmaK) {
-        __syncthreads();                                   // the previous step's tiles are consumed
-        // A: 16 node pairs x 32 quads of channels
-        for (int t = threadIdx.x; t < 16 * 32; t += kBwThreads) {
-            const int np = t & 15, jq = (t >> 4) * 4;
-            float x[2][4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int64_t row = r0 + 2 * np + h;
-                const int j = j0 + jq;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) x[h][q] = 0.f;
-                if (row < r_end) {
-                    const float be = __ldg(beta + row);
-                    if (j + 3 < d_out && vec_ok) {
-                        const float4 v = __ldg(reinterpret_cast<const float4*>(gz + row * ldz + j));
-                        x[h][0] = v.x * be, x[h][1] = v.y * be, x[h][2] = v.z * be, x[h][3] = v.w * be;
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (j + q < d_out) x[h][q] = __ldg(gz + row * ldz + j + q) * be;
-                    }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                unsigned short h0, m0, l0, h1, m1, l1;
-                split3(x[0][q], h0, m0, l0);
-                split3(x[1][q], h1, m1, l1);
-                const int at = (jq + q) * kMmaPitch + 2 * np;
-                *reinterpret_cast<uint32_t*>(&As[0 * kMmaTile * kMmaPitch + at]) = (uint32_t)h0 | ((uint32_t)h1 << 16);
-                *reinterpret_cast<uint32_t*>(&As[1 * kMmaTile * kMmaPitch + at]) = (uint32_t)m0 | ((uint32_t)m1 << 16);
-                *reinterpret_cast<uint32_t*>(&As[2 * kMmaTile * kMmaPitch + at]) = (uint32_t)l0 | ((uint32_t)l1 << 16);
-            }
-        }
-        // B: 16 node pairs x 4 words of 32 inputs, each word in two halves of 16
-        for (int t = threadIdx.x; t < 16 * 8; t += kBwThreads) {
-            const int np = t & 15, wd = (t >> 4) >> 1, half = (t >> 4) & 1;
-            const int kw = k0 + wd * 32;                   // first input of the word
-            uint32_t w0 = 0u, w1 = 0u;
-            const int64_t row = r0 + 2 * np;
-            if (kw < d_in) {
-                if (row < r_end) w0 = __ldg(bits + row * stride + (kw >> 5));
-                if (row + 1 < r_end) w1 = __ldg(bits + (row + 1) * stride + (kw >> 5));
-            }
-            const bool in0 = row < r_end, in1 = row + 1 < r_end;
-#pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                const int kb = half * 16 + b;
-                const bool kin = kw + kb < d_in;
-                const uint32_t lo = (kin && in0) ? (((w0 >> kb) & 1u) ? 0x3F80u : 0xBF80u) : 0u;
-                const uint32_t hi = (kin && in1) ? (((w1 >> kb) & 1u) ? 0x3F80u : 0xBF80u) : 0u;
-                *reinterpret_cast<uint32_t*>(&Bs[(wd * 32 + kb) * kMmaPitch + 2 * np]) = lo | (hi << 16);
-            }
-        }
-        __syncthreads();
-        mma_step(As, Bs, wr, wc, lane, acc);
-    }
-    float* slab = part + (int64_t)blockIdx.z * d_in * d_out;
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int mb = 0; mb < 2; ++mb)
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int j = j0 + wr * 32 + mb * 16 + g + 8 * half;
-            if (j >= d_out) continue;
-#pragma unroll
-            for (int nb = 0; nb < 8; ++nb)
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int k = k0 + wc * 64 + nb * 8 + 2 * t + q;
-                    if (k < d_in) slab[(int64_t)k * d_out + j] = acc[mb][nb][2 * half + q];
                 }
         }
 }
@@ -482,175 +408,169 @@ grad_h_tc_kernel(const float* __restrict__ gz, int64_t ldz, const float* __restr
 }
 
 // ---- G_W~ partial sums on the 5th-generation tensor cores -------------------------------------------------
-// The product of grad_wt_mma_kernel (transposed: C^T[j][k] = sum over nodes of (beta_i G_zeta[i][j]) F[i][k])
-// with tcgen05.mma kind::f16: M = 128 channels j, N = 64 / 128 / 256 >= d_in inputs k, the reduction over
-// the CTA's nodes in chunks of 64, all of them accumulated in one fp32 tile of tensor memory that is read
-// back once at the end and written as slab blockIdx.y of `part` ([k][j]: consecutive lanes write consecutive
-// j).  Both operands are node-major in global memory; the staging transposes them, two nodes per 32-bit store.
+// C^T[j][k] = sum over nodes of (beta_i G_zeta[i][j]) F[i][k] with tcgen05.mma kind::f16: M = 128 channels j, N = 64 / 128 /
+// 256 inputs k (blockIdx.z: slices of N), the reduction over the block's nodes, all of them accumulated in one fp32 tile of
+// tensor memory that is read back once at the end and written as slab blockIdx.y of `part` ([k][j]: consecutive lanes
+// write consecutive j).  Both operands are node-major in global memory and stay so in shared memory: M- and N-major operands
+// with 128-byte swizzle (64 channels or inputs of a node are 128 contiguous bytes), so nothing is transposed and every
+// store is a vector.  Chunks of 32 nodes, two stages: while one is multiplied the other is filled, and the chunk after
+// that is on its way in registers.  (With K-major operands every store was 4 bytes and the stages took turns: 2.4 M nodes,
+// 256 -> 256, 2.7 ms.)
+constexpr int kWtNodes = 32;                               // nodes per chunk
+constexpr int kWtAtom = kWtNodes * 128;                    // bytes of 64 columns of a chunk
+
 template <int N>
 __global__ void __launch_bounds__(kBwThreads, 2)
 grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float* __restrict__ beta,
                   const float* __restrict__ gz, int64_t ldz, int64_t n, int d_in, int d_out,
                   int64_t rows_per_split, float* __restrict__ part)
 {
-    constexpr int kRows = 128, kKc = 64;                   // channels per tile; nodes per chunk
-    constexpr int kCols = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
-    extern __shared__ __align__(128) unsigned char bw_smem[];
-    __shared__ __align__(8) uint64_t bar;
+    constexpr int kStage = 6 * kWtAtom + N / 64 * kWtAtom;  // three terms x two atoms of channels, N / 64 atoms of inputs
+    constexpr int kItems = kWtNodes * 32 / kBwThreads;      // 16-byte pieces of a chunk per thread
+    extern __shared__ unsigned char bw_raw[];
+    __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t tmem_base_s;
-    unsigned char* As = bw_smem;                            // [3][128 channels][64 nodes] bf16
-    unsigned char* Bs = bw_smem + 3 * kRows * 128;          // [N inputs][64 nodes] bf16
+    unsigned char* sm = bw_raw + ((1024u - (tc::smem_u32(bw_raw) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) tc::tmem_alloc(&tmem_base_s, kCols);
-    if (threadIdx.x == 0) tc::barrier_init(&bar);
+    if (warp == 0) tc::tmem_alloc(&tmem_base_s, N);
+    if (threadIdx.x == 0) {
+        tc::barrier_init(&bar[0]);
+        tc::barrier_init(&bar[1]);
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem_base = tmem_base_s;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
-    const uint32_t a_lbo = (kRows >> 3) * 128, b_lbo = (N >> 3) * 128, sbo = 128;
+    // D = f32, A = B = bf16, A M-major, B N-major, N, M = 128
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     const bool vec_ok = (ldz % 4 == 0) && (reinterpret_cast<uintptr_t>(gz) % 16 == 0);
-    const int j0 = blockIdx.x * kRows;
+    const int j0 = blockIdx.x * 128, k0 = blockIdx.z * N;
     const int64_t r_begin = (int64_t)blockIdx.y * rows_per_split;
     const int64_t r_end = min(n, r_begin + rows_per_split);
-    uint32_t phase = 0;
-    bool ok = true, any = false;
-    for (int64_t r0 = r_begin; r0 < r_end; r0 += kKc) {
-        // A: 32 node pairs x 32 quads of channels; all of a thread's loads are issued before the first is used
-        {
-            constexpr int kItems = 32 * 32 / kBwThreads;
-            float4 xv[kItems][2];
-            float bv[kItems][2];
+    const int n_chunks = r_begin < r_end ? (int)ceil_div(r_end - r_begin, kWtNodes) : 0;
+    // this thread's pieces: channels j .. j + 3 of nodes warp + 8 it; and word wd of node `lane`
+    const int j = j0 + 4 * lane, wd = (k0 >> 5) + warp;
+    const bool has_word = warp < N / 32 && wd < stride;
+    float4 xv[kItems];
+    float bv[kItems];
+    uint32_t word = 0u;
+    auto load = [&](int c) {
+        const int64_t r0 = r_begin + (int64_t)c * kWtNodes;
 #pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const int t = threadIdx.x + it * kBwThreads;
-                const int np = t & 31, jq = (t >> 5) * 4;
-                const int j = j0 + jq;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int64_t row = r0 + 2 * np + h;
-                    xv[it][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    bv[it][h] = 0.f;
-                    if (row < r_end) {
-                        bv[it][h] = __ldg(beta + row);
-                        if (j + 3 < d_out && vec_ok) {
-                            xv[it][h] = __ldg(reinterpret_cast<const float4*>(gz + row * ldz + j));
-                        } else {
-                            if (j < d_out) xv[it][h].x = __ldg(gz + row * ldz + j);
-                            if (j + 1 < d_out) xv[it][h].y = __ldg(gz + row * ldz + j + 1);
-                            if (j + 2 < d_out) xv[it][h].z = __ldg(gz + row * ldz + j + 2);
-                            if (j + 3 < d_out) xv[it][h].w = __ldg(gz + row * ldz + j + 3);
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const int t = threadIdx.x + it * kBwThreads;
-                const int np = t & 31, jq = (t >> 5) * 4;
-                const float x0[4] = {xv[it][0].x * bv[it][0], xv[it][0].y * bv[it][0], xv[it][0].z * bv[it][0], xv[it][0].w * bv[it][0]};
-                const float x1[4] = {xv[it][1].x * bv[it][1], xv[it][1].y * bv[it][1], xv[it][1].z * bv[it][1], xv[it][1].w * bv[it][1]};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    unsigned short h0, m0, l0, h1, m1, l1;
-                    split3(x0[u], h0, m0, l0);
-                    split3(x1[u], h1, m1, l1);
-                    const uint32_t off = tc::canon_off(kRows, jq + u, (2 * np) >> 3) + ((2 * np) & 7) * 2;
-                    *reinterpret_cast<uint32_t*>(As + 0 * kRows * 128 + off) = (uint32_t)h0 | ((uint32_t)h1 << 16);
-                    *reinterpret_cast<uint32_t*>(As + 1 * kRows * 128 + off) = (uint32_t)m0 | ((uint32_t)m1 << 16);
-                    *reinterpret_cast<uint32_t*>(As + 2 * kRows * 128 + off) = (uint32_t)l0 | ((uint32_t)l1 << 16);
+        for (int it = 0; it < kItems; ++it) {
+            const int64_t row = r0 + warp + 8 * it;
+            xv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+            bv[it] = 0.f;
+            if (row < r_end) {
+                bv[it] = __ldg(beta + row);
+                if (j + 3 < d_out && vec_ok) {
+                    xv[it] = __ldg(reinterpret_cast<const float4*>(gz + row * ldz + j));
+                } else {
+                    if (j < d_out) xv[it].x = __ldg(gz + row * ldz + j);
+                    if (j + 1 < d_out) xv[it].y = __ldg(gz + row * ldz + j + 1);
+                    if (j + 2 < d_out) xv[it].z = __ldg(gz + row * ldz + j + 2);
+                    if (j + 3 < d_out) xv[it].w = __ldg(gz + row * ldz + j + 3);
                 }
             }
         }
-        // B: 32 node pairs x (N / 32) packed words x 4 groups of 8 inputs (loads batched in the same way)
-        {
-            constexpr int kItems = 32 * (N / 32) * 4 / kBwThreads;
-            uint32_t w0v[kItems], w1v[kItems];
+        if (has_word) word = __ldg(bits + min(r0 + lane, r_end - 1) * stride + wd);   // (past the end: met by zeros)
+    };
+    // where they go inside a stage
+    uint32_t a_off[kItems];
 #pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const int t = threadIdx.x + it * kBwThreads;
-                const int np = t & 31, wd = (t >> 5) >> 2;
-                const int64_t row = r0 + 2 * np;
-                w0v[it] = 0u, w1v[it] = 0u;
-                if (wd * 32 < d_in) {
-                    if (row < r_end) w0v[it] = __ldg(bits + row * stride + wd);
-                    if (row + 1 < r_end) w1v[it] = __ldg(bits + (row + 1) * stride + wd);
+    for (int it = 0; it < kItems; ++it) {
+        const int node = warp + 8 * it;
+        a_off[it] = (uint32_t)((lane >> 4) * kWtAtom + (node >> 3) * 1024 + (node & 7) * 128 + ((((lane & 15) >> 1) ^ (node & 7)) << 4) + (lane & 1) * 8);
+    }
+    const uint32_t b_off = (uint32_t)(6 * kWtAtom + (warp >> 1) * kWtAtom + (lane >> 3) * 1024 + (lane & 7) * 128);
+    bool ok = true;
+    if (n_chunks > 0) load(0);
+    for (int c = 0; c < n_chunks; ++c) {
+        const int st = c & 1;
+        unsigned char* stage = sm + st * kStage;
+        if (c >= 2 && !tc::wait_barrier(&bar[st], (uint32_t)((c >> 1) + 1) & 1u)) {   // the products of chunk c - 2 are done
+            atomicExch(&g_bw_tc_timeout, 1);
+            ok = false;
+        }
+#pragma unroll
+        for (int it = 0; it < kItems; ++it) {
+            const float x[4] = {xv[it].x * bv[it], xv[it].y * bv[it], xv[it].z * bv[it], xv[it].w * bv[it]};
+            unsigned short hi[4], mid[4], lo[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) split3(x[u], hi[u], mid[u], lo[u]);
+            auto pack = [](const unsigned short (&h)[4]) { return make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16)); };
+            *reinterpret_cast<uint2*>(stage + 0 * kWtAtom + a_off[it]) = pack(hi);
+            *reinterpret_cast<uint2*>(stage + 2 * kWtAtom + a_off[it]) = pack(mid);
+            *reinterpret_cast<uint2*>(stage + 4 * kWtAtom + a_off[it]) = pack(lo);
+        }
+        if (warp < N / 32) {
+            const uint32_t minus = ~word;                   // bit 0: -1
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t o[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t two = minus >> (8 * q + 2 * r);
+                    o[r] = 0x3F803F80u | ((two & 1u) << 15) | ((two & 2u) << 30);
                 }
-            }
-#pragma unroll
-            for (int it = 0; it < kItems; ++it) {
-                const int t = threadIdx.x + it * kBwThreads;
-                const int np = t & 31, wd = (t >> 5) >> 2, part8 = (t >> 5) & 3;
-                const int kw = wd * 32;
-                const int64_t row = r0 + 2 * np;
-                const bool in0 = row < r_end, in1 = row + 1 < r_end;
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    const int kb = part8 * 8 + b, k = kw + kb;
-                    const bool kin = k < d_in;
-                    const uint32_t lo = (kin && in0) ? (((w0v[it] >> kb) & 1u) ? 0x3F80u : 0xBF80u) : 0u;
-                    const uint32_t hi = (kin && in1) ? (((w1v[it] >> kb) & 1u) ? 0x3F80u : 0xBF80u) : 0u;
-                    const uint32_t off = tc::canon_off(N, k, (2 * np) >> 3) + ((2 * np) & 7) * 2;
-                    *reinterpret_cast<uint32_t*>(Bs + off) = lo | (hi << 16);
-                }
+                *reinterpret_cast<uint4*>(stage + b_off + (((((warp & 1) * 4 + q)) ^ (lane & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
+        if (c + 1 < n_chunks) load(c + 1);
         tc::fence_async_smem();
         tc::fence_before_sync();
-        __syncthreads();
+        if (__syncthreads_or(!ok)) { ok = false; break; }   // leave together on a timeout
         tc::fence_after_sync();
         if (threadIdx.x == 0) {
-            const uint32_t a_base = tc::smem_u32(As), b_base = tc::smem_u32(Bs);
-            for (int ks = 0; ks < kKc / 16; ++ks) {
-                const uint64_t bd = tc::make_desc(b_base + 2 * ks * b_lbo, b_lbo, sbo);
+            const uint32_t base = tc::smem_u32(stage);
+            for (int ks = 0; ks < kWtNodes / 16; ++ks) {
+                const uint64_t bd = tc::make_desc(base + 6 * kWtAtom + ks * 2048, kWtAtom, 1024) | ((uint64_t)2 << 61);
 #pragma unroll
                 for (int sp = 0; sp < 3; ++sp) {
-                    const uint64_t ad = tc::make_desc(a_base + sp * kRows * 128 + 2 * ks * a_lbo, a_lbo, sbo);
-                    const uint32_t accum = (any || ks > 0 || sp > 0) ? 1u : 0u;
+                    const uint64_t ad = tc::make_desc(base + sp * 2 * kWtAtom + ks * 2048, kWtAtom, 1024) | ((uint64_t)2 << 61);
+                    const uint32_t accum = (c > 0 || ks > 0 || sp > 0) ? 1u : 0u;
                     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                                  ::"r"(tmem_base), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
                 }
             }
-            tc::commit_to(&bar);
+            tc::commit_to(&bar[st]);
         }
-        any = true;
-        if (!tc::wait_barrier(&bar, phase)) {
-            atomicExch(&g_bw_tc_timeout, 1);
-            ok = false;
-        }
-        phase ^= 1u;
-        tc::fence_after_sync();
-        if (__syncthreads_or(!ok)) { ok = false; break; }   // the operands may be overwritten; leave together on a timeout
     }
+    if (ok && n_chunks > 0 && !tc::wait_barrier(&bar[(n_chunks - 1) & 1], (uint32_t)((n_chunks - 1) >> 1) & 1u)) {
+        atomicExch(&g_bw_tc_timeout, 1);
+        ok = false;
+    }
+    tc::fence_after_sync();
+    ok = !__syncthreads_or(!ok);
     // ---- the slab: thread = channel j (tensor-memory lane), its warp's half of the inputs k
     if (ok) {
         float* slab = part + (int64_t)blockIdx.y * d_in * d_out;
         const int lane_base = 32 * (warp & 3);
-        const int j = j0 + lane_base + lane;
+        const int jj = j0 + lane_base + lane;
         const int c_begin = (warp >> 2) * (N / 2);
         for (int c0 = c_begin; c0 < c_begin + N / 2; c0 += 16) {
             uint32_t v[16];
-            if (any) tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)c0, v);
+            if (n_chunks > 0) tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)c0, v);
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
-                const int k = c0 + e;
-                if (j < d_out && k < d_in) slab[(int64_t)k * d_out + j] = any ? __uint_as_float(v[e]) : 0.f;
+                const int k = k0 + c0 + e;
+                if (jj < d_out && k < d_in) slab[(int64_t)k * d_out + jj] = n_chunks > 0 ? __uint_as_float(v[e]) : 0.f;
             }
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_free(tmem_base, kCols);
+    if (warp == 0) tc::tmem_free(tmem_base, N);
 }
 
 template <int N>
 cudaError_t launch_grad_wt_tc(cudaStream_t s, const uint32_t* bits, int64_t stride, const float* beta, const float* gz,
                               int64_t ldz, int64_t n, int d_in, int d_out, int n_splits, int64_t rows_per_split, float* part)
 {
-    const size_t smem = 3 * 128 * 128 + (size_t)N * 128;
+    const size_t smem = 2 * (6 + N / 64) * (size_t)kWtAtom + 1024;
     cudaError_t e = cudaFuncSetAttribute(grad_wt_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)ceil_div(d_out, 128), (unsigned)n_splits);
+    const dim3 grid((unsigned)ceil_div(d_out, 128), (unsigned)n_splits, (unsigned)ceil_div(d_in, N));
     grad_wt_tc_kernel<N><<<grid, kBwThreads, smem, s>>>(bits, stride, beta, gz, ldz, n, d_in, d_out, rows_per_split, part);
     return cudaGetLastError();
 }
@@ -667,51 +587,41 @@ cudaError_t launch_grad_h_tc(cudaStream_t s, const float* gz, int64_t ldz, const
     return cudaGetLastError();
 }
 
-// Eq. bp-W.  One block per 32 output channels: thread (tx, ty) sums G_W~_kj B_kj over k = ty, ty + 32, ...
-// for channel j0 + tx in double; the 32 partial sums of a channel are added in a fixed order; then
-// every element gets (1/d_in) B_ij col_j + alpha_j G_W~_ij [|W_ij| < 1].
+// Eq. bp-W.  A block per 32 channels x 32 inputs: thread (tx, ty) adds the partial column sums ty, ty + 32, ... of channel
+// j0 + tx in double, the 32 sums of a channel are added in order, and every element gets
+// (1/d_in) B_ij col_j + alpha_j G_W~_ij [|W_ij| < 1].
 __global__ void __launch_bounds__(1024)
-grad_w_kernel(const float* __restrict__ g_wt, const float* __restrict__ W, int64_t ldw,
+grad_w_kernel(const float* __restrict__ g_wt, const double* __restrict__ col_part, int n_part, const float* __restrict__ W, int64_t ldw,
               const float* __restrict__ alpha, int d_in, int d_out, float* __restrict__ g_w, int64_t ldgw)
 {
     __shared__ double part[32][33];
-    __shared__ double col[32];
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int j = blockIdx.x * 32 + tx;
+    const int j = blockIdx.x * 32 + tx, i = blockIdx.y * 32 + ty;
     double s = 0.0;
-    if (j < d_out)
-        for (int k = ty; k < d_in; k += 32) {
-            const float w = __ldg(W + (int64_t)k * ldw + j);
-            const double g = (double)__ldg(g_wt + (int64_t)k * d_out + j);
-            s += w >= 0.f ? g : -g;
-        }
+    if (j < d_out) {
+#pragma unroll 4
+        for (int q = ty; q < n_part; q += 32) s += __ldg(col_part + (int64_t)q * d_out + j);
+    }
     part[ty][tx] = s;
     __syncthreads();
-    if (ty == 0) {
-        double t = 0.0;
-        for (int r = 0; r < 32; ++r) t += part[r][tx];
-        col[tx] = t;
-    }
-    __syncthreads();
-    if (j < d_out) {
-        const double c = col[tx] / (double)d_in;
-        const float al = __ldg(alpha + j);
-        for (int i = ty; i < d_in; i += 32) {
-            const float w = __ldg(W + (int64_t)i * ldw + j);
-            double g = w >= 0.f ? c : -c;
-            if (fabsf(w) < 1.f) g += (double)al * (double)__ldg(g_wt + (int64_t)i * d_out + j);
-            g_w[(int64_t)i * ldgw + j] = (float)g;
-        }
-    }
+    if (j >= d_out || i >= d_in) return;
+    double c = 0.0;
+    for (int r = 0; r < 32; ++r) c += part[r][tx];
+    c /= (double)d_in;
+    const float w = __ldg(W + (int64_t)i * ldw + j);
+    double g = w >= 0.f ? c : -c;
+    if (fabsf(w) < 1.f) g += (double)__ldg(alpha + j) * (double)__ldg(g_wt + (int64_t)i * d_out + j);
+    g_w[(int64_t)i * ldgw + j] = (float)g;
 }
 
 int64_t pad4(int64_t d) { return (d + 3) / 4 * 4; }
 
+// Parts that the sum over the nodes is split into: two blocks per multiprocessor in all, at least 128 nodes each.
 int wt_splits(int64_t n, int d_in, int d_out)
 {
-    const int64_t tiles = ceil_div(d_in, kMmaTile) * ceil_div(d_out, kMmaTile);
-    const int64_t want = std::max<int64_t>(1, (sm_count() * 4) / tiles);               // about four blocks per SM in all
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(n, 4 * kMmaK)));
+    const int64_t tiles = ceil_div(d_in, 256) * ceil_div(d_out, 128);
+    const int64_t want = std::max<int64_t>(1, (sm_count() * 2) / tiles);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(n, 128)));
 }
 
 }  // namespace
@@ -731,6 +641,7 @@ size_t backward_scratch_bytes(int64_t n, int d_in, int d_out)
     total += up((size_t)n * pad4(d_out) * 4);                                    // G_zeta
     total += up((size_t)wt_splits(n, d_in, d_out) * d_in * d_out * 4);           // slabs of G_W~
     total += up((size_t)d_in * d_out * 4);                                       // G_W~
+    total += up((size_t)ceil_div(d_in, kRedRows) * d_out * 8);                   // column sums of Eq. bp-W
     total += up(spmm_scratch_bytes(n, 0, 0));
     return total;
 }
@@ -755,6 +666,9 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     base += up((size_t)n_splits * d_in * d_out * 4);
     float* g_wt = reinterpret_cast<float*>(base);
     base += up((size_t)d_in * d_out * 4);
+    const int n_part = (int)ceil_div(d_in, kRedRows);
+    double* col_part = reinterpret_cast<double*>(base);
+    base += up((size_t)n_part * d_out * 8);
     void* counter = base;
 
     // step 1a: G_zeta = A_tilde^T G' (A_tilde is symmetric: the forward aggregation on fp32 rows)
@@ -797,18 +711,11 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     {
         const int64_t rows_per_split = ceil_div(ceil_div(n, n_splits), 64) * 64;
         ++*launches;
-        if (d_in <= 256) {                                  // tcgen05 version: one tile covers all inputs
-            if (d_in <= 64) e = launch_grad_wt_tc<64>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
-            else if (d_in <= 128) e = launch_grad_wt_tc<128>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
-            else e = launch_grad_wt_tc<256>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
-            if (e != cudaSuccess) return e;
-        } else {
-            const dim3 grid((unsigned)ceil_div(d_out, kMmaTile), (unsigned)ceil_div(d_in, kMmaTile), (unsigned)n_splits);
-            grad_wt_mma_kernel<<<grid, kBwThreads, 0, s>>>(in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, rows_per_split, part);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        }
-        const int64_t elems = (int64_t)d_in * d_out;
-        grad_wt_reduce_kernel<<<(unsigned)ceil_div(elems, 256), 256, 0, s>>>(part, n_splits, elems, g_wt);
+        if (d_in <= 64) e = launch_grad_wt_tc<64>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
+        else if (d_in <= 128) e = launch_grad_wt_tc<128>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
+        else e = launch_grad_wt_tc<256>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
+        if (e != cudaSuccess) return e;
+        grad_wt_reduce_kernel<<<dim3((unsigned)ceil_div(d_out, 32), (unsigned)n_part), 32 * kRedRows * kRedGroups, 0, s>>>(part, n_splits, d_in, d_out, W, ldw, g_wt, col_part);
         ++*launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -827,7 +734,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
         }
     }
     // step 3: Eq. bp-W
-    grad_w_kernel<<<(unsigned)ceil_div(d_out, 32), dim3(32, 32), 0, s>>>(g_wt, W, ldw, alpha, d_in, d_out, g_w, ldgw);
+    grad_w_kernel<<<dim3((unsigned)ceil_div(d_out, 32), (unsigned)ceil_div(d_in, 32)), dim3(32, 32), 0, s>>>(g_wt, col_part, n_part, W, ldw, alpha, d_in, d_out, g_w, ldgw);
     ++*launches;
     return cudaGetLastError();
 }
