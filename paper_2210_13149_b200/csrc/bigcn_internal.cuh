@@ -125,6 +125,9 @@ bool bitgemm_tc_covers(int d_in, int d_out, int64_t stride_a, int64_t stride_b);
 cudaError_t launch_bitgemm_tc(cudaStream_t s, const uint32_t* A, int64_t stride_a, const uint32_t* BT, int64_t stride_b,
                               int64_t n, int d_in, int d_out, const float* beta, const float* alpha, int fmt, void* zeta,
                               int64_t ldz, int32_t* dbg_dot, float* dbg_zeta, float* nws = nullptr, float* col_b0 = nullptr, int row_tail = 0);
+bool bitgemm_takes_wide(int fmt, int64_t n, int d_in, int d_out);
+cudaError_t launch_bitgemm_wide(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
+                                const float* beta, const float* alpha, int fmt, void* zeta, int64_t ldz);
 int bitgemm_tc_timeouts();
 
 // Binning entropy estimate (entropy.cu): scratch = 2 * d uint32.

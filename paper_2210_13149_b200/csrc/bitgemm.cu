@@ -202,6 +202,10 @@ cudaError_t launch_bitgemm(cudaStream_t s, const uint32_t* A, int64_t stride_a,
         ++*launches;
         return launch_bitgemm_tc(s, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, fmt, zeta, ldz, dbg_dot, dbg_zeta, nullptr, nullptr, row_tail);
     }
+    if (path != 1 && !dbg_dot && !dbg_zeta && stride_a == stride_b && (path == 2 ? d_in > 256 && d_out <= 512 && fmt != kZetaI8 : bitgemm_takes_wide(fmt, n, d_in, d_out))) {
+        ++*launches;
+        return launch_bitgemm_wide(s, A, BT, stride_a, n, d_in, d_out, beta, alpha, fmt, zeta, ldz);
+    }
     const int kw = (d_in + 31) / 32;
     const int ldb = kw | 1;
     int tn = 8;

@@ -354,6 +354,187 @@ bitgemm_tc_kernel(const uint32_t* __restrict__ A, int64_t stride_a, const uint32
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(kCols) : "memory");
 }
 
+// The same product for layers of any d_in (more than 256: a tile's expanded rows no longer fit shared memory whole): K in
+// chunks of 256 positions, accumulated in tensor memory.  N = 64 or 128 channels (blockIdx.y: slices of N).  The expanded
+// weight panel stays in shared memory where that leaves room for a second block per multiprocessor or there is at most one tile
+// per multiprocessor (`resident`); otherwise a chunk of it is expanded again with every chunk of rows.  89,250 rows,
+// 500 -> 256: 100 us on the bit-count pipe; see bitgemm_takes_wide() for the line between the two.
+template <int N, int FMT>
+__global__ void __launch_bounds__(kTcThreads, 2)
+bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ BT, int64_t stride,
+                    int64_t n, int d_in, int d_out, const float* __restrict__ beta, const float* __restrict__ alpha,
+                    void* __restrict__ zeta, int64_t ldz, int resident)
+{
+    constexpr int kElt = TcOut<FMT>::kElt;                  // bytes per stored element = 16-byte pieces per chunk of 16 columns
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tmem_base_s;
+    __shared__ float al_s[N];
+    const int ch0 = blockIdx.y * N;                         // this block's channels
+    const int d_here = min(d_out - ch0, N);
+    BT += (int64_t)ch0 * stride;
+    const int K = (int)stride * 32, pieces = (int)(stride >> 2);         // a piece: 16 bytes of a packed row, 128 positions
+    const int pad = K - d_in;                               // padding positions: each contributes +1
+    const int n_chunks = (pieces + 1) >> 1;
+    unsigned char* As = tc_smem;                            // [128][256]; the epilogue's scratch too
+    unsigned char* Bs = tc_smem + kTcRows * 256;            // [N][K], or [N][256]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0) tc::tmem_alloc(&tmem_base_s, N);
+    if (threadIdx.x == 0) tc::barrier_init(&bar);
+    for (int j = threadIdx.x; j < N; j += kTcThreads) al_s[j] = j < d_here ? __ldg(alpha + ch0 + j) : 0.f;
+    if (resident) stage_operand(Bs, N, BT, stride, d_here);
+
+    const int64_t n_tiles = ceil_div(n, kTcRows);
+    const int64_t my_tiles = blockIdx.x < n_tiles ? ceil_div(n_tiles - blockIdx.x, (int64_t)gridDim.x) : 0;
+    auto tile_row0 = [&](int64_t i) { return (blockIdx.x + i * gridDim.x) * (int64_t)kTcRows; };
+    // piece of chunk c that this thread expands: row r, piece q (chunks of one piece: the lower half of the threads)
+    auto qc_of = [&](int c) { return min(2, pieces - 2 * c); };
+    auto fetch = [&](const uint32_t* src, int64_t rows, int c, int items) {
+        const int qc = qc_of(c), r = qc == 2 ? threadIdx.x >> 1 : threadIdx.x, q = qc == 2 ? threadIdx.x & 1 : 0;
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (r < items && r < rows) w = __ldg(reinterpret_cast<const uint4*>(src + r * stride) + 2 * c + q);
+        return w;
+    };
+    auto expand = [&](unsigned char* dst, int items, int64_t rows, int c, const uint4& w) {
+        const int qc = qc_of(c), r = qc == 2 ? threadIdx.x >> 1 : threadIdx.x, q = qc == 2 ? threadIdx.x & 1 : 0;
+        if (r >= items) return;
+        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
+            if (r < rows) expand_word(ws[u], lo, hi);
+            *reinterpret_cast<uint4*>(dst + canon_off(items, r, 2 * (4 * q + u))) = lo;
+            *reinterpret_cast<uint4*>(dst + canon_off(items, r, 2 * (4 * q + u) + 1)) = hi;
+        }
+    };
+    uint4 pre = make_uint4(0u, 0u, 0u, 0u), pre_b = pre;
+    if (my_tiles > 0) {
+        pre = fetch(A + tile_row0(0) * stride, n - tile_row0(0), 0, kTcRows);
+        if (!resident) pre_b = fetch(BT, d_here, 0, N);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem_base = tmem_base_s;
+    // instruction descriptor: D = s32, A = B = s8, both K-major, N, M = 128
+    const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
+    const uint32_t a_lbo = (kTcRows >> 3) * 128, b_lbo = (N >> 3) * 128, sbo = 128;
+    const int lane_base = 32 * (warp & 3);                  // a warp reads tensor-memory lanes 32 (warp % 4) .. + 31
+    const int c_begin = (warp >> 2) * (N / 2);              // warps 0-3: lower half of the columns, 4-7: upper half
+    constexpr int kRowBytes = (N / 2) * kElt;
+    constexpr int kPpr = kRowBytes >= 128 ? 8 : kRowBytes / 16;     // 16-byte pieces per row and pass (128 bytes at most)
+    constexpr int kChunksPerPass = kPpr / kElt;
+    constexpr int kPasses = kRowBytes / (16 * kPpr);
+    static_assert(kPpr % kElt == 0 && kRowBytes % (16 * kPpr) == 0, "a pass is a whole number of 16-column chunks");
+    unsigned char* scr = As + warp * 4096;                  // 32 rows x 128 bytes; piece p of row r at r * 128 + ((p ^ (r & 7)) * 16)
+    bool ok = true;
+    uint32_t phase = 0;
+    for (int64_t i = 0; i < my_tiles && ok; ++i) {
+        const int64_t rows = n - tile_row0(i);
+        for (int c = 0; c < n_chunks; ++c) {
+            expand(As, kTcRows, rows, c, pre);
+            if (!resident) expand(Bs, N, d_here, c, pre_b);
+            tc::fence_async_smem();
+            tc::fence_before_sync();
+            __syncthreads();
+            tc::fence_after_sync();
+            if (threadIdx.x == 0) {
+                const uint32_t a_base = smem_u32(As), b_base = smem_u32(Bs) + (resident ? 16u * (uint32_t)c * b_lbo : 0u);
+                for (int ks = 0; ks < 4 * qc_of(c); ++ks) {
+                    const uint64_t ad = make_desc(a_base + 2 * ks * a_lbo, a_lbo, sbo);
+                    const uint64_t bd = make_desc(b_base + 2 * ks * b_lbo, b_lbo, sbo);
+                    const uint32_t accum = c > 0 || ks > 0 ? 1u : 0u;
+                    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}\n"
+                                 ::"r"(tmem_base), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
+                }
+                tc::commit_to(&bar);
+            }
+            // the next chunk's bits, in flight while the products run
+            const bool last = c + 1 == n_chunks;
+            const int64_t r1 = tile_row0(last ? i + 1 : i);
+            if (!last || i + 1 < my_tiles) {
+                pre = fetch(A + r1 * stride, n - r1, last ? 0 : c + 1, kTcRows);
+                if (!resident) pre_b = fetch(BT, d_here, last ? 0 : c + 1, N);
+            }
+            if (!wait_barrier(&bar, phase)) {
+                atomicExch(&g_tc_timeout, 1);
+                ok = false;
+            }
+            phase ^= 1u;
+            tc::fence_after_sync();
+            if (__syncthreads_or(!ok)) { ok = false; break; }   // leave together if any wait ran out
+        }
+        if (!ok) break;
+        // ---- epilogue: a thread owns row lane_base + lane and walks over its warp's half of the columns
+        const int64_t row0 = tile_row0(i) + lane_base;
+        const float be = (FMT == kZetaF32 && row0 + lane < n) ? __ldg(beta + row0 + lane) : 0.f;
+#pragma unroll 1
+        for (int pass = 0; pass < kPasses; ++pass) {
+#pragma unroll
+            for (int ch = 0; ch < kChunksPerPass; ++ch) {
+                const int c0 = c_begin + (pass * kChunksPerPass + ch) * 16;
+                uint32_t v[16];
+                tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)c0, v);
+                int dot[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) dot[e] = (c0 + e < d_here) ? (int)v[e] - pad : 0;    // padding columns of zeta stay 0
+                uint4 out[kElt];
+                if constexpr (FMT == kZetaF16) {            // exact for |dot| <= 2048: int -> float without the conversion unit, then to half
+                    uint32_t h[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const __half2 r = __floats2half2_rn(__int_as_float(0x4B400000 + dot[2 * q]) - 12582912.f, __int_as_float(0x4B400000 + dot[2 * q + 1]) - 12582912.f);
+                        h[q] = *reinterpret_cast<const uint32_t*>(&r);
+                    }
+                    out[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                    out[1] = make_uint4(h[4], h[5], h[6], h[7]);
+                } else {
+                    TcOut<FMT>::pack(dot, be, al_s + c0, out);
+                }
+#pragma unroll
+                for (int u = 0; u < kElt; ++u) {
+                    const int piece = ch * kElt + u;
+                    *reinterpret_cast<uint4*>(scr + lane * 128 + ((piece ^ (lane & 7)) * 16)) = out[u];
+                }
+            }
+            __syncwarp();
+            // write the 32 rows x kPpr pieces out: a warp instruction covers 32 / kPpr whole row segments
+            const int64_t byte0 = (int64_t)(ch0 + c_begin + pass * kChunksPerPass * 16) * kElt;
+#pragma unroll
+            for (int it = 0; it < kPpr; ++it) {
+                const int r = it * (32 / kPpr) + lane / kPpr, pc = lane % kPpr;
+                const uint4 val = *reinterpret_cast<const uint4*>(scr + r * 128 + ((pc ^ (r & 7)) * 16));
+                const int64_t at = byte0 + pc * 16;
+                if (row0 + r < n && at < ldz * kElt)
+                    *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(zeta) + (row0 + r) * ldz * kElt + at) = val;
+            }
+            __syncwarp();
+        }
+        tc::fence_before_sync();
+        __syncthreads();                                    // the scratch is the next tile's operand space
+        tc::fence_after_sync();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_free(tmem_base, N);
+}
+
+template <int N, int FMT>
+cudaError_t launch_wide_inst(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
+                             const float* beta, const float* alpha, void* zeta, int64_t ldz)
+{
+    const int64_t tiles = ceil_div(n, kTcRows), gy = ceil_div(d_out, N);
+    const size_t panel = (size_t)N * stride * 32, a_bytes = (size_t)kTcRows * 256;
+    const bool resident = a_bytes + panel <= 110 * 1024 || (a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count());
+    const size_t smem = a_bytes + (resident ? panel : (size_t)N * 256);
+    cudaError_t e = cudaFuncSetAttribute(bitgemm_wide_kernel<N, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t fit = std::max<int64_t>(1, std::min<int64_t>(2, (int64_t)(227 * 1024) / (int64_t)(smem + 2048)));
+    const unsigned gx = (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, sm_count() * fit / gy));
+    bitgemm_wide_kernel<N, FMT><<<dim3(gx, (unsigned)gy), kTcThreads, smem, s>>>(A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz, resident ? 1 : 0);
+    return cudaGetLastError();
+}
+
 template <int N, int FMT>
 cudaError_t launch_tc_inst(cudaStream_t s, const uint32_t* A, int64_t stride_a, const uint32_t* BT, int64_t stride_b,
                            int64_t n, int d_in, int d_out, const float* beta, const float* alpha, void* zeta, int64_t ldz,
@@ -410,6 +591,31 @@ cudaError_t launch_bitgemm_tc(cudaStream_t s, const uint32_t* A, int64_t stride_
     if (d_out <= 64) return launch_tc_n<64>(s, fmt, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, row_tail);
     if (d_out <= 128) return launch_tc_n<128>(s, fmt, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, 0);
     return launch_tc_n<256>(s, fmt, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, 0);
+}
+
+// Whether a layer of more than 256 inputs runs on the tensor cores: from 3 x 2^23 word steps (rows x channels x packed words)
+// on.  Below, the bit-count kernel's smaller tiles occupy more of the GPU (a layer, bit counts -> tensor cores: 3,300 rows
+// 3,703 -> 64 25 -> 38 us, 8,000 rows 500 -> 256 29 -> 25 us, 89,250 rows 500 -> 256 157 -> 93 us, 233,000 rows 602 -> 256
+// 427 -> 247 us, all with the aggregation of an empty graph).
+bool bitgemm_takes_wide(int fmt, int64_t n, int d_in, int d_out)
+{
+    return d_in > 256 && d_out <= 512 && (fmt == kZetaF32 || fmt == kZetaF16 || fmt == kZetaI16) &&
+           n * (int64_t)d_out * ceil_div(d_in, 32) >= (int64_t(3) << 23);
+}
+
+cudaError_t launch_bitgemm_wide(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
+                                const float* beta, const float* alpha, int fmt, void* zeta, int64_t ldz)
+{
+#define BIGCN_WIDE_CALL(FMT) \
+    return d_out <= 64 ? launch_wide_inst<64, FMT>(s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz) \
+                       : launch_wide_inst<128, FMT>(s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz)
+    switch (fmt) {
+        case kZetaF32: BIGCN_WIDE_CALL(kZetaF32);
+        case kZetaF16: BIGCN_WIDE_CALL(kZetaF16);
+        case kZetaI16: BIGCN_WIDE_CALL(kZetaI16);
+        default: return cudaErrorInvalidValue;
+    }
+#undef BIGCN_WIDE_CALL
 }
 
 // Number of waits that ran out since the library was loaded on the current device (0 = none).
