@@ -24,6 +24,7 @@ constexpr int kBwThreads = 256;       // 8 warps per block
 __global__ void pad_rows_kernel(const float* __restrict__ src, int64_t n, int d, int64_t ld_in,
                                 float* __restrict__ dst, int64_t ld_out)
 {
+    pdl_enter();
     const int64_t total = n * ld_out;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / ld_out;
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(32 * kRedRows * kRedGroups)
 grad_wt_reduce_kernel(const float* __restrict__ part, int n_splits, int d_in, int d_out, const float* __restrict__ W, int64_t ldw,
                       float* __restrict__ g_wt, double* __restrict__ col_part /* [ceil(d_in / 4)][d_out] */)
 {
+    pdl_enter();
     __shared__ double s_sum[kRedGroups][kRedRows][33];
     const int tx = threadIdx.x & 31, r = (threadIdx.x >> 5) % kRedRows, zg = threadIdx.x / (32 * kRedRows);
     const int j = blockIdx.x * 32 + tx, k = blockIdx.y * kRedRows + r;
@@ -143,6 +145,7 @@ grad_h_mma_kernel(const float* __restrict__ gz, int64_t ldz, const float* __rest
                   const float* __restrict__ W, int64_t ldw, int64_t n, int d_in, int d_out,
                   float* __restrict__ g_h, int64_t ldh)
 {
+    pdl_enter();
     __shared__ __align__(16) unsigned short As[3 * kMmaTile * kMmaPitch];
     __shared__ __align__(16) unsigned short Bs[kMmaTile * kMmaPitch];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -229,6 +232,7 @@ grad_h_tc_kernel(const float* __restrict__ gz, int64_t ldz, const float* __restr
                  const float* __restrict__ W, int64_t ldw, int64_t n, int d_in, int d_out,
                  float* __restrict__ g_h, int64_t ldh)
 {
+    pdl_enter();
     constexpr int kRows = 128, kKc = 64;                   // tile rows; reduction elements per chunk
     constexpr int kCols = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
     extern __shared__ __align__(128) unsigned char bw_smem[];
@@ -425,6 +429,7 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
                   const float* __restrict__ gz, int64_t ldz, int64_t n, int d_in, int d_out,
                   int64_t rows_per_split, float* __restrict__ part)
 {
+    pdl_enter();
     constexpr int kStage = 6 * kWtAtom + N / 64 * kWtAtom;  // three terms x two atoms of channels, N / 64 atoms of inputs
     constexpr int kItems = kWtNodes * 32 / kBwThreads;      // 16-byte pieces of a chunk per thread
     extern __shared__ unsigned char bw_raw[];
@@ -571,7 +576,7 @@ cudaError_t launch_grad_wt_tc(cudaStream_t s, const uint32_t* bits, int64_t stri
     cudaError_t e = cudaFuncSetAttribute(grad_wt_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)ceil_div(d_out, 128), (unsigned)n_splits, (unsigned)ceil_div(d_in, N));
-    grad_wt_tc_kernel<N><<<grid, kBwThreads, smem, s>>>(bits, stride, beta, gz, ldz, n, d_in, d_out, rows_per_split, part);
+    launch_kernel(grad_wt_tc_kernel<N>, grid, kBwThreads, smem, s, bits, stride, beta, gz, ldz, n, d_in, d_out, rows_per_split, part);
     return cudaGetLastError();
 }
 
@@ -583,7 +588,7 @@ cudaError_t launch_grad_h_tc(cudaStream_t s, const float* gz, int64_t ldz, const
     cudaError_t e = cudaFuncSetAttribute(grad_h_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 128), sm_count() * 2);
-    grad_h_tc_kernel<N><<<grid, kBwThreads, smem, s>>>(gz, ldz, alpha, W, ldw, n, d_in, d_out, g_h, ldh);
+    launch_kernel(grad_h_tc_kernel<N>, grid, kBwThreads, smem, s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_h, ldh);
     return cudaGetLastError();
 }
 
@@ -594,6 +599,7 @@ __global__ void __launch_bounds__(1024)
 grad_w_kernel(const float* __restrict__ g_wt, const double* __restrict__ col_part, int n_part, const float* __restrict__ W, int64_t ldw,
               const float* __restrict__ alpha, int d_in, int d_out, float* __restrict__ g_w, int64_t ldgw)
 {
+    pdl_enter();
     __shared__ double part[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int j = blockIdx.x * 32 + tx, i = blockIdx.y * 32 + ty;
@@ -674,7 +680,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     // step 1a: G_zeta = A_tilde^T G' (A_tilde is symmetric: the forward aggregation on fp32 rows)
     const float* g_src = g_out;
     if (ldg != ldz || reinterpret_cast<uintptr_t>(g_out) % 16 != 0) {            // rows must be 16-byte vectors
-        pad_rows_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n * ldz, 256), sm_count() * 16), 256, 0, s>>>(g_out, n, d_out, ldg, g_pad, ldz);
+        launch_kernel(pad_rows_kernel, (unsigned)std::min<int64_t>(ceil_div(n * ldz, 256), sm_count() * 16), 256, 0, s, g_out, n, d_out, ldg, g_pad, ldz);
         ++*launches;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -715,7 +721,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
         else if (d_in <= 128) e = launch_grad_wt_tc<128>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
         else e = launch_grad_wt_tc<256>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
         if (e != cudaSuccess) return e;
-        grad_wt_reduce_kernel<<<dim3((unsigned)ceil_div(d_out, 32), (unsigned)n_part), 32 * kRedRows * kRedGroups, 0, s>>>(part, n_splits, d_in, d_out, W, ldw, g_wt, col_part);
+        launch_kernel(grad_wt_reduce_kernel, dim3((unsigned)ceil_div(d_out, 32), (unsigned)n_part), 32 * kRedRows * kRedGroups, 0, s, part, n_splits, d_in, d_out, W, ldw, g_wt, col_part);
         ++*launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -729,12 +735,12 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
             if (e != cudaSuccess) return e;
         } else {
             const dim3 grid((unsigned)ceil_div(n, kMmaTile), (unsigned)ceil_div(d_in, kMmaTile));
-            grad_h_mma_kernel<<<grid, kBwThreads, 0, s>>>(gz, ldz, alpha, W, ldw, n, d_in, d_out, g_in, ldgi);
+            launch_kernel(grad_h_mma_kernel, grid, kBwThreads, 0, s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_in, ldgi);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
     // step 3: Eq. bp-W
-    grad_w_kernel<<<dim3((unsigned)ceil_div(d_out, 32), (unsigned)ceil_div(d_in, 32)), dim3(32, 32), 0, s>>>(g_wt, col_part, n_part, W, ldw, alpha, d_in, d_out, g_w, ldgw);
+    launch_kernel(grad_w_kernel, dim3((unsigned)ceil_div(d_out, 32), (unsigned)ceil_div(d_in, 32)), dim3(32, 32), 0, s, g_wt, col_part, n_part, W, ldw, alpha, d_in, d_out, g_w, ldgw);
     ++*launches;
     return cudaGetLastError();
 }

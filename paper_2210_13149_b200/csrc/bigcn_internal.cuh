@@ -29,6 +29,31 @@ inline int zeta_elt_bytes(int fmt) { return fmt == kZetaF32 ? 4 : ((fmt == kZeta
 // fails, so that a grid derived from it stays valid).  Persistent grids are sized from it.
 int sm_count();
 
+// Programmatic dependent launch: a kernel started by launch_kernel() may be set up while the one before it on the stream still
+// runs -- a forward of a small graph is five kernels of 4 to 12 us with 2 us between them otherwise.  It therefore begins with
+// pdl_enter(): lets the kernel after it be set up likewise, and waits until the one before it is done and its writes are
+// visible.  (Transitive: a kernel is done only after its own wait.)
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- launchers (each returns the launch status; all asynchronous on `s`) ------------------------
 
 cudaError_t launch_pack_rows(cudaStream_t s, const float* H, int64_t n, int d, int64_t ld,

@@ -30,6 +30,7 @@ bitgemm_kernel(const uint32_t* __restrict__ A, int64_t stride_a,
                void* __restrict__ zeta, int64_t ldz,
                int32_t* __restrict__ dbg_dot, float* __restrict__ dbg_zeta)
 {
+    pdl_enter();
     constexpr int kTM = RW < 4 ? RW : 4, kRowsPerWarp = RW, kTileRows = RW * kGemmWarps;
     extern __shared__ __align__(16) uint32_t smem[];
     uint32_t* Bs = smem;                                   // [TN*32][ldb]
@@ -149,7 +150,7 @@ cudaError_t launch_inst(cudaStream_t s, const uint32_t* A, int64_t stride_a, con
     const int64_t n_tiles = ceil_div(n, RW * kGemmWarps);
     const unsigned gy = (unsigned)ceil_div(d_out, TN * 32);
     const unsigned gx = (unsigned)std::min<int64_t>(n_tiles, sm_count() * 8);
-    bitgemm_kernel<TN, FMT, DBG, RW><<<dim3(gx, gy), kGemmThreads, smem_bytes, s>>>(
+    launch_kernel(bitgemm_kernel<TN, FMT, DBG, RW>, dim3(gx, gy), kGemmThreads, smem_bytes, s, 
         A, stride_a, BT, stride_b, n, d_in, d_out, kw, ldb, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta);
     return cudaGetLastError();
 }

@@ -146,6 +146,7 @@ bitgemm_tc_kernel(const uint32_t* __restrict__ A, int64_t stride_a, const uint32
                   void* __restrict__ zeta, int64_t ldz, int32_t* __restrict__ dbg_dot, float* __restrict__ dbg_zeta,
                   float* __restrict__ nws, float* __restrict__ col_b0, int row_tail)
 {
+    pdl_enter();
     // row_tail (byte formats, N = 64, d_out <= 60): a row of zeta is 64 bytes and its last four bytes hold the row's
     // node factor as a float (beta_i, with the first feature sign for half-dot bytes), so that the aggregation of a
     // last layer fetches an entry's dots and its factor with one pair of 32-byte loads
@@ -365,6 +366,7 @@ bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__
                     int64_t n, int d_in, int d_out, const float* __restrict__ beta, const float* __restrict__ alpha,
                     void* __restrict__ zeta, int64_t ldz, int resident)
 {
+    pdl_enter();
     constexpr int kElt = TcOut<FMT>::kElt;                  // bytes per stored element = 16-byte pieces per chunk of 16 columns
     extern __shared__ __align__(128) unsigned char tc_smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -531,7 +533,7 @@ cudaError_t launch_wide_inst(cudaStream_t s, const uint32_t* A, const uint32_t* 
     if (e != cudaSuccess) return e;
     const int64_t fit = std::max<int64_t>(1, std::min<int64_t>(2, (int64_t)(227 * 1024) / (int64_t)(smem + 2048)));
     const unsigned gx = (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, sm_count() * fit / gy));
-    bitgemm_wide_kernel<N, FMT><<<dim3(gx, (unsigned)gy), kTcThreads, smem, s>>>(A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz, resident ? 1 : 0);
+    launch_kernel(bitgemm_wide_kernel<N, FMT>, dim3(gx, (unsigned)gy), kTcThreads, smem, s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz, resident ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -552,7 +554,7 @@ cudaError_t launch_tc_inst(cudaStream_t s, const uint32_t* A, int64_t stride_a, 
         // persistent blocks: as many as stay resident (tensor-memory columns, registers, and shared memory: 227 KB per SM)
         const int fit = (int)std::max<size_t>(1, std::min<size_t>((size_t)blocks_per_sm, (size_t)(227 * 1024) / (smem + 2048)));
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, kTcRows), (int64_t)sm_count() * fit);
-        kernel<<<grid, kTcThreads, smem, s>>>(A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, row_tail);
+        launch_kernel(kernel, grid, kTcThreads, smem, s, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, row_tail);
         return cudaGetLastError();
     };
     if (debug) return launch(bitgemm_tc_kernel<N, FMT, true>, 2);

@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(kEntThreads)
 range_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int64_t rows_per_block,
              uint32_t* __restrict__ key_min, uint32_t* __restrict__ key_max)
 {
+    pdl_enter();
     __shared__ float s_lo[kEntWarps][kWarp], s_hi[kEntWarps][kWarp];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = blockIdx.y * 32 + lane;
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(kEntThreads)
 init_kernel(uint32_t* __restrict__ key_min, uint32_t* __restrict__ key_max, int d, uint32_t* __restrict__ counts, int64_t n_counts,
             double* __restrict__ total)
 {
+    pdl_enter();
     const int64_t i0 = (int64_t)blockIdx.x * kEntThreads + threadIdx.x, step = (int64_t)gridDim.x * kEntThreads;
     for (int64_t i = i0; i < n_counts; i += step) counts[i] = 0u;
     for (int64_t i = i0; i < d; i += step) {
@@ -95,6 +97,7 @@ histogram_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int 
                  const uint32_t* __restrict__ key_min, const uint32_t* __restrict__ key_max,
                  float* __restrict__ col_min, float* __restrict__ col_max, uint32_t* __restrict__ counts)
 {
+    pdl_enter();
     extern __shared__ uint32_t hist[];                    // [n_bins][CW]
     constexpr int RPW = kWarp / CW;                       // rows per warp instruction
     constexpr int RPB = RPW * (kHistThreads / kWarp);     // rows per block step
@@ -150,6 +153,7 @@ histogram_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int 
 __global__ void __launch_bounds__(kEntThreads)
 entropy_kernel(const uint32_t* __restrict__ counts, int d, int n_bins, int64_t n, double* entropy, double* total)
 {
+    pdl_enter();
     __shared__ bool last_block;
     __shared__ double part[kEntWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -200,7 +204,7 @@ cudaError_t launch_histogram(cudaStream_t s, const float* H, int64_t n, int d, i
     // as many as it has counters to add up at the end
     const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, std::max(1024, n_bins)), (int64_t)sm_count() * per_sm / gy));
     const int64_t rows_per_block = ceil_div(n, gx);
-    histogram_kernel<CW><<<dim3((unsigned)gx, gy), kHistThreads, smem, s>>>(H, n, d, ld, n_bins, rows_per_block, key_min,
+    launch_kernel(histogram_kernel<CW>, dim3((unsigned)gx, gy), kHistThreads, smem, s, H, n, d, ld, n_bins, rows_per_block, key_min,
                                                                          key_max, col_min, col_max, counts);
     return cudaGetLastError();
 }
@@ -218,14 +222,14 @@ cudaError_t launch_entropy_bins(cudaStream_t s, const float* H, int64_t n, int d
     uint32_t* key_min = static_cast<uint32_t*>(scratch);
     uint32_t* key_max = key_min + d;
     const int64_t n_counts = (int64_t)d * n_bins;
-    init_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n_counts, kEntThreads * 4), (int64_t)sm_count() * 8), kEntThreads, 0, s>>>(key_min, key_max, d, counts, n_counts, total);
+    launch_kernel(init_kernel, (unsigned)std::min<int64_t>(ceil_div(n_counts, kEntThreads * 4), (int64_t)sm_count() * 8), kEntThreads, 0, s, key_min, key_max, d, counts, n_counts, total);
     ++*launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     {
         const unsigned gy = (unsigned)ceil_div(d, 32);
         const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), ceil_div((int64_t)sm_count() * 8, gy)));
-        range_kernel<<<dim3((unsigned)gx, gy), kEntThreads, 0, s>>>(H, n, d, ld, ceil_div(n, gx), key_min, key_max);
+        launch_kernel(range_kernel, dim3((unsigned)gx, gy), kEntThreads, 0, s, H, n, d, ld, ceil_div(n, gx), key_min, key_max);
         ++*launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -236,7 +240,7 @@ cudaError_t launch_entropy_bins(cudaStream_t s, const float* H, int64_t n, int d
     else e = launch_histogram<4>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
     ++*launches;
     if (e != cudaSuccess) return e;
-    entropy_kernel<<<(unsigned)d, kEntThreads, 0, s>>>(counts, d, n_bins, n, entropy, total);
+    launch_kernel(entropy_kernel, (unsigned)d, kEntThreads, 0, s, counts, d, n_bins, n, entropy, total);
     ++*launches;
     return cudaGetLastError();
 }

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(256)
 col_partial_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int64_t rows_per_chunk,
                    double* __restrict__ partial /* [chunks][d][2] */)
 {
+    pdl_enter();
     __shared__ double s_sum[8][33], s_sq[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + tx;
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(1024)
 col_final_kernel(const float* __restrict__ H, const double* __restrict__ partial, int chunks, int d, int64_t n, double eps,
                  float* __restrict__ shift, float* __restrict__ scale)
 {
+    pdl_enter();
     __shared__ double s_sum[32][33], s_sq[32][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + tx;
@@ -274,11 +276,11 @@ cudaError_t launch_col_stats(cudaStream_t s, const float* H, int64_t n, int d, i
     const int64_t rows_per_chunk = std::max<int64_t>(64, ceil_div(n, kStatChunksMax));
     const int chunks = (int)std::max<int64_t>(1, ceil_div(n, rows_per_chunk));
     double* partial = reinterpret_cast<double*>(scratch);
-    col_partial_kernel<<<dim3((unsigned)ceil_div(d, 32), (unsigned)chunks), 256, 0, s>>>(H, n, d, ld, rows_per_chunk, partial);
+    launch_kernel(col_partial_kernel, dim3((unsigned)ceil_div(d, 32), (unsigned)chunks), 256, 0, s, H, n, d, ld, rows_per_chunk, partial);
     ++*launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    col_final_kernel<<<(unsigned)ceil_div(d, 32), 1024, 0, s>>>(H, partial, chunks, d, n, (double)eps, shift, scale);
+    launch_kernel(col_final_kernel, (unsigned)ceil_div(d, 32), 1024, 0, s, H, partial, chunks, d, n, (double)eps, shift, scale);
     ++*launches;
     return cudaGetLastError();
 }

@@ -23,6 +23,7 @@ pack_rows_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld,
                  const float* __restrict__ shift, const float* __restrict__ scale,
                  uint32_t* __restrict__ bits, int64_t stride, float* __restrict__ beta)
 {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = (int64_t)blockIdx.x * kPackWarpsPerBlock + (threadIdx.x >> 5);
     const int64_t n_warps = (int64_t)gridDim.x * kPackWarpsPerBlock;
@@ -56,7 +57,7 @@ pack_rows_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld,
                 }
             };
             // rows of many words: the next chunk is asked for before this one is packed
-            constexpr bool kAhead = R <= 2;
+            constexpr bool kAhead = R == 1;
             if (kAhead) load(w0);
             for (int c0 = w0; c0 < wlast; c0 += WC) {
                 if (!kAhead) load(c0);
@@ -136,6 +137,7 @@ pack_rows_staged_kernel(const float* __restrict__ H, int64_t n, int d, int64_t l
                         const float* __restrict__ shift, const float* __restrict__ scale,
                         uint32_t* __restrict__ bits, int64_t stride, float* __restrict__ beta)
 {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char pack_smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(1024)
 pack_weights_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ldw,
                     uint32_t* __restrict__ bitsT, int64_t stride)
 {
+    pdl_enter();
     __shared__ unsigned char sgn[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int j0 = blockIdx.x * 32;
@@ -254,6 +257,7 @@ pack_weights_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ld
 __global__ void __launch_bounds__(1024)
 weight_scale_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ldw, float* __restrict__ alpha)
 {
+    pdl_enter();
     __shared__ double part[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int j = blockIdx.x * 32 + tx;
@@ -304,7 +308,7 @@ cudaError_t launch_pack_rows(cudaStream_t s, const float* H, int64_t n, int d, i
             per_sm = c.per_sm, n_sm = c.n_sm;
         }
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, (int64_t)kPackWarpsPerBlock * kStageRows), (int64_t)n_sm * std::max(per_sm, 1));
-        kernel<<<grid, kPackWarpsPerBlock * kWarp, staged_smem, s>>>(H, n, d, ld, shift, scale, bits, stride, beta);
+        launch_kernel(kernel, grid, kPackWarpsPerBlock * kWarp, staged_smem, s, H, n, d, ld, shift, scale, bits, stride, beta);
         ++*launches;
         return cudaGetLastError();
     }
@@ -313,7 +317,7 @@ cudaError_t launch_pack_rows(cudaStream_t s, const float* H, int64_t n, int d, i
     const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, (int64_t)kPackWarpsPerBlock * rows), sm_count() * 8);
     const dim3 block(kPackWarpsPerBlock * kWarp);
 #define BIGCN_PACK_LAUNCH(NORM, R, WC) \
-    pack_rows_kernel<NORM, R, WC><<<grid, block, 0, s>>>(H, n, d, ld, shift, scale, bits, stride, beta)
+    launch_kernel(pack_rows_kernel<NORM, R, WC>, grid, block, 0, s, H, n, d, ld, shift, scale, bits, stride, beta)
     if (shift) {
         if (rows == 8) BIGCN_PACK_LAUNCH(true, 8, 4);
         else if (rows == 4) BIGCN_PACK_LAUNCH(true, 4, 8);
@@ -335,11 +339,11 @@ cudaError_t launch_pack_weights(cudaStream_t s, const float* W, int d_in, int d_
 {
     const dim3 block(32, 32);
     const dim3 grid((unsigned)ceil_div(d_out, 32), (unsigned)stride);
-    pack_weights_kernel<<<grid, block, 0, s>>>(W, d_in, d_out, ldw, bitsT, stride);
+    launch_kernel(pack_weights_kernel, grid, block, 0, s, W, d_in, d_out, ldw, bitsT, stride);
     ++*launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    weight_scale_kernel<<<(unsigned)ceil_div(d_out, 32), block, 0, s>>>(W, d_in, d_out, ldw, alpha);
+    launch_kernel(weight_scale_kernel, (unsigned)ceil_div(d_out, 32), block, 0, s, W, d_in, d_out, ldw, alpha);
     ++*launches;
     return cudaGetLastError();
 }

@@ -1404,6 +1404,7 @@ template <int NV, bool kHalf, bool kTail = false, bool kNext = false>
 __global__ void __launch_bounds__(kLaneThreads, 2)
 spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
 {
+    pdl_enter();
     constexpr int NG4 = 4 * NV;
     extern __shared__ __align__(16) float lsm[];
     __shared__ int64_t long_rows[kLongQueue];
@@ -1436,10 +1437,11 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
     const int64_t n_runs = ceil_div(p.n, rows_per_warp);
     float4 t;
     float ws, wg;
-    for (;;) {
-        int64_t run = 0;
-        if (lane == 0) run = atomicAdd(p.run_counter, 1);
-        run = __shfl_sync(0xffffffffu, run, 0);
+    for (int64_t run = (int64_t)blockIdx.x * kLaneWarps + warp;; run = n_runs) {     // no counter: a run per warp at most
+        if (p.run_counter) {
+            if (lane == 0) run = atomicAdd(p.run_counter, 1);
+            run = __shfl_sync(0xffffffffu, run, 0);
+        }
         if (run >= n_runs) break;
         const int64_t warp_row0 = run * rows_per_warp;
         const int n_rows = (int)min((int64_t)rows_per_warp, p.n - warp_row0);
@@ -1531,11 +1533,12 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
     const int rows_per_warp = (int)std::min<int64_t>(kMaxRowsPerWarp, std::max<int64_t>(1, p.n / (kLaneWarps * sm_count() * 8)));
     cudaError_t e = cudaFuncSetAttribute(spmm_lane_kernel<NV, kHalf, kTail, kNext>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
     const int64_t wanted = ceil_div(ceil_div(p.n, rows_per_warp), kLaneWarps);
     const unsigned grid = (unsigned)std::min<int64_t>(wanted, sm_count() * 2);
-    spmm_lane_kernel<NV, kHalf, kTail, kNext><<<grid, kLaneThreads, smem, s>>>(p, rows_per_warp);
+    SpmmDev q = p;
+    if (wanted <= grid) q.run_counter = nullptr;              // a run per warp: nothing to hand out
+    else if ((e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s)) != cudaSuccess) return e;
+    launch_kernel(spmm_lane_kernel<NV, kHalf, kTail, kNext>, grid, kLaneThreads, smem, s, q, rows_per_warp);
     return cudaGetLastError();
 }
 
@@ -1604,6 +1607,7 @@ template <typename T, int LPR>
 __global__ void __launch_bounds__(kSpmmThreads, row_blocks(sizeof(T)))
 spmm_rows_kernel(const SpmmDev p, int rows_per_take, int dynamic)
 {
+    pdl_enter();
     constexpr int EPV = Elt<T>::kPerVec, kCols = LPR * EPV, S = row_lanes(LPR), R = 32 / S;
     using Set = RowSet<T, LPR, S>;
     using Wide = RowSet<T, LPR, 32>;
@@ -1758,6 +1762,7 @@ template <typename T, int NCH, int LPR, bool kFull, bool kAligned, bool kHalf = 
 __global__ void __launch_bounds__(kSpmmThreads, spmm_blocks_per_sm<NCH, LPR, kAligned, (int)sizeof(T)>())
 spmm_kernel(const SpmmDev p, int rows_per_warp)
 {
+    pdl_enter();
     static_assert(!kHalf || (sizeof(T) == 1 && LPR < 32), "half-dot bytes: rows of up to 256 signed bytes");
     static_assert(!kAligned || ((NCH == 1 || NCH == 2) && (LPR == 4 || LPR == 8 || LPR == 16)), "the multi-entry stream: 4, 8 or 16 lanes per row, one or two vectors per lane");
     using P = Pipe<NCH, LPR, kAligned>;
@@ -1780,10 +1785,11 @@ spmm_kernel(const SpmmDev p, int rows_per_warp)
 
     const int64_t n_runs = ceil_div(p.n, rows_per_warp);
     float acc[NCH][EPV];
-    for (;;) {
-        int64_t run = 0;
-        if (lane == 0) run = atomicAdd(p.run_counter, 1);
-        run = __shfl_sync(0xffffffffu, run, 0);
+    for (int64_t run = (int64_t)blockIdx.x * kSpmmWarps + warp;; run = n_runs) {     // no counter: a run per warp at most
+        if (p.run_counter) {
+            if (lane == 0) run = atomicAdd(p.run_counter, 1);
+            run = __shfl_sync(0xffffffffu, run, 0);
+        }
         if (run >= n_runs) break;
         const int64_t warp_row0 = run * rows_per_warp;
         const int n_rows = (int)min((int64_t)rows_per_warp, p.n - warp_row0);
@@ -1865,12 +1871,17 @@ cudaError_t launch_one(cudaStream_t s, const SpmmDev& p)
         cudaError_t e = cudaFuncSetAttribute(spmm_kernel<T, NCH, LPR, kFull, kAligned, kHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
     // one wave of resident blocks; the warps pull runs of rows until none are left
     const int64_t wanted = ceil_div(ceil_div(p.n, rows_per_warp), kSpmmWarps);
     const unsigned grid = (unsigned)std::min<int64_t>(wanted, sm_count() * spmm_blocks_per_sm<NCH, LPR, kAligned, (int)sizeof(T)>());
-    spmm_kernel<T, NCH, LPR, kFull, kAligned, kHalf><<<grid, kSpmmThreads, smem, s>>>(p, rows_per_warp);
+    SpmmDev q = p;
+    if (wanted <= grid) {
+        q.run_counter = nullptr;                              // a run per warp: nothing to hand out
+    } else {
+        cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
+    launch_kernel(spmm_kernel<T, NCH, LPR, kFull, kAligned, kHalf>, grid, kSpmmThreads, smem, s, q, rows_per_warp);
     return cudaGetLastError();
 }
 
@@ -1903,7 +1914,7 @@ cudaError_t launch_rows(cudaStream_t s, const SpmmDev& p, double mean_row)
         cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
-    spmm_rows_kernel<T, LPR><<<(unsigned)ceil_div(std::min(takes, warps), kSpmmWarps), kSpmmThreads, 0, s>>>(p, rows_per_take, dynamic);
+    launch_kernel(spmm_rows_kernel<T, LPR>, (unsigned)ceil_div(std::min(takes, warps), kSpmmWarps), kSpmmThreads, 0, s, p, rows_per_take, dynamic);
     return cudaGetLastError();
 }
 

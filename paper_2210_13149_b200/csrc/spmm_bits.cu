@@ -167,6 +167,7 @@ struct Walk {
 __global__ void __launch_bounds__(128) plan_kernel(const int64_t* __restrict__ rowptr, int n, int chunk_log2, int chunks,
                                                    int4* __restrict__ groups, int2* __restrict__ units, unsigned* __restrict__ used)
 {
+    pdl_enter();
     const int u = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (u >= chunks) return;
     Walk w{rowptr, n};
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const int64_t* __restrict__ r
 template <int K>
 __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_kernel(const AggDev d)
 {
+    pdl_enter();
     constexpr int kLaneBytes = K / 64;              // byte columns of a row that a lane takes: g, g + 8, ...
     constexpr int MT = K / 16;                      // 16-column products per window, and values per lane after the read-back
     constexpr int kAggWarps = agg_warps(K);
@@ -610,6 +612,7 @@ struct GemmDev {
 template <int NM, bool kBitsOnly, bool kOwn>
 __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDev p, const GemmDev d)
 {
+    pdl_enter();
     constexpr int kAcc = 4 / NM;
     extern __shared__ unsigned char gemm_raw[];
     unsigned char* sm = gemm_raw + ((1024u - (smem_u32(gemm_raw) & 1023u)) & 1023u);
@@ -877,7 +880,7 @@ cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const 
     unsigned* used = reinterpret_cast<unsigned*>(base + pl.graph_bytes() - 16);
     const cudaError_t e = cudaMemsetAsync(used, 0, 4, s);
     if (e != cudaSuccess) return e;
-    plan_kernel<<<(unsigned)ceil_div(pl.chunks, 128), 128, 0, s>>>(rowptr, (int)n, pl.chunk_log2, pl.chunks, reinterpret_cast<int4*>(base), units, used);
+    launch_kernel(plan_kernel, (unsigned)ceil_div(pl.chunks, 128), 128, 0, s, rowptr, (int)n, pl.chunk_log2, pl.chunks, reinterpret_cast<int4*>(base), units, used);
     if (launches) ++*launches;
     return cudaGetLastError();
 }
@@ -914,7 +917,7 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
         cudaError_t err = cudaFuncSetAttribute(agg_bits_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (err != cudaSuccess) return err;
         const unsigned grid = (unsigned)std::min<int64_t>(ceil_div((int64_t)g.chunks * g.slices, kAggWarps), (int64_t)sm_count() * agg_blocks(K));
-        agg_bits_kernel<K><<<grid, 32 * kAggWarps, smem, s>>>(g);
+        launch_kernel(agg_bits_kernel<K>, grid, 32 * kAggWarps, smem, s, g);
         if (launches) ++*launches;
         return cudaGetLastError();
     };
@@ -961,7 +964,7 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
     auto gemm = [&](auto kernel) -> cudaError_t {
         cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (err != cudaSuccess) return err;
-        kernel<<<(unsigned)std::min(d.tiles, sm_count()), kGemmThreads, smem, s>>>(p, d);
+        launch_kernel(kernel, (unsigned)std::min(d.tiles, sm_count()), kGemmThreads, smem, s, p, d);
         if (launches) ++*launches;
         return cudaGetLastError();
     };

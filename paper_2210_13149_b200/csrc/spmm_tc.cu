@@ -582,6 +582,7 @@ template <bool kHalf, bool kBitsOnly, bool kFull>
 __global__ void __launch_bounds__(kThreads, 4)
 spmm_tc_kernel(const SpmmDev p)
 {
+    pdl_enter();
     extern __shared__ unsigned char tca_raw[];
     unsigned char* sm = tca_raw + ((1024u - (smem_u32(tca_raw) & 1023u)) & 1023u);   // the swizzled operands want 1024-byte alignment
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kOffBars);
@@ -624,7 +625,7 @@ cudaError_t launch_spmm_tc(cudaStream_t s, const SpmmDev& p)
     auto launch = [&](auto kernel) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
-        kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
+        launch_kernel(kernel, grid, kThreads, kSmemBytes, s, p);
         return cudaGetLastError();
     };
     const bool full = p.nv == 16 && p.d_out == 256;
