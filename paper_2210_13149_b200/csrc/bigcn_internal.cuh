@@ -29,13 +29,14 @@ inline int zeta_elt_bytes(int fmt) { return fmt == kZetaF32 ? 4 : ((fmt == kZeta
 // fails, so that a grid derived from it stays valid).  Persistent grids are sized from it.
 int sm_count();
 
-// Programmatic dependent launch: a kernel started by launch_kernel() may be set up while the one before it on the stream still
-// runs -- a forward of a small graph is five kernels of 4 to 12 us with 2 us between them otherwise.  It therefore begins with
-// pdl_enter(): lets the kernel after it be set up likewise, and waits until the one before it is done and its writes are
-// visible.  (Transitive: a kernel is done only after its own wait.)
+// Programmatic dependent launch: a kernel started by launch_kernel() is set up as the blocks of the one before it on the stream
+// leave, and begins with pdl_enter(), which waits until that one is done and its writes are visible.  A forward of a small graph
+// is four to six kernels of 4 to 12 us, with about 2 us between them otherwise (2,708 nodes, 1433-64-7: 43.1 -> 34.2 us).
+// Kernels do not call launch_dependents: blocks that come early fill the SMs that happen to be free, several to one SM, and
+// stay there -- 3,327 nodes, 3703-64-6 from packed rows: 54.8 us with it at the start of each kernel, 43.1 us without any
+// early launch, 35.5 us like this.
 __device__ __forceinline__ void pdl_enter()
 {
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 template <typename... P, typename... A>
