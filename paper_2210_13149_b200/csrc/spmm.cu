@@ -1437,11 +1437,10 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
     const int64_t n_runs = ceil_div(p.n, rows_per_warp);
     float4 t;
     float ws, wg;
-    for (int64_t run = (int64_t)blockIdx.x * kLaneWarps + warp;; run = n_runs) {     // no counter: a run per warp at most
-        if (p.run_counter) {
-            if (lane == 0) run = atomicAdd(p.run_counter, 1);
-            run = __shfl_sync(0xffffffffu, run, 0);
-        }
+    for (;;) {
+        int64_t run = 0;
+        if (lane == 0) run = atomicAdd(p.run_counter, 1);
+        run = __shfl_sync(0xffffffffu, run, 0);
         if (run >= n_runs) break;
         const int64_t warp_row0 = run * rows_per_warp;
         const int n_rows = (int)min((int64_t)rows_per_warp, p.n - warp_row0);
@@ -1535,10 +1534,9 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
     if (e != cudaSuccess) return e;
     const int64_t wanted = ceil_div(ceil_div(p.n, rows_per_warp), kLaneWarps);
     const unsigned grid = (unsigned)std::min<int64_t>(wanted, sm_count() * 2);
-    SpmmDev q = p;
-    if (wanted <= grid) q.run_counter = nullptr;              // a run per warp: nothing to hand out
-    else if ((e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s)) != cudaSuccess) return e;
-    launch_kernel(spmm_lane_kernel<NV, kHalf, kTail, kNext>, grid, kLaneThreads, smem, s, q, rows_per_warp);
+    e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    launch_kernel(spmm_lane_kernel<NV, kHalf, kTail, kNext>, grid, kLaneThreads, smem, s, p, rows_per_warp);
     return cudaGetLastError();
 }
 
@@ -1785,11 +1783,10 @@ spmm_kernel(const SpmmDev p, int rows_per_warp)
 
     const int64_t n_runs = ceil_div(p.n, rows_per_warp);
     float acc[NCH][EPV];
-    for (int64_t run = (int64_t)blockIdx.x * kSpmmWarps + warp;; run = n_runs) {     // no counter: a run per warp at most
-        if (p.run_counter) {
-            if (lane == 0) run = atomicAdd(p.run_counter, 1);
-            run = __shfl_sync(0xffffffffu, run, 0);
-        }
+    for (;;) {
+        int64_t run = 0;
+        if (lane == 0) run = atomicAdd(p.run_counter, 1);
+        run = __shfl_sync(0xffffffffu, run, 0);
         if (run >= n_runs) break;
         const int64_t warp_row0 = run * rows_per_warp;
         const int n_rows = (int)min((int64_t)rows_per_warp, p.n - warp_row0);
@@ -1874,14 +1871,9 @@ cudaError_t launch_one(cudaStream_t s, const SpmmDev& p)
     // one wave of resident blocks; the warps pull runs of rows until none are left
     const int64_t wanted = ceil_div(ceil_div(p.n, rows_per_warp), kSpmmWarps);
     const unsigned grid = (unsigned)std::min<int64_t>(wanted, sm_count() * spmm_blocks_per_sm<NCH, LPR, kAligned, (int)sizeof(T)>());
-    SpmmDev q = p;
-    if (wanted <= grid) {
-        q.run_counter = nullptr;                              // a run per warp: nothing to hand out
-    } else {
-        cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
-        if (e != cudaSuccess) return e;
-    }
-    launch_kernel(spmm_kernel<T, NCH, LPR, kFull, kAligned, kHalf>, grid, kSpmmThreads, smem, s, q, rows_per_warp);
+    cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    launch_kernel(spmm_kernel<T, NCH, LPR, kFull, kAligned, kHalf>, grid, kSpmmThreads, smem, s, p, rows_per_warp);
     return cudaGetLastError();
 }
 

@@ -199,7 +199,6 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
     const bool odd = t & 1;
     Slot<K>* const slots = reinterpret_cast<Slot<K>*>(agg_smem) + 2 * warp;
     float* const facc = reinterpret_cast<float*>(reinterpret_cast<Slot<K>*>(agg_smem) + 2 * kAggWarps) + K * warp;   // an open row's sums: value i of lane 4 g + odd at 16 i + 2 g + odd
-    const int n = d.n;
     const uint32_t slot0 = smem_u32(slots);
     const uint32_t my_ld = kHalves == 2 ? (uint32_t)(lane * 32 + (((lane >> 2) & 1) << 4)) : (uint32_t)(lane * 16);
 
