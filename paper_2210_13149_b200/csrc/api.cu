@@ -161,10 +161,11 @@ void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 
 // One layer on already validated arguments.  `zeta` is `room` bytes of scratch: the contraction's rows in its first zbytes and
 // the aggregation's counter behind them, or (bits first) what spmm_bits_scratch_bytes() counts and the graph's plan, made here
-// unless `planned`.
+// unless `planned`.  any_order: H' may be summed in the order that is the fastest (the logits of a forward); a layer called by
+// itself keeps one order, so that thresholds taken from its H' are met by its own sums.
 bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer,
                        const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool planned,
-                       float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,
+                       bool any_order, float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,
                        float* next_beta, int32_t* dbg_dot, float* dbg_zeta,
                        cudaEvent_t ev_mid /*nullable*/)
 {
@@ -240,7 +241,8 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
     a.next_beta = next ? next_beta : nullptr;
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
-    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, a.h_out != nullptr);
+    a.any_order = any_order;
+    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, a.h_out != nullptr && !any_order);
     a.scratch = scratch;
     a.scratch_bytes = spmm_scratch_bytes(g->n, g->nnz, layer->d_out);
     e = launch_spmm(ctx->stream, a, &ctx->launches_i);
@@ -329,7 +331,7 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     for (int l = 0; l < n_layers; ++l) {
         const bool last = (l == n_layers - 1);
         const int o = (l + 1) & 1;
-        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, zbytes, room, planned,
+        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, zbytes, room, planned, true,
                                     last ? logits_out : nullptr, ldo, last ? nullptr : &layers[l + 1],
                                     bits[o], beta[o], nullptr, nullptr, stats ? ev[2 + 2 * l] : nullptr);
         if (st != BIGCN_OK) return st;
@@ -637,7 +639,7 @@ bigcn_status bigcn_layer_forward(bigcn_ctx* ctx, const bigcn_graph* graph, const
     const size_t zbytes = up(zeta_bytes_max(graph->n, dims, 1));
     const size_t need = zbytes + up(spmm_scratch_bytes(graph->n, graph->nnz, layer->d_out));
     if (!ctx->ws || ctx->ws_bytes < need) return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace, has %zu", need, ctx->ws_bytes);
-    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, zbytes, ctx->ws_bytes, false, h_out, ldh, next, next_bits, next_beta,
+    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, zbytes, ctx->ws_bytes, false, false, h_out, ldh, next, next_bits, next_beta,
                    dbg_dot, dbg_zeta, nullptr);
     finish_call(ctx);
     return st;

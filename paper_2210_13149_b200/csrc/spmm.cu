@@ -1546,8 +1546,8 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
 // share instructions.  A chunk is S stored entries of each of the rows: lane i of the S loads entry i's column, value and
 // factor -- column and value one chunk ahead, across rows -- and then every entry's row is fetched by the LPR lanes of one
 // of the S / LPR lane groups, up to eight fetches in flight.  Rows of more than 8 S entries are taken by the whole warp,
-// those above long_row by the block.  The order of summation differs from stream_entries()'s: for launches that write no H'
-// and for gradients (any_order).
+// those above long_row by the block.  The order of summation differs from stream_entries()'s: for launches that write no H',
+// for gradients and for the logits of a forward (any_order).
 //
 // Against stream_entries(), which its ring in shared memory and the bookkeeping around it bound at 21 instructions per
 // entry and 110 per row: see rows_pays().

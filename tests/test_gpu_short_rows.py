@@ -43,6 +43,7 @@ def test_hidden_and_narrow_layers(ctx, n, e, seed, d_in, d_out):
     assert bad == 0, "%d of %d flips away from the threshold" % (bad, flips)
     np.testing.assert_allclose(out["next_beta"].cpu().numpy(), beta, rtol=10 * RTOL, atol=ATOL * float(scale.max()))
     assert_close(ctx.layer_forward(G, layer, bits_to_dev(t.bits), dev(t.beta))["h"], t.H_out, "H'")
+    assert_close(ctx.forward_packed(G, [layer], bits_to_dev(t.bits), dev(t.beta)), t.H_out, "logits")
 
 
 @pytest.mark.parametrize("d_out", [1, 4, 13, 32, 64])
