@@ -145,12 +145,12 @@ bigcn_status check_layer(bigcn_ctx* ctx, const bigcn_layer* l, const char* name)
 
 // Whether a layer aggregates the packed bits before the contraction (spmm_bits.cu), in `room` bytes of scratch.  Options that
 // name a storage format or a kernel of the other order, and the debug taps on the contraction, keep to that order; so does
-// by default a launch that writes H' in fp32 (not bits_only), whose values then round as they always did.
-bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer, size_t room, bool bits_only, bool taps, bool own = false)
+// by default a layer called for H' alone (not hidden), whose values then round as they always did.
+bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer, size_t room, bool hidden, bool taps, bool own = false)
 {
     return ctx->order != 1 && ctx->zeta_format == 0 && ctx->contraction == 0 && ctx->byte_path == 0 && ctx->long_row == 0 && !taps &&
            spmm_bits_covers(g->n, g->nnz, layer->d_in, layer->d_out, own) &&
-           (ctx->order == 2 || (bits_only && spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out))) &&
+           (ctx->order == 2 || (hidden && spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out))) &&
            spmm_bits_scratch_bytes(g->n, g->nnz, layer->d_in) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
 }
 // The plan of the graph sits at the end of the scratch.
@@ -170,7 +170,7 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
                        cudaEvent_t ev_mid /*nullable*/)
 {
     const int64_t stride_in = bigcn_packed_stride_words(layer->d_in);
-    if (bits_first(ctx, g, layer, room, h_out == nullptr, dbg_dot || dbg_zeta) && (!next || aligned(next_bits, 16))) {
+    if (bits_first(ctx, g, layer, room, next != nullptr, dbg_dot || dbg_zeta) && (!next || aligned(next_bits, 16))) {
         if (ev_mid) BIGCN_CUDA(ctx, cudaEventRecord(ev_mid, ctx->stream));
         SpmmArgs a = {};
         a.n = g->n;
@@ -242,7 +242,7 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
     a.any_order = any_order;
-    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, a.h_out != nullptr && !any_order);
+    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, !next && !any_order);
     a.scratch = scratch;
     a.scratch_bytes = spmm_scratch_bytes(g->n, g->nnz, layer->d_out);
     e = launch_spmm(ctx->stream, a, &ctx->launches_i);
@@ -1046,7 +1046,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.next_beta = next ? next_beta : nullptr;
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
-    if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, h_out == nullptr, false, /*own=*/true) && (!next || aligned(next_bits, 16))) {
+    if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, next != nullptr, false, /*own=*/true) && (!next || aligned(next_bits, 16))) {
         const OwnTerm own = {reinterpret_cast<const int16_t*>(base), zeta_ld(d_out, kZetaI16), self_layer->alpha};
         a.scratch = zeta_nbr;
         void* plan = plan_at(mean_graph, zeta_nbr, ctx->ws_bytes - zbytes);
@@ -1073,7 +1073,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.zeta = zeta_nbr;
     a.ldz = ldz;
     a.byte_path = ctx->byte_path;
-    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, a.h_out != nullptr);
+    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, !next);
     a.scratch = counter;
     a.scratch_bytes = spmm_scratch_bytes(n, mean_graph->nnz, d_out);
     e = launch_spmm(ctx->stream, a, &ctx->launches_i);

@@ -1546,8 +1546,8 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
 // share instructions.  A chunk is S stored entries of each of the rows: lane i of the S loads entry i's column, value and
 // factor -- column and value one chunk ahead, across rows -- and then every entry's row is fetched by the LPR lanes of one
 // of the S / LPR lane groups, up to eight fetches in flight.  Rows of more than 8 S entries are taken by the whole warp,
-// those above long_row by the block.  The order of summation differs from stream_entries()'s: for launches that write no H',
-// for gradients and for the logits of a forward (any_order).
+// those above long_row by the block.  The order of summation differs from stream_entries()'s: for hidden layers, whether or not
+// they also write H', for gradients and for the logits of a forward (any_order).
 //
 // Against stream_entries(), which its ring in shared memory and the bookkeeping around it bound at 21 instructions per
 // entry and 110 per row: see rows_pays().
@@ -1882,11 +1882,11 @@ cudaError_t launch_one(cudaStream_t s, const SpmmDev& p)
 // 1,636 / 2,774 us; 600 K rows of 51, 32 columns 807 -> 523 us; 20 K rows of 6, 3 columns 30 -> 20 us; gradients, 1.4 M rows of
 // 21, 32 columns 1,556 -> 1,153 us.  Not for rows of 32 vectors (2.4 M rows of 13, 256 columns 4.6 -> 5.1 ms), nor for 8 and
 // more on graphs that leave most warps without a row, where the ring keeps more fetches of a longer row in flight (2,500
-// rows of 31, 64 columns: 24 -> 30 us); nor, beyond one vector, where H' is written (the order of summation differs).
+// rows of 31, 64 columns: 24 -> 30 us); nor, beyond one vector, where a layer called by itself writes H' and no bits (the order of summation differs).
 bool rows_pays(const SpmmDev& p, int elt_bytes, double mean_row)
 {
     if (p.half_dots || p.nv > 16) return false;
-    if (p.h_out && !p.any_order && p.nv > 1) return false;
+    if (!p.next_bits && !p.any_order && p.nv > 1) return false;
     if (elt_bytes == 1 && p.nv > 8 && !(mean_row > 0.0 && mean_row < 8.0)) return false;   // the row-aligned byte stream
     return !(p.nv > 4 && p.n < 12000 && mean_row > 12.0);
 }
