@@ -551,16 +551,26 @@ def run_ours(args):
         if last and elt == 1 and 32 < dims[l + 1] <= 60 and on_tc:
             ldz = 64
         out_bytes = n * dims[l + 1] * 4.0 if last else n * (binding.packed_stride_words(dims[l + 1]) * 4.0 + 4.0)
-        lower, upper, expected = spmm_bytes_model(n, nnz, ldz * elt, out_bytes, deg_cum)
+        # a hidden layer whose two times meet at its start aggregated the packed bits before the contraction: 16 or 32 bytes
+        # per operand row, and four digit bytes per input column and node written and read between its two kernels
+        bits_first = not last and gemm_ms[l] < 0.02 * spmm_ms[l]
+        row_bytes = binding.packed_stride_words(dims[l]) * 4 if bits_first else ldz * elt
+        if bits_first:
+            out_bytes += 8.0 * n * row_bytes * 8
+        lower, upper, expected = spmm_bytes_model(n, nnz, row_bytes, out_bytes, deg_cum)
         t = spmm_ms[l] * 1e-3
         # the library's rule for the aggregation kernel: tcgen05 products for a hidden layer (only bits and beta wanted) of
         # 129..256 byte columns on a graph whose rows average at least 8 stored entries, unless another path is asked for
         on_tc_agg = (elt == 1 and 128 < dims[l + 1] <= 256 and not last and nnz < (1 << 31)
                      and (args.byte_aggregation == 3 or (args.byte_aggregation == 0 and nnz >= 8 * n)))
         agg_name = "spmm_tc_kernel" if on_tc_agg else ("spmm_lane_kernel" if (last and elt == 1 and 32 < dims[l + 1] <= 64 and nnz >= 8 * n) else "spmm_kernel")
+        if bits_first:
+            agg_name = "agg_bits_kernel + bits_gemm_kernel"
         kernels["spmm_l%d" % l] = {"ms": spmm_ms[l], "kernel": agg_name, "GBps_cached_model": expected / t / 1e9,
                                    "GBps_lower_model": lower / t / 1e9, "GBps_no_reuse_model": upper / t / 1e9,
-                                   "bytes_cached_model": expected, "row_bytes": ldz * elt, "zeta_format": {1: "f32", 2: "i16", 3: "i8", 4: "f16", 5: "i8h"}[f]}
+                                   "bytes_cached_model": expected, "row_bytes": row_bytes, "zeta_format": "bits" if bits_first else {1: "f32", 2: "i16", 3: "i8", 4: "f16", 5: "i8h"}[f]}
+        if bits_first:
+            continue
         ops = 2.0 * n * dims[l] * dims[l + 1]
         words = n * dims[l + 1] * ((dims[l] + 31) // 32)                  # XOR + bit-count + add steps
         popc_peak = extras.get("popc_word_steps_per_s")
@@ -585,7 +595,8 @@ def run_ours(args):
                 "bound": "hbm", "achieved": achieved, "peak": peak, "peak_kind": "%s copy bandwidth" % peak_kind,
                 "unit": "GB/s", "frac": achieved / peak, "traffic": traffic_record(dom_key),
                 "algorithmic_bytes": kernels["spmm_l%d" % dom]["bytes_cached_model"],
-                "note": "byte rows (i8 / i8h) halve the DRAM traffic of the 256-column aggregations and leave them bound by "
+                "note": "bits: the gathers stay in the L2 and the layer is bound by instruction issue (agg_bits_kernel); "
+                        "byte rows (i8 / i8h) halve the DRAM traffic of the 256-column aggregations and leave them bound by "
                         "the per-chunk chain of hand-offs (tcgen05 products, the default) or by instruction issue (the fp32 "
                         "FMA stream, extras.spmm_fma_stream_ms), not HBM; with fp16 rows (--zeta-format 4) the same layer is "
                         "HBM-bound: see extras.spmm_fp16_rows_ms and kernels.*",
@@ -609,7 +620,7 @@ def run_ours(args):
         except Exception as exc:      # the oracle is optional equipment for the bench
             cpu = {"value": None, "unit": UNIT, "cores": 0, "kind": "oracle", "sample": "failed: %r" % (exc,)}
 
-    on_tc_layers = [kernels["bitgemm_l%d" % l]["path"].startswith("tcgen05") for l in range(L)]
+    on_tc_layers = [kernels.get("bitgemm_l%d" % l, {"path": "tcgen05 int8"})["path"].startswith("tcgen05") for l in range(L)]
     dtype = DTYPE_TC if all(on_tc_layers) else (DTYPE if not any(on_tc_layers) else DTYPE_TC + " / " + DTYPE)
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
