@@ -217,194 +217,189 @@ grad_h_mma_kernel(const float* __restrict__ gz, int64_t ldz, const float* __rest
 }
 
 // ---- G_H on the 5th-generation tensor cores ---------------------------------------------------------------
-// The same product as grad_h_mma_kernel with tcgen05.mma kind::f16 (bf16 operands, fp32 accumulators in
-// tensor memory): M = 128 rows, N = 64 / 128 / 256 >= d_in, the reduction over the output channels in
-// chunks of 64 (128 bytes per operand row: the three terms of the fp32 operand take 48 KB, the +-1
-// operand N x 128 bytes).  Two CTAs per SM overlap each other's staging, products and epilogue.  Operands
-// are K-major no-swizzle (core matrices of 8 rows x 16 bytes).  The epilogue reads the accumulators back
-// (a thread owns one row), clips (Eq. bp-H) and writes through shared memory as 128-byte row segments.
+// The same product as grad_h_mma_kernel with tcgen05.mma kind::f16 (bf16 operands, fp32 accumulators in tensor memory):
+// M = 128 rows, N = 64 / 128 / 256 inputs (blockIdx.y: slices of N), the reduction over the output channels in chunks of 64.
+// Both operands are K-major with 128-byte swizzle: 64 channels of a row are 128 contiguous bytes, so a warp reads and stages
+// two whole row pieces without bank conflicts.  One block of 16 warps per multiprocessor.  The fp32 operand has two stages of
+// its three terms: while one is multiplied the other is filled, and the chunk after that is on its way in registers; two
+// accumulators, so that a tile is read back, clipped (Eq. bp-H) and written under the products of the next one.  The signs of
+// W stay in shared memory for all tiles where all of their chunks fit (d_out <= 65536 / N); longer ones pass through
+// two stages.  (One stage, the signs rebuilt for every chunk of every tile, stores that met in the banks eight at a time:
+// 2.4 M nodes, 256 -> 256, 2.8 ms; now 1.37 ms.)
 // Needs d_in a multiple of 4 and 16-byte aligned rows of g_h; every mbarrier wait is bounded.
 __device__ int g_bw_tc_timeout;
 
+constexpr int kGhThreads = 512, kGhRows = 128, kGhK = 64;
+constexpr int kGhTerm = kGhRows * 128;                      // bytes of one term of a chunk
+constexpr int kGhStage = 3 * kGhTerm;
+__host__ __device__ constexpr int gh_slots(int n) { return 1024 / n; }         // chunks of signs that stay: 128 KB
+
 template <int N>
-__global__ void __launch_bounds__(kBwThreads, 2)
+__global__ void __launch_bounds__(kGhThreads, 1)
 grad_h_tc_kernel(const float* __restrict__ gz, int64_t ldz, const float* __restrict__ alpha,
                  const float* __restrict__ W, int64_t ldw, int64_t n, int d_in, int d_out,
                  float* __restrict__ g_h, int64_t ldh)
 {
     pdl_enter();
-    constexpr int kRows = 128, kKc = 64;                   // tile rows; reduction elements per chunk
-    constexpr int kCols = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
-    extern __shared__ __align__(128) unsigned char bw_smem[];
-    __shared__ __align__(8) uint64_t bar;
+    constexpr int kBChunk = N * 128;
+    constexpr int kItems = kGhRows * (kGhK / 4) / kGhThreads, kBItems = N * (kGhK / 4) / kGhThreads;
+    constexpr int kCols = 2 * N;                            // two accumulators
+    extern __shared__ unsigned char bw_raw[];
+    __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t tmem_base_s;
-    unsigned char* As = bw_smem;                            // [3][128][128 bytes]; also the epilogue's scratch (>= 32 KB)
-    unsigned char* Bs = bw_smem + 3 * kRows * 128;          // [N][128 bytes]
+    unsigned char* sm = bw_raw + ((1024u - (tc::smem_u32(bw_raw) & 1023u)) & 1023u);
+    unsigned char* Bs = sm + 2 * kGhStage;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) tc::tmem_alloc(&tmem_base_s, kCols);
-    if (threadIdx.x == 0) tc::barrier_init(&bar);
+    if (threadIdx.x == 0) {
+        tc::barrier_init(&bar[0]);
+        tc::barrier_init(&bar[1]);
+    }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem_base = tmem_base_s;
     // instruction descriptor: D = f32, A = B = bf16, both K-major, N, M = 128
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
-    const uint32_t a_lbo = (kRows >> 3) * 128, b_lbo = (N >> 3) * 128, sbo = 128;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kGhRows >> 4) << 24);
     const bool vec_ok = (ldz % 4 == 0) && (reinterpret_cast<uintptr_t>(gz) % 16 == 0);
     const bool w_vec_ok = (ldw % 4 == 0) && (reinterpret_cast<uintptr_t>(W) % 16 == 0);
-    const int n_chunks = (d_out + kKc - 1) / kKc;
-    const int64_t n_tiles = ceil_div(n, kRows);
-    const int lane_base = 32 * (warp & 3);
-    const int c_begin = (warp >> 2) * (N / 2);
-    unsigned char* scr = As + warp * 4096;                  // 32 rows x 128 bytes, pieces swizzled by (row & 7)
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        const int64_t i0 = tile * kRows;
-        for (int ch = 0; ch < n_chunks; ++ch) {
-            const int j0 = ch * kKc;
-            // A: 128 rows x 16 quads of channels -> three bf16 terms of G_zeta * alpha.  All of a thread's loads are
-            // issued before the first is used (8 independent 16-byte loads in flight per thread).
-            {
-                constexpr int kItems = kRows * (kKc / 4) / kBwThreads;
-                float4 xv[kItems], av[kItems];
+    const int k0 = blockIdx.y * N;
+    const int n_chunks = (d_out + kGhK - 1) / kGhK;
+    const bool resident = n_chunks <= gh_slots(N);
+    const int64_t n_tiles = ceil_div(n, kGhRows);
+    const int64_t my_tiles = n_tiles > blockIdx.x ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int64_t total = my_tiles * n_chunks;              // chunks of all tiles of this block, one after the other
+    // this thread's pieces of a chunk: channels jq .. jq + 3 of rows threadIdx.x / 16 + 32 it, of both operands
+    const int jq = (threadIdx.x & 15) * 4, r0 = threadIdx.x >> 4;
+    const uint32_t off = (uint32_t)((r0 >> 3) * 1024 + (r0 & 7) * 128 + (((jq >> 3) ^ (r0 & 7)) << 4) + (jq & 7) * 2);   // + 4096 it
+    auto load4 = [](const float* src, bool whole, int left) {                  // the first `left` of four floats
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (whole && left >= 4) return __ldg(reinterpret_cast<const float4*>(src));
+        if (left > 0) v.x = __ldg(src);
+        if (left > 1) v.y = __ldg(src + 1);
+        if (left > 2) v.z = __ldg(src + 2);
+        if (left > 3) v.w = __ldg(src + 3);
+        return v;
+    };
+    float4 xv[kItems], av;
+    auto load = [&](int64_t tile, int ch) {
+        const int j = ch * kGhK + jq;
 #pragma unroll
-                for (int it = 0; it < kItems; ++it) {
-                    const int t = threadIdx.x + it * kBwThreads;
-                    const int jq = (t & 15) * 4, r = t >> 4;
-                    const int j = j0 + jq;
-                    const int64_t row = i0 + r;
-                    xv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    av[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (row < n) {
-                        if (j + 3 < d_out && vec_ok) {
-                            xv[it] = __ldg(reinterpret_cast<const float4*>(gz + row * ldz + j));
-                        } else {
-                            if (j < d_out) xv[it].x = __ldg(gz + row * ldz + j);
-                            if (j + 1 < d_out) xv[it].y = __ldg(gz + row * ldz + j + 1);
-                            if (j + 2 < d_out) xv[it].z = __ldg(gz + row * ldz + j + 2);
-                            if (j + 3 < d_out) xv[it].w = __ldg(gz + row * ldz + j + 3);
-                        }
-                    }
-                    if (j < d_out) av[it].x = __ldg(alpha + j);
-                    if (j + 1 < d_out) av[it].y = __ldg(alpha + j + 1);
-                    if (j + 2 < d_out) av[it].z = __ldg(alpha + j + 2);
-                    if (j + 3 < d_out) av[it].w = __ldg(alpha + j + 3);
-                }
-#pragma unroll
-                for (int it = 0; it < kItems; ++it) {
-                    const int t = threadIdx.x + it * kBwThreads;
-                    const int jq = (t & 15) * 4, r = t >> 4;
-                    const float x[4] = {__fmul_rn(xv[it].x, av[it].x), __fmul_rn(xv[it].y, av[it].y), __fmul_rn(xv[it].z, av[it].z), __fmul_rn(xv[it].w, av[it].w)};
-                    unsigned short hi[4], mid[4], lo[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) split3(x[u], hi[u], mid[u], lo[u]);
-                    auto pack = [](const unsigned short (&h)[4]) { return make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16)); };
-                    const uint32_t off = tc::canon_off(kRows, r, jq >> 3) + (jq & 7) * 2;
-                    *reinterpret_cast<uint2*>(As + 0 * kRows * 128 + off) = pack(hi);
-                    *reinterpret_cast<uint2*>(As + 1 * kRows * 128 + off) = pack(mid);
-                    *reinterpret_cast<uint2*>(As + 2 * kRows * 128 + off) = pack(lo);
-                }
-            }
-            // B: N inputs x 16 quads of channels -> sign of W as +-1 (loads batched in the same way)
-            {
-                constexpr int kItems = N * (kKc / 4) / kBwThreads;
-                float4 wv[kItems];
-#pragma unroll
-                for (int it = 0; it < kItems; ++it) {
-                    const int t = threadIdx.x + it * kBwThreads;
-                    const int jq = (t & 15) * 4, k = t >> 4;
-                    const int j = j0 + jq;
-                    wv[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (k < d_in) {
-                        if (j + 3 < d_out && w_vec_ok) {
-                            wv[it] = __ldg(reinterpret_cast<const float4*>(W + (int64_t)k * ldw + j));
-                        } else {
-                            if (j < d_out) wv[it].x = __ldg(W + (int64_t)k * ldw + j);
-                            if (j + 1 < d_out) wv[it].y = __ldg(W + (int64_t)k * ldw + j + 1);
-                            if (j + 2 < d_out) wv[it].z = __ldg(W + (int64_t)k * ldw + j + 2);
-                            if (j + 3 < d_out) wv[it].w = __ldg(W + (int64_t)k * ldw + j + 3);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int it = 0; it < kItems; ++it) {
-                    const int t = threadIdx.x + it * kBwThreads;
-                    const int jq = (t & 15) * 4, k = t >> 4;
-                    const int j = j0 + jq;
-                    const bool kin = k < d_in;
-                    const float w[4] = {wv[it].x, wv[it].y, wv[it].z, wv[it].w};
-                    uint32_t sg[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) sg[u] = (kin && j + u < d_out) ? (w[u] >= 0.f ? 0x3F80u : 0xBF80u) : 0u;
-                    const uint32_t off = tc::canon_off(N, k, jq >> 3) + (jq & 7) * 2;
-                    *reinterpret_cast<uint2*>(Bs + off) = make_uint2(sg[0] | (sg[1] << 16), sg[2] | (sg[3] << 16));
-                }
-            }
-            tc::fence_async_smem();
-            tc::fence_before_sync();
-            __syncthreads();                                // operands complete; previous tile's accumulator reads are over
-            tc::fence_after_sync();
-            if (threadIdx.x == 0) {
-                const uint32_t a_base = tc::smem_u32(As), b_base = tc::smem_u32(Bs);
-                for (int ks = 0; ks < kKc / 16; ++ks) {
-                    const uint64_t bd = tc::make_desc(b_base + 2 * ks * b_lbo, b_lbo, sbo);
-#pragma unroll
-                    for (int sp = 0; sp < 3; ++sp) {
-                        const uint64_t ad = tc::make_desc(a_base + sp * kRows * 128 + 2 * ks * a_lbo, a_lbo, sbo);
-                        const uint32_t accum = (ch > 0 || ks > 0 || sp > 0) ? 1u : 0u;
-                        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                     ::"r"(tmem_base), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
-                    }
-                }
-                tc::commit_to(&bar);
-            }
-            if (!tc::wait_barrier(&bar, phase)) {
-                atomicExch(&g_bw_tc_timeout, 1);
-                ok = false;
-            }
-            phase ^= 1u;
-            tc::fence_after_sync();
-            if (__syncthreads_or(!ok)) { ok = false; break; }   // the operands may be overwritten; leave together on a timeout
+        for (int it = 0; it < kItems; ++it) {
+            const int64_t row = tile * kGhRows + r0 + 32 * it;
+            xv[it] = load4(gz + row * ldz + j, vec_ok, row < n ? d_out - j : 0);
         }
-        if (!ok) break;
-        // ---- epilogue: clip and write the tile (a thread owns row lane_base + lane, its warp's half of the columns)
-        const int64_t row0 = i0 + lane_base;
-        constexpr int kPasses = (N / 2) * 4 / 128 > 0 ? (N / 2) * 4 / 128 : 1;    // 32 columns = 128 bytes per pass
-        constexpr int kPpr = (N / 2) * 4 >= 128 ? 8 : (N / 2) * 4 / 16;
+        av = load4(alpha + j, false, d_out - j);
+    };
+    auto wait = [&](int64_t c) {                            // until the products of chunk c are done
+        const bool in_time = __all_sync(0xffffffffu, tc::wait_barrier(&bar[c & 1], (uint32_t)(c >> 1) & 1u));
+        if (!in_time) atomicExch(&g_bw_tc_timeout, 1);
+        return in_time;
+    };
+    // a finished tile: a thread owns row 32 (warp % 4) + lane, its warp a quarter of the columns, 16 at a time, which leave
+    // as 64-byte pieces of rows through 2 KB of a free stage
+    const int lane_base = 32 * (warp & 3), c_begin = (warp >> 2) * (N / 4);
+    auto finish = [&](int64_t tile, int acc, unsigned char* scratch) {
+        unsigned char* scr = scratch + warp * 2048;
+        const int64_t row0 = tile * kGhRows + lane_base;
 #pragma unroll 1
-        for (int pass = 0; pass < kPasses; ++pass) {
+        for (int c0 = c_begin; c0 < c_begin + N / 4; c0 += 16) {
+            uint32_t v[16];
+            tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)(acc * N + c0), v);
 #pragma unroll
-            for (int c2 = 0; c2 < kPpr / 4; ++c2) {
-                const int c0 = c_begin + pass * 32 + c2 * 16;
-                uint32_t v[16];
-                tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)c0, v);
+            for (int u = 0; u < 4; ++u) {
+                float f[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float f[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float a = __uint_as_float(v[4 * u + e]);
-                        f[e] = fabsf(a) < 1.f ? a : 0.f;                                  // Eq. bp-H
-                    }
-                    const int piece = c2 * 4 + u;
-                    *reinterpret_cast<uint4*>(scr + lane * 128 + ((piece ^ (lane & 7)) * 16)) =
-                        make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+                for (int e = 0; e < 4; ++e) {
+                    const float g = __uint_as_float(v[4 * u + e]);
+                    f[e] = fabsf(g) < 1.f ? g : 0.f;                                      // Eq. bp-H
                 }
+                *reinterpret_cast<float4*>(scr + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) = make_float4(f[0], f[1], f[2], f[3]);
             }
             __syncwarp();
-            const int col0 = c_begin + pass * 32;
 #pragma unroll
-            for (int it = 0; it < kPpr; ++it) {
-                const int r = it * (32 / kPpr) + lane / kPpr, pc = lane % kPpr;
-                const uint4 val = *reinterpret_cast<const uint4*>(scr + r * 128 + ((pc ^ (r & 7)) * 16));
-                const int col = col0 + pc * 4;
-                if (row0 + r < n && col < d_in) *reinterpret_cast<uint4*>(g_h + (row0 + r) * ldh + col) = val;
+            for (int it = 0; it < 4; ++it) {
+                const int r = it * 8 + (lane >> 2), u = lane & 3;
+                const float4 val = *reinterpret_cast<const float4*>(scr + r * 64 + ((u ^ ((r >> 1) & 3)) << 4));
+                const int col = k0 + c0 + 4 * u;
+                if (row0 + r < n && col < d_in) *reinterpret_cast<float4*>(g_h + (row0 + r) * ldh + col) = val;
             }
             __syncwarp();
         }
+    };
+    bool ok = true;
+    int64_t tile = blockIdx.x;
+    int ch = 0, acc = 0;
+    if (total > 0) load(tile, 0);
+    for (int64_t c = 0; c < total; ++c) {
+        const int st = (int)(c & 1);
+        unsigned char* stage = sm + st * kGhStage;
+        unsigned char* signs = Bs + (resident ? ch : st) * kBChunk;
+        if (c >= 2) ok = wait(c - 2) && ok;
+        const float a4[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+        for (int it = 0; it < kItems; ++it) {
+            const float x[4] = {__fmul_rn(xv[it].x, a4[0]), __fmul_rn(xv[it].y, a4[1]), __fmul_rn(xv[it].z, a4[2]), __fmul_rn(xv[it].w, a4[3])};
+            unsigned short hi[4], mid[4], lo[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) split3(x[u], hi[u], mid[u], lo[u]);
+            auto pack = [](const unsigned short (&h)[4]) { return make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16)); };
+            *reinterpret_cast<uint2*>(stage + 0 * kGhTerm + off + 4096 * it) = pack(hi);
+            *reinterpret_cast<uint2*>(stage + 1 * kGhTerm + off + 4096 * it) = pack(mid);
+            *reinterpret_cast<uint2*>(stage + 2 * kGhTerm + off + 4096 * it) = pack(lo);
+        }
+        if (!resident || c < n_chunks) {
+            const int j = ch * kGhK + jq;
+#pragma unroll
+            for (int it = 0; it < kBItems; ++it) {
+                const int k = k0 + r0 + 32 * it;
+                const int left = k < d_in ? d_out - j : 0;
+                const float4 wv = load4(W + (int64_t)k * ldw + j, w_vec_ok, left);
+                const float w[4] = {wv.x, wv.y, wv.z, wv.w};
+                uint32_t sg[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sg[u] = u < left ? (w[u] >= 0.f ? 0x3F80u : 0xBF80u) : 0u;
+                *reinterpret_cast<uint2*>(signs + off + 4096 * it) = make_uint2(sg[0] | (sg[1] << 16), sg[2] | (sg[3] << 16));
+            }
+        }
+        const int64_t cur_tile = tile;
+        const int cur_ch = ch;
+        if (++ch == n_chunks) {
+            ch = 0;
+            tile += gridDim.x;
+        }
+        if (c + 1 < total) load(tile, ch);
+        tc::fence_async_smem();
         tc::fence_before_sync();
-        __syncthreads();                                    // the scratch is the next tile's operand space
+        if (__syncthreads_or(!ok)) { ok = false; break; }   // operands complete; leave together on a timeout
+        tc::fence_after_sync();
+        if (threadIdx.x == 0) {
+            const uint32_t a_base = tc::smem_u32(stage), b_base = tc::smem_u32(signs);
+            for (int ks = 0; ks < kGhK / 16; ++ks) {
+                const uint64_t bd = tc::make_desc(b_base + ks * 32, 16, 1024) | ((uint64_t)2 << 61);
+#pragma unroll
+                for (int sp = 0; sp < 3; ++sp) {
+                    const uint64_t ad = tc::make_desc(a_base + sp * kGhTerm + ks * 32, 16, 1024) | ((uint64_t)2 << 61);
+                    const uint32_t accum = (cur_ch > 0 || ks > 0 || sp > 0) ? 1u : 0u;
+                    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                                 ::"r"(tmem_base + (uint32_t)(acc * N)), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
+                }
+            }
+            tc::commit_to(&bar[st]);
+        }
+        if (cur_ch == 0 && c > 0) {                         // the tile before, from the other accumulator, by way of the other stage
+            ok = wait(c - 1) && ok;
+            tc::fence_after_sync();
+            if (ok) finish(cur_tile - gridDim.x, acc ^ 1, sm + (st ^ 1) * kGhStage);
+            tc::fence_before_sync();
+            __syncthreads();                                // that stage is filled next
+        }
+        if (cur_ch == n_chunks - 1) acc ^= 1;
+    }
+    if (total > 0 && ok) {
+        ok = wait(total - 1);
+        tc::fence_after_sync();
+        if (ok) finish(tile - gridDim.x, acc ^ 1, sm + (total & 1) * kGhStage);
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -584,11 +579,13 @@ template <int N>
 cudaError_t launch_grad_h_tc(cudaStream_t s, const float* gz, int64_t ldz, const float* alpha, const float* W, int64_t ldw,
                              int64_t n, int d_in, int d_out, float* g_h, int64_t ldh)
 {
-    const size_t smem = 3 * 128 * 128 + (size_t)N * 128;
+    const int chunks = (int)ceil_div(d_out, kGhK);
+    const size_t smem = 2 * kGhStage + (size_t)(chunks <= gh_slots(N) ? chunks : 2) * N * 128 + 1024;
     cudaError_t e = cudaFuncSetAttribute(grad_h_tc_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 128), sm_count() * 2);
-    launch_kernel(grad_h_tc_kernel<N>, grid, kBwThreads, smem, s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_h, ldh);
+    const unsigned slices = (unsigned)ceil_div(d_in, N);
+    const dim3 grid((unsigned)std::min<int64_t>(ceil_div(n, kGhRows), std::max(1, sm_count() / (int)slices)), slices);
+    launch_kernel(grad_h_tc_kernel<N>, grid, kGhThreads, smem, s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_h, ldh);
     return cudaGetLastError();
 }
 
@@ -728,7 +725,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     // step 1c + 2: G_H = clip(G_zeta W~^T)
     if (g_in) {
         ++*launches;
-        if (d_in <= 256 && d_in % 4 == 0 && ldgi % 4 == 0 && reinterpret_cast<uintptr_t>(g_in) % 16 == 0) {   // tcgen05 version
+        if (d_in % 4 == 0 && ldgi % 4 == 0 && reinterpret_cast<uintptr_t>(g_in) % 16 == 0) {   // tcgen05 version
             if (d_in <= 64) e = launch_grad_h_tc<64>(s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_in, ldgi);
             else if (d_in <= 128) e = launch_grad_h_tc<128>(s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_in, ldgi);
             else e = launch_grad_h_tc<256>(s, gz, ldz, alpha, W, ldw, n, d_in, d_out, g_in, ldgi);
