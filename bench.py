@@ -588,6 +588,8 @@ def run_ours(args):
     pack_bytes = n * (dims[0] * 4.0 + binding.packed_stride_words(dims[0]) * 4.0 + 4.0)
     kernels["pack_features"] = {"ms": pack_ms, "GBps": pack_bytes / (pack_ms * 1e-3) / 1e9,
                                 "frac_of_hbm_peak": pack_bytes / (pack_ms * 1e-3) / 1e9 / peak}
+    if any(k["kernel"].startswith("agg_bits") for name, k in kernels.items() if name.startswith("spmm_l")):
+        kernels["pack_features"]["includes"] = "plan_kernel (the split of the aggregation's work, once per forward)"
     achieved = kernels["spmm_l%d" % dom]["GBps_cached_model"]
     dom_name = kernels["spmm_l%d" % dom]["kernel"]
     dom_key = "%s/%s/%s/l%d" % (dom_name, spec.name, kernels["spmm_l%d" % dom]["zeta_format"], dom)

@@ -16,8 +16,8 @@
 // (bytes & 0x01010101 << j) IS the operand of column j scaled by 2^j, which the read-back removes: one logic instruction per
 // four bits.  The mma.sync form is taken because it alone lets the operand be built in registers; tcgen05 wants it in shared
 // memory, where the expanded bytes would cost two passes over 256 bytes per entry.  P leaves as its four digit bytes, in the
-// layout the next kernel reads.  Bound: instruction issue (55 to 60 % of the slots, the logic pipe 55 %, the tensor pipe
-// 18 %; 256 columns, 31.5 M entries 0.79 ms).
+// layout the next kernel reads.  Bound: instructions at the few warps that the accumulators leave room for (53 to 58 % of the issue
+// slots, the logic pipe 57 %, the tensor pipe 18 %; 256 columns, 31.5 M entries 0.79 ms).
 //
 // bits_gemm_kernel: H' = P B diag(alpha) as tcgen05.mma.kind::i8.  The digits of 32 rows are one operand of N = 128 (row,
 // digit) columns, K-major with 128-byte swizzle, fetched by bulk copies; the other is the weights expanded to +-1 bytes
