@@ -260,13 +260,23 @@ size_t zeta_bytes_max(int64_t n, const int32_t* dims, int n_layers)
     return m;
 }
 
-// Scratch between the kernels of a layer, the larger of the two orders over all layers.
+// Scratch of the contraction-first order: the contraction's rows, the aggregation's counter.
+size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers)
+{
+    return up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
+}
+
+// Scratch between the kernels of a layer, the larger of the two orders over all layers, and behind it the graph's plan, which
+// layers of both orders leave alone.
 size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers)
 {
-    size_t m = up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
+    size_t m = contraction_first_bytes(n, nnz, dims, n_layers), plan = 0;
     for (int l = 0; l < n_layers; ++l)
-        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]) + spmm_bits_plan_bytes(n, nnz) + kAlign);
-    return m;
+        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) {
+            m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]));
+            plan = spmm_bits_plan_bytes(n, nnz);
+        }
+    return m + plan;
 }
 
 // Bytes of a slot's input staging buffer: the fp32 features, or -- whichever is larger -- the packed input
@@ -298,8 +308,9 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     const size_t zbytes = up(zeta_bytes_max(n, dims, n_layers));
     size_t others = 0;                                       // what else the step keeps
     for (int i = 0; i < 2; ++i) others += up((size_t)n * stride_max * 4) + up((size_t)n * 4);
+    const size_t least = contraction_first_bytes(n, graph->nnz, dims, n_layers);
     size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers);
-    if (up(ws.off) + room + others > ws.size) room = zbytes + up(spmm_scratch_bytes(n, graph->nnz, 0));   // a workspace without room for P
+    if (up(ws.off) + room + others > ws.size) room = least;  // a workspace without room for P
     void* zeta = ws.take(room);
     uint32_t* bits[2];
     float* beta[2];
@@ -321,8 +332,10 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
         cur_bits = bits[0];
         cur_beta = beta[0];
     }
-    bool planned = false;                                    // the layers share the graph's plan
-    for (int l = 0; l < n_layers && !planned; ++l) planned = bits_first(ctx, graph, &layers[l], room, l < n_layers - 1, false);
+    // The layers share the graph's plan where the scratch of the contraction-first ones ends before it; otherwise each that
+    // needs it makes its own.
+    bool planned = false;
+    for (int l = 0; l < n_layers && !planned && room >= least + spmm_bits_plan_bytes(n, graph->nnz); ++l) planned = bits_first(ctx, graph, &layers[l], room, l < n_layers - 1, false);
     if (planned) {
         cudaError_t e = launch_spmm_bits_plan(ctx->stream, n, graph->nnz, graph->rowptr, plan_at(graph, zeta, room), &ctx->launches_i);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");
