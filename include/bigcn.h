@@ -115,7 +115,11 @@ enum {
      *     graph let it expect to be the faster; 1 otherwise.
      * A layer keeps to 1 when one of the options above is set or a debug tap is asked for.  Both orders meet the same
      * tolerance; their fp32 sums differ in rounding. */
-    BIGCN_OPT_ORDER = 5
+    BIGCN_OPT_ORDER = 5,
+    /* Bound of every wait of one part of a thread block for another in the product P B of order 2, in tries of up to a
+     * microsecond: 0 = default (2^20), at most 2^20.  A block whose wait runs out ends early, its outputs unwritten, and
+     * bigcn_sync_check() reports BIGCN_ERR_INTERNAL from then on.  For tests of that path. */
+    BIGCN_OPT_WAIT_TRIES = 6
 };
 
 /* Context: binds a device and a stream.  `cuda_stream` is a cudaStream_t (0 = default stream). */

@@ -22,6 +22,7 @@ struct bigcn_ctx {
     int zeta_format;             // 0 = auto
     int64_t long_row;            // 0 = default
     int contraction;             // 0 = auto, 1 = bit-count pipe, 2 = tensor cores wherever covered
+    int wait_tries;              // 0 = default
     int order;                   // 0 = the faster one, 1 = contraction first, 2 = aggregation first wherever covered
     int byte_path;               // aggregation of 129..256 byte columns: 0 / 1 = fp32 FMA stream, 2 = integer tensor-core products
     cudaEvent_t ev[2 * BIGCN_MAX_LAYERS + 2];
@@ -189,6 +190,7 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
         a.next_shift = next ? next->in_shift : nullptr;
         a.next_scale = next ? next->in_scale : nullptr;
         a.scratch = zeta;
+        a.wait_tries = ctx->wait_tries;
         void* plan = plan_at(g, zeta, room);
         cudaError_t e = planned ? cudaSuccess : launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
         if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, nullptr, &ctx->launches_i);
@@ -467,6 +469,10 @@ bigcn_status bigcn_set_option(bigcn_ctx* ctx, int32_t option, int64_t value)
         case BIGCN_OPT_ORDER:
             if (value < 0 || value > 2) return fail(ctx, BIGCN_ERR_SHAPE, "order %lld not in 0..2", (long long)value);
             ctx->order = (int)value;
+            return BIGCN_OK;
+        case BIGCN_OPT_WAIT_TRIES:
+            if (value < 0 || value > (int64_t(1) << 20)) return fail(ctx, BIGCN_ERR_SHAPE, "wait tries %lld not in 0..2^20", (long long)value);
+            ctx->wait_tries = (int)value;
             return BIGCN_OK;
         case BIGCN_OPT_BYTE_AGGREGATION:
             if (value < 0 || value > 3) return fail(ctx, BIGCN_ERR_SHAPE, "byte aggregation path %lld not in 0..3", (long long)value);
@@ -1062,6 +1068,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     if (bits_first(ctx, mean_graph, nbr_layer, ctx->ws_bytes - zbytes, next != nullptr, false, /*own=*/true) && (!next || aligned(next_bits, 16))) {
         const OwnTerm own = {reinterpret_cast<const int16_t*>(base), zeta_ld(d_out, kZetaI16), self_layer->alpha};
         a.scratch = zeta_nbr;
+        a.wait_tries = ctx->wait_tries;
         void* plan = plan_at(mean_graph, zeta_nbr, ctx->ws_bytes - zbytes);
         e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, self_layer->alpha,
                            kZetaI16, base, own.ld, nullptr, nullptr, &ctx->launches_i, ctx->contraction);

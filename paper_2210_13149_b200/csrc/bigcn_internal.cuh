@@ -102,6 +102,7 @@ struct SpmmArgs {
     int64_t long_row;        // rows with more entries are split (0 = never)
     void* scratch;           // partial sums of split rows
     size_t scratch_bytes;
+    int wait_tries = 0;      // launch_spmm_bits(): bound of the waits inside a block (0 = default)
 };
 cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches);
 size_t spmm_scratch_bytes(int64_t n, int64_t nnz, int d_out);

@@ -549,7 +549,7 @@ constexpr int kGemmStages = 3;
 constexpr int kOwnElts = 2 * kTileRows * 256;       // two tiles of up to 256 columns or four of up to 128
 constexpr int kEpiGroups = 4;                       // warpgroups that read accumulators back
 constexpr int kGemmThreads = 128 * kEpiGroups + 64; // + a copying and an issuing warp
-constexpr int kTries = 1 << 20;                     // bound of every wait: tries of up to 1 us
+constexpr int kTries = 1 << 20;                     // bound of a wait: tries of up to 1 us (a single one does not linger)
 
 struct GemmMisc {
     uint64_t full[kGemmStages], empty[kGemmStages];
@@ -569,13 +569,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
-// false when the block gives up
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort)
+// false when the block gives up, which threads that wait for the same barrier may learn differently: one sees it complete,
+// another the end of its tries
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int tries)
 {
-    for (int it = 0; it < kTries; ++it) {
+    for (int it = 0; it < tries; ++it) {
         uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, 1000;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(smem_u32(bar)), "r"(parity), "r"(tries > 1 ? 1000u : 0u) : "memory");
         if (done) return true;
         if (*abort) return false;
     }
@@ -584,13 +585,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
-// Waits for a copy of this thread's own before the block ends (bounded; at once unless the block gave up).
+// Waits for a copy or product of this thread's own before the block ends (bounded; at once unless the block gave up).
 __device__ __forceinline__ void wait_landed(uint64_t* bar, uint32_t parity)
 {
     uint32_t done = 0;
     for (int it = 0; it < kTries && !done; ++it)
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, 1000;\nselp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+}
+// A named barrier of `threads` threads that tells each whether all of them were ok.
+__device__ __forceinline__ bool meet(int id, int threads, bool ok)
+{
+    uint32_t all;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 p, %3, 0;\nbarrier.cta.red.and.aligned.pred q, %1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(all) : "r"(id), "r"(threads), "r"(ok ? 1u : 0u) : "memory");
+    return all != 0;
 }
 __device__ __forceinline__ void copy_bulk(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar)
 {
@@ -606,6 +615,7 @@ struct GemmDev {
     const uint32_t* w_bits;
     int w_stride;
     int tiles;
+    int tries;                                      // bound of the waits between the block's roles
     const int16_t* own;                             // kOwn: the nodes' own dots, rows of own_ld
     int own_ld;
     const float* own_alpha;
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                 bool ok = true;
                 for (int kc = 0; kc < d.n_kc && ok; ++kc, ++s) {
                     const int st = s % kGemmStages;
-                    if (s >= kGemmStages) ok = mbar_wait(&m->empty[st], (uint32_t)(s / kGemmStages + 1) & 1u, abort);
+                    if (s >= kGemmStages) ok = mbar_wait(&m->empty[st], (uint32_t)(s / kGemmStages + 1) & 1u, abort, d.tries);
                     if (!ok) break;
                     copy_bulk(smem_u32(stages + st * kTileChunk), src + (int64_t)kc * kTileChunk, kTileChunk, &m->full[st]);
                 }
@@ -690,19 +700,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
             // D = s32, A = B = s8, both K-major, N = 128, M = 128
             const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
             const uint32_t a_base = smem_u32(a_op), s_base = smem_u32(stages);
-            int s = 0, i = 0;
+            int s = 0, i = 0, owns = 0;
             for (; i < my_tiles; ++i) {
                 const int acc = i % kAcc;
-                if (i >= kAcc && !mbar_wait(&m->acc_empty[acc], (uint32_t)(i / kAcc + 1) & 1u, abort)) break;
+                if (i >= kAcc && !mbar_wait(&m->acc_empty[acc], (uint32_t)(i / kAcc + 1) & 1u, abort, d.tries)) break;
                 if constexpr (kOwn) {
                     const int64_t r0 = (int64_t)(blockIdx.x + i * gridDim.x) * kTileRows;
                     const uint32_t bytes = (uint32_t)min((int64_t)kTileRows, p.n - r0) * (uint32_t)(2 * d.own_ld);
                     copy_bulk(smem_u32(own_s + acc * kTileRows * d.own_ld), d.own + r0 * d.own_ld, bytes, &m->own_full[acc]);
+                    ++owns;
                 }
                 bool ok = true;
                 for (int kc = 0; kc < d.n_kc; ++kc, ++s) {
                     const int st = s % kGemmStages;
-                    ok = mbar_wait(&m->full[st], (uint32_t)(s / kGemmStages) & 1u, abort);
+                    ok = mbar_wait(&m->full[st], (uint32_t)(s / kGemmStages) & 1u, abort, d.tries);
                     if (!ok) break;
                     tc::fence_after_sync();
                     for (int h = 0; h < NM; ++h)
@@ -717,8 +728,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                 if (!ok) break;
                 tc::commit_to(&m->acc_full[acc]);
             }
-            if constexpr (kOwn)
-                for (int q = max(0, i + 1 - kAcc); q < min(i + 1, my_tiles); ++q) wait_landed(&m->own_full[q % kAcc], (uint32_t)(q / kAcc) & 1u);
+            // what was issued is done before the block frees its memory, also where the block gave up
+            if (s > 0) wait_landed(&m->empty[(s - 1) % kGemmStages], (uint32_t)((s - 1) / kGemmStages) & 1u);
+            for (int q = max(0, owns - kAcc); q < owns; ++q) wait_landed(&m->own_full[q % kAcc], (uint32_t)(q / kAcc) & 1u);
         }
     } else {                                                          // epilogue
         const int wg = warp >> 2, wq = warp & 3, h = wg % NM, acc = wg / NM;
@@ -735,54 +747,56 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
             m->rows[warp][0][lane] = __ldg(d.row_scale + my_row);
             if constexpr (kOwn) m->rows[warp][1][lane] = __ldg(d.own_beta + my_row);
             __syncwarp();
-            if (!mbar_wait(&m->acc_full[acc], (uint32_t)(i / kAcc) & 1u, abort)) break;
-            if constexpr (kOwn) {
-                if (!mbar_wait(&m->own_full[acc], (uint32_t)(i / kAcc) & 1u, abort)) break;
-            }
+            bool ok = mbar_wait(&m->acc_full[acc], (uint32_t)(i / kAcc) & 1u, abort, d.tries);
+            if constexpr (kOwn) ok = ok && mbar_wait(&m->own_full[acc], (uint32_t)(i / kAcc) & 1u, abort, d.tries);
+            ok = __all_sync(0xffffffffu, ok);
             const int16_t* own = own_s + acc * kTileRows * d.own_ld + ch;
-            tc::fence_after_sync();
             uint32_t word = 0u;
             float l1_row = 0.f;                                       // lane r: the warp's sum of |x| over row r
+            if (ok) {
+                tc::fence_after_sync();
 #pragma unroll 1
-            for (int rb = 0; rb < kTileRows / 4; ++rb) {              // four rows at a time
-                uint32_t v[16];
-                tc::tmem_ld16(t_addr + (uint32_t)(rb * 16), v);
-                float l1[4];
-                const float4 rs4 = *reinterpret_cast<const float4*>(&m->rows[warp][0][4 * rb]);
-                const float rs[4] = {rs4.x, rs4.y, rs4.z, rs4.w};
+                for (int rb = 0; rb < kTileRows / 4; ++rb) {              // four rows at a time
+                    uint32_t v[16];
+                    tc::tmem_ld16(t_addr + (uint32_t)(rb * 16), v);
+                    float l1[4];
+                    const float4 rs4 = *reinterpret_cast<const float4*>(&m->rows[warp][0][4 * rb]);
+                    const float rs[4] = {rs4.x, rs4.y, rs4.z, rs4.w};
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int lo = (int)v[4 * r] + ((int)v[4 * r + 1] << 8), hi = (int)v[4 * r + 2] + ((int)v[4 * r + 3] << 8);
-                    float x = fmaf((float)hi, 65536.f, (float)lo) * (rs[r] * alpha);
-                    if constexpr (kOwn) {
-                        if (in) x += __fmul_rn(__fmul_rn(m->rows[warp][1][4 * rb + r], own_alpha), (float)own[(4 * rb + r) * d.own_ld]);
+                    for (int r = 0; r < 4; ++r) {
+                        const int lo = (int)v[4 * r] + ((int)v[4 * r + 1] << 8), hi = (int)v[4 * r + 2] + ((int)v[4 * r + 3] << 8);
+                        float x = fmaf((float)hi, 65536.f, (float)lo) * (rs[r] * alpha);
+                        if constexpr (kOwn) {
+                            if (in) x += __fmul_rn(__fmul_rn(m->rows[warp][1][4 * rb + r], own_alpha), (float)own[(4 * rb + r) * d.own_ld]);
+                        }
+                        if constexpr (!kBitsOnly) {
+                            const int row = row0 + 4 * rb + r;
+                            if (row < p.n && in && p.h_out) p.h_out[(int64_t)row * p.ldh + ch] = x;
+                        }
+                        const float xh = __fmul_rn(__fsub_rn(x, shift), scale);
+                        const uint32_t b = __ballot_sync(0xffffffffu, in && xh >= 0.f);
+                        if (lane == 4 * rb + r) word = b;
+                        l1[r] = fabsf(xh);
                     }
-                    if constexpr (!kBitsOnly) {
-                        const int row = row0 + 4 * rb + r;
-                        if (row < p.n && in && p.h_out) p.h_out[(int64_t)row * p.ldh + ch] = x;
-                    }
-                    const float xh = __fmul_rn(__fsub_rn(x, shift), scale);
-                    const uint32_t b = __ballot_sync(0xffffffffu, in && xh >= 0.f);
-                    if (lane == 4 * rb + r) word = b;
-                    l1[r] = fabsf(xh);
-                }
-                if (kBitsOnly || p.next_bits) {                       // four sums over the warp: lanes 4 q + r end with row r's
-                    const bool b0 = lane & 1, b1 = lane & 2;
-                    const float s0 = (b0 ? l1[1] : l1[0]) + __shfl_xor_sync(0xffffffffu, b0 ? l1[0] : l1[1], 1);
-                    const float s1 = (b0 ? l1[3] : l1[2]) + __shfl_xor_sync(0xffffffffu, b0 ? l1[2] : l1[3], 1);
-                    float s = (b1 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, b1 ? s0 : s1, 2);
+                    if (kBitsOnly || p.next_bits) {                       // four sums over the warp: lanes 4 q + r end with row r's
+                        const bool b0 = lane & 1, b1 = lane & 2;
+                        const float s0 = (b0 ? l1[1] : l1[0]) + __shfl_xor_sync(0xffffffffu, b0 ? l1[0] : l1[1], 1);
+                        const float s1 = (b0 ? l1[3] : l1[2]) + __shfl_xor_sync(0xffffffffu, b0 ? l1[2] : l1[3], 1);
+                        float s = (b1 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, b1 ? s0 : s1, 2);
 #pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                    if ((lane >> 2) == rb) l1_row = s;
+                        for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                        if ((lane >> 2) == rb) l1_row = s;
+                    }
                 }
+                tc::fence_before_sync();
+                __syncwarp();                                         // (also: rows[] is written again for the next tile)
+                if (lane == 0) mbar_arrive(&m->acc_empty[acc]);
             }
-            tc::fence_before_sync();
-            __syncwarp();                                             // (also: rows[] is written again for the next tile)
-            if (lane == 0) mbar_arrive(&m->acc_empty[acc]);
             if (kBitsOnly || p.next_bits) {
                 m->words[turn][wg][lane][wq] = word;
                 m->l1[turn][wg][wq][lane] = l1_row;
-                asm volatile("barrier.cta.sync.aligned %0, %1;\n" ::"r"(1 + acc), "n"(128 * NM) : "memory");
+                // the warps of an accumulator leave together: one that went on alone would wait here for the others
+                if (!meet(1 + acc, 128 * NM, ok)) break;
                 const int tid = 32 * wq + lane;
                 if (tid < kTileRows && row0 + tid < p.n)              // this warpgroup's 128 columns of row tid
                     *reinterpret_cast<uint4*>(p.next_bits + (int64_t)(row0 + tid) * p.next_stride + 4 * h) = *reinterpret_cast<const uint4*>(m->words[turn][wg][tid]);
@@ -791,6 +805,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                     if constexpr (NM == 2) s += (m->l1[turn][wg + 1][0][lane] + m->l1[turn][wg + 1][1][lane]) + (m->l1[turn][wg + 1][2][lane] + m->l1[turn][wg + 1][3][lane]);
                     p.next_beta[row0 + lane] = s * p.inv_d_out;
                 }
+            } else if (!ok) {
+                break;
             }
         }
     }
@@ -961,6 +977,7 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
     d.w_bits = w_bits;
     d.w_stride = (int)stride;
     d.tiles = (int)ceil_div(a.n, kTileRows);
+    d.tries = a.wait_tries > 0 ? std::min(a.wait_tries, kTries) : kTries;
     d.own = own ? own->dots : nullptr;
     d.own_ld = own ? (int)own->ld : 0;
     d.own_alpha = own ? own->alpha : nullptr;
