@@ -278,23 +278,36 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
             }
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
-        float m0 = 0.f, m1 = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            w[i] *= bt[i];
-            if (32 * i + lane < g_mid) m0 = fmaxf(m0, fabsf(w[i]));
-            else m1 = fmaxf(m1, fabsf(w[i]));
-        }
-        // |w| < 2^(x - 126): q = round(w 2^(156 - lc - x)), at most 2^lc of them: sum |q| <= 2^30
-        uint32_t x0 = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)) >> 23, 40u), 245u);
-        const uint32_t x1 = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m1)) >> 23, 40u), 245u);
-        int lc0 = 32 - __clz(max(g_mid, 1) - 1);
-        const int lc1 = 32 - __clz(max(g_cnt - g_mid, 1) - 1);
+        for (int i = 0; i < 4; ++i) w[i] *= bt[i];
+        uint32_t x0, x1 = 40u;
+        int lc0 = 0, lc1 = 0;
         int flags = g_flags;
-        if (!(flags & kDirect)) {
-            // a piece of a row: |q| <= 2^30.  Up to three pieces share a scale (with 3 bits to spare for larger weights) and
-            // one read-back: the two low digits' sums of 384 entries just fit 32 bits
-            lc0 = 0;
+        if (flags & kDirect) {
+            // Whole rows: q = round(w 2^(156 - lc - x)) with sum |w| <= 2^(x + lc - 126), so that sum |q| <= 2^30 (and a half per
+            // entry) and a weight is off by 2^-30 of sum |w| at most, whatever share of it the largest has.  (A scale of
+            // entries times the largest weight was off by 2^-24 of that.)  x is the exponent of the largest of the lanes' sums;
+            // these are added up in units of 2^(x - 146), rounded up.
+            float m0 = 0.f, m1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (32 * i + lane < g_mid) m0 += fabsf(w[i]);
+                else m1 += fabsf(w[i]);
+            }
+            auto scale = [](float m, uint32_t& x) {
+                x = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m)) >> 23, 40u), 245u);
+                const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)__float2int_ru(m * __uint_as_float((273u - x) << 23)));
+                return max(12 - __clz((int)t - 1), -1);
+            };
+            lc0 = scale(m0, x0);
+            if (flags & kPair) lc1 = scale(m1, x1);
+        } else {
+            // a piece of a row: |q| <= 2^30 by its largest weight.  Up to three pieces share a scale (with 3 bits to spare for
+            // larger weights) and one read-back: the two low digits' sums of 384 entries just fit 32 bits
+            float m0 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m0 = fmaxf(m0, fabsf(w[i]));
+            x0 = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)) >> 23, 40u), 245u);
             if (!(flags & kFirst) && chain + g_cnt <= 384 && x0 <= chain_x) {
                 x0 = chain_x;
                 chain += g_cnt;
