@@ -24,6 +24,9 @@
 // (M = 128 output columns, resident).  The epilogue combines a row's four digit sums (exact int32), scales by the row's power
 // of two and alpha, and stores H' and / or packs it for the next layer.
 //
+// Rows whose weights have no common fixed point -- a non-finite one, or magnitudes outside 2^-87 .. 2^104 -- carry a mark for
+// their scale, and the second kernel sums them as they are written, in fp32 (literal_row).
+//
 // Two kernels and not one: with both in one kernel the code of all roles did not stay in the instruction cache, and
 // tiles waited for their longest row; P costs one write and one read of 4 bytes per input column and node, which the first
 // kernel's arithmetic hides and the second is bound by.
@@ -75,6 +78,18 @@ struct AggDev {
 };
 
 enum Flags : int { kPair = 1, kDirect = 2, kFirst = 4, kLast = 8, kStarts = 16, kWhole = 32, kMore = 64 };
+
+// Biased exponents of a row's largest weight (of a whole row: of the largest of the lanes' sums) that have a fixed point here.  A row
+// without one gets a scale whose exponent is zero, all ones or beyond, which marks it for literal_row(); what its integers
+// are is of no account then.
+constexpr uint32_t kExpLow = 40, kExpHigh = 230;
+__device__ __forceinline__ bool is_literal(float scale) { return __float_as_uint(scale) - 1u >= 0x7f7fffffu; }
+__device__ __forceinline__ float max_nan(float a, float b)   // NaN if either is
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 
 // Warps per block and resident blocks per multiprocessor: what the registers leave room for beside 64, 32 or 16 accumulators
 // per lane.
@@ -280,7 +295,7 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
         asm volatile("cp.async.commit_group;\n" ::: "memory");
 #pragma unroll
         for (int i = 0; i < 4; ++i) w[i] *= bt[i];
-        uint32_t x0, x1 = 40u;
+        uint32_t x0, x1 = kExpLow, s0, s1 = 0;      // s: exponents of what an integer stands for
         int lc0 = 0, lc1 = 0;
         int flags = g_flags;
         if (flags & kDirect) {
@@ -294,20 +309,26 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
                 if (32 * i + lane < g_mid) m0 += fabsf(w[i]);
                 else m1 += fabsf(w[i]);
             }
-            auto scale = [](float m, uint32_t& x) {
-                x = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m)) >> 23, 40u), 245u);
+            auto scale = [](float m, uint32_t& x, uint32_t& s) {
+                const uint32_t most = __reduce_max_sync(0xffffffffu, __float_as_uint(m));   // (as integers, NaN is the largest of all)
+                x = max(most >> 23, kExpLow);
+                if (x > kExpHigh) x = 320u;          // s from 271 on
                 const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)__float2int_ru(m * __uint_as_float((273u - x) << 23)));
-                return max(12 - __clz((int)t - 1), -1);
+                const int lc = 12 - __clz((int)t - 1);   // -20 to 12 (a row of zeros); below -10, sum |w| < 2^-96, s is 0 or less
+                s = x + lc - 29u;
+                return lc;
             };
-            lc0 = scale(m0, x0);
-            if (flags & kPair) lc1 = scale(m1, x1);
+            lc0 = scale(m0, x0, s0);
+            if (flags & kPair) lc1 = scale(m1, x1, s1);
         } else {
             // a piece of a row: |q| <= 2^30 by its largest weight.  Up to three pieces share a scale (with 3 bits to spare for
             // larger weights) and one read-back: the two low digits' sums of 384 entries just fit 32 bits
+            // (weights too small for a fixed point count only where the whole row has no larger ones: finish())
             float m0 = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) m0 = fmaxf(m0, fabsf(w[i]));
-            x0 = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)) >> 23, 40u), 245u);
+            for (int i = 0; i < 4; ++i) m0 = max_nan(m0, fabsf(w[i]));
+            x0 = max(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)) >> 23, kExpLow);
+            if (x0 > kExpHigh) x0 = 281u;           // bound infinite or NaN, also with 3 bits to spare
             if (!(flags & kFirst) && chain + g_cnt <= 384 && x0 <= chain_x) {
                 x0 = chain_x;
                 chain += g_cnt;
@@ -317,6 +338,7 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
                 chain_x = x0;
                 chain = g_cnt;
             }
+            s0 = x0 - 29u;
         }
         const float f0 = __uint_as_float((283u - lc0 - x0) << 23), f1 = __uint_as_float((283u - lc1 - x1) << 23);
         int w0 = 0, w1 = 0, mag = 0;
@@ -338,18 +360,18 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
             }
         }
         w0 = __reduce_add_sync(0xffffffffu, w0);
-        w1 = __reduce_add_sync(0xffffffffu, w1);
+        if ((flags & (kDirect | kPair)) != kDirect) w1 = __reduce_add_sync(0xffffffffu, w1);
         if (!(flags & kDirect)) mag = __reduce_add_sync(0xffffffffu, mag);
         if (lane == 0) {
             *reinterpret_cast<int4*>(&sl->windows) = make_int4((g_cnt + 31) >> 5, flags, g_row, g_where);
-            *reinterpret_cast<int4*>(&sl->w0) = make_int4(w0, w1, (int)(x0 + lc0 - 29u), flags & kDirect ? (int)(x1 + lc1 - 29u) : mag);
+            *reinterpret_cast<int4*>(&sl->w0) = make_int4(w0, w1, (int)s0, flags & kDirect ? (int)s1 : mag);
         }
     };
     auto tile_of = [&](int row, int pb) { return d.p + (int64_t)(row >> 5) * d.n_kc * kTileChunk + (d.first_kc + (pb >> 7)) * kTileChunk; };
     // facc -> digits of one row
     auto finish = [&](int row, int sli, float bound) {        // bound >= sum |w| of the row: the same for all slices
         __syncwarp();
-        const uint32_t x = min(max(__float_as_uint(bound * 1.0009765625f) >> 23, 40u), 245u);
+        const uint32_t b = __float_as_uint(bound * 1.0009765625f), x = max(b >> 23, kExpLow);
         const float up = __uint_as_float((283u - x) << 23);   // |f| < 2^(x - 126): q = round(f 2^(156 - x))
         // values i .. i + V - 1 of lane 4 g' + odd', V = K / 32 of its MT
         constexpr int V = K / 32;
@@ -374,7 +396,7 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
             else if constexpr (V == 4) *reinterpret_cast<uint32_t*>(dst) = o[i][0];
             else *reinterpret_cast<uint16_t*>(dst) = (uint16_t)o[i][0];
         }
-        if (lane == 0) d.row_scale[row] = __uint_as_float((x - 29u) << 23);
+        if (lane == 0) d.row_scale[row] = __uint_as_float((b < (kExpLow << 23) || b >= ((kExpHigh + 1) << 23) ? 0u : x - 29u) << 23);
         __syncwarp();
     };
 
@@ -633,7 +655,56 @@ struct GemmDev {
     int own_ld;
     const float* own_alpha;
     const float* own_beta;
+    const uint32_t* bits;                           // packed input rows of w_stride words
 };
+
+// One row by one warp, as it is written: every entry's integer dot with every channel times its weight, in fp32, then alpha, the
+// node's own term, and what the epilogue does with a row.  For rows without a fixed point; speed does not matter.
+__device__ __noinline__ void literal_row(const SpmmDev& p, const GemmDev& d, int64_t row, int lane)
+{
+    float acc[8];                                   // channels 32 t + lane
+#pragma unroll
+    for (int t = 0; t < 8; ++t) acc[t] = 0.f;
+    const int kw = (d.d_in + 31) >> 5;
+    const uint32_t last = 0xffffffffu >> (32 * kw - d.d_in);
+    const int64_t end = __ldg(p.rowptr + row + 1);
+    for (int64_t e = __ldg(p.rowptr + row); e < end; ++e) {
+        const int c = __ldg(p.colidx + e);
+        const float w = __ldg(p.val + e) * __ldg(p.node_w + c);
+        const uint32_t* f = d.bits + (int64_t)c * d.w_stride;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const int ch = 32 * t + lane;
+            if (ch >= p.d_out) break;
+            int differ = 0;
+            for (int k = 0; k < kw; ++k) differ += __popc((__ldg(f + k) ^ __ldg(d.w_bits + (int64_t)ch * d.w_stride + k)) & (k == kw - 1 ? last : 0xffffffffu));
+            acc[t] = fmaf(w, (float)(d.d_in - 2 * differ), acc[t]);
+        }
+    }
+    float l1 = 0.f;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int ch = 32 * t + lane;
+        const bool in = ch < p.d_out;
+        float x = 0.f, xh = 0.f;
+        if (in) {
+            x = acc[t] * __ldg(p.col_w + ch);
+            if (d.own) x += __fmul_rn(__fmul_rn(__ldg(d.own_beta + row), __ldg(d.own_alpha + ch)), (float)d.own[row * d.own_ld + ch]);
+            if (p.h_out) p.h_out[row * p.ldh + ch] = x;
+            xh = p.next_shift ? __fmul_rn(__fsub_rn(x, __ldg(p.next_shift + ch)), __ldg(p.next_scale + ch)) : x;
+            l1 += fabsf(xh);
+        }
+        if (p.next_bits && t < p.next_stride) {
+            const uint32_t word = __ballot_sync(0xffffffffu, in && xh >= 0.f);
+            if (lane == 0) p.next_bits[row * p.next_stride + t] = word;
+        }
+    }
+    if (p.next_bits) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+        if (lane == 0) p.next_beta[row] = l1 * p.inv_d_out;
+    }
+}
 
 // NM: blocks of 128 output columns.  Accumulators: 4 / NM tiles in tensor memory, each with a warpgroup per block of columns.
 // kOwn (Bi-GraphSAGE): the node's own term, beta_i alpha_j dot_ij, is added to the row.  Its dots come as 16-bit integers by bulk
@@ -690,6 +761,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = m->tmem;
+    bool literal = false;                                             // a row of this warp's tiles is to be summed as it is written
     const int my_tiles = (int)blockIdx.x < d.tiles ? (d.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
     if (warp == 4 * kEpiGroups) {                                     // copies
@@ -757,7 +829,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
         for (int i = acc; i < my_tiles; i += kAcc) {
             const int row0 = (int)(blockIdx.x + i * gridDim.x) * kTileRows, turn = (i / kAcc) & 1;
             const int my_row = (int)min((int64_t)row0 + lane, p.n - 1);
-            m->rows[warp][0][lane] = __ldg(d.row_scale + my_row);
+            const float scale_row = __ldg(d.row_scale + my_row);
+            literal = literal || is_literal(scale_row);
+            m->rows[warp][0][lane] = scale_row;
             if constexpr (kOwn) m->rows[warp][1][lane] = __ldg(d.own_beta + my_row);
             __syncwarp();
             bool ok = mbar_wait(&m->acc_full[acc], (uint32_t)(i / kAcc) & 1u, abort, d.tries);
@@ -778,7 +852,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const int lo = (int)v[4 * r] + ((int)v[4 * r + 1] << 8), hi = (int)v[4 * r + 2] + ((int)v[4 * r + 3] << 8);
-                        float x = fmaf((float)hi, 65536.f, (float)lo) * (rs[r] * alpha);
+                        float x = fmaf((float)hi, 65536.f, (float)lo) * rs[r] * alpha;
                         if constexpr (kOwn) {
                             if (in) x += __fmul_rn(__fmul_rn(m->rows[warp][1][4 * rb + r], own_alpha), (float)own[(4 * rb + r) * d.own_ld]);
                         }
@@ -824,8 +898,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
         }
     }
     tc::fence_before_sync();
-    __syncthreads();
+    literal = __syncthreads_or(literal) && !*abort;
     if (warp == 0) tc::tmem_free(m->tmem, 512);
+    if (literal) {
+        for (int i = warp; i < my_tiles; i += kGemmThreads / 32) {
+            const int row0 = (int)(blockIdx.x + i * gridDim.x) * kTileRows;
+            const bool mine = row0 + lane < p.n && is_literal(__ldg(d.row_scale + row0 + lane));
+            for (unsigned todo = __ballot_sync(0xffffffffu, mine); todo; todo &= todo - 1) literal_row(p, d, row0 + __ffs(todo) - 1, lane);
+        }
+    }
 }
 
 int gemm_smem(int nm, int n_kc, bool own) { return kGemmStages * kTileChunk + nm * 128 * 128 * n_kc + (own ? kOwnElts * 2 : 0) + (int)sizeof(GemmMisc) + 1024; }
@@ -972,6 +1053,10 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
 
     SpmmDev p = {};
     p.n = a.n;
+    p.rowptr = a.rowptr;
+    p.colidx = a.colidx;
+    p.val = a.val;
+    p.node_w = a.node_w;
     p.d_out = a.d_out;
     p.col_w = a.col_w;
     p.h_out = a.h_out;
@@ -995,6 +1080,7 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
     d.own_ld = own ? (int)own->ld : 0;
     d.own_alpha = own ? own->alpha : nullptr;
     d.own_beta = a.node_w;
+    d.bits = bits;
     const int nm = a.d_out > 128 ? 2 : 1;
     const int smem = gemm_smem(nm, pl.n_kc, own != nullptr);
     const bool bits_only = p.next_bits && !p.h_out;
