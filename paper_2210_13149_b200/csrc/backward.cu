@@ -408,9 +408,12 @@ grad_h_tc_kernel(const float* __restrict__ gz, int64_t ldz, const float* __restr
 
 // ---- G_W~ partial sums on the 5th-generation tensor cores -------------------------------------------------
 // C^T[j][k] = sum over nodes of (beta_i G_zeta[i][j]) F[i][k] with tcgen05.mma kind::f16: M = 128 channels j, N = 64 / 128 /
-// 256 inputs k (blockIdx.z: slices of N), the reduction over the block's nodes, all of them accumulated in one fp32 tile of
-// tensor memory that is read back once at the end and written as slab blockIdx.y of `part` ([k][j]: consecutive lanes
-// write consecutive j).  Both operands are node-major in global memory and stay so in shared memory: M- and N-major operands
+// 256 inputs k (blockIdx.z: slices of N), the reduction over the block's nodes, accumulated in fp32 tiles of tensor memory
+// that are read back at the end, added and written as slab blockIdx.y of `part` ([k][j]: consecutive lanes write
+// consecutive j): one tile for 256 inputs, for fewer two of half the chunks each, which halves the rounding of the long sums
+// where a block has twice the nodes (100 K nodes, 64 -> 64: G_W off by 1.1e-6 of its norm with one tile, 6e-7 with two; as
+// many blocks more instead of tiles: 127 -> 132 us).  Both operands are node-major in global memory and stay so in shared
+// memory: M- and N-major operands
 // with 128-byte swizzle (64 channels or inputs of a node are 128 contiguous bytes), so nothing is transposed and every
 // store is a vector.  Chunks of 32 nodes, two stages: while one is multiplied the other is filled, and the chunk after
 // that is on its way in registers.  (With K-major operands every store was 4 bytes and the stages took turns: 2.4 M nodes,
@@ -427,12 +430,13 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
     pdl_enter();
     constexpr int kStage = 6 * kWtAtom + N / 64 * kWtAtom;  // three terms x two atoms of channels, N / 64 atoms of inputs
     constexpr int kItems = kWtNodes * 32 / kBwThreads;      // 16-byte pieces of a chunk per thread
+    constexpr int kTiles = N <= 128 ? 2 : 1;                // accumulators
     extern __shared__ unsigned char bw_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t tmem_base_s;
     unsigned char* sm = bw_raw + ((1024u - (tc::smem_u32(bw_raw) & 1023u)) & 1023u);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) tc::tmem_alloc(&tmem_base_s, N);
+    if (warp == 0) tc::tmem_alloc(&tmem_base_s, kTiles * N);
     if (threadIdx.x == 0) {
         tc::barrier_init(&bar[0]);
         tc::barrier_init(&bar[1]);
@@ -448,6 +452,7 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
     const int64_t r_begin = (int64_t)blockIdx.y * rows_per_split;
     const int64_t r_end = min(n, r_begin + rows_per_split);
     const int n_chunks = r_begin < r_end ? (int)ceil_div(r_end - r_begin, kWtNodes) : 0;
+    const int second = kTiles == 2 ? (n_chunks + 1) / 2 : n_chunks;      // first chunk of the second accumulator
     // this thread's pieces: channels j .. j + 3 of nodes warp + 8 it; and word wd of node `lane`
     const int j = j0 + 4 * lane, wd = (k0 >> 5) + warp;
     const bool has_word = warp < N / 32 && wd < stride;
@@ -522,15 +527,15 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
         if (__syncthreads_or(!ok)) { ok = false; break; }   // leave together on a timeout
         tc::fence_after_sync();
         if (threadIdx.x == 0) {
-            const uint32_t base = tc::smem_u32(stage);
+            const uint32_t base = tc::smem_u32(stage), acc = tmem_base + (c >= second ? (uint32_t)N : 0u);
             for (int ks = 0; ks < kWtNodes / 16; ++ks) {
                 const uint64_t bd = tc::make_desc(base + 6 * kWtAtom + ks * 2048, kWtAtom, 1024) | ((uint64_t)2 << 61);
 #pragma unroll
                 for (int sp = 0; sp < 3; ++sp) {
                     const uint64_t ad = tc::make_desc(base + sp * 2 * kWtAtom + ks * 2048, kWtAtom, 1024) | ((uint64_t)2 << 61);
-                    const uint32_t accum = (c > 0 || ks > 0 || sp > 0) ? 1u : 0u;
+                    const uint32_t accum = ((c > 0 && c != second) || ks > 0 || sp > 0) ? 1u : 0u;
                     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                                 ::"r"(tmem_base), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
+                                 ::"r"(acc), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
                 }
             }
             tc::commit_to(&bar[st]);
@@ -551,6 +556,12 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
         for (int c0 = c_begin; c0 < c_begin + N / 2; c0 += 16) {
             uint32_t v[16];
             if (n_chunks > 0) tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)c0, v);
+            if (second < n_chunks) {
+                uint32_t u[16];
+                tc::tmem_ld16(tmem_base + ((uint32_t)lane_base << 16) + (uint32_t)(N + c0), u);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(u[e]));
+            }
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const int k = k0 + c0 + e;
@@ -560,7 +571,7 @@ grad_wt_tc_kernel(const uint32_t* __restrict__ bits, int64_t stride, const float
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_free(tmem_base, N);
+    if (warp == 0) tc::tmem_free(tmem_base, kTiles * N);
 }
 
 template <int N>
@@ -619,11 +630,15 @@ grad_w_kernel(const float* __restrict__ g_wt, const double* __restrict__ col_par
 
 int64_t pad4(int64_t d) { return (d + 3) / 4 * 4; }
 
-// Parts that the sum over the nodes is split into: two blocks per multiprocessor in all, at least 128 nodes each.
+// Parts that the sum over the nodes is split into: two blocks per multiprocessor in all, at least 128 nodes each.  Twice as many
+// where an odd number of 128 inputs above 256 would leave fewer than four per multiprocessor and 128 x 128 weights: a part
+// is one fp32 accumulation, whose rounding grows with its length (100 K nodes, 300 -> 200: G_W off by 3.3e-6 of its norm with
+// 74 parts, by 2.4e-6 with 98).
 int wt_splits(int64_t n, int d_in, int d_out)
 {
-    const int64_t tiles = ceil_div(d_in, 256) * ceil_div(d_out, 128);
-    const int64_t want = std::max<int64_t>(1, (sm_count() * 2) / tiles);
+    const int64_t tiles = ceil_div(d_in, 256) * ceil_div(d_out, 128), squares = ceil_div(d_in, 128) * ceil_div(d_out, 128);
+    const int64_t wave = std::max<int64_t>(1, sm_count() * 2 / tiles);
+    const int64_t want = d_in > 256 && sm_count() * 4 / squares > wave ? 2 * wave : wave;
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, ceil_div(n, 128)));
 }
 
