@@ -84,9 +84,9 @@ init_kernel(uint32_t* __restrict__ key_min, uint32_t* __restrict__ key_max, int 
 // Pass 2.  Block (x, y) histograms its share of the rows for the strip of CW columns CW y ..: a warp
 // instruction covers 32 / CW rows x CW columns (CW * 4 contiguous bytes per row); the strip's M x CW
 // counters sit in shared memory and are added to the global ones once per block.  The counters of a column stay in
-// the 32 / CW banks of its own: with CW = 32 (M <= 1,750) the 32 atomic adds of a warp never meet in a bank.  (With the
-// counters of a column contiguous they met in random banks, about 3.5 of 32 in the fullest, and that bounded the pass:
-// 0.49 ms for 2.4 M x 128 values and 1,000 intervals, now 0.25 ms; reading them takes 0.19 ms.)  The rows are taken from the
+// the 32 / CW banks of its own.  (With the counters of a column contiguous the atomic adds of a warp met in random banks,
+// about 3.5 of 32 in the fullest, and that bounded the pass: 0.49 ms for 2.4 M x 128 values and 1,000 intervals, now
+// 0.25 ms; reading them takes 0.19 ms.)  The rows are taken from the
 // last to the first, because pass 1 has just left the last ones of every share in the L2.  The interval of a
 // value is decided in fp32 exactly as documented for the entry point: (x - min) * (M / (max - min)),
 // truncated, clamped to M - 1; a constant column has scale 0 and lands in interval 0.
@@ -233,9 +233,16 @@ cudaError_t launch_entropy_bins(cudaStream_t s, const float* H, int64_t n, int d
         ++*launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    // the widest strip whose counters fit a block's shared memory
-    if (n_bins <= 1750) e = launch_histogram<32>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
-    else if (n_bins <= 3500) e = launch_histogram<16>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
+    // Strips of 16 columns where their counters fit a block's shared memory; of 8 where that leaves fewer lanes past the
+    // last of up to 24 columns (beyond, the half as long row pieces cost more).  Strips of 32 have no two lanes in a bank, but
+    // twice the counters to clear and to add up, which only the rows of a long matrix that is one such strip make up for.
+    // All of the estimate, strips of 32 / 16 / 8: 2.4 M rows, 100 intervals, 8 columns 98 / 77 / 67 us, 24: 138 / 146 / 140, 31:
+    // 156 / 171 / 181, 48: 251 / 230 / 258, 128: 452 / 450 / 486; 1,000 intervals, 24: 163 / 157 / 146, 31: 179 / 185 / 187, 128:
+    // 469 / 460 / 492; 300,000 rows, 100 intervals, 8: 38 / 28 / 24, 24: 42 / 36 / 31, 48: 58 / 46 / 46, 128: 93 / 85 / 87.
+    const bool one = d > 16 && d <= 32 && n >= (int64_t(1) << 20) && n_bins <= (d > 24 ? 1750 : 200);
+    const bool narrow = d <= 24 && round_up(d, 8) < round_up(d, 16) && n_bins <= 1750;
+    if (one) e = launch_histogram<32>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
+    else if (n_bins <= 3500 && !narrow) e = launch_histogram<16>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
     else if (n_bins <= 7000) e = launch_histogram<8>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
     else e = launch_histogram<4>(s, H, n, d, ld, n_bins, key_min, key_max, col_min, col_max, counts);
     ++*launches;
