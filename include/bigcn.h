@@ -85,8 +85,8 @@ enum {
     BIGCN_OPT_LONG_ROW = 2,
     /* How the binary contraction runs.  0 = default: as int8 tensor-core products (tcgen05, the packed bits
      * expanded to +1 / -1 bytes in shared memory; the same integers) for layers with d_in <= 256 and
-     * d_out <= 256 and at least 2^20 outputs, and for layers of more inputs from 3 * 2^23 word steps (n * d_out *
-     * ceil(d_in / 32)) on; on the XOR / bit-count pipe otherwise, and for the debug taps above 256 inputs;
+     * d_out <= 256 and at least 2^20 outputs, and for layers of more inputs from about 10,000 nodes and 33
+     * columns on (fewer nodes for wider layers, 77,000 for narrower ones); on the XOR / bit-count pipe otherwise, and for the debug taps above 256 inputs;
      * 1 = always on the XOR / bit-count pipe; 2 = tensor cores wherever they serve the layer. */
     BIGCN_OPT_CONTRACTION = 3,
     /* How rows of 129..256 signed bytes (zeta formats 3 and 5) are aggregated.

@@ -595,14 +595,20 @@ cudaError_t launch_bitgemm_tc(cudaStream_t s, const uint32_t* A, int64_t stride_
     return launch_tc_n<256>(s, fmt, A, stride_a, BT, stride_b, n, d_in, d_out, beta, alpha, zeta, ldz, dbg_dot, dbg_zeta, nws, col_b0, 0);
 }
 
-// Whether a layer of more than 256 inputs runs on the tensor cores: from 3 x 2^23 word steps (rows x channels x packed words)
-// on.  Below, the bit-count kernel's smaller tiles occupy more of the GPU (a layer, bit counts -> tensor cores: 3,300 rows
-// 3,703 -> 64 25 -> 38 us, 8,000 rows 500 -> 256 29 -> 25 us, 89,250 rows 500 -> 256 157 -> 93 us, 233,000 rows 602 -> 256
-// 427 -> 247 us, all with the aggregation of an empty graph).
+// Whether a layer of more than 256 inputs runs on the tensor cores: by the blocks of work it has, tiles of 128 rows x slices of 64
+// or 128 channels.  Both kernels' times grow alike with d_in, so it does not move the line, but the bit-count kernel's
+// tiles of 16 rows fill multiprocessors that these leave idle below 80 blocks -- 44 where the weights of more than 64
+// channels are long: that kernel reads them all again.  Up to 32 channels it has half the products of these; they win by
+// their reads of the rows alone, from 600 blocks on.
+// Measured, a layer with the aggregation of an empty graph, bit counts / tensor cores: 3,703 -> 64: 4,000 rows (32 blocks) 24 /
+// 36 us, 8,000 (63) 32 / 38, 12,000 (94) 42 / 38; 300 -> 64: 8,192 (64) 13 / 15, 12,000 (94) 15 / 15, 16,384 (128) 17 / 15;
+// 300 -> 256: 4,096 (64) 25 / 25, 8,192 (128) 29 / 27; 1,433 -> 256: 2,000 (32) 27 / 29, 3,000 (48) 33 / 29, 6,000 (94) 43 / 31;
+// 16,000 -> 128: 6,000 (47) 198 / 126; 602 -> 16: 40,000 (313) 33 / 35, 200,000 (1,563) 74 / 68; 89,250 rows 500 -> 256 157 / 93.
 bool bitgemm_takes_wide(int fmt, int64_t n, int d_in, int d_out)
 {
+    const int64_t blocks = ceil_div(n, kTcRows) * ceil_div(d_out, d_out <= 64 ? 64 : 128);
     return d_in > 256 && d_out <= 512 && (fmt == kZetaF32 || fmt == kZetaF16 || fmt == kZetaI16) &&
-           n * (int64_t)d_out * ceil_div(d_in, 32) >= (int64_t(3) << 23);
+           blocks >= (d_out <= 32 ? 600 : (d_out > 64 && d_in > 1024 ? 44 : 80));
 }
 
 cudaError_t launch_bitgemm_wide(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
