@@ -35,13 +35,16 @@ constexpr size_t kAlign = 256;
 // Rows longer than this are split over the warps of a block.  A warp of the machine (148 multiprocessors x 24) has nnz / 3,552
 // entries to do on average, and what the launch waits for is a row of many times that: small graphs split their hub rows
 // earlier (2,708 nodes, hub rows of 300 entries: 13.5 us where the average warp has 4 entries), but only rows well above
-// the mean, because a block takes its split rows one after the other.
-// fp32 rows of more than kLongRowNodes nodes keep the one length: there are enough short rows beside the hub rows to hide them.
-constexpr int64_t kLongRowMax = 2048, kLongRowMin = 64, kLongRowNodes = 32768;
-int64_t default_long_row(int64_t n, int64_t nnz, bool fp32_rows)
+// the mean, because a block takes its split rows one after the other; and, up to 64 columns, only from 128 entries on, because
+// a warp takes narrow rows in fewer steps (a hidden layer, rows of 8 entries, split from 64 / 128 on: 2,700 nodes, 32 columns
+// 19.5 / 17.4 us, 6,000, 16 columns 19.5 / 17.4, 20,000, 64 columns 50 / 47; 6,000, rows of 4, 256 columns 24 / 28).
+// H' of a layer called by itself keeps the one length above kLongRowNodes nodes, and with it the order of its sums; what that
+// costs: 60,000 nodes, rows of 15, 128 columns 168 us, split like the others 96; 250,000 nodes 298, 295.
+constexpr int64_t kLongRowMax = 2048, kLongRowNodes = 32768;
+int64_t default_long_row(int64_t n, int64_t nnz, int d_out, bool fp32_rows)
 {
     if (fp32_rows && n > kLongRowNodes) return kLongRowMax;
-    return std::min(kLongRowMax, std::max(std::max(kLongRowMin, 4 * nnz / std::max<int64_t>(n, 1)), nnz / (148 * 24)));
+    return std::min(kLongRowMax, std::max(std::max<int64_t>(d_out <= 64 ? 128 : 64, 4 * nnz / std::max<int64_t>(n, 1)), nnz / (148 * 24)));
 }
 
 bigcn_status fail(bigcn_ctx* ctx, bigcn_status s, const char* fmt, ...)
@@ -244,7 +247,7 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
     a.next_shift = next ? next->in_shift : nullptr;
     a.next_scale = next ? next->in_scale : nullptr;
     a.any_order = any_order;
-    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, !next && !any_order);
+    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, a.d_out, !next && !any_order);
     a.scratch = scratch;
     a.scratch_bytes = spmm_scratch_bytes(g->n, g->nnz, layer->d_out);
     e = launch_spmm(ctx->stream, a, &ctx->launches_i);
@@ -940,7 +943,7 @@ bigcn_status bigcn_layer_backward(bigcn_ctx* ctx, const bigcn_graph* graph, cons
         return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace (bigcn_backward_workspace_bytes)", backward_scratch_bytes(n, d_in, d_out));
     cudaError_t e = launch_layer_backward(ctx->stream, n, graph->rowptr, graph->colidx, graph->val, d_in, d_out, W, ldw,
                                           layer->alpha, in_bits, bigcn_packed_stride_words(d_in), in_beta, g_out, ldg,
-                                          g_in, ldgi, g_w, ldgw, ctx->long_row ? ctx->long_row : default_long_row(n, graph->nnz, false), ctx->ws,
+                                          g_in, ldgi, g_w, ldgw, ctx->long_row ? ctx->long_row : default_long_row(n, graph->nnz, d_out, false), ctx->ws,
                                           &ctx->launches_i);
     finish_call(ctx);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "backward launch");
@@ -1093,7 +1096,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.zeta = zeta_nbr;
     a.ldz = ldz;
     a.byte_path = ctx->byte_path;
-    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, !next);
+    a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, d_out, !next);
     a.scratch = counter;
     a.scratch_bytes = spmm_scratch_bytes(n, mean_graph->nnz, d_out);
     e = launch_spmm(ctx->stream, a, &ctx->launches_i);
