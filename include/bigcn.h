@@ -109,8 +109,9 @@ enum {
      * 1 = the contraction F B first, then the aggregation of its rows (the kernels the options above choose among);
      * 2 = the aggregation of the packed bits first, P = (A_tilde diag(beta)) F, then P B, both as exact integer products of
      *     fixed-point weights; for d_out <= 256 and weights that fit shared memory (d_in <= 1280, or 640 above 128
-     *     columns), graphs of fewer than about 2^31 entries and rows, and a workspace of bigcn_workspace_bytes();
-     *     otherwise 1.  Edge values of either sign;
+     *     columns), graphs of fewer than about 2^31 entries and rows, and a workspace with room for P; otherwise 1.
+     *     bigcn_workspace_bytes() counts P where the default may take this order and where it is below 64 MB; elsewhere add
+     *     600 bytes per node and 128 inputs and 9 bytes per stored entry and 256 inputs.  Edge values of either sign;
      * 0 = default: 2 for a launch that wants only the next layer's sign bits and beta, where the sizes of the layer and the
      *     graph let it expect to be the faster; 1 otherwise.
      * A layer keeps to 1 when one of the options above is set or a debug tap is asked for.  Both orders meet the same

@@ -272,15 +272,21 @@ size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int 
 }
 
 // Scratch between the kernels of a layer, the larger of the two orders over all layers, and behind it the graph's plan, which
-// layers of both orders leave alone.
-size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers)
+// layers of both orders leave alone.  The packed bits first take 512 bytes per node and 128 inputs, many times the other
+// order's rows for a wide input and few outputs, so they are counted only for layers that may run so by default (one by
+// itself may be called as a hidden layer) or that ask for little, where the option can be tried; `every`: for all that can.
+constexpr size_t kLittle = size_t(64) << 20;
+size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers, bool every)
 {
     size_t m = contraction_first_bytes(n, nnz, dims, n_layers), plan = 0;
-    for (int l = 0; l < n_layers; ++l)
-        if (n > 0 && nnz >= 0 && spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) {
-            m = std::max(m, spmm_bits_scratch_bytes(n, nnz, dims[l]));
-            plan = spmm_bits_plan_bytes(n, nnz);
-        }
+    for (int l = 0; l < n_layers; ++l) {
+        if (n <= 0 || nnz < 0 || !spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) continue;
+        const size_t bytes = spmm_bits_scratch_bytes(n, nnz, dims[l]);
+        const bool hidden = l < n_layers - 1 || n_layers == 1;
+        if (!every && bytes > kLittle && !(hidden && spmm_bits_pays(n, nnz, dims[l], dims[l + 1]))) continue;
+        m = std::max(m, bytes);
+        plan = spmm_bits_plan_bytes(n, nnz);
+    }
     return m + plan;
 }
 
@@ -314,7 +320,8 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     size_t others = 0;                                       // what else the step keeps
     for (int i = 0; i < 2; ++i) others += up((size_t)n * stride_max * 4) + up((size_t)n * 4);
     const size_t least = contraction_first_bytes(n, graph->nnz, dims, n_layers);
-    size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers);
+    size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, ctx->order == 2);
+    if (up(ws.off) + room + others > ws.size) room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, false);
     if (up(ws.off) + room + others > ws.size) room = least;  // a workspace without room for P
     void* zeta = ws.take(room);
     uint32_t* bits[2];
@@ -516,7 +523,7 @@ size_t bigcn_workspace_bytes(int64_t n, int64_t nnz, const int32_t* dims, int32_
         if (l < n_layers && bigcn_packed_stride_words(dims[l]) > stride_max) stride_max = bigcn_packed_stride_words(dims[l]);
         if (dims[l] > d_max) d_max = dims[l];
     }
-    size_t total = layer_scratch_bytes(n, nnz, dims, n_layers);
+    size_t total = layer_scratch_bytes(n, nnz, dims, n_layers, false);
     total += 2 * (up((size_t)n * stride_max * 4) + up((size_t)n * 4));
     size_t aux = up(normalize_scratch_bytes(n));
     if (up(col_stats_scratch_bytes(d_max)) > aux) aux = up(col_stats_scratch_bytes(d_max));

@@ -19,6 +19,7 @@ from paper_2210_13149_b200 import binding as B, synth
 ctx = B.BiGCN(0)
 ctx.set_option(B.OPT_ORDER, 2)
 n = 200000
+ctx.ensure_workspace(2 << 30)           # room for this order in every case from the first call on
 pattern = synth.power_law_graph(n, 300000, 1, device="cuda")
 G, M = ctx.normalize_adjacency(*pattern), ctx.mean_adjacency(*pattern)
 cases = []
