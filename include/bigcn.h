@@ -232,14 +232,16 @@ bigcn_status bigcn_layer_forward(bigcn_ctx* ctx, const bigcn_graph* graph, const
                                  const bigcn_layer* next, uint32_t* next_bits, float* next_beta,
                                  int32_t* dbg_dot, float* dbg_zeta);
 
-/* Per-step device times of one bigcn_forward() call, in milliseconds (CUDA events). */
+/* Per-step device times of one bigcn_forward() call, in milliseconds (CUDA events).  A layer's two products are timed in
+ * the order they run in (BIGCN_OPT_ORDER); the second of them re-binarizes.  The first layer that aggregates the packed bits
+ * also splits the graph's entries into units of work for all that do, within its ms_spmm. */
 typedef struct {
     int32_t n_layers;
     int32_t launches;
     float ms_total;
     float ms_pack;                       /* binarize + pack of X */
-    float ms_gemm[BIGCN_MAX_LAYERS];     /* binary contraction + rescale */
-    float ms_spmm[BIGCN_MAX_LAYERS];     /* aggregation (+ re-binarization) */
+    float ms_gemm[BIGCN_MAX_LAYERS];     /* contraction + rescale */
+    float ms_spmm[BIGCN_MAX_LAYERS];     /* aggregation */
 } bigcn_stats;
 
 /* L stacked layers from fp32 features to logits (H^(0) = X, Sec. 3.2; every layer binarized, the

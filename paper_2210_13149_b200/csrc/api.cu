@@ -165,17 +165,17 @@ void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 
 // One layer on already validated arguments.  `zeta` is `room` bytes of scratch: the contraction's rows in its first zbytes and
 // the aggregation's counter behind them, or (bits first) what spmm_bits_scratch_bytes() counts and the graph's plan, made here
-// unless `planned`.  any_order: H' may be summed in the order that is the fastest (the logits of a forward); a layer called by
+// unless *planned.  ev_mid is recorded between the layer's two products, aggregated_first tells their order.  any_order: H' may be summed in the order that is the fastest (the logits of a forward); a layer called by
 // itself keeps one order, so that thresholds taken from its H' are met by its own sums.
 bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer,
-                       const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool planned,
+                       const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool* planned /*nullable*/,
                        bool any_order, float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,
                        float* next_beta, int32_t* dbg_dot, float* dbg_zeta,
-                       cudaEvent_t ev_mid /*nullable*/)
+                       cudaEvent_t ev_mid /*nullable*/, bool* aggregated_first = nullptr)
 {
     const int64_t stride_in = bigcn_packed_stride_words(layer->d_in);
     if (bits_first(ctx, g, layer, room, next != nullptr, dbg_dot || dbg_zeta) && (!next || aligned(next_bits, 16))) {
-        if (ev_mid) BIGCN_CUDA(ctx, cudaEventRecord(ev_mid, ctx->stream));
+        if (aggregated_first) *aggregated_first = true;
         SpmmArgs a = {};
         a.n = g->n;
         a.nnz = g->nnz;
@@ -195,8 +195,9 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
         a.scratch = zeta;
         a.wait_tries = ctx->wait_tries;
         void* plan = plan_at(g, zeta, room);
-        cudaError_t e = planned ? cudaSuccess : launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
-        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, nullptr, &ctx->launches_i);
+        cudaError_t e = planned && *planned ? cudaSuccess : launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
+        if (planned) *planned = true;
+        if (e == cudaSuccess) e = launch_spmm_bits(ctx->stream, a, plan, in_bits, stride_in, layer->d_in, layer->w_bitsT, nullptr, &ctx->launches_i, ev_mid);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
@@ -344,21 +345,17 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
         cur_bits = bits[0];
         cur_beta = beta[0];
     }
-    // The layers share the graph's plan where the scratch of the contraction-first ones ends before it; otherwise each that
-    // needs it makes its own.
-    bool planned = false;
-    for (int l = 0; l < n_layers && !planned && room >= least + spmm_bits_plan_bytes(n, graph->nnz); ++l) planned = bits_first(ctx, graph, &layers[l], room, l < n_layers - 1, false);
-    if (planned) {
-        cudaError_t e = launch_spmm_bits_plan(ctx->stream, n, graph->nnz, graph->rowptr, plan_at(graph, zeta, room), &ctx->launches_i);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");
-    }
+    // The layers share the graph's plan, made by the first that needs it, where the scratch of the contraction-first ones ends
+    // before it; otherwise each makes its own.
+    const bool shared = room >= least + spmm_bits_plan_bytes(n, graph->nnz);
+    bool planned = false, aggregated_first[BIGCN_MAX_LAYERS] = {};
     if (stats) BIGCN_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
     for (int l = 0; l < n_layers; ++l) {
         const bool last = (l == n_layers - 1);
         const int o = (l + 1) & 1;
-        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, zbytes, room, planned, true,
+        bigcn_status st = run_layer(ctx, graph, &layers[l], cur_bits, cur_beta, zeta, zbytes, room, shared ? &planned : nullptr, true,
                                     last ? logits_out : nullptr, ldo, last ? nullptr : &layers[l + 1],
-                                    bits[o], beta[o], nullptr, nullptr, stats ? ev[2 + 2 * l] : nullptr);
+                                    bits[o], beta[o], nullptr, nullptr, stats ? ev[2 + 2 * l] : nullptr, &aggregated_first[l]);
         if (st != BIGCN_OK) return st;
         if (stats) BIGCN_CUDA(ctx, cudaEventRecord(ev[3 + 2 * l], ctx->stream));
         cur_bits = bits[o];
@@ -371,8 +368,8 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
         stats->launches = ctx->launches_i;
         cudaEventElapsedTime(&stats->ms_pack, ev[0], ev[1]);
         for (int l = 0; l < n_layers; ++l) {
-            cudaEventElapsedTime(&stats->ms_gemm[l], ev[1 + 2 * l], ev[2 + 2 * l]);
-            cudaEventElapsedTime(&stats->ms_spmm[l], ev[2 + 2 * l], ev[3 + 2 * l]);
+            cudaEventElapsedTime(aggregated_first[l] ? &stats->ms_spmm[l] : &stats->ms_gemm[l], ev[1 + 2 * l], ev[2 + 2 * l]);
+            cudaEventElapsedTime(aggregated_first[l] ? &stats->ms_gemm[l] : &stats->ms_spmm[l], ev[2 + 2 * l], ev[3 + 2 * l]);
         }
         cudaEventElapsedTime(&stats->ms_total, ev[0], ev[1 + 2 * n_layers]);
     }
@@ -668,7 +665,7 @@ bigcn_status bigcn_layer_forward(bigcn_ctx* ctx, const bigcn_graph* graph, const
     const size_t zbytes = up(zeta_bytes_max(graph->n, dims, 1));
     const size_t need = zbytes + up(spmm_scratch_bytes(graph->n, graph->nnz, layer->d_out));
     if (!ctx->ws || ctx->ws_bytes < need) return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace, has %zu", need, ctx->ws_bytes);
-    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, zbytes, ctx->ws_bytes, false, false, h_out, ldh, next, next_bits, next_beta,
+    st = run_layer(ctx, graph, layer, in_bits, in_beta, ctx->ws, zbytes, ctx->ws_bytes, nullptr, false, h_out, ldh, next, next_bits, next_beta,
                    dbg_dot, dbg_zeta, nullptr);
     finish_call(ctx);
     return st;

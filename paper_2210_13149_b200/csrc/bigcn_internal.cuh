@@ -124,7 +124,8 @@ size_t spmm_bits_plan_bytes(int64_t n, int64_t nnz);
 cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const int64_t* rowptr, void* plan, int* launches);
 size_t spmm_bits_scratch_bytes(int64_t n, int64_t nnz, int d_in);
 cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan, const uint32_t* bits, int64_t stride, int d_in,
-                             const uint32_t* w_bits, const OwnTerm* own, int* launches);
+                             const uint32_t* w_bits, const OwnTerm* own, int* launches,
+                             cudaEvent_t between = nullptr /* recorded between the two products */);
 int spmm_bits_timeouts();
 
 cudaError_t launch_normalize_adjacency(cudaStream_t s, int64_t n, int64_t nnz_in,

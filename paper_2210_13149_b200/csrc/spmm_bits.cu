@@ -1003,7 +1003,7 @@ cudaError_t launch_spmm_bits_plan(cudaStream_t s, int64_t n, int64_t nnz, const 
 }
 
 cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan, const uint32_t* bits, int64_t stride, int d_in,
-                             const uint32_t* w_bits, const OwnTerm* own, int* launches)
+                             const uint32_t* w_bits, const OwnTerm* own, int* launches, cudaEvent_t between)
 {
     if (a.n == 0) return cudaSuccess;
     const Plan pl = make_plan(a.n, a.nnz, d_in);
@@ -1050,6 +1050,7 @@ cudaError_t launch_spmm_bits(cudaStream_t s, const SpmmArgs& a, const void* plan
         g.counters = counters + (size_t)pl.chunks * pl.full;
         if ((e = pl.rest > 64 ? agg(std::integral_constant<int, 128>()) : agg(std::integral_constant<int, 64>())) != cudaSuccess) return e;
     }
+    if (between && (e = cudaEventRecord(between, s)) != cudaSuccess) return e;
 
     SpmmDev p = {};
     p.n = a.n;
