@@ -112,10 +112,13 @@ enum {
      *     columns), graphs of fewer than about 2^31 entries and rows, and a workspace with room for P; otherwise 1.
      *     bigcn_workspace_bytes() counts P where the default may take this order and where it is below 64 MB; elsewhere add
      *     600 bytes per node and 128 inputs and 9 bytes per stored entry and 256 inputs.  Edge values of either sign;
-     * 0 = default: 2 for a launch that wants only the next layer's sign bits and beta, where the sizes of the layer and the
-     *     graph let it expect to be the faster; 1 otherwise.
+     * 0 = default: 2 for a layer with a next one, whether or not its H' is wanted too, where the sizes of the layer and the
+     *     graph let it expect to be the faster; 1 otherwise, in particular for a layer of which only H' is wanted.  So H' of
+     *     a call without a next layer and of a call with one may round differently; a forward's sign bits follow from the
+     *     latter.
      * A layer keeps to 1 when one of the options above is set or a debug tap is asked for.  Both orders meet the same
-     * tolerance; their fp32 sums differ in rounding. */
+     * tolerance; their fp32 sums differ in rounding.  In order 2 a row of A_tilde diag(beta) with a NaN or an infinity, or
+     * without a fixed point because all of it is below 2^-87 or some of it above 2^104, is summed in fp32 as it is written. */
     BIGCN_OPT_ORDER = 5,
     /* Bound of every wait of one part of a thread block for another in the product P B of order 2, in tries of up to a
      * microsecond: 0 = default (2^20), at most 2^20.  A block whose wait runs out ends early, its outputs unwritten, and
