@@ -165,8 +165,9 @@ void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 
 // One layer on already validated arguments.  `zeta` is `room` bytes of scratch: the contraction's rows in its first zbytes and
 // the aggregation's counter behind them, or (bits first) what spmm_bits_scratch_bytes() counts and the graph's plan, made here
-// unless *planned.  ev_mid is recorded between the layer's two products, aggregated_first tells their order.  any_order: H' may be summed in the order that is the fastest (the logits of a forward); a layer called by
-// itself keeps one order, so that thresholds taken from its H' are met by its own sums.
+// unless *planned.  ev_mid is recorded between the layer's two products, aggregated_first tells their order.  any_order: H' may
+// be summed in the order that is the fastest (the logits of a forward); a layer called by itself keeps one order, so that
+// thresholds taken from its H' are met by its own sums.
 bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer,
                        const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool* planned /*nullable*/,
                        bool any_order, float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,
