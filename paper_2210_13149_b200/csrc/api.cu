@@ -106,6 +106,42 @@ int pick_format(const bigcn_ctx* ctx, int d_in, int d_out, int64_t n, bool allow
     return f;
 }
 
+// How the contraction's rows lie in the zeta scratch.
+struct ZetaRows {
+    int fmt;
+    bool half, tail;
+    int64_t ld;
+    float* nws;      // half-dot bytes: the node factors carrying the first feature sign and the columns' first weight signs follow
+    float* col_b0;   // the byte rows inside the scratch (which is sized for fp32 rows, four times as much)
+    void hand_over(SpmmArgs& a, const float* beta) const
+    {
+        a.fmt = half ? kZetaI8 : fmt;
+        a.ldz = ld;
+        a.node_w = half ? nws : beta;
+        a.half_dots = half;
+        a.col_b0 = col_b0;
+        a.row_tail = tail;
+    }
+};
+// 33..60 byte columns for the lane-per-entry stream (narrow_bytes), on the tensor-core contraction: 64-byte rows that carry the
+// node factor in their last four bytes, so that the aggregation needs two lookups per entry, not four or five.
+ZetaRows zeta_rows(const bigcn_ctx* ctx, const bigcn_graph* g, int d_in, int d_out, void* zeta, bool allow_half, bool narrow_bytes)
+{
+    const int64_t stride = bigcn_packed_stride_words(d_in);
+    ZetaRows z = {};
+    z.fmt = pick_format(ctx, d_in, d_out, g->n, allow_half, narrow_bytes);
+    z.half = z.fmt == kZetaI8H;
+    z.tail = (z.fmt == kZetaI8 || z.half) && narrow_bytes && d_out > 32 && d_out <= 60 &&
+             bitgemm_takes_tc(z.fmt, z.half ? 2 : ctx->contraction, g->n, d_in, d_out, stride, stride);
+    z.ld = z.tail ? 64 : zeta_ld(d_out, z.fmt);
+    if (z.half) {
+        char* after = static_cast<char*>(zeta) + up((size_t)g->n * z.ld);
+        z.nws = reinterpret_cast<float*>(after);
+        z.col_b0 = reinterpret_cast<float*>(after + up((size_t)g->n * 4));
+    }
+    return z;
+}
+
 struct Carver {
     char* base;
     size_t size, off;
@@ -203,26 +239,11 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
         return BIGCN_OK;
     }
     void* const scratch = static_cast<char*>(zeta) + zbytes;
-    const bool lane_stream = (next == nullptr && h_out != nullptr) || (next != nullptr && g->nnz >= 8 * g->n);
-    const int fmt = pick_format(ctx, layer->d_in, layer->d_out, g->n, /*allow_half=*/true, /*narrow_bytes=*/lane_stream);
-    const bool half = fmt == kZetaI8H;
-    // 33..60 byte columns for the lane-per-entry stream, on the tensor-core contraction: 64-byte rows that carry the node
-    // factor in their last four bytes, so that the aggregation needs two lookups per entry, not four or five
-    const bool row_tail = (fmt == kZetaI8 || half) && lane_stream && layer->d_out > 32 && layer->d_out <= 60 &&
-                          bitgemm_takes_tc(fmt, half ? 2 : ctx->contraction, g->n, layer->d_in, layer->d_out, stride_in, stride_in);
-    const int64_t ldz = row_tail ? 64 : zeta_ld(layer->d_out, fmt);
-    // half-dot bytes: the node factors carrying the first feature sign and the columns' first weight signs follow
-    // the byte rows inside the zeta scratch (which is sized for fp32 rows, four times as much)
-    float* nws = nullptr;
-    float* col_b0 = nullptr;
-    if (half) {
-        char* after = static_cast<char*>(zeta) + up((size_t)g->n * ldz);
-        nws = reinterpret_cast<float*>(after);
-        col_b0 = reinterpret_cast<float*>(after + up((size_t)g->n * 4));
-    }
+    const ZetaRows z = zeta_rows(ctx, g, layer->d_in, layer->d_out, zeta, /*allow_half=*/true,
+                                 /*narrow_bytes=*/(next == nullptr && h_out != nullptr) || (next != nullptr && g->nnz >= 8 * g->n));
     cudaError_t e = launch_bitgemm(ctx->stream, in_bits, stride_in, layer->w_bitsT, stride_in, g->n,
-                                   layer->d_in, layer->d_out, in_beta, layer->alpha, fmt, zeta, ldz,
-                                   dbg_dot, dbg_zeta, &ctx->launches_i, half ? 2 : ctx->contraction, nws, col_b0, row_tail ? 1 : 0);
+                                   layer->d_in, layer->d_out, in_beta, layer->alpha, z.fmt, zeta, z.ld,
+                                   dbg_dot, dbg_zeta, &ctx->launches_i, z.half ? 2 : ctx->contraction, z.nws, z.col_b0, z.tail ? 1 : 0);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "bit-GEMM launch");
     if (ev_mid) BIGCN_CUDA(ctx, cudaEventRecord(ev_mid, ctx->stream));
     SpmmArgs a;
@@ -231,16 +252,11 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
     a.rowptr = g->rowptr;
     a.colidx = g->colidx;
     a.val = g->val;
-    a.fmt = half ? kZetaI8 : fmt;
     a.zeta = zeta;
-    a.ldz = ldz;
+    z.hand_over(a, in_beta);
     a.d_out = layer->d_out;
-    a.node_w = half ? nws : in_beta;
     a.col_w = layer->alpha;
-    a.half_dots = half;
     a.byte_path = ctx->byte_path;
-    a.row_tail = row_tail;
-    a.col_b0 = col_b0;
     a.h_out = h_out;
     a.ldh = ldh;
     a.next_bits = next ? next_bits : nullptr;
@@ -1092,14 +1108,15 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
     a.add = zeta_self;
     a.ld_add = ld_self;
-    const int fmt = pick_format(ctx, d_in, d_out, n);
-    const int64_t ldz = zeta_ld(d_out, fmt);
-    e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out,
-                       in_beta, nbr_layer->alpha, fmt, zeta_nbr, ldz, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
+    // 33..48 columns on rows not much shorter than a pass: bytes, for the lane-per-entry stream (2.4 M nodes, 126 M entries, 256 -> 47:
+    // 4.3 ms with fp16 rows on the general stream, 3.0 like this); rows of bytes of more columns have no stream with an own term
+    const bool narrow = d_out > 32 && d_out <= 48 && mean_graph->nnz >= 8 * n;
+    const ZetaRows z = zeta_rows(ctx, mean_graph, d_in, d_out, zeta_nbr, /*allow_half=*/narrow, narrow);
+    e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, nbr_layer->alpha,
+                       z.fmt, zeta_nbr, z.ld, nullptr, nullptr, &ctx->launches_i, z.half ? 2 : ctx->contraction, z.nws, z.col_b0, z.tail ? 1 : 0);
     if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (neighbour term) launch"); }
-    a.fmt = fmt;
     a.zeta = zeta_nbr;
-    a.ldz = ldz;
+    z.hand_over(a, in_beta);
     a.byte_path = ctx->byte_path;
     a.long_row = ctx->long_row > 0 ? ctx->long_row : default_long_row(a.n, a.nnz, d_out, !next);
     a.scratch = counter;

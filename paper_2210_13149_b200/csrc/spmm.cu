@@ -1190,11 +1190,14 @@ constexpr int kLaneWarps = 8;
 constexpr int kLaneThreads = kLaneWarps * kWarp;
 constexpr int kLanePitch = 68;                                // floats per lane in the reduction buffer (64 + 4: 16-byte stores of 8 lanes fall into distinct banks)
 
+// Whether rows of nv vectors may have a row added (kAdd): four leave no registers for it.
+__host__ __device__ constexpr bool lane_may_add(int nv) { return nv < 4; }
+
 // Streams rows [row_lo, row_hi) of a run (kPartial: the stored entries [e0, e0 + n_ent) as one row, whose sums are
 // handed back in `out` / `wsum` / `wsgn` instead of being written).
 // kTail: a row of zeta is 64 bytes, 32-byte aligned, and carries its node factor in its last four bytes: an entry's
 // dots and factor come with one pair of 32-byte loads (two tag lookups per entry instead of NV + 1).
-template <int NV, bool kHalf, bool kPartial, bool kTail = false, bool kNext = false>
+template <int NV, bool kHalf, bool kPartial, bool kTail = false, bool kNext = false, bool kAdd = false>
 __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, int lane, int64_t e0, int n_ent,
                                                  int64_t warp_row0, int row_lo, int row_hi, int rp_rel,
                                                  const float (&al)[4], const float (&b0)[4], float4& out, float& wsum_out, float& wsgn_out,
@@ -1268,6 +1271,12 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
         w1 = w2;
         gather(c1);                                           // the next pass's operand rows
         fetch_indices(c2, w2);                                // the indices of the pass after that
+        float own[NV];                                        // the row's added values, asked for before its last products
+        if (kAdd && !kPartial && row_start(cr) + co + 32 >= row_end(cr)) {
+            const float* src = p.add + (warp_row0 + cr) * p.ld_add + (lane >> 1);
+#pragma unroll
+            for (int q = 0; q < NV; ++q) own[q] = 16 * q + (lane >> 1) < p.d_out ? __ldg(src + 16 * q) : 0.f;
+        }
         const float wa = kHalf ? fabsf(wt) : wt;              // half-dot bytes: the sign carries the source's first feature sign
         if (kHalf) { ws += wa; wg += wt; }
 #pragma unroll
@@ -1316,6 +1325,7 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
             for (int q = 0; q < NV; ++q) {
                 if (kHalf) x[q] = fmaf(2.f, x[q], fmaf(b02[q], wg, ws));
                 x[q] *= al2[q];
+                if (kAdd) x[q] += own[q];
             }
             if ((!kNext || p.h_out) && (lane & 1) == 0) {
                 float* dst = p.h_out + (warp_row0 + cr) * p.ldh + j;
@@ -1400,7 +1410,7 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
     }
 }
 
-template <int NV, bool kHalf, bool kTail = false, bool kNext = false>
+template <int NV, bool kHalf, bool kTail = false, bool kNext = false, bool kAdd = false>
 __global__ void __launch_bounds__(kLaneThreads, 2)
 spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
 {
@@ -1459,7 +1469,7 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
             const int rl = rest ? ra + (__ffs(rest) - 1) : n_rows;
             if (rl > ra) {
                 const int64_t e0 = __shfl_sync(0xffffffffu, rp_reg, ra);
-                stream_rows_lane<NV, kHalf, false, kTail, kNext>(p, red, lane, e0, 0, warp_row0, ra, rl, (int)(rp_reg - e0), al, b0, t, ws, wg, al2, b02);
+                stream_rows_lane<NV, kHalf, false, kTail, kNext, kAdd>(p, red, lane, e0, 0, warp_row0, ra, rl, (int)(rp_reg - e0), al, b0, t, ws, wg, al2, b02);
             }
             ra = rl + 1;
         }
@@ -1492,6 +1502,7 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
                 for (int i = 0; i < 4; ++i) {
                     if (kHalf) x[i] = fmaf(2.f, x[i], fmaf(b0[i], swg, sws));
                     x[i] *= al[i];
+                    if (kAdd && 4 * cg + i < p.d_out) x[i] += __ldg(p.add + lrow * p.ld_add + 4 * cg + i);
                     if ((!kNext || p.h_out) && 4 * cg + i < p.d_out) p.h_out[lrow * p.ldh + 4 * cg + i] = x[i];
                 }
             }
@@ -1525,19 +1536,28 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
     }
 }
 
-template <int NV, bool kHalf, bool kTail = false, bool kNext = false>
-cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
+template <int NV, bool kHalf, bool kTail, bool kNext, bool kAdd>
+cudaError_t launch_lane_inst(cudaStream_t s, const SpmmDev& p)
 {
     constexpr size_t smem = ((size_t)kLaneWarps * 32 * kLanePitch + (size_t)kLaneWarps * (NV * 16 + 4)) * sizeof(float);
     const int rows_per_warp = (int)std::min<int64_t>(kMaxRowsPerWarp, std::max<int64_t>(1, p.n / (kLaneWarps * sm_count() * 8)));
-    cudaError_t e = cudaFuncSetAttribute(spmm_lane_kernel<NV, kHalf, kTail, kNext>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(spmm_lane_kernel<NV, kHalf, kTail, kNext, kAdd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t wanted = ceil_div(ceil_div(p.n, rows_per_warp), kLaneWarps);
     const unsigned grid = (unsigned)std::min<int64_t>(wanted, sm_count() * 2);
     e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    launch_kernel(spmm_lane_kernel<NV, kHalf, kTail, kNext>, grid, kLaneThreads, smem, s, p, rows_per_warp);
+    launch_kernel(spmm_lane_kernel<NV, kHalf, kTail, kNext, kAdd>, grid, kLaneThreads, smem, s, p, rows_per_warp);
     return cudaGetLastError();
+}
+
+template <int NV, bool kHalf, bool kTail = false, bool kNext = false>
+cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
+{
+    if constexpr (lane_may_add(NV)) {
+        if (p.add) return launch_lane_inst<NV, kHalf, kTail, kNext, true>(s, p);
+    }
+    return launch_lane_inst<NV, kHalf, kTail, kNext, false>(s, p);
 }
 
 // ---- short rows ----------------------------------------------------------------------------------------------------
@@ -1922,7 +1942,7 @@ cudaError_t dispatch(cudaStream_t s, const SpmmDev& p, double mean_row)
     if constexpr (sizeof(T) == 1) {
         // 33..64 byte columns, written out as fp32 (a last layer) or re-binarized (a hidden layer), rows not much
         // shorter than a pass: one entry per lane
-        if ((nv == 3 || nv == 4) && (p.h_out || p.next_bits) && !p.add && p.byte_path != 2 && !(mean_row > 0.0 && mean_row < 8.0)) {
+        if ((nv == 3 || nv == 4) && (p.h_out || p.next_bits) && (!p.add || lane_may_add(p.d_out <= 48 ? 3 : 4)) && p.byte_path != 2 && !(mean_row > 0.0 && mean_row < 8.0)) {
             if (p.next_bits) {
                 if (p.row_tail && nv == 4) {
                     const bool three = p.d_out <= 48;
