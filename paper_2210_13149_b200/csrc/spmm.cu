@@ -1565,7 +1565,7 @@ cudaError_t launch_lane(cudaStream_t s, const SpmmDev& p)
 // hold its vectors where those are more), so a warp takes 32 / S rows at once, and their bookkeeping, gathers and epilogues
 // share instructions.  A chunk is S stored entries of each of the rows: lane i of the S loads entry i's column, value and
 // factor -- column and value one chunk ahead, across rows -- and then every entry's row is fetched by the LPR lanes of one
-// of the S / LPR lane groups, up to eight fetches in flight.  Rows of more than 8 S entries are taken by the whole warp,
+// of the S / LPR lane groups, up to eight fetches in flight.  Rows of more than wide_from entries are taken by the whole warp,
 // those above long_row by the block.  The order of summation differs from stream_entries()'s: for hidden layers, whether or not
 // they also write H', for gradients and for the logits of a forward (any_order).
 //
@@ -1623,7 +1623,7 @@ __host__ __device__ constexpr int row_blocks(int elt_bytes) { return elt_bytes =
 
 template <typename T, int LPR>
 __global__ void __launch_bounds__(kSpmmThreads, row_blocks(sizeof(T)))
-spmm_rows_kernel(const SpmmDev p, int rows_per_take, int dynamic)
+spmm_rows_kernel(const SpmmDev p, int rows_per_take, int wide_from, int dynamic)
 {
     pdl_enter();
     constexpr int EPV = Elt<T>::kPerVec, kCols = LPR * EPV, S = row_lanes(LPR), R = 32 / S;
@@ -1682,7 +1682,7 @@ spmm_rows_kernel(const SpmmDev p, int rows_per_take, int dynamic)
             if (slot < kLongQueue) long_rows[slot] = row0 + lane;
             else is_long = false;
         }
-        const bool wide = lane < n_rows && !is_long && (S == 32 || rp_next - rp > 8 * S);
+        const bool wide = lane < n_rows && !is_long && (S == 32 || rp_next - rp > wide_from);
         unsigned wide_mask = __ballot_sync(0xffffffffu, wide);
         if constexpr (S < 32) {
             // lane i: row i's entries, or -1 where the rows below do not take it
@@ -1919,14 +1919,22 @@ cudaError_t launch_rows(cudaStream_t s, const SpmmDev& p, double mean_row)
     // rows that a warp takes at a time: four sets (four rows where most of them take a whole warp), fewer where that would
     // leave warps without rows
     const int unit = mean_row > 32.0 ? 1 : R;
-    const int rows_per_take = (int)std::min<int64_t>(4, std::max<int64_t>(1, p.n / (2 * warps * unit))) * unit;
+    // On graphs of fewer rows than there are warps a launch is one row's chain of dependent fetches: a warp takes one row, with all of
+    // its lanes where the row has more than S entries (3,327 rows of 4, 64 / 16 / 6 columns: 15.6 / 9.1 / 8.8 us four rows to a warp,
+    // 9.2 / 6.4 / 6.2 like this; 4,000 of 11: 19.0 / 11.3 / 11.2, 12.7 / 9.1 / 8.6).
+    constexpr int S = row_lanes(LPR);
+    const bool one = p.n <= warps;
+    const int rows_per_take = one ? 1 : (int)std::min<int64_t>(4, std::max<int64_t>(1, p.n / (2 * warps * unit))) * unit;
     const int64_t takes = ceil_div(p.n, rows_per_take);
     const int dynamic = takes > 2 * warps ? 1 : 0;            // (on small graphs the counter's latency is not worth it)
     if (dynamic) {
         cudaError_t e = cudaMemsetAsync(p.run_counter, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
-    launch_kernel(spmm_rows_kernel<T, LPR>, (unsigned)ceil_div(std::min(takes, warps), kSpmmWarps), kSpmmThreads, 0, s, p, rows_per_take, dynamic);
+    // rows of more entries are taken by the whole warp: it takes them in fewer steps, but one after the other, while the other row
+    // sets of the warp wait (19,717 rows of 5.5, 64 columns, from 64 / 32 entries on: 17.7 / 16.3 us; 8,000 of 26, 7 columns: 14.7 / 16.1)
+    const int wide_from = one ? S : (!dynamic && mean_row <= 8.0 ? 4 * S : 8 * S);
+    launch_kernel(spmm_rows_kernel<T, LPR>, (unsigned)ceil_div(std::min(takes, warps), kSpmmWarps), kSpmmThreads, 0, s, p, rows_per_take, wide_from, dynamic);
     return cudaGetLastError();
 }
 
