@@ -230,48 +230,42 @@ pack_rows_staged_kernel(const float* __restrict__ H, int64_t n, int d, int64_t l
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
-// Weights: W is [d_in x d_out] row-major and the packed output is transposed (one row per output
-// channel, packed along d_in).  A 32 x 32 tile is read coalesced along d_out, the sign bits go
-// through shared memory, and warp t ballots the 32 k-values of channel j0 + t.
+// Weights: W is [d_in x d_out] row-major and the packed output is transposed (one row per output channel, packed along d_in).
+// Blocks (x, y > 0): word y - 1 of channels 32 x ..: a 32 x 32 tile is read coalesced along d_out, the sign bits go through
+// shared memory, and warp t ballots the 32 k-values of channel 32 x + t.  Blocks (x, 0), first because they take longest:
+// alpha_j = ||W_:,j||_1 / d_in; thread (tx, ty) sums rows ty, ty + 32, ... of column 32 x + tx in double, then the 32 partial
+// sums of a column are added in a fixed order.  One kernel for both, which a training step calls for every layer.
 __global__ void __launch_bounds__(1024)
 pack_weights_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ldw,
-                    uint32_t* __restrict__ bitsT, int64_t stride)
+                    uint32_t* __restrict__ bitsT, int64_t stride, float* __restrict__ alpha)
 {
     pdl_enter();
-    __shared__ unsigned char sgn[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int j0 = blockIdx.x * 32;
-    const int w = blockIdx.y;                 // word index along d_in; words >= ceil(d_in/32) are padding
+    const int j0 = blockIdx.x * 32, j = j0 + tx;
+    if (blockIdx.y == 0) {
+        __shared__ double part[32][33];
+        double s = 0.0;
+        if (j < d_out)
+#pragma unroll 8
+            for (int k = ty; k < d_in; k += 32) s += (double)fabsf(__ldg(W + (int64_t)k * ldw + j));
+        part[ty][tx] = s;
+        __syncthreads();
+        if (ty == 0 && j < d_out) {
+            double t = 0.0;
+            for (int r = 0; r < 32; ++r) t += part[r][tx];
+            alpha[j] = (float)(t / (double)d_in);
+        }
+        return;
+    }
+    __shared__ unsigned char sgn[32][33];
+    const int w = blockIdx.y - 1;             // word index along d_in; words >= ceil(d_in/32) are padding
     const int k = w * 32 + ty;
-    const int j = j0 + tx;
     bool pos = false;
     if (k < d_in && j < d_out) pos = __ldg(W + (int64_t)k * ldw + j) >= 0.f;
     sgn[ty][tx] = pos ? 1 : 0;
     __syncthreads();
     const uint32_t word = __ballot_sync(0xffffffffu, sgn[tx][ty] != 0);   // lane tx = k offset, channel j0 + ty
     if (tx == 0 && j0 + ty < d_out) bitsT[(int64_t)(j0 + ty) * stride + w] = word;
-}
-
-// alpha_j = ||W_:,j||_1 / d_in.  One block per 32 channels; thread (tx, ty) sums rows ty, ty+32, ...
-// of column j0 + tx in double, then the 32 partial sums of a column are added in a fixed order.
-__global__ void __launch_bounds__(1024)
-weight_scale_kernel(const float* __restrict__ W, int d_in, int d_out, int64_t ldw, float* __restrict__ alpha)
-{
-    pdl_enter();
-    __shared__ double part[32][33];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int j = blockIdx.x * 32 + tx;
-    double s = 0.0;
-    if (j < d_out)
-#pragma unroll 8
-        for (int k = ty; k < d_in; k += 32) s += (double)fabsf(__ldg(W + (int64_t)k * ldw + j));
-    part[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0 && j < d_out) {
-        double t = 0.0;
-        for (int r = 0; r < 32; ++r) t += part[r][tx];
-        alpha[j] = (float)(t / (double)d_in);
-    }
 }
 
 }  // namespace
@@ -338,12 +332,8 @@ cudaError_t launch_pack_weights(cudaStream_t s, const float* W, int d_in, int d_
                                 uint32_t* bitsT, int64_t stride, float* alpha, int* launches)
 {
     const dim3 block(32, 32);
-    const dim3 grid((unsigned)ceil_div(d_out, 32), (unsigned)stride);
-    launch_kernel(pack_weights_kernel, grid, block, 0, s, W, d_in, d_out, ldw, bitsT, stride);
-    ++*launches;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    launch_kernel(weight_scale_kernel, (unsigned)ceil_div(d_out, 32), block, 0, s, W, d_in, d_out, ldw, alpha);
+    const dim3 grid((unsigned)ceil_div(d_out, 32), (unsigned)stride + 1);
+    launch_kernel(pack_weights_kernel, grid, block, 0, s, W, d_in, d_out, ldw, bitsT, stride, alpha);
     ++*launches;
     return cudaGetLastError();
 }
