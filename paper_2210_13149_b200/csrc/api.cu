@@ -16,7 +16,7 @@ struct bigcn_ctx {
     char err[512];
     void* ws;
     size_t ws_bytes;
-    int* d_flag;                 // device status words (owned)
+    int* d_flag;                 // device status words (owned), and behind the first kFlagBytes the counters of column statistics
     int launches_i;              // launches of the call in progress
     int64_t launches;
     int zeta_format;             // 0 = auto
@@ -31,7 +31,7 @@ struct bigcn_ctx {
 
 namespace {
 
-constexpr size_t kAlign = 256;
+constexpr size_t kAlign = 256, kFlagBytes = 256;
 // Rows longer than this are split over the warps of a block.  A warp of the machine (148 multiprocessors x 24) has nnz / 3,552
 // entries to do on average, and what the launch waits for is a row of many times that: small graphs split their hub rows
 // earlier (2,708 nodes, hub rows of 300 entries: 13.5 us where the average warp has 4 entries), but only rows well above
@@ -449,8 +449,9 @@ bigcn_status bigcn_create(bigcn_ctx** out, int device, void* cuda_stream)
     memset(ctx, 0, sizeof(*ctx));
     ctx->device = device;
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMalloc(reinterpret_cast<void**>(&ctx->d_flag), 256) != cudaSuccess ||
-        cudaMemset(ctx->d_flag, 0, 256) != cudaSuccess) {
+    constexpr size_t owned = kFlagBytes + kStatGroups * sizeof(unsigned);
+    if (cudaMalloc(reinterpret_cast<void**>(&ctx->d_flag), owned) != cudaSuccess ||
+        cudaMemset(ctx->d_flag, 0, owned) != cudaSuccess) {
         delete ctx;
         return BIGCN_ERR_CUDA;
     }
@@ -903,7 +904,8 @@ bigcn_status bigcn_col_stats(bigcn_ctx* ctx, const float* H, int64_t n, int32_t 
     if (n < 0 || d < 1 || ld < d || !(eps >= 0.f)) return fail(ctx, BIGCN_ERR_SHAPE, "n=%lld d=%d ld=%lld eps=%g", (long long)n, d, (long long)ld, (double)eps);
     if (!shift_out || !scale_out || (n > 0 && !H)) return fail(ctx, BIGCN_ERR_NULL, "H, shift_out or scale_out is null");
     if (!ctx->ws || ctx->ws_bytes < col_stats_scratch_bytes(d)) return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace", col_stats_scratch_bytes(d));
-    cudaError_t e = launch_col_stats(ctx->stream, H, n, d, ld, eps, shift_out, scale_out, ctx->ws, &ctx->launches_i);
+    cudaError_t e = launch_col_stats(ctx->stream, H, n, d, ld, eps, shift_out, scale_out, ctx->ws,
+                                     reinterpret_cast<unsigned*>(reinterpret_cast<char*>(ctx->d_flag) + kFlagBytes), &ctx->launches_i);
     finish_call(ctx);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "col_stats launch");
     return BIGCN_OK;

@@ -139,8 +139,10 @@ cudaError_t launch_adjacency_from_edges(cudaStream_t s, int64_t n, int64_t m, co
                                         int64_t* rowptr, int32_t* colidx, void* scratch, int* flag, int* launches);
 size_t edges_scratch_bytes(int64_t m);
 
+// done: kStatGroups counters that are zero before and after
+constexpr int kStatGroups = 4096;
 cudaError_t launch_col_stats(cudaStream_t s, const float* H, int64_t n, int d, int64_t ld, float eps,
-                             float* shift, float* scale, void* scratch, int* launches);
+                             float* shift, float* scale, void* scratch, unsigned* done, int* launches);
 size_t col_stats_scratch_bytes(int d);
 
 cudaError_t measure_popc_peak(cudaStream_t s, void* scratch, double* word_steps_per_s, int* launches);

@@ -170,21 +170,25 @@ fill_kernel(int64_t n, const int64_t* __restrict__ rowptr_A, const int32_t* __re
 
 constexpr int kStatChunksMax = 1024;
 
+// Block (x, y) sums chunk y of the rows over columns 32 x .. 32 x + 31.  The block of a column group that ends last (counted in
+// done[x], which is zero before and after) adds the chunks up, thread (tx, ty) chunks ty, ty + 8, ..., then the eight sums in
+// order.  One wave of blocks: with chunks of 64 rows and a second kernel for the sums, 19,717 x 500 took 28 us.
 __global__ void __launch_bounds__(256)
-col_partial_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int64_t rows_per_chunk,
-                   double* __restrict__ partial /* [chunks][d][2] */)
+col_stats_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int64_t rows_per_chunk, double eps,
+                 double* __restrict__ partial /* [chunks][d][2] */, unsigned* __restrict__ done, float* __restrict__ shift, float* __restrict__ scale)
 {
     pdl_enter();
     __shared__ double s_sum[8][33], s_sq[8][33];
+    __shared__ bool last;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + tx;
     const int64_t r0 = (int64_t)blockIdx.y * rows_per_chunk;
     const int64_t r1 = min(n, r0 + rows_per_chunk);
     // sums of (x - pivot) and (x - pivot)^2 around the column's first value: the variance formed from them does
     // not cancel for a column with a large offset, and is exactly 0 for a constant one
-    double s = 0.0, q = 0.0;
-    if (j < d) {
-        const double pivot = (double)__ldg(H + j);
+    double s = 0.0, q = 0.0, pivot = 0.0;
+    if (j < d && n > 0) {
+        pivot = (double)__ldg(H + j);
 #pragma unroll 8
         for (int64_t r = r0 + ty; r < r1; r += 8) {
             const double x = (double)__ldg(H + r * ld + j) - pivot;
@@ -192,47 +196,44 @@ col_partial_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, in
             q += x * x;
         }
     }
-    s_sum[ty][tx] = s;
-    s_sq[ty][tx] = q;
-    __syncthreads();
-    if (ty == 0 && j < d) {
-        double ts = 0.0, tq = 0.0;
-        for (int r = 0; r < 8; ++r) { ts += s_sum[r][tx]; tq += s_sq[r][tx]; }
-        partial[((int64_t)blockIdx.y * d + j) * 2] = ts;
-        partial[((int64_t)blockIdx.y * d + j) * 2 + 1] = tq;
-    }
-}
-
-// A block per 32 columns; thread (tx, ty) adds chunks ty, ty + 32, ... of column tx, the 32 sums are added in order.  (A
-// thread per column walked through all chunks alone: 18 us for 78 chunks.)
-__global__ void __launch_bounds__(1024)
-col_final_kernel(const float* __restrict__ H, const double* __restrict__ partial, int chunks, int d, int64_t n, double eps,
-                 float* __restrict__ shift, float* __restrict__ scale)
-{
-    pdl_enter();
-    __shared__ double s_sum[32][33], s_sq[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int j = blockIdx.x * 32 + tx;
-    double s = 0.0, q = 0.0;
-    if (j < d) {
-#pragma unroll 4
-        for (int c = ty; c < chunks; c += 32) {
-            const double2 v = __ldg(reinterpret_cast<const double2*>(partial) + (int64_t)c * d + j);
-            s += v.x;
-            q += v.y;
+    auto add_up = [&]() {                             // the totals, in the threads ty = 0
+        s_sum[ty][tx] = s;
+        s_sq[ty][tx] = q;
+        __syncthreads();
+        if (ty == 0) {
+            for (int r = 1; r < 8; ++r) {
+                s += s_sum[r][tx];
+                q += s_sq[r][tx];
+            }
         }
+    };
+    add_up();
+    if (gridDim.y > 1) {
+        if (ty == 0 && j < d) {
+            double2* to = reinterpret_cast<double2*>(partial) + (int64_t)blockIdx.y * d + j;
+            __stcg(to, make_double2(s, q));
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(done + blockIdx.x, 1u) == gridDim.y - 1;
+        __syncthreads();
+        if (!last) return;
+        if (threadIdx.x == 0) done[blockIdx.x] = 0u;
+        __threadfence();
+        s = q = 0.0;
+        if (j < d) {
+#pragma unroll 8
+            for (int c = ty; c < (int)gridDim.y; c += 8) {
+                const double2 v = __ldcg(reinterpret_cast<const double2*>(partial) + (int64_t)c * d + j);
+                s += v.x;
+                q += v.y;
+            }
+        }
+        add_up();
     }
-    s_sum[ty][tx] = s;
-    s_sq[ty][tx] = q;
-    __syncthreads();
     if (ty != 0 || j >= d) return;
-    s = q = 0.0;
-    for (int r = 0; r < 32; ++r) {
-        s += s_sum[r][tx];
-        q += s_sq[r][tx];
-    }
     const double off = n > 0 ? s / (double)n : 0.0;                       // mean of x - pivot
-    const double mean = n > 0 ? (double)__ldg(H + j) + off : 0.0;
+    const double mean = n > 0 ? pivot + off : 0.0;
     double var = n > 0 ? q / (double)n - off * off : 0.0;
     if (var < 0.0) var = 0.0;
     shift[j] = (float)mean;
@@ -271,16 +272,15 @@ cudaError_t launch_normalize_adjacency(cudaStream_t s, int64_t n, int64_t nnz_in
 size_t col_stats_scratch_bytes(int d) { return (size_t)kStatChunksMax * (size_t)d * 16; }
 
 cudaError_t launch_col_stats(cudaStream_t s, const float* H, int64_t n, int d, int64_t ld, float eps,
-                             float* shift, float* scale, void* scratch, int* launches)
+                             float* shift, float* scale, void* scratch, unsigned* done, int* launches)
 {
-    const int64_t rows_per_chunk = std::max<int64_t>(64, ceil_div(n, kStatChunksMax));
+    const int64_t groups = ceil_div(d, 32);
+    // one wave of blocks (eight to a multiprocessor), of at least 64 rows each
+    const int64_t wanted = groups > kStatGroups ? 1 : std::min<int64_t>(kStatChunksMax, std::max<int64_t>(1, 8 * sm_count() / groups));
+    const int64_t rows_per_chunk = std::max<int64_t>(64, ceil_div(n, wanted));
     const int chunks = (int)std::max<int64_t>(1, ceil_div(n, rows_per_chunk));
-    double* partial = reinterpret_cast<double*>(scratch);
-    launch_kernel(col_partial_kernel, dim3((unsigned)ceil_div(d, 32), (unsigned)chunks), 256, 0, s, H, n, d, ld, rows_per_chunk, partial);
-    ++*launches;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    launch_kernel(col_final_kernel, (unsigned)ceil_div(d, 32), 1024, 0, s, H, partial, chunks, d, n, (double)eps, shift, scale);
+    launch_kernel(col_stats_kernel, dim3((unsigned)groups, (unsigned)chunks), 256, 0, s, H, n, d, ld, rows_per_chunk, (double)eps,
+                  static_cast<double*>(scratch), done, shift, scale);
     ++*launches;
     return cudaGetLastError();
 }
