@@ -53,6 +53,10 @@ __device__ int g_bits_timeout;                      // set when a bounded wait r
 
 constexpr int kGroup = 128;                         // stored entries of a group
 constexpr int kRowCost = 4;                         // what a row counts beside its entries where work is split
+// Entries of a row under one scale: their sum of |q| >> kMagShift fits 32 bits.  From kChainAny on, pieces whose largest weight is
+// less than a quarter of the scale's start another, so that they are not rounded more coarsely for it.  (Up to three pieces
+// whatever the row: 60,000 nodes in rows of 470, 256 inputs, one read-back for three pieces 506 us, 488 now.)
+constexpr int kChain = 2048, kChainAny = 384, kMagShift = 10;
 constexpr int kTileRows = 32;                       // rows of a tile of P
 constexpr int kTileChunk = 128 * 128;               // bytes of 128 input columns of a tile: 32 rows x 4 digits x 128
 
@@ -321,15 +325,15 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
             lc0 = scale(m0, x0, s0);
             if (flags & kPair) lc1 = scale(m1, x1, s1);
         } else {
-            // a piece of a row: |q| <= 2^30 by its largest weight.  Up to three pieces share a scale (with 3 bits to spare for
-            // larger weights) and one read-back: the two low digits' sums of 384 entries just fit 32 bits
+            // a piece of a row: |q| <= 2^30 by its largest weight.  The pieces of a unit share a scale (with 3 bits to spare for
+            // larger weights) and one read-back, as long as none has a larger weight, or from kChainAny entries on much smaller ones
             // (weights too small for a fixed point count only where the whole row has no larger ones: finish())
             float m0 = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) m0 = max_nan(m0, fabsf(w[i]));
             x0 = max(__reduce_max_sync(0xffffffffu, __float_as_uint(m0)) >> 23, kExpLow);
             if (x0 > kExpHigh) x0 = 281u;           // bound infinite or NaN, also with 3 bits to spare
-            if (!(flags & kFirst) && chain + g_cnt <= 384 && x0 <= chain_x) {
+            if (!(flags & kFirst) && x0 <= chain_x && (chain + g_cnt <= kChainAny || (chain + g_cnt <= kChain && x0 + 5u >= chain_x))) {
                 x0 = chain_x;
                 chain += g_cnt;
                 if (lane == 0) slots[(k & 1) ^ 1].flags |= kMore;
@@ -356,7 +360,7 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
                 const int hi = (q + 0x8080) >> 16;
                 w0 += q - hi * 65536;
                 w1 += hi;
-                mag += (abs(q) >> 8) + 1;
+                mag += (abs(q) >> kMagShift) + 1;
             }
         }
         w0 = __reduce_add_sync(0xffffffffu, w0);
@@ -520,16 +524,19 @@ __global__ void __launch_bounds__(32 * agg_warps(K), agg_blocks(K)) agg_bits_ker
                     const float sc = __uint_as_float((uint32_t)hw.z << 23);
                     const bool first = !row_open;
                     row_open = true;
-                    bound = first ? (float)wmag * (256.f * sc) : fmaf((float)wmag, 256.f * sc, bound);
+                    constexpr float kMag = (float)(1 << kMagShift);
+                    bound = first ? (float)(unsigned)wmag * (kMag * sc) : fmaf((float)(unsigned)wmag, kMag * sc, bound);
                     float* f = facc + 2 * g + (odd ? 1 : 0);
 #pragma unroll
                     for (int i = 0; i < MT / 2; ++i) {
 #pragma unroll
                         for (int q = 0; q < 2; ++q) {
-                            int low, high;
-                            halves(i, q, low, high);
-                            const int bit = K > 64 ? 2 * (i & 3) + q : 2 * i + q + (odd ? 4 : 0);
-                            const float x = fmaf((float)(2 * (high >> bit) - whi), 65536.f, (float)(2 * (low >> bit) - wlo)) * sc;
+                            // (shifted before the digits are put together, so that kChain entries fit)
+                            const int bit = K > 64 ? 2 * (i & 3) + q : 2 * i + q, bit_up = K > 64 ? bit : bit + 4;
+                            const int lo = (c[i][2 * q + 1] >> bit) * 256 + (c[i][2 * q] >> bit);
+                            const int up = (c[i + MT / 2][2 * q + 1] >> bit_up) * 256 + (c[i + MT / 2][2 * q] >> bit_up);
+                            const int got = __shfl_xor_sync(0xffffffffu, odd ? lo : up, 1);
+                            const float x = fmaf((float)(2 * (odd ? up : got) - whi), 65536.f, (float)(2 * (odd ? got : lo) - wlo)) * sc;
                             if (t < 2) f[16 * (2 * i + q)] = first ? x : x + f[16 * (2 * i + q)];
                         }
                     }
