@@ -679,7 +679,7 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
     base += up((size_t)n * ldz * 4);
     float* gz = reinterpret_cast<float*>(base);
     base += up((size_t)n * ldz * 4);
-    const int n_splits = wt_splits(n, d_in, d_out);
+    int n_splits = wt_splits(n, d_in, d_out);
     float* part = reinterpret_cast<float*>(base);
     base += up((size_t)n_splits * d_in * d_out * 4);
     float* g_wt = reinterpret_cast<float*>(base);
@@ -727,7 +727,11 @@ cudaError_t launch_layer_backward(cudaStream_t s, int64_t n, const int64_t* rowp
 
     // step 1b: G_W~ = H~^T G_zeta, split over the rows, slabs added in a fixed order
     {
-        const int64_t rows_per_split = ceil_div(ceil_div(n, n_splits), 64) * 64;
+        // whole pairs of chunks; of few nodes whole chunks, and no part without nodes (19,717 nodes, 500 -> 64: 103 parts of 192 nodes and
+        // 45 empty ones, now 124 of 160)
+        const int64_t each = ceil_div(n, n_splits), unit = each <= 8 * kWtNodes ? kWtNodes : 2 * kWtNodes;
+        const int64_t rows_per_split = std::max<int64_t>(1, ceil_div(each, unit)) * unit;
+        n_splits = (int)std::max<int64_t>(1, ceil_div(n, rows_per_split));
         ++*launches;
         if (d_in <= 64) e = launch_grad_wt_tc<64>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
         else if (d_in <= 128) e = launch_grad_wt_tc<128>(s, in_bits, stride_in, in_beta, gz, ldz, n, d_in, d_out, n_splits, rows_per_split, part);
