@@ -66,7 +66,7 @@ enum {
      * 0 = choose per layer (default: for 129..256 output columns, where the aggregation streams 256-byte
      *     rows, and for 33..64 output columns of a layer whose result is only written out as fp32 (no next
      *     layer) or of a hidden layer on a graph whose rows average at least 8 stored entries (the aggregation
-     *     then streams one stored entry per lane), 3 when d_in <= 127 and 5 when 128 <= d_in <= 256 and the
+     *     then streams one stored entry per lane, or takes groups of them as integer products), 3 when d_in <= 127 and 5 when 128 <= d_in <= 256 and the
      *     layer has at least 2^20 outputs;
      *     otherwise 4 when d_in <= 2048, else 2);
      * 1 = fp32 zeta_ij = (beta_i alpha_j) dot_ij, exactly Eq. "cdot-op";
@@ -92,7 +92,7 @@ enum {
     /* How rows of 129..256 signed bytes (zeta formats 3 and 5) are aggregated.
      * 1 = the fp32 FMA stream (bytes converted to fp32 one by one; with format 5 this stream takes the edge values
      *     as non-negative, as those of the normalized adjacency are);
-     * 2 = exact integer products on the tensor cores through mma.sync (s8 x s8 -> s32: the edge weights of up to 32
+     * 2 = (also for rows of 33..64 bytes, see below) exact integer products on the tensor cores through mma.sync (s8 x s8 -> s32: the edge weights of up to 32
      *     stored entries of a row in 28..31-bit fixed point against a common power of two, split into four signed
      *     base-256 digits; the digit sums recombined in fp32 when the row ends; edge values of either sign);
      * 3 = the same fixed-point digits on the 5th-generation tensor cores (tcgen05.mma kind::i8: the gathered rows
@@ -102,7 +102,11 @@ enum {
      * 0 = default: 3 for a launch that wants only the next layer's sign bits and beta (a hidden layer inside
      *     bigcn_forward) on a graph whose rows average at least 8 stored entries, 1 otherwise.  Measured on the two
      *     256-column layers of a 2.4 M-node, 126 M-entry graph, bits and beta only: 4.9 / 5.2 ms for 3,
-     *     5.7-5.9 / 5.9-6.1 ms for 1, 8.0 / 8.3 ms for 2.  All paths meet the same tolerance; their fp32 sums differ
+     *     5.7-5.9 / 5.9-6.1 ms for 1, 8.0 / 8.3 ms for 2.
+     * Rows of 33..64 bytes take such products by default, in groups of up to 128 stored entries, on graphs whose rows average 40
+     * entries and that hold 4 million, in a workspace with room for what they sum in parts (bigcn_workspace_bytes() counts it
+     * there), and with 2 wherever the workspace has room; otherwise, and with an option that names a format or another
+     * kernel, fp32 streams.  Edge values of either sign; rows without a fixed point are summed in fp32 as they are written.  All paths meet the same tolerance; their fp32 sums differ
      *     in rounding, so a re-binarized bit at the threshold may differ between them. */
     BIGCN_OPT_BYTE_AGGREGATION = 4,
     /* Order of a layer's two products, H' = A_tilde (diag(beta) F B diag(alpha)).

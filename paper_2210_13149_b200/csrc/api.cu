@@ -193,6 +193,16 @@ bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* l
            (ctx->order == 2 || (hidden && spmm_bits_pays(g->n, g->nnz, layer->d_in, layer->d_out))) &&
            spmm_bits_scratch_bytes(g->n, g->nnz, layer->d_in) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
 }
+// Whether byte rows of 33..64 columns are aggregated as grouped integer products (spmm_bytes.cu), whose scratch lies at `at` of `room`
+// bytes, before the plan: where that pays, or wherever covered by option.  Options that name a storage format or another kernel keep
+// to the streams.
+bool grouped_bytes(const bigcn_ctx* ctx, const bigcn_graph* g, int d_in, int d_out, size_t at, size_t room)
+{
+    const bool wanted = ctx->byte_path == 2 ? spmm_bytes_covers(g->n, g->nnz, d_in, d_out)
+                                            : ctx->zeta_format == 0 && ctx->contraction == 0 && ctx->byte_path == 0 && ctx->long_row == 0 && spmm_bytes_pays(g->n, g->nnz, d_in, d_out);
+    return wanted &&
+           at + up(spmm_bytes_scratch_bytes(g->n, g->nnz)) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
+}
 // The plan of the graph sits at the end of the scratch.
 void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 {
@@ -247,6 +257,15 @@ bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* 
     if (e != cudaSuccess) return cuda_fail(ctx, e, "bit-GEMM launch");
     if (ev_mid) BIGCN_CUDA(ctx, cudaEventRecord(ev_mid, ctx->stream));
     SpmmArgs a;
+    const size_t parts_at = zbytes + up(spmm_scratch_bytes(g->n, g->nnz, layer->d_out));
+    if ((z.half || z.fmt == kZetaI8) && grouped_bytes(ctx, g, layer->d_in, layer->d_out, parts_at, room)) {
+        void* plan = plan_at(g, zeta, room);
+        if (!planned || !*planned) e = launch_spmm_bits_plan(ctx->stream, g->n, g->nnz, g->rowptr, plan, &ctx->launches_i);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");
+        if (planned) *planned = true;
+        a.plan = plan;
+        a.parts = static_cast<char*>(zeta) + parts_at;
+    }
     a.n = g->n;
     a.nnz = g->nnz;
     a.rowptr = g->rowptr;
@@ -283,10 +302,14 @@ size_t zeta_bytes_max(int64_t n, const int32_t* dims, int n_layers)
     return m;
 }
 
-// Scratch of the contraction-first order: the contraction's rows, the aggregation's counter.
-size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers)
+// Scratch of the contraction-first order: the contraction's rows, the aggregation's counter and, where grouped, what grouped byte
+// rows sum in parts.
+size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers, bool grouped)
 {
-    return up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0));
+    size_t parts = 0;
+    for (int l = 0; l < n_layers && grouped; ++l)
+        if (spmm_bytes_pays(n, nnz, dims[l], dims[l + 1])) parts = up(spmm_bytes_scratch_bytes(n, nnz));
+    return up(zeta_bytes_max(n, dims, n_layers)) + up(spmm_scratch_bytes(n, nnz, 0)) + parts;
 }
 
 // Scratch between the kernels of a layer, the larger of the two orders over all layers, and behind it the graph's plan, which
@@ -296,8 +319,9 @@ size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int 
 constexpr size_t kLittle = size_t(64) << 20;
 size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers, bool every)
 {
-    size_t m = contraction_first_bytes(n, nnz, dims, n_layers), plan = 0;
+    size_t m = contraction_first_bytes(n, nnz, dims, n_layers, true), plan = 0;
     for (int l = 0; l < n_layers; ++l) {
+        if (spmm_bytes_pays(n, nnz, dims[l], dims[l + 1])) plan = spmm_bits_plan_bytes(n, nnz);
         if (n <= 0 || nnz < 0 || !spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) continue;
         const size_t bytes = spmm_bits_scratch_bytes(n, nnz, dims[l]);
         const bool hidden = l < n_layers - 1 || n_layers == 1;
@@ -337,7 +361,7 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     const size_t zbytes = up(zeta_bytes_max(n, dims, n_layers));
     size_t others = 0;                                       // what else the step keeps
     for (int i = 0; i < 2; ++i) others += up((size_t)n * stride_max * 4) + up((size_t)n * 4);
-    const size_t least = contraction_first_bytes(n, graph->nnz, dims, n_layers);
+    const size_t first = contraction_first_bytes(n, graph->nnz, dims, n_layers, true), least = contraction_first_bytes(n, graph->nnz, dims, n_layers, false);
     size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, ctx->order == 2);
     if (up(ws.off) + room + others > ws.size) room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, false);
     if (up(ws.off) + room + others > ws.size) room = least;  // a workspace without room for P
@@ -364,7 +388,7 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     }
     // The layers share the graph's plan, made by the first that needs it, where the scratch of the contraction-first ones ends
     // before it; otherwise each makes its own.
-    const bool shared = room >= least + spmm_bits_plan_bytes(n, graph->nnz);
+    const bool shared = room >= first + spmm_bits_plan_bytes(n, graph->nnz);
     bool planned = false, aggregated_first[BIGCN_MAX_LAYERS] = {};
     if (stats) BIGCN_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
     for (int l = 0; l < n_layers; ++l) {
@@ -1112,11 +1136,19 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     a.ld_add = ld_self;
     // 33..48 columns on rows not much shorter than a pass: bytes, for the lane-per-entry stream (2.4 M nodes, 126 M entries, 256 -> 47:
     // 4.3 ms with fp16 rows on the general stream, 3.0 like this); rows of bytes of more columns have no stream with an own term
-    const bool narrow = d_out > 32 && d_out <= 48 && mean_graph->nnz >= 8 * n;
+    const bool grouped = grouped_bytes(ctx, mean_graph, d_in, d_out, need, ctx->ws_bytes);
+    const bool narrow = grouped || (d_out > 32 && d_out <= 48 && mean_graph->nnz >= 8 * n);
     const ZetaRows z = zeta_rows(ctx, mean_graph, d_in, d_out, zeta_nbr, /*allow_half=*/narrow, narrow);
     e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, nbr_layer->alpha,
                        z.fmt, zeta_nbr, z.ld, nullptr, nullptr, &ctx->launches_i, z.half ? 2 : ctx->contraction, z.nws, z.col_b0, z.tail ? 1 : 0);
     if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (neighbour term) launch"); }
+    if (grouped && (z.half || z.fmt == kZetaI8)) {
+        void* plan = plan_at(mean_graph, base, ctx->ws_bytes);
+        e = launch_spmm_bits_plan(ctx->stream, n, mean_graph->nnz, mean_graph->rowptr, plan, &ctx->launches_i);
+        if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "plan launch"); }
+        a.plan = plan;
+        a.parts = base + need;
+    }
     a.zeta = zeta_nbr;
     z.hand_over(a, in_beta);
     a.byte_path = ctx->byte_path;

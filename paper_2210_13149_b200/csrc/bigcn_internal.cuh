@@ -102,10 +102,16 @@ struct SpmmArgs {
     int64_t long_row;        // rows with more entries are split (0 = never)
     void* scratch;           // partial sums of split rows
     size_t scratch_bytes;
+    const void* plan = nullptr;      // byte rows of 33..64 columns: the graph's plan, with which they are aggregated as grouped integer
+    void* parts = nullptr;           // products (spmm_bytes.cu); `parts` is spmm_bytes_scratch_bytes() more scratch
     int wait_tries = 0;      // launch_spmm_bits(): bound of the waits inside a block (0 = default)
 };
 cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches);
 size_t spmm_scratch_bytes(int64_t n, int64_t nnz, int d_out);
+// Rows of 33..64 signed bytes as grouped integer products (spmm_bytes.cu).
+bool spmm_bytes_covers(int64_t n, int64_t nnz, int d_in, int d_out);
+bool spmm_bytes_pays(int64_t n, int64_t nnz, int d_in, int d_out);
+size_t spmm_bytes_scratch_bytes(int64_t n, int64_t nnz);
 
 // A layer with the aggregation before the contraction, on the packed bits (spmm_bits.cu).  `plan` (spmm_bits_plan_bytes(), made by
 // launch_spmm_bits_plan() from the graph alone) serves any number of layers.  `a` as for launch_spmm(), its zeta fields

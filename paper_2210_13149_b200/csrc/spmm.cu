@@ -2065,6 +2065,7 @@ cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches)
     // the sign bits and beta are wanted, on a graph whose rows are not much shorter than its chunks' eight segments allow
     const bool tc_default = a.byte_path == 0 && a.next_bits && !a.h_out && !a.add && mean_row >= 8.0;
     if (a.fmt == kZetaI8 && (a.byte_path == 3 || tc_default) && a.nnz > 0 && a.nnz < (int64_t(1) << 31) && spmm_tc_covers(p)) return launch_spmm_tc(s, p);
+    if (a.plan) return launch_spmm_bytes(s, p, a.nnz, a.plan, a.parts);
     switch (a.fmt) {
         case kZetaF32: return dispatch<float>(s, p, mean_row);
         case kZetaF16: return dispatch<__half>(s, p, mean_row);

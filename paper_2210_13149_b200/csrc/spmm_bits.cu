@@ -39,20 +39,20 @@
 
 #include "bigcn_internal.cuh"
 #include "spmm_dev.cuh"
+#include "spmm_groups.cuh"
 #include "tc_common.cuh"
 
 namespace bigcn {
 
 namespace {
 
+using namespace groups;
 using tc::smem_u32;
 
 __device__ int g_bits_timeout;                      // set when a bounded wait ran out
 
 // ---- P -------------------------------------------------------------------------------------------------------------
 
-constexpr int kGroup = 128;                         // stored entries of a group
-constexpr int kRowCost = 4;                         // what a row counts beside its entries where work is split
 // Entries of a row under one scale: their sum of |q| >> kMagShift fits 32 bits.  From kChainAny on, pieces whose largest weight is
 // less than a quarter of the scale's start another, so that they are not rounded more coarsely for it.  (Up to three pieces
 // whatever the row: 60,000 nodes in rows of 470, 256 inputs, one read-back for three pieces 506 us, 488 now.)
@@ -81,12 +81,10 @@ struct AggDev {
     unsigned* counters;                             // [slices][chunks] pieces done; zeroed before
 };
 
-enum Flags : int { kPair = 1, kDirect = 2, kFirst = 4, kLast = 8, kStarts = 16, kWhole = 32, kMore = 64 };
+constexpr int kMore = 64;                           // beside Flags, of a group in a slot: the next one adds to its products
 
-// Biased exponents of a row's largest weight (of a whole row: of the largest of the lanes' sums) that have a fixed point here.  A row
-// without one gets a scale whose exponent is zero, all ones or beyond, which marks it for literal_row(); what its integers
-// are is of no account then.
-constexpr uint32_t kExpLow = 40, kExpHigh = 230;
+// A row without a fixed point (by the exponent of its largest weight, of a whole row: of the largest of the lanes' sums) gets a scale
+// whose exponent is zero, all ones or beyond, which marks it for literal_row(); what its integers are is of no account then.
 __device__ __forceinline__ bool is_literal(float scale) { return __float_as_uint(scale) - 1u >= 0x7f7fffffu; }
 __device__ __forceinline__ float max_nan(float a, float b)   // NaN if either is
 {
@@ -116,14 +114,6 @@ __device__ __forceinline__ void imma(int (&c)[4], uint32_t a0, uint32_t a1, uint
                  : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// Two 16 x 16 byte matrices, transposed: lane 4 g + t gets byte g (r[0]) and byte g + 8 (r[1]) of rows 4 t .. 4 t + 3 of the
-// first, r[2] and r[3] of the second; lane l gives the address of row l of the 32.
-__device__ __forceinline__ void ldmatrix_bytes(uint32_t saddr, uint32_t (&r)[4])
-{
-    asm volatile("ldmatrix.sync.aligned.m16n16.x2.trans.shared.b8 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(saddr) : "memory");
-}
-constexpr uint32_t kFlip = 0x80808080u;             // (v + kFlip) ^ kFlip: the balanced digits of v, one per byte
 // byte d of four words, for d = 0..3
 __device__ __forceinline__ void transpose4(const uint32_t (&u)[4], uint32_t (&o)[4])
 {
@@ -1003,6 +993,11 @@ bool spmm_bits_pays(int64_t n, int64_t nnz, int d_in, int d_out)
     return 65e6 + here_entry * nnz + here_row * n < 0.95 * (10e6 + there_entry * nnz + there_row * n);
 }
 
+groups::GraphPlan spmm_bits_plan_at(int64_t n, int64_t nnz, const void* plan)
+{
+    const Plan pl = make_plan(n, nnz, 1);
+    return {pl.chunk_log2, pl.chunks, static_cast<const int4*>(plan), reinterpret_cast<const int2*>(static_cast<const char*>(plan) + pl.groups_bytes)};
+}
 size_t spmm_bits_plan_bytes(int64_t n, int64_t nnz) { return make_plan(n, nnz, 1).graph_bytes(); }
 size_t spmm_bits_scratch_bytes(int64_t n, int64_t nnz, int d_in) { return make_plan(n, nnz, d_in).layer_bytes(); }
 

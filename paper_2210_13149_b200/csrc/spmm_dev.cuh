@@ -43,4 +43,7 @@ bool spmm_tc_covers(const SpmmDev& p);
 cudaError_t launch_spmm_tc(cudaStream_t s, const SpmmDev& p);
 int spmm_tc_timeouts();
 
+// The aggregation of rows of 33..64 signed bytes as integer products (spmm_bytes.cu); plan: of the graph (launch_spmm_bits_plan()).
+cudaError_t launch_spmm_bytes(cudaStream_t s, const SpmmDev& p, int64_t nnz, const void* plan, void* scratch);
+
 }  // namespace bigcn
