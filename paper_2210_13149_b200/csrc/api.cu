@@ -1094,7 +1094,7 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
     const size_t need = 2 * zbytes + up(spmm_scratch_bytes(n, mean_graph->nnz, d_out));
     if (!ctx->ws || ctx->ws_bytes < need) return fail(ctx, BIGCN_ERR_WORKSPACE, "needs %zu bytes of workspace, has %zu", need, ctx->ws_bytes);
     char* base = static_cast<char*>(ctx->ws);
-    float* zeta_self = reinterpret_cast<float*>(base);                   // literal fp32 zeta of the node's own term
+    float* zeta_self = reinterpret_cast<float*>(base);                   // the node's own term: fp32 zeta, or its dots
     void* zeta_nbr = base + zbytes;
     void* counter = base + 2 * zbytes;
     const int64_t stride_in = bigcn_packed_stride_words(d_in);
@@ -1128,17 +1128,26 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
-    const int64_t ld_self = zeta_ld(d_out, kZetaF32);
-    e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out,
-                                   in_beta, self_layer->alpha, kZetaF32, zeta_self, ld_self, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
-    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
-    a.add = zeta_self;
-    a.ld_add = ld_self;
     // 33..48 columns on rows not much shorter than a pass: bytes, for the lane-per-entry stream (2.4 M nodes, 126 M entries, 256 -> 47:
     // 4.3 ms with fp16 rows on the general stream, 3.0 like this); rows of bytes of more columns have no stream with an own term
     const bool grouped = grouped_bytes(ctx, mean_graph, d_in, d_out, need, ctx->ws_bytes);
     const bool narrow = grouped || (d_out > 32 && d_out <= 48 && mean_graph->nnz >= 8 * n);
     const ZetaRows z = zeta_rows(ctx, mean_graph, d_in, d_out, zeta_nbr, /*allow_half=*/narrow, narrow);
+    // the own term: integer dots where the aggregation scales them (the same products), fp32 rows otherwise
+    const bool own_dots = (z.fmt == kZetaF16 || z.fmt == kZetaI16) && d_in <= 32767;
+    const int self_fmt = own_dots ? kZetaI16 : kZetaF32;
+    const int64_t ld_self = zeta_ld(d_out, self_fmt);
+    e = launch_bitgemm(ctx->stream, in_bits, stride_in, self_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, self_layer->alpha,
+                       self_fmt, zeta_self, ld_self, nullptr, nullptr, &ctx->launches_i, ctx->contraction);
+    if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (self term) launch"); }
+    if (own_dots) {
+        a.own = reinterpret_cast<const int16_t*>(zeta_self);
+        a.own_ld = ld_self;
+        a.own_alpha = self_layer->alpha;
+    } else {
+        a.add = zeta_self;
+        a.ld_add = ld_self;
+    }
     e = launch_bitgemm(ctx->stream, in_bits, stride_in, nbr_layer->w_bitsT, stride_in, n, d_in, d_out, in_beta, nbr_layer->alpha,
                        z.fmt, zeta_nbr, z.ld, nullptr, nullptr, &ctx->launches_i, z.half ? 2 : ctx->contraction, z.nws, z.col_b0, z.tail ? 1 : 0);
     if (e != cudaSuccess) { finish_call(ctx); return cuda_fail(ctx, e, "bit-GEMM (neighbour term) launch"); }

@@ -91,6 +91,9 @@ struct SpmmArgs {
     bool row_tail = false;           // byte rows of 64 bytes whose last four bytes hold the source's node factor (see bitgemm_tc.cu)
     const float* add = nullptr;   // optional fp32 [n x ld_add] added to every aggregated row (Bi-GraphSAGE self term)
     int64_t ld_add = 0;
+    const int16_t* own = nullptr; // the same as integer dots (rows of 16-bit integers): node_w_i own_alpha_j own_ij is added
+    int64_t own_ld = 0;
+    const float* own_alpha = nullptr;
     bool any_order = false;          // h_out: the order of summation is free (see spmm.cu)
     float* h_out;            // nullable
     int64_t ldh;

@@ -123,7 +123,7 @@ __device__ __forceinline__ void reduce_groups(float (&acc)[NCH][EPV])
 // Per-column constants of the row epilogue, staged once per thread block: four arrays of kCols
 // floats -- the column factor (0 for padding columns, 1 when there is none), the next layer's shift and
 // scale (0 and 1 where there are none, so that applying them changes nothing), and the first weight
-// sign of the column (half-dot bytes only, else 0).  Inside an array the 16-byte chunks are ordered so that the
+// sign of the column (half-dot bytes), or the factor of the own dots (else 0).  Inside an array the 16-byte chunks are ordered so that the
 // lanes' reads in the row epilogue are contiguous: a lane holds EPV consecutive columns (EPV / 4 chunks) and reads
 // its q-th chunk together with the other lanes, so chunk q of vector v sits at position q * (kCols / EPV) + v
 // (in column order the reads of 8- and 16-column vectors fall 32 and 64 bytes apart: 2- and 4-way bank conflicts).
@@ -144,7 +144,7 @@ __device__ __forceinline__ void fill_col_table(const SpmmDev& p, float* ctab)
         ctab[at] = in ? (p.col_w ? __ldg(p.col_w + col) : 1.f) : 0.f;
         ctab[kCols + at] = (in && p.next_shift) ? __ldg(p.next_shift + col) : 0.f;
         ctab[2 * kCols + at] = (in && p.next_shift) ? __ldg(p.next_scale + col) : 1.f;
-        ctab[3 * kCols + at] = (in && p.col_b0) ? __ldg(p.col_b0 + col) : 0.f;
+        ctab[3 * kCols + at] = !in ? 0.f : (p.own ? __ldg(p.own_alpha + col) : (p.col_b0 ? __ldg(p.col_b0 + col) : 0.f));
     }
 }
 
@@ -184,10 +184,28 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
             x[4 * q + 2] = t[2] * a.z;
             x[4 * q + 3] = t[3] * a.w;
         }
-        if (p.add) {
+        if constexpr (EPV != 8) {
+            if (p.add) {
 #pragma unroll
-            for (int i = 0; i < EPV; ++i)
-                if ((S == 32 || on) && col0 + i < p.d_out) x[i] += __ldg(p.add + row * p.ld_add + col0 + i);
+                for (int i = 0; i < EPV; ++i)
+                    if ((S == 32 || on) && col0 + i < p.d_out) x[i] += __ldg(p.add + row * p.ld_add + col0 + i);
+            }
+        } else {
+            if (p.own && (S == 32 || on) && col0 < p.own_ld) {               // (one load; as fp32 rows it was eight, of twice the bytes)
+                const uint4 v = __ldg(reinterpret_cast<const uint4*>(p.own + row * p.own_ld + col0));
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+                const float be = __ldg(p.node_w + row);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const float4 a = *reinterpret_cast<const float4*>(ctab + 3 * kCols + ctab_at<kCols, EPV>(col0 + 4 * q));
+                    const float oa[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int dot = (int)(u[2 * q + (i >> 1)] << (i & 1 ? 0 : 16)) >> 16;
+                        x[4 * q + i] += __fmul_rn(__fmul_rn(be, oa[i]), (float)dot);
+                    }
+                }
+            }
         }
         if (p.h_out && g == 0 && vec < p.nv_fin && (S == 32 || on)) {
             float* dst = p.h_out + row * p.ldh + col0;
@@ -2038,6 +2056,11 @@ cudaError_t launch_spmm(cudaStream_t s, const SpmmArgs& a, int* launches)
     p.node_w = a.fmt == kZetaF32 ? nullptr : a.node_w;
     p.col_w = a.fmt == kZetaF32 ? nullptr : a.col_w;
     p.add = a.add;
+    p.own = a.own;
+    p.own_ld = a.own_ld;
+    p.own_alpha = a.own_alpha;
+    const bool halves = a.fmt == kZetaF16 || a.fmt == kZetaI16;
+    if ((a.own && !halves) || (a.add && halves)) return cudaErrorInvalidValue;
     p.col_b0 = a.half_dots ? a.col_b0 : nullptr;
     p.half_dots = a.half_dots ? 1 : 0;
     p.byte_path = a.byte_path;

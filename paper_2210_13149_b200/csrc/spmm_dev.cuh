@@ -21,8 +21,11 @@ struct SpmmDev {
     int half_dots;           // zeta holds s = (dot' - 1) / 2; node_w carries the first feature sign
     int byte_path;           // 129..256 byte columns: 0 / 1 the FMA stream, 2 integer tensor-core products
     int row_tail;            // rows of 64 bytes whose last four bytes hold the source's node factor as a float
-    const float* add;        // nullable: fp32 [n x ld_add] added to the aggregated row (after col_w)
+    const float* add;        // nullable: fp32 [n x ld_add] added to the aggregated row (after col_w); not for fp16 and 16-bit zeta
     int64_t ld_add;
+    const int16_t* own;      // nullable: node_w_i own_alpha_j own_ij is added (fp16 and 16-bit zeta only); rows of own_ld, a multiple of 8
+    int64_t own_ld;
+    const float* own_alpha;
     float* h_out;
     int64_t ldh;
     int h_vec;               // 1: rows of h_out can be stored as float4
