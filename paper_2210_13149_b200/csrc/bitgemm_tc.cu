@@ -50,10 +50,10 @@ __device__ __forceinline__ void expand_word(uint32_t w, uint4& lo, uint4& hi)
 // Expands `rows_valid` packed rows (stride words each, read 16 bytes at a time) into the canonical
 // operand of `rows` rows; rows past rows_valid become zero bytes.
 __device__ __forceinline__ void stage_operand(unsigned char* dst, int rows, const uint32_t* __restrict__ src,
-                                              int64_t stride, int64_t rows_valid)
+                                              int64_t stride, int64_t rows_valid, int threads = kTcThreads)
 {
     const int q = (int)(stride >> 2);                       // 16-byte pieces per packed row
-    for (int t = threadIdx.x; t < rows * q; t += kTcThreads) {
+    for (int t = threadIdx.x; t < rows * q; t += threads) {
         const int r = t / q, piece = t - r * q;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         const bool in = r < rows_valid;
@@ -356,10 +356,9 @@ bitgemm_tc_kernel(const uint32_t* __restrict__ A, int64_t stride_a, const uint32
 }
 
 // The same product for layers of any d_in (more than 256: a tile's expanded rows no longer fit shared memory whole): K in
-// chunks of 256 positions, accumulated in tensor memory.  N = 64 or 128 channels (blockIdx.y: slices of N).  The expanded
-// weight panel stays in shared memory where that leaves room for a second block per multiprocessor or there is at most one tile
-// per multiprocessor (`resident`); otherwise a chunk of it is expanded again with every chunk of rows.  89,250 rows,
-// 500 -> 256: 100 us on the bit-count pipe; see bitgemm_takes_wide() for the line between the two.
+// chunks of 256 positions, accumulated in tensor memory.  N = 64 or 128 channels (blockIdx.y: slices of N).  For panels that leave
+// the pipeline below no room: the expanded weight panel stays in shared memory where it fits and there is at most one tile per
+// multiprocessor (`resident`); otherwise a chunk of it is expanded again with every chunk of rows.
 template <int N, int FMT>
 __global__ void __launch_bounds__(kTcThreads, 2)
 bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ BT, int64_t stride,
@@ -521,13 +520,277 @@ bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__
     if (warp == 0) tc::tmem_free(tmem_base, N);
 }
 
+// Layers of more than 256 inputs as a pipeline, one block per multiprocessor: expanding, multiplying and converting run side by
+// side.  In the kernel above a tile is a chain of them, barrier after barrier (89,250 rows, 500 -> 256: 8 us per tile where the
+// products take 0.6 and the instructions of both other steps 2.4), and two blocks per multiprocessor hide little of it.  Warps 0-7 expand
+// chunks of 256 positions of the packed rows into a ring of operand tiles (each thread has the bits of its next two chunks in
+// flight); one thread of warp 8 issues the products into one of two accumulators; warps 9-16 convert and write the other one.
+// N = 256 halves the expansions: up to 512 inputs its panel leaves room for two operand tiles.
+// Measured, the kernel above / this one: 89,250 rows 500 -> 256 35 / 21 us, 60,000 rows 602 -> 256 38 / 25, 200,000 rows
+// 1,000 -> 100 68 / 52 and 602 -> 41 35 / 32, 1,000,000 rows 500 -> 64 123 / 101, 10,240 rows 300 -> 128 7.9 / 7.1, 19,717 rows
+// 500 -> 64 8.5 / 8.5 and 22,000 rows 300 -> 64 7.8 / 7.9 (one or two tiles per block: nothing to overlap).  Up to 256 inputs a tile is one chunk, three blocks of bitgemm_tc_kernel overlap as well, and the two are level (169,343 rows
+// 256 -> 256 30 / 28, 128 -> 256 as floats 36 / 38, 255 -> 100 17 / 18): that kernel stays.
+constexpr int kPipeThreads = 17 * 32;
+constexpr int kPipeStages = 4;                // operand tiles at most; as many as fit
+
+__device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* bar)
+{
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+
+template <int N, int FMT>
+__global__ void __launch_bounds__(kPipeThreads, 1)
+bitgemm_pipe_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ BT, int64_t stride,
+                    int64_t n, int d_in, int d_out, const float* __restrict__ beta, const float* __restrict__ alpha,
+                    void* __restrict__ zeta, int64_t ldz, int stages)
+{
+    pdl_enter();
+    constexpr int kElt = TcOut<FMT>::kElt;
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    // an operand tile is complete / read; an accumulator is complete / read
+    __shared__ __align__(8) uint64_t full[kPipeStages], empty[kPipeStages], done[2], taken[2], drain;
+    __shared__ uint32_t tmem_base_s;
+    __shared__ float al_s[N];
+    const int ch0 = blockIdx.y * N;                         // this block's channels
+    const int d_here = min(d_out - ch0, N);
+    BT += (int64_t)ch0 * stride;
+    const int K = (int)stride * 32, pieces = (int)(stride >> 2);         // a piece: 16 bytes of a packed row, 128 positions
+    const int pad = K - d_in;                               // padding positions: each contributes +1
+    const int n_chunks = (pieces + 1) >> 1;
+    constexpr int tile_bytes = kTcRows * 256;
+    unsigned char* Bs = tc_smem;                            // [N][K]
+    unsigned char* As = Bs + (size_t)N * K;                 // stages of [128][256]
+    unsigned char* scratch = As + stages * tile_bytes;      // 4 KB per converting warp
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0) tc::tmem_alloc(&tmem_base_s, 2 * N);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kPipeStages; ++s) bar_init(&full[s], 8), bar_init(&empty[s], 1);
+        for (int b = 0; b < 2; ++b) bar_init(&done[b], 1), bar_init(&taken[b], 8);
+        bar_init(&drain, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    for (int j = threadIdx.x; j < N; j += kPipeThreads) al_s[j] = j < d_here ? __ldg(alpha + ch0 + j) : 0.f;
+    stage_operand(Bs, N, BT, stride, d_here, kPipeThreads);
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem_base = tmem_base_s;
+
+    const int64_t n_tiles = ceil_div(n, kTcRows);
+    const int64_t my_tiles = blockIdx.x < n_tiles ? ceil_div(n_tiles - blockIdx.x, (int64_t)gridDim.x) : 0;
+    auto tile_row0 = [&](int64_t i) { return (blockIdx.x + i * gridDim.x) * (int64_t)kTcRows; };
+    auto qc_of = [&](int c) { return min(2, pieces - 2 * c); };         // pieces of chunk c
+    bool ok = true;
+    if (warp < 8) {
+        // ---- expand: two threads per row (one, by the lower half of the threads, where a chunk is one piece)
+        struct Next { int64_t i; int c; };
+        auto advance = [&](Next& x) { if (++x.c == n_chunks) x.c = 0, ++x.i; };
+        auto fetch = [&](const Next& x) {
+            uint4 w = make_uint4(0u, 0u, 0u, 0u);
+            if (x.i >= my_tiles) return w;
+            const int qc = qc_of(x.c), r = qc == 2 ? threadIdx.x >> 1 : threadIdx.x, q = qc == 2 ? threadIdx.x & 1 : 0;
+            const int64_t row = tile_row0(x.i) + r;
+            if (r < kTcRows && row < n) w = __ldg(reinterpret_cast<const uint4*>(A + row * stride) + 2 * x.c + q);
+            return w;
+        };
+        Next at{0, 0}, ahead{0, 0};
+        uint4 pre[2];
+        pre[0] = fetch(ahead), advance(ahead);
+        pre[1] = fetch(ahead), advance(ahead);
+        int s = 0;
+        uint32_t lap = 0;
+        auto step = [&](uint4& w) {
+            if (!(ok = __all_sync(~0u, wait_barrier(&empty[s], lap ^ 1u)))) return;
+            const int qc = qc_of(at.c), r = qc == 2 ? threadIdx.x >> 1 : threadIdx.x, q = qc == 2 ? threadIdx.x & 1 : 0;
+            if (r < kTcRows) {
+                unsigned char* dst = As + s * tile_bytes;
+                const bool in = tile_row0(at.i) + r < n;
+                const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;
+                    if (in) expand_word(ws[u], lo, hi);
+                    *reinterpret_cast<uint4*>(dst + canon_off(kTcRows, r, 2 * (4 * q + u))) = lo;
+                    *reinterpret_cast<uint4*>(dst + canon_off(kTcRows, r, 2 * (4 * q + u) + 1)) = hi;
+                }
+            }
+            w = fetch(ahead);
+            advance(ahead), advance(at);
+            tc::fence_async_smem();
+            __syncwarp();
+            if (lane == 0) bar_arrive(&full[s]);
+            if (++s == stages) s = 0, lap ^= 1u;
+        };
+        while (ok && at.i < my_tiles) {
+            step(pre[0]);
+            if (ok && at.i < my_tiles) step(pre[1]);
+        }
+    } else if (warp == 8) {
+        // ---- products: all K steps of a chunk, then its operand tile is free; after the last one the accumulator is complete
+        if (lane == 0) {
+            // instruction descriptor: D = s32, A = B = s8, both K-major, N, M = 128
+            const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
+            const uint32_t a_lbo = (kTcRows >> 3) * 128, b_lbo = (N >> 3) * 128, sbo = 128;
+            int s = 0;
+            uint32_t lap = 0;
+            for (int64_t i = 0; ok && i < my_tiles; ++i) {
+                const int b = (int)(i & 1);
+                ok = wait_barrier(&taken[b], ((uint32_t)(i >> 1) & 1u) ^ 1u);
+                for (int c = 0; ok && c < n_chunks; ++c) {
+                    if (!(ok = wait_barrier(&full[s], lap))) break;
+                    tc::fence_after_sync();
+                    const uint32_t a_base = smem_u32(As) + s * tile_bytes, b_base = smem_u32(Bs) + 16u * (uint32_t)c * b_lbo;
+                    for (int ks = 0; ks < 4 * qc_of(c); ++ks) {
+                        const uint64_t ad = make_desc(a_base + 2 * ks * a_lbo, a_lbo, sbo);
+                        const uint64_t bd = make_desc(b_base + 2 * ks * b_lbo, b_lbo, sbo);
+                        const uint32_t accum = c > 0 || ks > 0 ? 1u : 0u;
+                        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}\n"
+                                     ::"r"(tmem_base + b * N), "l"(ad), "l"(bd), "r"(idesc), "r"(accum) : "memory");
+                    }
+                    tc::commit_to(&empty[s]);
+                    if (c + 1 == n_chunks) tc::commit_to(&done[b]);
+                    if (++s == stages) s = 0, lap ^= 1u;
+                }
+            }
+            if (!ok) {                                      // what was issued ends before the accumulators are given back
+                tc::commit_to(&drain);
+                wait_barrier(&drain, 0);
+            }
+        }
+    } else {
+        // ---- convert: a thread owns row lane_base + lane and walks over its warp's half of the columns
+        const int half = (warp - 9) >> 2;
+        const int lane_base = 32 * (warp & 3);              // a warp reads tensor-memory lanes 32 (warp % 4) .. + 31
+        const int c_begin = half * (N / 2);
+        constexpr int kRowBytes = (N / 2) * kElt;
+        constexpr int kPpr = kRowBytes >= 128 ? 8 : kRowBytes / 16;     // 16-byte pieces per row and pass (128 bytes at most)
+        constexpr int kChunksPerPass = kPpr / kElt;
+        constexpr int kPasses = kRowBytes / (16 * kPpr);
+        static_assert(kPpr % kElt == 0 && kRowBytes % (16 * kPpr) == 0, "a pass is a whole number of 16-column chunks");
+        constexpr int kBatch = kChunksPerPass < 2 ? kChunksPerPass : 2; // loads of tensor memory in flight
+        static_assert(kChunksPerPass % kBatch == 0, "whole batches");
+        unsigned char* scr = scratch + (warp - 9) * 4096;   // 32 rows x 128 bytes; piece p of row r at r * 128 + ((p ^ (r & 7)) * 16)
+        for (int64_t i = 0; i < my_tiles; ++i) {
+            const int64_t row0 = tile_row0(i) + lane_base;
+            const float be = (FMT == kZetaF32 && row0 + lane < n) ? __ldg(beta + row0 + lane) : 0.f;
+            const int b = (int)(i & 1);
+            if (!(ok = __all_sync(~0u, wait_barrier(&done[b], (uint32_t)(i >> 1) & 1u)))) break;
+            tc::fence_after_sync();
+#pragma unroll 1
+            for (int pass = 0; pass < kPasses; ++pass) {
+#pragma unroll
+                for (int ch1 = 0; ch1 < kChunksPerPass; ch1 += kBatch) {
+                    uint32_t v[kBatch][16];
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u)
+                        tc::tmem_ld16_nowait(tmem_base + b * N + ((uint32_t)lane_base << 16) + (uint32_t)(c_begin + (pass * kChunksPerPass + ch1 + u) * 16), v[u]);
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) tc::tmem_wait16(v[u]);
+#pragma unroll
+                    for (int u1 = 0; u1 < kBatch; ++u1) {
+                        const int ch = ch1 + u1, c0 = c_begin + (pass * kChunksPerPass + ch) * 16;
+                        int dot[16];
+                        const bool whole = c0 + 16 <= d_here;       // every column of the chunk exists: no per-column tests
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) dot[e] = (int)v[u1][e] - pad;
+                        if (!whole) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) dot[e] = (c0 + e < d_here) ? dot[e] : 0;       // padding columns of zeta stay 0
+                        }
+                        uint4 out[kElt];
+                        if constexpr (FMT == kZetaF16) {    // exact for |dot| <= 2048: int -> float without the conversion unit, then to half
+                            uint32_t h[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const __half2 r = __floats2half2_rn(__int_as_float(0x4B400000 + dot[2 * q]) - 12582912.f, __int_as_float(0x4B400000 + dot[2 * q + 1]) - 12582912.f);
+                                h[q] = *reinterpret_cast<const uint32_t*>(&r);
+                            }
+                            out[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                            out[1] = make_uint4(h[4], h[5], h[6], h[7]);
+                        } else {
+                            TcOut<FMT>::pack(dot, be, al_s + c0, out);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kElt; ++u) {
+                            const int piece = ch * kElt + u;
+                            *reinterpret_cast<uint4*>(scr + lane * 128 + ((piece ^ (lane & 7)) * 16)) = out[u];
+                        }
+                    }
+                }
+                if (pass + 1 == kPasses) {                  // the accumulator is free before its rows are written
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(&taken[b]);
+                } else {
+                    __syncwarp();
+                }
+                // write the 32 rows x kPpr pieces out: a warp instruction covers 32 / kPpr whole row segments
+                const int64_t byte0 = (int64_t)(ch0 + c_begin + pass * kChunksPerPass * 16) * kElt;
+#pragma unroll
+                for (int it = 0; it < kPpr; ++it) {
+                    const int r = it * (32 / kPpr) + lane / kPpr, pc = lane % kPpr;
+                    const uint4 val = *reinterpret_cast<const uint4*>(scr + r * 128 + ((pc ^ (r & 7)) * 16));
+                    const int64_t at = byte0 + pc * 16;
+                    if (row0 + r < n && at < ldz * kElt)
+                        *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(zeta) + (row0 + r) * ldz * kElt + at) = val;
+                }
+                __syncwarp();
+            }
+        }
+    }
+    if (!ok) atomicExch(&g_tc_timeout, 1);
+    __syncwarp();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_free(tmem_base, 2 * N);
+}
+
+// Dynamic shared memory of the pipeline without its operand tiles, and the tiles that fit (less than two: not covered)
+size_t pipe_fixed_bytes(int N, int64_t stride) { return (size_t)N * stride * 32 + 8 * 4096; }
+int pipe_stages(int N, int64_t stride)
+{
+    const size_t limit = (227 - 2) * 1024, fixed = pipe_fixed_bytes(N, stride);          // 2 KB: what the kernel declares
+    const size_t tile = (size_t)kTcRows * 256;
+    return fixed + 2 * tile > limit ? 0 : (int)std::min<size_t>(kPipeStages, (limit - fixed) / tile);
+}
+
+template <int N, int FMT>
+cudaError_t launch_pipe_inst(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
+                             const float* beta, const float* alpha, void* zeta, int64_t ldz)
+{
+    const int stages = pipe_stages(N, stride);
+    const size_t smem = pipe_fixed_bytes(N, stride) + (size_t)stages * kTcRows * 256;
+    cudaError_t e = cudaFuncSetAttribute(bitgemm_pipe_kernel<N, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = ceil_div(n, kTcRows), gy = ceil_div(d_out, N);
+    const unsigned gx = (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(1, sm_count() / gy));
+    launch_kernel(bitgemm_pipe_kernel<N, FMT>, dim3(gx, (unsigned)gy), kPipeThreads, smem, s, A, BT, stride, n, d_in, d_out, beta, alpha,
+                  zeta, ldz, stages);
+    return cudaGetLastError();
+}
+
+// Channels per block of the pipeline, 0 where it does not run.  256 only where slices of 128 are more than a block per
+// multiprocessor: 5,120 rows 500 -> 256 (80 slices) 10.2 us with 256 and 7.6 with 128, 8,000 rows 300 -> 256 (126) 9.0 and 6.8;
+// 12,000 rows 500 -> 256 (188) 10.4 where slices of 128 took 10.8 with the kernel above, 30,000 rows (470) 13 and 17.
+int pipe_width(int64_t n, int d_out, int64_t stride)
+{
+    const bool wide = d_out > 128 && ceil_div(n, kTcRows) * ceil_div(d_out, 128) > sm_count() && pipe_stages(256, stride) >= 2;
+    const int N = d_out <= 64 ? 64 : (wide ? 256 : 128);
+    return pipe_stages(N, stride) < 2 ? 0 : N;
+}
+
 template <int N, int FMT>
 cudaError_t launch_wide_inst(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
                              const float* beta, const float* alpha, void* zeta, int64_t ldz)
 {
     const int64_t tiles = ceil_div(n, kTcRows), gy = ceil_div(d_out, N);
     const size_t panel = (size_t)N * stride * 32, a_bytes = (size_t)kTcRows * 256;
-    const bool resident = a_bytes + panel <= 110 * 1024 || (a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count());
+    const bool resident = a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count();
     const size_t smem = a_bytes + (resident ? panel : (size_t)N * 256);
     cudaError_t e = cudaFuncSetAttribute(bitgemm_wide_kernel<N, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -603,7 +866,8 @@ cudaError_t launch_bitgemm_tc(cudaStream_t s, const uint32_t* A, int64_t stride_
 // Measured, a layer with the aggregation of an empty graph, bit counts / tensor cores: 3,703 -> 64: 4,000 rows (32 blocks) 24 /
 // 36 us, 8,000 (63) 32 / 38, 12,000 (94) 42 / 38; 300 -> 64: 8,192 (64) 13 / 15, 12,000 (94) 15 / 15, 16,384 (128) 17 / 15;
 // 300 -> 256: 4,096 (64) 25 / 25, 8,192 (128) 29 / 27; 1,433 -> 256: 2,000 (32) 27 / 29, 3,000 (48) 33 / 29, 6,000 (94) 43 / 31;
-// 16,000 -> 128: 6,000 (47) 198 / 126; 602 -> 16: 40,000 (313) 33 / 35, 200,000 (1,563) 74 / 68; 89,250 rows 500 -> 256 157 / 93.
+// 16,000 -> 128: 6,000 (47) 198 / 126; 602 -> 16: 40,000 (313) 33 / 35, 200,000 (1,563) 74 / 68; 89,250 rows 500 -> 256 157 / 93
+// (with bitgemm_wide_kernel; the pipeline is level with it near the line and faster far from it).
 bool bitgemm_takes_wide(int fmt, int64_t n, int d_in, int d_out)
 {
     const int64_t blocks = ceil_div(n, kTcRows) * ceil_div(d_out, d_out <= 64 ? 64 : 128);
@@ -614,9 +878,14 @@ bool bitgemm_takes_wide(int fmt, int64_t n, int d_in, int d_out)
 cudaError_t launch_bitgemm_wide(cudaStream_t s, const uint32_t* A, const uint32_t* BT, int64_t stride, int64_t n, int d_in, int d_out,
                                 const float* beta, const float* alpha, int fmt, void* zeta, int64_t ldz)
 {
-#define BIGCN_WIDE_CALL(FMT) \
-    return d_out <= 64 ? launch_wide_inst<64, FMT>(s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz) \
-                       : launch_wide_inst<128, FMT>(s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz)
+    const int N = pipe_width(n, d_out, stride);
+#define BIGCN_WIDE_ARGS (s, A, BT, stride, n, d_in, d_out, beta, alpha, zeta, ldz)
+#define BIGCN_WIDE_CALL(FMT)                                           \
+    return N == 64    ? launch_pipe_inst<64, FMT> BIGCN_WIDE_ARGS      \
+           : N == 128 ? launch_pipe_inst<128, FMT> BIGCN_WIDE_ARGS     \
+           : N == 256 ? launch_pipe_inst<256, FMT> BIGCN_WIDE_ARGS     \
+           : d_out <= 64 ? launch_wide_inst<64, FMT> BIGCN_WIDE_ARGS   \
+                         : launch_wide_inst<128, FMT> BIGCN_WIDE_ARGS
     switch (fmt) {
         case kZetaF32: BIGCN_WIDE_CALL(kZetaF32);
         case kZetaF16: BIGCN_WIDE_CALL(kZetaF16);
@@ -624,6 +893,7 @@ cudaError_t launch_bitgemm_wide(cudaStream_t s, const uint32_t* A, const uint32_
         default: return cudaErrorInvalidValue;
     }
 #undef BIGCN_WIDE_CALL
+#undef BIGCN_WIDE_ARGS
 }
 
 // Number of waits that ran out since the library was loaded on the current device (0 = none).
