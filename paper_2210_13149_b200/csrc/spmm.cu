@@ -225,16 +225,16 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                 sh[4 * q] = a.x, sh[4 * q + 1] = a.y, sh[4 * q + 2] = a.z, sh[4 * q + 3] = a.w;
                 sc[4 * q] = b.x, sc[4 * q + 1] = b.y, sc[4 * q + 2] = b.z, sc[4 * q + 3] = b.w;
             }
+            const int n_valid = min(max(p.d_out - col0, 0), EPV);            // padding columns pack as 0 and do not count
             uint32_t bits = 0u;
             float l1c = 0.f;
 #pragma unroll
             for (int i = 0; i < EPV; ++i) {
-                const float xh = __fmul_rn(__fsub_rn(x[i], sh[i]), sc[i]);   // padding columns: (0 - 0) * 1
+                const float xh = __fmul_rn(__fsub_rn(x[i], sh[i]), sc[i]);
                 if (xh >= 0.f) bits |= 1u << i;
-                l1c += fabsf(xh);
+                if (i < n_valid) l1c += fabsf(xh);                           // (a factor of infinity times a padding 0 is a NaN)
             }
             if (vec < p.nv_fin) l1 += l1c;            // lanes past the last vector accumulated nothing meaningful
-            const int n_valid = min(max(p.d_out - col0, 0), EPV);            // padding columns pack as 0
             bits &= (n_valid >= 32) ? 0xffffffffu : ((1u << n_valid) - 1u);
             uint32_t word = bits << ((col0) & 31);
 #pragma unroll
