@@ -1284,7 +1284,8 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
         uint4 v[NV];
 #pragma unroll
         for (int q = 0; q < NV; ++q) v[q] = vn[q];
-        const float wt = c1 >= 0 ? w1 * nwn : 0.f;            // lanes past the row's end add nothing
+        // lanes past the row's end add nothing; half-dot bytes: the factor's sign is the source's first feature sign, not the weight's
+        float wt = c1 >= 0 ? w1 * nwn : 0.f, wa = kHalf ? (c1 >= 0 ? w1 * fabsf(nwn) : 0.f) : wt;
         c1 = c2;
         w1 = w2;
         gather(c1);                                           // the next pass's operand rows
@@ -1295,7 +1296,24 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
 #pragma unroll
             for (int q = 0; q < NV; ++q) own[q] = 16 * q + (lane >> 1) < p.d_out ? __ldg(src + 16 * q) : 0.f;
         }
-        const float wa = kHalf ? fabsf(wt) : wt;              // half-dot bytes: the sign carries the source's first feature sign
+        if constexpr (kHalf && kAdd) {
+            // a weight that is not finite meets whole dots: in the three sums of half-dots, infinities of either sign would meet
+            const bool whole = !(fabsf(wt) <= 3.402823466e38f);
+            if (__any_sync(0xffffffffu, whole) && whole) {
+                const bool neg = signbit(wt) != signbit(wa);
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float b = 16 * q + i < p.d_out ? __ldg(p.col_b0 + 16 * q + i) : 0.f;
+                        const int s = (int)(u[i >> 2] << (24 - 8 * (i & 3))) >> 24;
+                        acc[q][i] = fmaf(wa, (float)(2 * s + 1) + (neg ? -b : b), acc[q][i]);
+                    }
+                }
+                wt = wa = 0.f;
+            }
+        }
         if (kHalf) { ws += wa; wg += wt; }
 #pragma unroll
         for (int q = 0; q < NV; ++q) fma_bytes16(wa, v[q], acc[q]);
@@ -1499,7 +1517,7 @@ spmm_lane_kernel(const SpmmDev p, int rows_per_warp)
         const int64_t ls = __ldg(p.rowptr + lrow), le = __ldg(p.rowptr + lrow + 1);
         const int64_t slice = round_up(ceil_div(le - ls, kLaneWarps), 32);
         const int64_t s0 = min(le, ls + warp * slice), s1 = min(le, s0 + slice);
-        stream_rows_lane<NV, kHalf, true, kTail>(p, red, lane, s0, (int)(s1 - s0), 0, 0, (s1 > s0) ? 1 : 0, 0, al, b0, t, ws, wg, al2, b02);
+        stream_rows_lane<NV, kHalf, true, kTail, false, kAdd>(p, red, lane, s0, (int)(s1 - s0), 0, 0, (s1 > s0) ? 1 : 0, 0, al, b0, t, ws, wg, al2, b02);
         if (lane < NG4) *reinterpret_cast<float4*>(part + warp * kPartPitch + 4 * cg) = t;
         if (lane == 0) {
             part[warp * kPartPitch + NG4 * 4] = ws;
