@@ -14,7 +14,10 @@
 // Half-dot bytes (kHalf): zeta holds s = (dot' - 1) / 2 and the node factor carries the first feature sign f; sum w dot = 2 sum w s +
 // sum w + b0_j sum w f.  The two sums over the weights are two columns of one more A operand, all ones and the signs.
 //
-// Rows whose weights have no fixed point (not finite, or outside 2^-87 .. 2^104) are summed as they are written, in fp32.
+// Weights that have no fixed point (a piece's largest not finite, or outside 2^-87 .. 2^104) meet their dots one by one in fp32, from the
+// byte rows in shared memory, while their digits are 0: the other pieces of a row are summed like any, so that such a weight beside a
+// hub row costs what its 128 entries do.  (Summed from memory by the warp that ends it, a row of 100,000 entries with one NaN took
+// 49 ms, with all of the row's 0.23 now.)
 #include <algorithm>
 #include <type_traits>
 
@@ -40,13 +43,13 @@ struct Slot {                                       // of a warp
     uint8_t rows[kRing][kWindowBytes];              // byte rows of the windows of the group at hand and of the next; 16-byte pieces of entry e exchanged by (e / 2) % 4
     uint2 q[2][32][2];                              // [window / 2][entry][window % 2]: digits of the entry's weight under the group's two rows (0 under the other)
     uint8_t sign[kGroup];                           // first feature signs, +-1
-    float sums[16 * MT];                            // an open row's sums
+    float sums[2][16 * MT];                         // an open row's sums; of a direct group, what its rows sum in fp32
 };
 
 struct BytesDev {
     SpmmDev p;
     GraphPlan plan;
-    float* parts;                                   // [chunks][2][16 MT + 4]: pieces of rows cut by a unit's end, and whether one has no fixed point
+    float* parts;                                   // [chunks][2][16 MT]: pieces of rows cut by a unit's end
     unsigned* counters;                             // [chunks] pieces done; zeroed before
 };
 
@@ -55,29 +58,6 @@ __device__ __forceinline__ void imma(int (&c)[4], uint32_t a0, uint32_t a1, uint
     asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};\n"
         : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// sum_e w_e dot_ej of one row in fp32, as written, into out[column]
-template <bool kHalf>
-__device__ __forceinline__ void literal_sums(const SpmmDev& p, int row, int cols, int lane, float* out)
-{
-    const int64_t e0 = __ldg(p.rowptr + row), e1 = __ldg(p.rowptr + row + 1);
-#pragma unroll 1
-    for (int j = lane; j < cols; j += 32) {
-        float s = 0.f;
-        if (j < p.d_out) {
-            const float b0 = kHalf ? __ldg(p.col_b0 + j) : 0.f;
-#pragma unroll 1
-            for (int64_t e = e0; e < e1; ++e) {
-                const int c = __ldg(p.colidx + e);
-                const float f = __ldg(p.node_w + c);
-                const float b = (float)reinterpret_cast<const signed char*>(p.zeta)[(int64_t)c * p.nv * 16 + j];
-                const float dot = kHalf ? 2.f * b + 1.f + (signbit(f) ? -b0 : b0) : b;
-                s = fmaf(__ldg(p.val + e) * (kHalf ? fabsf(f) : f), dot, s);
-            }
-        }
-        out[j] = s;
-    }
 }
 
 // kTail: a byte row is 64 bytes and carries its node factor in the last four.  kAdd: rows of p.add are added.
@@ -180,7 +160,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
         if (t < 2) {
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
-                float* f = slot->sums + 16 * m + my_col;
+                float* f = slot->sums[0] + 16 * m + my_col;
                 *f = row_open ? *f + x[m] : x[m];
             }
         }
@@ -230,7 +210,23 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
     auto no_fixed_point = [](uint32_t most) { return most != 0u && ((most >> 23) < kExpLow || (most >> 23) > kExpHigh); };
     auto exponent = [](uint32_t most) { return min(max(most >> 23, kExpLow), kExpHigh + 1u); };
 
-    bool literal = false;                           // the open row is to be summed as it is written
+    // adds sum_e w_e dot_ej over entries [from, to) of the group whose windows lie at `at`, in fp32, to (or, fresh, as) sums[h].
+    // slot->q holds the weights, slot->sign the signs
+    auto sum_written = [&](int at, int from, int to, int h, bool fresh) {
+#pragma unroll 1
+        for (int j = lane; j < 16 * MT; j += 32) {
+            float s = 0.f;
+#pragma unroll 4
+            for (int e = from; e < to; ++e) {
+                const int i = e >> 5, r = e & 31;
+                const float b = (float)(signed char)slot->rows[ring(at + i)][r * kRowBytes + (((j >> 4) ^ ((r >> 1) & 3)) << 4) + (j & 15)];
+                float dot = b;
+                if constexpr (kHalf) dot = 2.f * b + 1.f + ((slot->sign[e] & 0x80) ? -tab[j].y : tab[j].y);
+                s = fmaf(__uint_as_float(slot->q[i >> 1][r][i & 1].x), dot, s);
+            }
+            slot->sums[h][j] = fresh ? s : slot->sums[h][j] + s;
+        }
+    };
     bool have_a = false, have_b = false, have_c = c_group.next(d.plan);
     if (have_c) c_group.load(p.colidx, p.val, lane);
     for (;;) {
@@ -281,12 +277,12 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
             }
             m0 = __reduce_max_sync(0xffffffffu, m0);
             m1 = flags & kPair ? __reduce_max_sync(0xffffffffu, m1) : 0u;
-            uint32_t x0 = exponent(m0);
+            const bool written0 = no_fixed_point(m0), written1 = no_fixed_point(m1);
+            uint32_t x0 = written0 ? kExpLow : exponent(m0);
             const uint32_t x1 = exponent(m1);
-            const bool literal1 = no_fixed_point(m1);
             if (flags & (kDirect | kFirst)) {
                 clear();
-                literal = row_open = false;
+                row_open = false;
                 if (!(flags & (kDirect | kLast))) x0 += 3;
                 chain_x = x0;
                 chain = cnt;
@@ -299,7 +295,23 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
                 chain_x = x0;
                 chain = cnt;
             }
-            literal = literal || no_fixed_point(m0);
+            if (written0 || written1) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    slot->q[i >> 1][lane][i & 1].x = __float_as_uint(w[i]);
+                    if constexpr (kHalf) slot->sign[32 * i + lane] = signbit(fac[i]) ? 0xffu : 1u;
+                }
+                __syncwarp();
+                if (written0) {
+                    sum_written(at_a, 0, mid, 0, !row_open);
+                    row_open = !(flags & kDirect);
+                }
+                if (written1) sum_written(at_a, mid, cnt, 1, true);
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (32 * i + lane < mid ? written0 : written1) w[i] = 0.f;
+            }
             const float f0 = __uint_as_float((283u - x0) << 23), f1 = __uint_as_float((283u - x1) << 23);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -338,22 +350,25 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
             asm volatile("cp.async.commit_group;\n" ::: "memory");
             if (flags & (kDirect | kLast)) {
                 float x[MT];
-                bool literal0 = literal, done = true;
+                bool done = true;
                 if (flags & kDirect) {
                     read_back(__uint_as_float(((t < 2 ? x0 : x1) - 29u) << 23), x);
+                    if (t < 2 ? written0 : written1) {
+#pragma unroll
+                        for (int m = 0; m < MT; ++m) x[m] = slot->sums[t >> 1][16 * m + my_col];
+                    }
                 } else {
                     move();
                     done = flags & kWhole;
                     __syncwarp();
                     if (!done) {
                         // the row reaches over several units: leave this one's sums; whoever comes last adds them up in order
-                        constexpr int kPart = 16 * MT + 4;
+                        constexpr int kPart = 16 * MT;
                         const int u0 = ((int)__ldg(p.rowptr + row) + kRowCost * row) >> d.plan.chunk_log2;
                         const int u1 = ((int)__ldg(p.rowptr + row + 1) + kRowCost * (row + 1) - 1) >> d.plan.chunk_log2;
                         float* part = d.parts + ((int64_t)place * 2 + ((flags & kStarts) ? 1 : 0)) * kPart;
 #pragma unroll 1
-                        for (int i = lane; i < 16 * MT; i += 32) part[i] = slot->sums[i];
-                        if (lane == 0) part[16 * MT] = literal ? 1.f : 0.f;
+                        for (int i = lane; i < kPart; i += 32) part[i] = slot->sums[0][i];
                         __threadfence();
                         __syncwarp();
                         unsigned before = 0;
@@ -361,34 +376,17 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
                         done = __shfl_sync(0xffffffffu, before, 0) == (unsigned)(u1 - u0);
                         if (done) {
                             __threadfence();
-                            float any = 0.f;
 #pragma unroll 1
-                            for (int i = lane; i < 16 * MT + 32; i += 32) {
-                                const int j = min(i, 16 * MT);
-                                float s = __ldcg(d.parts + ((int64_t)u0 * 2 + 1) * kPart + j);
-                                for (int u = u0 + 1; u <= u1; ++u) s += __ldcg(d.parts + (int64_t)u * 2 * kPart + j);
-                                if (j < 16 * MT) slot->sums[j] = s;
-                                else any = s;
+                            for (int i = lane; i < kPart; i += 32) {
+                                float s = __ldcg(d.parts + ((int64_t)u0 * 2 + 1) * kPart + i);
+                                for (int u = u0 + 1; u <= u1; ++u) s += __ldcg(d.parts + (int64_t)u * 2 * kPart + i);
+                                slot->sums[0][i] = s;
                             }
-                            literal0 = any != 0.f;
                             __syncwarp();
                         }
                     }
 #pragma unroll
-                    for (int m = 0; m < MT; ++m) x[m] = slot->sums[16 * m + my_col];
-                }
-                if (done && (literal0 || literal1)) {
-#pragma unroll 1
-                    for (int h = 0; h < 2; ++h) {
-                        if (!(h ? literal1 : literal0)) continue;
-                        __syncwarp();
-                        literal_sums<kHalf>(p, row + h, 16 * MT, lane, slot->sums);
-                        __syncwarp();
-                        if ((t >> 1) == h) {
-#pragma unroll
-                            for (int m = 0; m < MT; ++m) x[m] = slot->sums[16 * m + my_col];
-                        }
-                    }
+                    for (int m = 0; m < MT; ++m) x[m] = slot->sums[0][16 * m + my_col];
                 }
                 if (done) finish(x, own, row, flags & kPair);
             }
@@ -403,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) agg_bytes_kernel(const __gr
 }
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
-size_t parts_bytes(int chunks) { return up256((size_t)chunks * 2 * (64 + 4) * 4); }
+size_t parts_bytes(int chunks) { return up256((size_t)chunks * 2 * 64 * 4); }
 
 template <int MT, bool kHalf, bool kTail, bool kAdd>
 cudaError_t launch_inst(cudaStream_t s, const BytesDev& d)
