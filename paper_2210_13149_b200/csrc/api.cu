@@ -317,11 +317,11 @@ size_t contraction_first_bytes(int64_t n, int64_t nnz, const int32_t* dims, int 
 // order's rows for a wide input and few outputs, so they are counted only for layers that may run so by default (one by
 // itself may be called as a hidden layer) or that ask for little, where the option can be tried; `every`: for all that can.
 constexpr size_t kLittle = size_t(64) << 20;
-size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers, bool every)
+size_t layer_scratch_bytes(int64_t n, int64_t nnz, const int32_t* dims, int n_layers, bool every, bool grouped)
 {
-    size_t m = contraction_first_bytes(n, nnz, dims, n_layers, true), plan = 0;
+    size_t m = contraction_first_bytes(n, nnz, dims, n_layers, grouped), plan = 0;
     for (int l = 0; l < n_layers; ++l) {
-        if (spmm_bytes_pays(n, nnz, dims[l], dims[l + 1])) plan = spmm_bits_plan_bytes(n, nnz);
+        if (grouped && spmm_bytes_pays(n, nnz, dims[l], dims[l + 1])) plan = spmm_bits_plan_bytes(n, nnz);
         if (n <= 0 || nnz < 0 || !spmm_bits_covers(n, nnz, dims[l], dims[l + 1], false)) continue;
         const size_t bytes = spmm_bits_scratch_bytes(n, nnz, dims[l]);
         const bool hidden = l < n_layers - 1 || n_layers == 1;
@@ -361,10 +361,15 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
     const size_t zbytes = up(zeta_bytes_max(n, dims, n_layers));
     size_t others = 0;                                       // what else the step keeps
     for (int i = 0; i < 2; ++i) others += up((size_t)n * stride_max * 4) + up((size_t)n * 4);
-    const size_t first = contraction_first_bytes(n, graph->nnz, dims, n_layers, true), least = contraction_first_bytes(n, graph->nnz, dims, n_layers, false);
-    size_t room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, ctx->order == 2);
-    if (up(ws.off) + room + others > ws.size) room = layer_scratch_bytes(n, graph->nnz, dims, n_layers, false);
-    if (up(ws.off) + room + others > ws.size) room = least;  // a workspace without room for P
+    const size_t least = contraction_first_bytes(n, graph->nnz, dims, n_layers, false);
+    // a workspace without room for what grouped byte rows sum in parts does without that before it does without P
+    size_t room = least;
+    for (int i = 0; i < 4; ++i) {
+        const size_t wanted = layer_scratch_bytes(n, graph->nnz, dims, n_layers, /*every=*/ctx->order == 2 && i < 2, /*grouped=*/i % 2 == 0);
+        if (up(ws.off) + wanted + others > ws.size) continue;
+        room = wanted;
+        break;
+    }
     void* zeta = ws.take(room);
     uint32_t* bits[2];
     float* beta[2];
@@ -386,9 +391,9 @@ bigcn_status forward_impl(bigcn_ctx* ctx, const bigcn_graph* graph, const bigcn_
         cur_bits = bits[0];
         cur_beta = beta[0];
     }
-    // The layers share the graph's plan, made by the first that needs it, where the scratch of the contraction-first ones ends
-    // before it; otherwise each makes its own.
-    const bool shared = room >= first + spmm_bits_plan_bytes(n, graph->nnz);
+    // The layers share the graph's plan, made by the first that needs it, where the rows of the contraction-first ones end before it (the
+    // parts of grouped ones always do); otherwise each makes its own.
+    const bool shared = room >= least + spmm_bits_plan_bytes(n, graph->nnz);
     bool planned = false, aggregated_first[BIGCN_MAX_LAYERS] = {};
     if (stats) BIGCN_CUDA(ctx, cudaEventRecord(ev[1], ctx->stream));
     for (int l = 0; l < n_layers; ++l) {
@@ -562,7 +567,7 @@ size_t bigcn_workspace_bytes(int64_t n, int64_t nnz, const int32_t* dims, int32_
         if (l < n_layers && bigcn_packed_stride_words(dims[l]) > stride_max) stride_max = bigcn_packed_stride_words(dims[l]);
         if (dims[l] > d_max) d_max = dims[l];
     }
-    size_t total = layer_scratch_bytes(n, nnz, dims, n_layers, false);
+    size_t total = layer_scratch_bytes(n, nnz, dims, n_layers, false, true);
     total += 2 * (up((size_t)n * stride_max * 4) + up((size_t)n * 4));
     size_t aux = up(normalize_scratch_bytes(n));
     if (up(col_stats_scratch_bytes(d_max)) > aux) aux = up(col_stats_scratch_bytes(d_max));
