@@ -154,11 +154,13 @@ __device__ __forceinline__ void fill_col_table(const SpmmDev& p, float* ctab)
 // kHalf (half-dot bytes): the accumulators hold sum_k w_k s_kj with s = (dot' - 1) / 2; the row's sum of the
 // edge weights `wsum` and their sum signed by the sources' first feature sign `wsgn` give back
 // sum_k w_k dot_kj = 2 acc_j + wsum + b0_j wsgn before the column factor is applied.
-template <typename T, int NCH, int LPR, bool kHalf = false, int S = 32>
+// kStream: a launch of a stream, not of the short-row kernel.
+template <typename T, int NCH, int LPR, bool kHalf = false, int S = 32, bool kStream = true>
 __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, int64_t row, int lane,
                                            float (&acc)[NCH][Elt<T>::kPerVec], float wsum = 0.f, float wsgn = 0.f, bool on = true)
 {
     constexpr int EPV = Elt<T>::kPerVec;
+    constexpr bool kAgain = kStream && EPV < 16;
     constexpr int LW = 32 / EPV;                  // lanes that share one packed word
     constexpr int kCols = NCH * (LPR < 32 ? LPR : 32) * EPV;
     const int g = (lane % S) / LPR, l = lane % LPR;
@@ -225,16 +227,33 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                 sh[4 * q] = a.x, sh[4 * q + 1] = a.y, sh[4 * q + 2] = a.z, sh[4 * q + 3] = a.w;
                 sc[4 * q] = b.x, sc[4 * q + 1] = b.y, sc[4 * q + 2] = b.z, sc[4 * q + 3] = b.w;
             }
-            const int n_valid = min(max(p.d_out - col0, 0), EPV);            // padding columns pack as 0 and do not count
+            auto columns = [&]() { return min(max(p.d_out - col0, 0), EPV); };
+            const int n_first = kAgain ? 0 : columns();
             uint32_t bits = 0u;
             float l1c = 0.f;
 #pragma unroll
             for (int i = 0; i < EPV; ++i) {
                 const float xh = __fmul_rn(__fsub_rn(x[i], sh[i]), sc[i]);
                 if (xh >= 0.f) bits |= 1u << i;
-                if (i < n_valid) l1c += fabsf(xh);                           // (a factor of infinity times a padding 0 is a NaN)
+                // padding columns do not count (an infinite factor times 0 is a NaN)
+                if (kAgain || i < n_first) l1c += fabsf(xh);
+                x[i] = xh;
+            }
+            // The streams of 16- and 32-bit rows add a vector with padding up again, in a loop: with a condition per column they compile to slower
+            // ones, also where they write H' alone (a million rows of 9, 128 columns: 636 like this, 777 us); byte rows and short rows the
+            // other way round (a million rows of 9, 200 columns, H' and bits: 1,434 and 1,218 us).
+            if (kAgain && col0 + EPV > p.d_out) {
+                l1c = 0.f;
+#pragma unroll 1
+                for (int i = 0; i < p.d_out - col0; ++i) {
+                    float v = x[0];
+#pragma unroll
+                    for (int k = 1; k < EPV; ++k) v = k == i ? x[k] : v;
+                    l1c += fabsf(v);
+                }
             }
             if (vec < p.nv_fin) l1 += l1c;            // lanes past the last vector accumulated nothing meaningful
+            const int n_valid = kAgain ? columns() : n_first;                // padding columns pack as 0
             bits &= (n_valid >= 32) ? 0xffffffffu : ((1u << n_valid) - 1u);
             uint32_t word = bits << ((col0) & 31);
 #pragma unroll
@@ -1764,14 +1783,14 @@ spmm_rows_kernel(const SpmmDev p, int rows_per_take, int wide_from, int dynamic)
                     Set::reduce(acc[0]);
                 }
                 if (__any_sync(0xffffffffu, n_cur >= 0))
-                    finish_row<T, 1, LPR, false, S>(p, ctab, row0 + r0 + lane / S, lane, acc, 0.f, 0.f, n_cur >= 0);
+                    finish_row<T, 1, LPR, false, S, false>(p, ctab, row0 + r0 + lane / S, lane, acc, 0.f, 0.f, n_cur >= 0);
             }
         }
         for (; wide_mask; wide_mask &= wide_mask - 1) {
             const int r = __ffs(wide_mask) - 1;
             const int64_t s = __shfl_sync(0xffffffffu, rp, r);
             whole(s, __shfl_sync(0xffffffffu, rp_next, r) - s);
-            finish_row<T, 1, LPR>(p, ctab, row0 + r, lane, acc);
+            finish_row<T, 1, LPR, false, 32, false>(p, ctab, row0 + r, lane, acc);
         }
         if (!dynamic) take += (int)gridDim.x * kSpmmWarps;
     }
@@ -1796,7 +1815,7 @@ spmm_rows_kernel(const SpmmDev p, int rows_per_take, int wide_from, int dynamic)
                 for (int w = 0; w < kSpmmWarps; ++w) s += part[w][(lane % LPR) * EPV + i];
                 acc[0][i] = s;
             }
-            finish_row<T, 1, LPR>(p, ctab, lrow, lane, acc);
+            finish_row<T, 1, LPR, false, 32, false>(p, ctab, lrow, lane, acc);
         }
         __syncthreads();
     }
