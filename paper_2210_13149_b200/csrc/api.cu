@@ -203,6 +203,18 @@ bool grouped_bytes(const bigcn_ctx* ctx, const bigcn_graph* g, int d_in, int d_o
     return wanted &&
            at + up(spmm_bytes_scratch_bytes(g->n, g->nnz)) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
 }
+// Whether the neighbours' rows of a Bi-GraphSAGE layer of 33..48 outputs are bytes for the lane-per-entry stream (of more outputs it has
+// no registers for an own term), not 16-bit rows for the general stream or, where a next layer follows, for the short-row kernel.
+// Measured, a layer of 256 inputs and 47 outputs, 16-bit rows / bytes, in us.  H': 40,000 nodes in rows of 9 61 / 61, of 15 84 / 68, of
+// 30 130 / 87; 200,000 nodes in rows of 9 159 / 198, of 15 201 / 209, of 20 236 / 221, of 30 305 / 246; a million in rows of 15 749 /
+// 899, of 20 878 / 936 (100 inputs: 847 / 828), of 30 1,151 / 1,020.  Bits: 40,000 in rows of 15 56 / 74, of 30 77 / 83, of 60
+// 124 / 106; 200,000 in rows of 20 214 / 232, of 30 282 / 258; a million in rows of 9 500 / 914, of 30 1,017 / 1,082.
+bool sage_lane_pays(int64_t n, int64_t nnz, int d_out, bool next)
+{
+    if (d_out <= 32 || d_out > 48) return false;
+    if (next) return nnz >= 30 * n && nnz < (int64_t(1) << 24);
+    return nnz >= 20 * n || (nnz >= 8 * n && n <= 65536);
+}
 // The plan of the graph sits at the end of the scratch.
 void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 {
@@ -1133,10 +1145,8 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
-    // 33..48 columns on rows not much shorter than a pass: bytes, for the lane-per-entry stream (2.4 M nodes, 126 M entries, 256 -> 47:
-    // 4.3 ms with fp16 rows on the general stream, 3.0 like this); rows of bytes of more columns have no stream with an own term
     const bool grouped = grouped_bytes(ctx, mean_graph, d_in, d_out, need, ctx->ws_bytes);
-    const bool narrow = grouped || (d_out > 32 && d_out <= 48 && mean_graph->nnz >= 8 * n);
+    const bool narrow = grouped || sage_lane_pays(n, mean_graph->nnz, d_out, next != nullptr);
     const ZetaRows z = zeta_rows(ctx, mean_graph, d_in, d_out, zeta_nbr, /*allow_half=*/narrow, narrow);
     // the own term: integer dots where the aggregation scales them (the same products), fp32 rows otherwise
     const bool own_dots = (z.fmt == kZetaF16 || z.fmt == kZetaI16) && d_in <= 32767;

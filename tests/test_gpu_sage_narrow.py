@@ -1,6 +1,7 @@
-"""Bi-GraphSAGE layers of 33..64 outputs, whose neighbour term is gathered as byte rows by the lane-per-entry stream with the node's own
-term added at a row's end: plain and half-dot bytes, rows with and without the node factor in their tail, three and four vectors, with
-and without a next layer; against the oracle under the tolerance of the other layers."""
+"""Bi-GraphSAGE layers of 33..64 outputs against the oracle under the tolerance of the other layers.  Where sage_lane_pays() says so, the
+neighbours of a layer of 33..48 outputs are byte rows for the lane-per-entry stream, with the node's own term added at a row's end: plain
+bytes up to 127 inputs, half-dot bytes with the node factor in the rows' tail from 2^20 outputs on; elsewhere, and for 49..64 outputs,
+16-bit rows."""
 import numpy as np
 import pytest
 
@@ -34,3 +35,22 @@ def test_narrow_sage_logits(ctx, n, e, d_in, d_out):  # noqa: F811
     out = ctx.sage_layer_forward(G, B.make_layer(d_in, d_out, bits_to_dev(t.bitsT_self), dev(t.alpha_self)),
                                  B.make_layer(d_in, d_out, bits_to_dev(t.bitsT_nbr), dev(t.alpha_nbr)), bits_to_dev(t.bits), dev(t.beta))
     assert_close(out["h"], t.H_out, "logits")
+
+
+# byte rows: plain ones on a dense graph, half-dot ones; their hub rows are split over a block
+BYTE_ROWS = [(3000, 900000, 100, 47), (3000, 900000, 127, 33), (24000, 800000, 256, 47), (24000, 800000, 255, 48), (32700, 1000000, 128, 33)]
+
+
+@pytest.mark.parametrize("n,e,d_in,d_out", BYTE_ROWS)
+def test_narrow_sage_logits_of_split_rows(ctx, n, e, d_in, d_out):  # noqa: F811
+    rows = np.diff(synth.power_law_graph(n, e, 300 + n)[0].numpy())
+    mean = rows.sum() // n
+    assert mean >= 20 and (d_in <= 127 or n * d_out >= 1 << 20)                # byte rows
+    assert n <= 32768 and rows.max() > max(128, 4 * (mean + 1), rows.sum() // 3552)   # the default length from which H' splits a row
+    test_narrow_sage_logits(ctx, n, e, d_in, d_out)
+
+
+@pytest.mark.parametrize("n,e,d_in,d_out", BYTE_ROWS)
+def test_narrow_sage_layers_of_split_rows(ctx, n, e, d_in, d_out):  # noqa: F811
+    assert synth.power_law_graph(n, e, 200 + n)[1].numel() >= 30 * n           # byte rows where a next layer follows, too
+    check_sage_layer(ctx, 0, n, e, d_in, d_out)
