@@ -869,7 +869,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                         if ((lane >> 2) == rb) l1_row = s;
                     }
                 };
-                // the next four's sums are on their way under the arithmetic of these (100 -> 256, 2.4 M rows: 681 -> 629 us; with 256
+                // the next four's sums are on their way under the arithmetic of these, by loads without a condition: between a load and its
+                // wait the registers must not pass a merge of control flow, where they may be copied (100 -> 256, 2.4 M rows: 681 -> 629 us; with 256
                 // inputs the copies of P bound the kernel: 827 / 836, more of them in flight 852)
                 uint32_t v[2][16];
                 tc::tmem_ld16_nowait(t_addr, v[0]);
@@ -879,7 +880,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) bits_gemm_kernel(const SpmmDe
                     tc::tmem_ld16_nowait(t_addr + (uint32_t)(rb * 16 + 16), v[1]);
                     four(rb, v[0]);
                     tc::tmem_wait16(v[1]);
-                    if (rb + 2 < kTileRows / 4) tc::tmem_ld16_nowait(t_addr + (uint32_t)(rb * 16 + 32), v[0]);
+                    tc::tmem_ld16_nowait(t_addr + (uint32_t)(min(rb + 2, kTileRows / 4 - 2) * 16), v[0]);   // (the last one again)
                     four(rb + 1, v[1]);
                     tc::tmem_wait16(v[0]);
                 }
