@@ -172,8 +172,12 @@ constexpr int kStatChunksMax = 1024;
 
 // Block (x, y) sums chunk y of the rows over columns 32 x .. 32 x + 31.  The block of a column group that ends last (counted in
 // done[x], which is zero before and after) adds the chunks up, thread (tx, ty) chunks ty, ty + 8, ..., then the eight sums in
-// order.  One wave of blocks: with chunks of 64 rows and a second kernel for the sums, 19,717 x 500 took 28 us.
-__global__ void __launch_bounds__(256)
+// order.  One wave of blocks, as many as a multiprocessor's registers hold; for 8 they would keep fewer loads in flight.  Measured,
+// chunks of 64 rows and a second kernel for the sums / 8 blocks' worth of chunks on 6 / 8 blocks resident / 6 and 6 chunks, in us:
+// 19,717 x 500 28.7 / 19.6 / 18.9 / 16.9, 250,000 x 256 118 / 68 / 75 / 61, 250,000 x 64 40 / 34 / 36 / 27, 2.4 M x 100 489 / 247 /
+// 286 / 193 (5.1 TB/s).
+constexpr int kStatBlocks = 6;
+__global__ void __launch_bounds__(256, kStatBlocks)
 col_stats_kernel(const float* __restrict__ H, int64_t n, int d, int64_t ld, int64_t rows_per_chunk, double eps,
                  double* __restrict__ partial /* [chunks][d][2] */, unsigned* __restrict__ done, float* __restrict__ shift, float* __restrict__ scale)
 {
@@ -275,8 +279,8 @@ cudaError_t launch_col_stats(cudaStream_t s, const float* H, int64_t n, int d, i
                              float* shift, float* scale, void* scratch, unsigned* done, int* launches)
 {
     const int64_t groups = ceil_div(d, 32);
-    // one wave of blocks (eight to a multiprocessor), of at least 64 rows each
-    const int64_t wanted = groups > kStatGroups ? 1 : std::min<int64_t>(kStatChunksMax, std::max<int64_t>(1, 8 * sm_count() / groups));
+    // one wave of blocks, of at least 64 rows each
+    const int64_t wanted = groups > kStatGroups ? 1 : std::min<int64_t>(kStatChunksMax, std::max<int64_t>(1, kStatBlocks * sm_count() / groups));
     const int64_t rows_per_chunk = std::max<int64_t>(64, ceil_div(n, wanted));
     const int chunks = (int)std::max<int64_t>(1, ceil_div(n, rows_per_chunk));
     launch_kernel(col_stats_kernel, dim3((unsigned)groups, (unsigned)chunks), 256, 0, s, H, n, d, ld, rows_per_chunk, (double)eps,

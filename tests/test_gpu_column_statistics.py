@@ -7,7 +7,7 @@ from parity_util import dev
 pytestmark = pytest.mark.gpu
 
 
-# one block and several per column group; rows on either side of a chunk of 64; one column, ragged and many groups (above 592 one chunk each)
+# one block and several per column group; rows on either side of a chunk of 64; one column, ragged and many groups (above 444 one chunk each)
 @pytest.mark.parametrize("n,d", [(1, 1), (64, 33), (65, 33), (129, 600), (20000, 500), (70000, 7), (130, 20000)])
 def test_column_statistics(n, d):
     from paper_2210_13149_b200 import binding as B
