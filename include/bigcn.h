@@ -11,8 +11,8 @@
  * General rules
  *   - Every data pointer is a DEVICE pointer owned by the caller unless a comment says "host".
  *     The library allocates no data buffers: scratch comes from the workspace the caller attaches
- *     with bigcn_set_workspace().  A context owns only a few hundred bytes of device status words
- *     and some CUDA events.
+ *     with bigcn_set_workspace().  A context owns only 17 KB of device memory (status words and
+ *     the counters of bigcn_col_stats()) and some CUDA events.
  *   - All work is enqueued on the stream given to bigcn_create() (borrowed, not owned).  Calls are
  *     asynchronous unless stated; results are ready once that stream has been synchronised.
  *   - Matrices are row-major; leading dimensions ("ld") are in elements, packed strides in 32-bit
@@ -103,11 +103,13 @@ enum {
      *     bigcn_forward) on a graph whose rows average at least 8 stored entries, 1 otherwise.  Measured on the two
      *     256-column layers of a 2.4 M-node, 126 M-entry graph, bits and beta only: 4.9 / 5.2 ms for 3,
      *     5.7-5.9 / 5.9-6.1 ms for 1, 8.0 / 8.3 ms for 2.
-     * Rows of 33..64 bytes take such products by default, in groups of up to 128 stored entries, on graphs whose rows average 40
-     * entries and that hold 4 million, in a workspace with room for what they sum in parts (bigcn_workspace_bytes() counts it
-     * there), and with 2 wherever the workspace has room; otherwise, and with an option that names a format or another
-     * kernel, fp32 streams.  Edge values of either sign; rows without a fixed point are summed in fp32 as they are written.  All paths meet the same tolerance; their fp32 sums differ
-     *     in rounding, so a re-binarized bit at the threshold may differ between them. */
+     * Rows of 33..64 bytes of layers with up to 256 inputs take such products by default, in groups of up to 128 stored entries, on
+     *     graphs whose rows average 40 entries and that hold 4 million, in a workspace with room for what they sum in parts
+     *     (bigcn_workspace_bytes() counts it there), and with 2 wherever the workspace has room, whatever the format, contraction
+     *     and row length asked for; otherwise, and by default with any of those three options set, fp32 streams.  Edge values of
+     *     either sign; weights without a fixed point are summed in fp32.
+     * All paths meet the same tolerance; their fp32 sums differ in rounding, so a re-binarized bit at the threshold may differ between
+     *     them, and H' of the same call may round differently in a workspace without room for the parts. */
     BIGCN_OPT_BYTE_AGGREGATION = 4,
     /* Order of a layer's two products, H' = A_tilde (diag(beta) F B diag(alpha)).
      * 1 = the contraction F B first, then the aggregation of its rows (the kernels the options above choose among);

@@ -194,8 +194,8 @@ bool bits_first(const bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* l
            spmm_bits_scratch_bytes(g->n, g->nnz, layer->d_in) + spmm_bits_plan_bytes(g->n, g->nnz) <= room;
 }
 // Whether byte rows of 33..64 columns are aggregated as grouped integer products (spmm_bytes.cu), whose scratch lies at `at` of `room`
-// bytes, before the plan: where that pays, or wherever covered by option.  Options that name a storage format or another kernel keep
-// to the streams.
+// bytes, before the plan: where that pays and no option names a storage format, a contraction, another kernel or a length of split
+// rows; with BIGCN_OPT_BYTE_AGGREGATION = 2 wherever covered, whatever the other options.
 bool grouped_bytes(const bigcn_ctx* ctx, const bigcn_graph* g, int d_in, int d_out, size_t at, size_t room)
 {
     const bool wanted = ctx->byte_path == 2 ? spmm_bytes_covers(g->n, g->nnz, d_in, d_out)
@@ -224,8 +224,9 @@ void* plan_at(const bigcn_graph* g, void* scratch, size_t room)
 // One layer on already validated arguments.  `zeta` is `room` bytes of scratch: the contraction's rows in its first zbytes and
 // the aggregation's counter behind them, or (bits first) what spmm_bits_scratch_bytes() counts and the graph's plan, made here
 // unless *planned.  ev_mid is recorded between the layer's two products, aggregated_first tells their order.  any_order: H' may
-// be summed in the order that is the fastest (the logits of a forward); a layer called by itself keeps one order, so that
-// thresholds taken from its H' are met by its own sums.
+// be summed in the order that is the fastest (the logits of a forward); a layer called by itself keeps to the kernels that a call with a
+// next layer has too, so that thresholds taken from its H' are met by its own sums: the streams, or, for byte rows of 33..64 columns on
+// long rows, grouped products where there is room for their parts.
 bigcn_status run_layer(bigcn_ctx* ctx, const bigcn_graph* g, const bigcn_layer* layer,
                        const uint32_t* in_bits, const float* in_beta, void* zeta, size_t zbytes, size_t room, bool* planned /*nullable*/,
                        bool any_order, float* h_out, int64_t ldh, const bigcn_layer* next, uint32_t* next_bits,

@@ -7,9 +7,9 @@
 // beta_e in fixed point against a power of two of the row's largest (|q| <= 2^30), split into four balanced base-256 digits: columns
 // 0..3 for the first row, 4..7 for the second.  The digit sums are exact in 32 bits; a lane pair recombines them at a row's end, and
 // a lane holds the row's columns 16 m + g + 8 odd.  Pieces of a row share a scale (with 3 bits to spare) and the accumulators until one
-// has a larger weight or 480 entries are summed; what there is then moves to an fp32 sum.  A weight is off by at most 2^-31 of the
-// largest of its row, in rows of more than 128 entries 2^-28 of the largest of its piece; the fp32 sums that this replaces rounded
-// every addition to 2^-24.
+// has a larger weight or 480 entries are summed; what there is then moves to an fp32 sum.  A weight is off by at most 2^-30 of the
+// largest of its row, in rows of more than 128 entries 2^-27 of the largest of the piece that set its scale; the fp32 sums that this
+// replaces rounded every addition to 2^-24.
 //
 // Half-dot bytes (kHalf): zeta holds s = (dot' - 1) / 2 and the node factor carries the first feature sign f; sum w dot = 2 sum w s +
 // sum w + b0_j sum w f.  The two sums over the weights are two columns of one more A operand, all ones and the signs.
@@ -17,7 +17,7 @@
 // Weights that have no fixed point (a piece's largest not finite, or outside 2^-87 .. 2^104) meet their dots one by one in fp32, from the
 // byte rows in shared memory, while their digits are 0: the other pieces of a row are summed like any, so that such a weight beside a
 // hub row costs what its 128 entries do.  (Summed from memory by the warp that ends it, a row of 100,000 entries with one NaN took
-// 49 ms, with all of the row's 0.23 now.)
+// 49 ms, with 0.22 for the launch now.)
 #include <algorithm>
 #include <type_traits>
 

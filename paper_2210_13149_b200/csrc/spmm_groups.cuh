@@ -36,7 +36,8 @@ __device__ __forceinline__ void ldmatrix_bytes(uint32_t saddr, uint32_t (&r)[4])
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // The groups of a warp's units of work, one after the other, with the column indices and values of their entries; a group is
-// asked for one ahead.
+// asked for one ahead.  (agg_bits_kernel, at its limit of registers, has a walk of its own: a unit there is one slice of columns of a
+// unit here, and it holds the column indices and values of one group, this struct those of a second beside the caller's.)
 struct Stream {
     int unit, step;                                 // the unit after the one at hand; warps of the grid
     int where;                                      // the unit at hand

@@ -59,7 +59,7 @@ def weighted(rng, lens, n, make):
 
 
 @pytest.mark.parametrize("entries", [1, 31, 64, 65, 128, 129, 480, 481, 2000, 4500])
-@pytest.mark.parametrize("weights", ["both signs, wide", "largest last", "not finite", "tiny"])
+@pytest.mark.parametrize("weights", ["both signs, wide", "largest first", "largest last", "not finite", "tiny"])
 def test_any_weights(ctx, entries, weights):
     """No less precise than the literal fp32 order (BIGCN_OPT_ZETA_FORMAT = 1); weights without a fixed point are summed as written."""
     from paper_2210_13149_b200 import binding as B
@@ -71,8 +71,8 @@ def test_any_weights(ctx, entries, weights):
         w = 0.5 + rng.random(k)
         if weights == "both signs, wide":
             w *= np.exp2(rng.uniform(-12, 0, k)) * rng.choice([-1.0, 1.0], k)
-        elif weights == "largest last" and k:
-            w[-1] = 1e4
+        elif weights in ("largest first", "largest last") and k:
+            w[0 if weights == "largest first" else -1] = 1e4
         elif weights == "not finite" and k:
             w[rng.integers(k)] = rng.choice([np.inf, np.nan, 1e38])
         elif weights == "tiny":
@@ -97,6 +97,39 @@ def test_any_weights(ctx, entries, weights):
     assert not np.isfinite(got[5][~np.isfinite(exact).all(1)]).all(1).any()
     rms = {f: np.sqrt(np.mean(((h[finite] - exact[finite]) / np.maximum(unit[finite], 1e-300)) ** 2)) for f, h in got.items()}
     assert rms[5] <= rms[1] * 1.05 + 2.0 ** -30
+
+
+@pytest.mark.parametrize("entries", [100, 128, 129, 480, 481, 2000])
+@pytest.mark.parametrize("where", ["first", "last"])
+@pytest.mark.parametrize("d_in,d_out,fmt", [(126, 47, 3), (200, 47, 5), (200, 64, 5)])
+def test_columns_in_which_the_largest_weight_meets_a_dot_of_zero(ctx, entries, where, d_in, d_out, fmt):
+    """Single sums against what the digits of weights a thousand times smaller leave of them."""
+    from paper_2210_13149_b200 import binding as B
+    n, rows = 4000, 40
+    rng = np.random.default_rng(entries + d_in)
+    lens = np.where(np.arange(n) < rows, entries, 1)
+    make = lambda k: np.where(np.arange(k) == (0 if where == "first" else k - 1), 1.0, (0.5 + rng.random(k)) * 2.0 ** -10)
+    rowptr, cols, val = weighted(rng, lens, n, make)
+    F, beta = oracle.binarize_rows(rng.standard_normal((n, d_in)).astype(np.float32))
+    signs, alpha = oracle.binarize_cols((rng.standard_normal((d_in, d_out)) * d_in ** -0.5).astype(np.float32))
+    ctx.set_option(B.OPT_ZETA_FORMAT, fmt)
+    G, layer = B.make_graph(dev(rowptr), dev(cols), dev(val)), B.make_layer(d_in, d_out, bits_to_dev(oracle.pack_cols(signs)), dev(alpha))
+    h = ctx.layer_forward(G, layer, bits_to_dev(oracle.pack_rows(F)), dev(beta))["h"].cpu().numpy().astype(np.float64)
+    dots = F.astype(np.float64) @ signs.astype(np.float64)
+    w = (val * beta[cols]).astype(np.float64)                                  # the fp32 product every order starts from
+    seen = 0
+    for r in range(rows):
+        a, b = rowptr[r], rowptr[r + 1]
+        top = cols[a if where == "first" else b - 1]
+        zero = dots[top] == 0
+        terms = w[a:b, None] * dots[cols[a:b]][:, zero]
+        # A weight is off by 2^-30 of its row's largest, 2^-27 of its scale's where a row has several pieces; sums of pieces are fp32 (three
+        # roundings each), and so are the three sums of half-dot bytes, each as large as sum |w|, in which the largest weight cancels.
+        off = 2.0 ** (-30 if entries <= 128 else -27) * w[a:b].max() * np.abs(dots[cols[a:b]][:, zero]).sum(0)
+        fp32 = sum(np.abs(terms[i:i + 128]).sum(0) for i in range(0, b - a, 128)) + (0 if fmt == 3 else 4 * w[a:b].sum())
+        assert np.all(np.abs(h[r, zero] - terms.sum(0) * alpha[zero]) <= alpha[zero] * (off + 2.0 ** -22 * fp32))
+        seen += zero.sum()
+    assert seen > 20
 
 
 @pytest.mark.parametrize("d_in,d_out", [(127, 33), (255, 47), (128, 60), (200, 64)])
