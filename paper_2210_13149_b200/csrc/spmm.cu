@@ -1303,8 +1303,10 @@ __device__ __forceinline__ void stream_rows_lane(const SpmmDev& p, float* red, i
         uint4 v[NV];
 #pragma unroll
         for (int q = 0; q < NV; ++q) v[q] = vn[q];
-        // lanes past the row's end add nothing; half-dot bytes: the factor's sign is the source's first feature sign, not the weight's
-        float wt = c1 >= 0 ? w1 * nwn : 0.f, wa = kHalf ? (c1 >= 0 ? w1 * fabsf(nwn) : 0.f) : wt;
+        // Lanes past the row's end add nothing.  Half-dot bytes: the factor's sign is the source's first feature sign.  With an own term the
+        // weight keeps the edge value's sign; without, where edge values are those of the normalised adjacency, the one instruction per
+        // entry would cost 1.5 % (169,343 rows of 15, 256 -> 40: 129 / 131 us).
+        float wt = c1 >= 0 ? w1 * nwn : 0.f, wa = kHalf ? (kAdd ? copysignf(wt, w1) : fabsf(wt)) : wt;
         c1 = c2;
         w1 = w2;
         gather(c1);                                           // the next pass's operand rows
