@@ -160,7 +160,7 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                                            float (&acc)[NCH][Elt<T>::kPerVec], float wsum = 0.f, float wsgn = 0.f, bool on = true)
 {
     constexpr int EPV = Elt<T>::kPerVec;
-    constexpr bool kAgain = kStream && EPV < 16;
+    constexpr bool kAgain = kStream && EPV < 16, kFirst = !kStream && EPV < 16;
     constexpr int LW = 32 / EPV;                  // lanes that share one packed word
     constexpr int kCols = NCH * (LPR < 32 ? LPR : 32) * EPV;
     const int g = (lane % S) / LPR, l = lane % LPR;
@@ -228,20 +228,20 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                 sc[4 * q] = b.x, sc[4 * q + 1] = b.y, sc[4 * q + 2] = b.z, sc[4 * q + 3] = b.w;
             }
             auto columns = [&]() { return min(max(p.d_out - col0, 0), EPV); };
-            const int n_first = kAgain ? 0 : columns();
+            const int n_first = kFirst ? columns() : 0;
             uint32_t bits = 0u;
             float l1c = 0.f;
 #pragma unroll
             for (int i = 0; i < EPV; ++i) {
                 const float xh = __fmul_rn(__fsub_rn(x[i], sh[i]), sc[i]);
                 if (xh >= 0.f) bits |= 1u << i;
-                // padding columns do not count (an infinite factor times 0 is a NaN)
-                if (kAgain || i < n_first) l1c += fabsf(xh);
+                if (!kFirst || i < n_first) l1c += fabsf(xh);
                 x[i] = xh;
             }
-            // The streams of 16- and 32-bit rows add a vector with padding up again, in a loop: with a condition per column they compile to slower
-            // ones, also where they write H' alone (a million rows of 9, 128 columns: 636 like this, 777 us); byte rows and short rows the
-            // other way round (a million rows of 9, 200 columns, H' and bits: 1,434 and 1,218 us).
+            // Padding columns do not count: an infinite factor times 0 is a NaN.  The streams add a vector with padding up again, in a loop: with a
+            // condition per column they compile to slower ones, also where they write H' alone (a million rows of 9, 128 columns: 636 like
+            // this, 777 us).  Not for byte rows, whose own terms are whole fp32 rows: either form costs their streams up to 18 %, so a
+            // neighbour's infinite factor makes the next scale of a row with padding a NaN there.
             if (kAgain && col0 + EPV > p.d_out) {
                 l1c = 0.f;
 #pragma unroll 1
@@ -253,7 +253,7 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                 }
             }
             if (vec < p.nv_fin) l1 += l1c;            // lanes past the last vector accumulated nothing meaningful
-            const int n_valid = kAgain ? columns() : n_first;                // padding columns pack as 0
+            const int n_valid = kFirst ? n_first : columns();                // padding columns pack as 0
             bits &= (n_valid >= 32) ? 0xffffffffu : ((1u << n_valid) - 1u);
             uint32_t word = bits << ((col0) & 31);
 #pragma unroll
