@@ -575,7 +575,7 @@ def run_ours(args):
         # 129..256 byte columns on a graph whose rows average at least 8 stored entries, unless another path is asked for
         on_tc_agg = (elt == 1 and 128 < dims[l + 1] <= 256 and not last and nnz < (1 << 31)
                      and (args.byte_aggregation == 3 or (args.byte_aggregation == 0 and nnz >= 8 * n)))
-        grouped = args.byte_aggregation == 0 and args.zeta_format == 0 and nnz >= 40 * n and nnz >= (4 << 20)   # narrow byte rows as grouped products
+        grouped = args.byte_aggregation == 0 and args.zeta_format == 0 and nnz >= 40 * n and nnz >= ((5 if dims[l + 1] <= 48 else 4) << 20)   # narrow byte rows as grouped products
         narrow = last and elt == 1 and 32 < dims[l + 1] <= 64 and nnz >= 8 * n
         agg_name = "spmm_tc_kernel" if on_tc_agg else (("agg_bytes_kernel" if grouped else "spmm_lane_kernel") if narrow else "spmm_kernel")
         if bits_first[l]:

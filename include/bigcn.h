@@ -104,7 +104,7 @@ enum {
      *     256-column layers of a 2.4 M-node, 126 M-entry graph, bits and beta only: 4.9 / 5.2 ms for 3,
      *     5.7-5.9 / 5.9-6.1 ms for 1, 8.0 / 8.3 ms for 2.
      * Rows of 33..64 bytes of layers with up to 256 inputs take such products by default, in groups of up to 128 stored entries, on
-     *     graphs whose rows average 40 entries and that hold 4 million, in a workspace with room for what they sum in parts
+     *     graphs whose rows average 40 entries and that hold 5 * 2^20 (4 * 2^20 above 48 columns), in a workspace with room for what they sum in parts
      *     (bigcn_workspace_bytes() counts it there), and with 2 wherever the workspace has room, whatever the format, contraction
      *     and row length asked for; otherwise, and by default with any of those three options set, fp32 streams.  Edge values of
      *     either sign; weights without a fixed point are summed in fp32.

@@ -438,10 +438,12 @@ bool spmm_bytes_covers(int64_t n, int64_t nnz, int d_in, int d_out)
 // layer may have to make for itself, is small beside the launch.  256 inputs, the aggregation alone (and the plan) against the
 // stream: 2.4 M rows of 51, 47 columns 2.19 (0.06) / 2.59 ms, 64 columns 2.38 / 3.25; 800,000 of 30, 40 columns 569 (63) / 642 us;
 // 200,000 of 60, 40 columns 232 (23) / 270, of 30 189 (21) / 196; 30,000 of 200 117 (12) / 154, of 60 65 (12) / 74; 169,343 of
-// 15 140 (19) / 121.
+// 15 140 (19) / 121.  Whole layers, stream / products with the plan, power-law graphs in rows of 42 and 60: 4.3 M entries, 40 columns 137 /
+// 153 and 122 / 140, 64 columns 164 / 169 and 153 / 155; 6 M entries, 40 columns 180 / 178 and 164 / 159, 64 columns 219 / 195 and 188 /
+// 165; so rows of three products, which the stream takes with fewer registers, need 5 Mi entries, and rows of four 4 Mi.
 bool spmm_bytes_pays(int64_t n, int64_t nnz, int d_in, int d_out)
 {
-    return spmm_bytes_covers(n, nnz, d_in, d_out) && nnz >= 40 * n && nnz >= (int64_t(4) << 20);
+    return spmm_bytes_covers(n, nnz, d_in, d_out) && nnz >= 40 * n && nnz >= (int64_t(d_out <= 48 ? 5 : 4) << 20);
 }
 
 size_t spmm_bytes_scratch_bytes(int64_t n, int64_t nnz)

@@ -34,3 +34,12 @@ def test_layers_that_may_aggregate_first_get_room_for_their_sums(workspace, dims
 @pytest.mark.parametrize("n,nnz,dims", [(2500, 6500, [257, 47]), (400, 5400, [602, 200]), (60000, 210000, [33, 256])])
 def test_small_graphs_have_room_for_either_order(workspace, n, nnz, dims):
     assert workspace(n, nnz, dims) >= n * 512 * -(-dims[0] // 128) + n * 16
+
+
+@pytest.mark.parametrize("d_out,least", [(33, 5 << 20), (48, 5 << 20), (49, 4 << 20), (64, 4 << 20)])
+def test_grouped_rows_get_room_for_their_parts_and_the_plan(workspace, d_out, least):
+    """From the first graph that takes them by default on: a record of 16 bytes per group (at least one per 128 entries), two rows of sums
+    per unit of work (at most 2,048 entries)."""
+    n, dims = 100_000, [700, 100, d_out]
+    with_parts, without = workspace(n, least, dims), workspace(n, least - 1, dims)
+    assert with_parts - without >= least // 128 * 16 + least // 2048 * 2 * 48 * 4
