@@ -356,9 +356,9 @@ bitgemm_tc_kernel(const uint32_t* __restrict__ A, int64_t stride_a, const uint32
 }
 
 // The same product for layers of any d_in (more than 256: a tile's expanded rows no longer fit shared memory whole): K in
-// chunks of 256 positions, accumulated in tensor memory.  N = 64 or 128 channels (blockIdx.y: slices of N).  For panels that leave
-// the pipeline below no room: the expanded weight panel stays in shared memory where it fits and there is at most one tile per
-// multiprocessor (`resident`); otherwise a chunk of it is expanded again with every chunk of rows.
+// chunks of 256 positions, accumulated in tensor memory.  N = 64 or 128 channels (blockIdx.y: slices of N).  Where the pipeline
+// below is not the faster one (pipe_width()): the expanded weight panel stays in shared memory where two fit or there is at most one tile
+// per multiprocessor (`resident`); otherwise a chunk of it is expanded again with every chunk of rows.
 template <int N, int FMT>
 __global__ void __launch_bounds__(kTcThreads, 2)
 bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__ BT, int64_t stride,
@@ -528,7 +528,7 @@ bitgemm_wide_kernel(const uint32_t* __restrict__ A, const uint32_t* __restrict__
 // N = 256 halves the expansions: up to 512 inputs its panel leaves room for two operand tiles.
 // Measured, the kernel above / this one: 89,250 rows 500 -> 256 35 / 21 us, 60,000 rows 602 -> 256 38 / 25, 200,000 rows
 // 1,000 -> 100 68 / 52 and 602 -> 41 35 / 32, 1,000,000 rows 500 -> 64 123 / 101, 10,240 rows 300 -> 128 7.9 / 7.1, 19,717 rows
-// 500 -> 64 8.5 / 8.5 and 22,000 rows 300 -> 64 7.8 / 7.9 (one or two tiles per block: nothing to overlap).  Up to 256 inputs a tile is one chunk, three blocks of bitgemm_tc_kernel overlap as well, and the two are level (169,343 rows
+// 500 -> 64 8.5 / 8.5 and 22,000 rows 300 -> 64 7.8 / 7.9 (one or two tiles per block: nothing to overlap, see pipe_width()).  Up to 256 inputs a tile is one chunk, three blocks of bitgemm_tc_kernel overlap as well, and the two are level (169,343 rows
 // 256 -> 256 30 / 28, 128 -> 256 as floats 36 / 38, 255 -> 100 17 / 18): that kernel stays.
 constexpr int kPipeThreads = 17 * 32;
 constexpr int kPipeStages = 4;                // operand tiles at most; as many as fit
@@ -774,12 +774,25 @@ cudaError_t launch_pipe_inst(cudaStream_t s, const uint32_t* A, const uint32_t* 
     return cudaGetLastError();
 }
 
+// Whether two blocks of bitgemm_wide_kernel with their whole panels fit a multiprocessor.
+bool wide_resident_twice(int N, int64_t stride) { return (size_t)kTcRows * 256 + (size_t)N * stride * 32 <= 110 * 1024; }
+
 // Channels per block of the pipeline, 0 where it does not run.  256 only where slices of 128 are more than a block per
 // multiprocessor: 5,120 rows 500 -> 256 (80 slices) 10.2 us with 256 and 7.6 with 128, 8,000 rows 300 -> 256 (126) 9.0 and 6.8;
 // 12,000 rows 500 -> 256 (188) 10.4 where slices of 128 took 10.8 with the kernel above, 30,000 rows (470) 13 and 17.
+// Between one slice per multiprocessor and two, bitgemm_wide_kernel takes all of them in one wave, two blocks to a multiprocessor, and
+// the pipeline in two rounds.  It is the slower one there where its panel is wide (602 inputs and more: few operand tiles fit beside it),
+// where slices of 64 have little to expand, and where slices of 256 leave most of the second unused.  Kernel above / pipeline, in us:
+// 19,000 rows 1,000 -> 128 13.6 / 15.9, 602 -> 128 10.7 / 11.4, 500 -> 128 10.0 / 9.3; 25,000 rows 1,433 -> 64 16.6 / 17.6, 1,000 -> 64
+// 15.1 / 13.3, 300 -> 41 7.6 / 7.9; 12,000 rows 300 -> 300 9.8 / 11.2, 1,000 -> 256 14.9 / 16.1, 500 -> 256 10.8 / 10.1.
 int pipe_width(int64_t n, int d_out, int64_t stride)
 {
-    const bool wide = d_out > 128 && ceil_div(n, kTcRows) * ceil_div(d_out, 128) > sm_count() && pipe_stages(256, stride) >= 2;
+    const int64_t tiles = ceil_div(n, kTcRows), slices = tiles * ceil_div(d_out, d_out <= 64 ? 64 : 128);
+    if (slices > sm_count() && slices <= 2 * sm_count()) {
+        const bool panel_fits_twice = wide_resident_twice(d_out <= 64 ? 64 : 128, stride);
+        if (d_out <= 64 ? stride <= 16 || !panel_fits_twice : !panel_fits_twice || (d_out > 256 && tiles * ceil_div(d_out, 256) > sm_count())) return 0;
+    }
+    const bool wide = d_out > 128 && slices > sm_count() && pipe_stages(256, stride) >= 2;
     const int N = d_out <= 64 ? 64 : (wide ? 256 : 128);
     return pipe_stages(N, stride) < 2 ? 0 : N;
 }
@@ -790,7 +803,7 @@ cudaError_t launch_wide_inst(cudaStream_t s, const uint32_t* A, const uint32_t* 
 {
     const int64_t tiles = ceil_div(n, kTcRows), gy = ceil_div(d_out, N);
     const size_t panel = (size_t)N * stride * 32, a_bytes = (size_t)kTcRows * 256;
-    const bool resident = a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count();
+    const bool resident = wide_resident_twice(N, stride) || (a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count());
     const size_t smem = a_bytes + (resident ? panel : (size_t)N * 256);
     cudaError_t e = cudaFuncSetAttribute(bitgemm_wide_kernel<N, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
