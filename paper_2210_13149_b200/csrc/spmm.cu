@@ -236,7 +236,7 @@ __device__ __forceinline__ void finish_row(const SpmmDev& p, const float* ctab, 
                 const float xh = __fmul_rn(__fsub_rn(x[i], sh[i]), sc[i]);
                 if (xh >= 0.f) bits |= 1u << i;
                 if (!kFirst || i < n_first) l1c += fabsf(xh);
-                x[i] = xh;
+                if constexpr (kAgain) x[i] = xh;
             }
             // Padding columns do not count: an infinite factor times 0 is a NaN.  The streams add a vector with padding up again, in a loop: with a
             // condition per column they compile to slower ones, also where they write H' alone (a million rows of 9, 128 columns: 636 like
