@@ -1146,7 +1146,10 @@ bigcn_status bigcn_sage_layer_forward(bigcn_ctx* ctx, const bigcn_graph* mean_gr
         if (e != cudaSuccess) return cuda_fail(ctx, e, "layer launch (bits first)");
         return BIGCN_OK;
     }
-    const bool grouped = grouped_bytes(ctx, mean_graph, d_in, d_out, need, ctx->ws_bytes);
+    // (where a next layer follows, rows of four products are held against 16-bit rows on the short-row kernel: 106,000 nodes in rows of 40,
+    // 256 -> 64 172 us with those, 200 grouped; 140,000 in rows of 42 221 and 231, in rows of 60 224 and 206)
+    const bool grouped = (!next || ctx->byte_path == 2 || mean_graph->nnz >= (int64_t(5) << 20)) &&
+                         grouped_bytes(ctx, mean_graph, d_in, d_out, need, ctx->ws_bytes);
     const bool narrow = grouped || sage_lane_pays(n, mean_graph->nnz, d_out, next != nullptr);
     const ZetaRows z = zeta_rows(ctx, mean_graph, d_in, d_out, zeta_nbr, /*allow_half=*/narrow, narrow);
     // the own term: integer dots where the aggregation scales them (the same products), fp32 rows otherwise
