@@ -33,3 +33,10 @@ def test_wide_contraction_equals_the_bit_count_pipe(n, d_in, d_out):
         ctx.sync_check()
         assert torch.equal(got, want)
     ctx.close()
+
+
+# between one slice and two per multiprocessor, and on either side: two blocks with a whole panel, a panel in chunks, three slices of 128
+@pytest.mark.parametrize("n,d_in,d_out", [(18944, 1000, 128), (18945, 1000, 128), (37888, 300, 41), (37889, 300, 41), (25000, 1433, 64),
+                                          (12601, 300, 300), (12545, 1000, 256)])
+def test_one_wave_of_the_wide_contraction(n, d_in, d_out):
+    test_wide_contraction_equals_the_bit_count_pipe(n, d_in, d_out)
