@@ -774,26 +774,22 @@ cudaError_t launch_pipe_inst(cudaStream_t s, const uint32_t* A, const uint32_t* 
     return cudaGetLastError();
 }
 
-// Whether two blocks of bitgemm_wide_kernel with their whole panels fit a multiprocessor.
-bool wide_resident_twice(int N, int64_t stride) { return (size_t)kTcRows * 256 + (size_t)N * stride * 32 <= 110 * 1024; }
-
 // Channels per block of the pipeline, 0 where it does not run.  256 only where slices of 128 are more than a block per
 // multiprocessor: 5,120 rows 500 -> 256 (80 slices) 10.2 us with 256 and 7.6 with 128, 8,000 rows 300 -> 256 (126) 9.0 and 6.8;
 // 12,000 rows 500 -> 256 (188) 10.4 where slices of 128 took 10.8 with the kernel above, 30,000 rows (470) 13 and 17.
 // Between one slice per multiprocessor and two, bitgemm_wide_kernel takes all of them in one wave, two blocks to a multiprocessor, and
-// the pipeline in two rounds.  It is the slower one there where its panel is wide (602 inputs and more: few operand tiles fit beside it),
-// where slices of 64 have little to expand, and where slices of 256 leave most of the second unused.  Kernel above / pipeline, in us:
-// 19,000 rows 1,000 -> 128 13.6 / 15.9, 602 -> 128 10.7 / 11.4, 500 -> 128 10.0 / 9.3; 25,000 rows 1,433 -> 64 16.6 / 17.6, 1,000 -> 64
-// 15.1 / 13.3, 300 -> 41 7.6 / 7.9; 12,000 rows 300 -> 300 9.8 / 11.2, 1,000 -> 256 14.9 / 16.1, 500 -> 256 10.8 / 10.1.
+// the pipeline in two rounds.  It is the slower one there beside panels of 96 KB and more, which leave room for few operand tiles, and where
+// slices of 256 leave most of the second unused.  Two layers of packed input among others, kernel above / pipeline, in us: 19,717 rows
+// 1,000 -> 128 49.9 / 50.9, 602 -> 128 46.6 / 46.3, 500 -> 128 44.6 / 44.5; 25,000 rows 1,433 -> 64 43.2 / 43.6, 602 -> 64 36.7 / 36.7,
+// 300 -> 41 35.2 / 35.1; 12,000 rows 300 -> 300 57.4 / 58.1, 1,000 -> 256 46.8 / 47.7.  (Alone, 19,000 rows 1,000 -> 128 13.6 / 15.9.)
 int pipe_width(int64_t n, int d_out, int64_t stride)
 {
-    const int64_t tiles = ceil_div(n, kTcRows), slices = tiles * ceil_div(d_out, d_out <= 64 ? 64 : 128);
-    if (slices > sm_count() && slices <= 2 * sm_count()) {
-        const bool panel_fits_twice = wide_resident_twice(d_out <= 64 ? 64 : 128, stride);
-        if (d_out <= 64 ? stride <= 16 || !panel_fits_twice : !panel_fits_twice || (d_out > 256 && tiles * ceil_div(d_out, 256) > sm_count())) return 0;
-    }
+    const int narrow = d_out <= 64 ? 64 : 128;
+    const int64_t tiles = ceil_div(n, kTcRows), slices = tiles * ceil_div(d_out, narrow);
+    if (slices > sm_count() && slices <= 2 * sm_count() &&
+        (narrow * stride * 32 >= 96 * 1024 || (d_out > 256 && tiles * ceil_div(d_out, 256) > sm_count()))) return 0;
     const bool wide = d_out > 128 && slices > sm_count() && pipe_stages(256, stride) >= 2;
-    const int N = d_out <= 64 ? 64 : (wide ? 256 : 128);
+    const int N = wide ? 256 : narrow;
     return pipe_stages(N, stride) < 2 ? 0 : N;
 }
 
@@ -803,7 +799,7 @@ cudaError_t launch_wide_inst(cudaStream_t s, const uint32_t* A, const uint32_t* 
 {
     const int64_t tiles = ceil_div(n, kTcRows), gy = ceil_div(d_out, N);
     const size_t panel = (size_t)N * stride * 32, a_bytes = (size_t)kTcRows * 256;
-    const bool resident = wide_resident_twice(N, stride) || (a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count());
+    const bool resident = a_bytes + panel <= 110 * 1024 || (a_bytes + panel <= 200 * 1024 && tiles * gy <= sm_count());
     const size_t smem = a_bytes + (resident ? panel : (size_t)N * 256);
     cudaError_t e = cudaFuncSetAttribute(bitgemm_wide_kernel<N, FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
